@@ -50,9 +50,7 @@ __device__ __forceinline__ void rope_rotate(float a, float b, float c, float s, 
     nb = __fmaf_rn(a, s, __fmul_rn(b, c));
 }
 #endif
-int num_sms();
-// (cos, sin) of every (token, pair m < rot_dim / 2) at pos * base^(-2m / rot_dim), [n_tokens][rot_dim / 2] (rope.cu).
-int launch_rope_table(const float *pos, int64_t n_tokens, int rot_dim, double base, float2 *out, cudaStream_t st);                              // multiprocessors of the current device (api.cu)
+int num_sms();                              // multiprocessors of the current device (api.cu)
 
 // ---- device helpers ----------------------------------------------------------------
 #ifdef __CUDACC__

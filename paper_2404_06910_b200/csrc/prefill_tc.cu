@@ -22,8 +22,8 @@
 // share an SM (256 TMEM columns each).  A small plan kernel turns the ragged layout into a
 // tile list.  Every mbarrier wait is bounded: on expiry the block records a timeout in the
 // workspace status word, unwinds, frees its TMEM and exits.
-// Compile-time variants: ALIBI adds the position bias to the scores; ROPE takes an unrotated Q and has the
-// softmax warps rotate each query tile in shared memory before its first use (sp_superpose_prefill_rope).
+// Compile-time variant: ALIBI adds the position bias to the scores.  sp_superpose_prefill_rope rotates Q into `out` first
+// and runs the same kernel on it.
 #include <cstdlib>
 
 #include "common.cuh"
@@ -104,8 +104,6 @@ struct TcParams {
     int64_t total_tokens;
     float scale_log2e;
     const float *pos, *slopes;        // ALiBi variant: token positions [T], head slopes [H]
-    const float2 *rope_cs;            // ROPE variant: (cos, sin) of every (token, pair), [T][64]
-    int rope_pairing;
     int stall_producer;               // test hook: the producer issues no load, so every wait runs out
 };
 
@@ -189,7 +187,7 @@ struct Cursor {
 // wrong fill.
 enum { BAR_Q_FULL = 0, BAR_Q_EMPTY, BAR_K_FULL, BAR_V_FULL = BAR_K_FULL + 2, BAR_S_FULL = BAR_V_FULL + 2,
        BAR_P_FULL = BAR_S_FULL + 2, BAR_O_DONE = BAR_P_FULL + 2, BAR_L_READY = BAR_O_DONE + 2,
-       BAR_X_FREE = BAR_L_READY + 2, BAR_O_FREE = BAR_X_FREE + 2, BAR_V_CLEAN, BAR_Q_ROT = BAR_V_CLEAN + 2, BAR_DRAIN,
+       BAR_X_FREE = BAR_L_READY + 2, BAR_O_FREE = BAR_X_FREE + 2, BAR_V_CLEAN, BAR_DRAIN = BAR_V_CLEAN + 2,
        BAR_COUNT = BAR_DRAIN + 2 };      // DRAIN: one per issuing thread
 
 template <int N> __device__ __forceinline__ void reg_alloc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
@@ -197,9 +195,7 @@ template <int N> __device__ __forceinline__ void reg_dealloc() { asm volatile("s
 
 // ALIBI: scores get -slope_h * |pos_q - pos_k| before the softmax (Section 3.2.2: real-valued
 // positions are no obstacle for ALiBi); the plain instantiation carries none of that code.
-// ROPE: Q arrives unrotated; the softmax warps rotate each query tile in shared memory, at the tokens' real-valued
-// positions (Section 3.2.2, footnote on RoPE), between its arrival and the item's first S = Q K^T.
-template <bool ALIBI, bool ROPE>
+template <bool ALIBI>
 __global__ void __launch_bounds__(kTcThreads, 2) prefill_tc_kernel(const __grid_constant__ TcParams p)
 {
     extern __shared__ unsigned char smem_raw[];
@@ -216,7 +212,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) prefill_tc_kernel(const __grid_
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int i = 0; i < BAR_COUNT; ++i)
-            mbar_init(&bars[i], ((i >= BAR_P_FULL && i < BAR_P_FULL + 2) || (i >= BAR_L_READY && i <= BAR_O_FREE) || i == BAR_Q_ROT) ? 128 : 1);
+            mbar_init(&bars[i], ((i >= BAR_P_FULL && i < BAR_P_FULL + 2) || (i >= BAR_L_READY && i <= BAR_O_FREE)) ? 128 : 1);
         fence_mbar_init();
         for (int i = 0; i < 3; ++i) prefetch_tmap(&p.mq[i]);
         for (int i = 0; i < 2; ++i) { prefetch_tmap(&p.mk[i]); prefetch_tmap(&p.mv[i]); }
@@ -279,7 +275,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) prefill_tc_kernel(const __grid_
 #pragma unroll 1
                 for (cs.init(p.tiles, n_items, p.n_heads); cs.valid && ok; cs.next()) {
                     const uint32_t st = cs.g & 1;
-                    if (cs.j == 0 && !(ok = mbar_wait(&bars[ROPE ? BAR_Q_ROT : BAR_Q_FULL], cs.item_no & 1))) break;
+                    if (cs.j == 0 && !(ok = mbar_wait(&bars[BAR_Q_FULL], cs.item_no & 1))) break;
                     if (!(ok = mbar_wait(&bars[BAR_K_FULL + st], (cs.g >> 1) & 1))) break;
                     // S(g) lands on the columns of P(g-2): the O += P V that reads them (issued by the other
                     // issuing thread) must be complete
@@ -442,55 +438,6 @@ __global__ void __launch_bounds__(kTcThreads, 2) prefill_tc_kernel(const __grid_
             if (ALIBI) {
                 if (lane < kt.n_valid) kp0 = __ldg(p.pos + kt.row0 + lane);
                 if (32 + lane < kt.n_valid) kp1 = __ldg(p.pos + kt.row0 + 32 + lane);
-            }
-            if (ROPE && first) {
-                // This thread's row of the new query tile: 8 pieces of 16 bytes in each 64-column half (the 128-byte
-                // swizzle permutes the pieces of a row by its index mod 8); the (cos, sin) pairs come from the
-                // per-token table.  The arithmetic is the standalone rotation's, so the tile equals what that
-                // kernel would have stored.
-                if (!(ok = mbar_wait_warp(&bars[BAR_Q_FULL], c.item_no & 1))) break;
-                if (row < t.n_rows) {
-                    unsigned char *h0 = sQ + row * 128, *h1 = h0 + (32 << q_box_sel(t.n_rows)) * 128;
-                    const float4 *tab = reinterpret_cast<const float4 *>(p.rope_cs + (int64_t)(t.q_row + row) * (kHD / 2));
-                    const bool half_split = p.rope_pairing == SP_ROPE_HALF_SPLIT;
-#pragma unroll 1
-                    for (int pc = 0; pc < 8; ++pc) {
-                        uint4 *pa = reinterpret_cast<uint4 *>(h0 + ((pc ^ (row & 7)) << 4));
-                        uint4 *pb = reinterpret_cast<uint4 *>(h1 + ((pc ^ (row & 7)) << 4));
-                        uint4 va = *pa, vb = *pb;
-                        uint32_t *ua = reinterpret_cast<uint32_t *>(&va), *ub = reinterpret_cast<uint32_t *>(&vb);
-                        if (half_split) {            // element j of the piece in half 0 pairs with element j in half 1
-#pragma unroll
-                            for (int j2 = 0; j2 < 4; ++j2) {
-                                const float4 w = __ldg(tab + pc * 4 + j2);      // pairs 8 pc + 2 j2, + 1
-                                const float a0 = __uint_as_float(ua[j2] << 16), a1 = __uint_as_float(ua[j2] & 0xffff0000u);
-                                const float b0 = __uint_as_float(ub[j2] << 16), b1 = __uint_as_float(ub[j2] & 0xffff0000u);
-                                float na0, nb0, na1, nb1;
-                                rope_rotate(a0, b0, w.x, w.y, na0, nb0);
-                                rope_rotate(a1, b1, w.z, w.w, na1, nb1);
-                                ua[j2] = pack_bf16x2(na0, na1);
-                                ub[j2] = pack_bf16x2(nb0, nb1);
-                            }
-                        } else {                     // neighbours pair up: pair 4 pc + j2 in half 0, 32 + 4 pc + j2 in half 1
-#pragma unroll
-                            for (int j2 = 0; j2 < 4; j2 += 2) {
-                                const float4 wa = __ldg(tab + pc * 2 + (j2 >> 1)), wb = __ldg(tab + 16 + pc * 2 + (j2 >> 1));
-                                float n0, n1;
-                                rope_rotate(__uint_as_float(ua[j2] << 16), __uint_as_float(ua[j2] & 0xffff0000u), wa.x, wa.y, n0, n1);
-                                ua[j2] = pack_bf16x2(n0, n1);
-                                rope_rotate(__uint_as_float(ua[j2 + 1] << 16), __uint_as_float(ua[j2 + 1] & 0xffff0000u), wa.z, wa.w, n0, n1);
-                                ua[j2 + 1] = pack_bf16x2(n0, n1);
-                                rope_rotate(__uint_as_float(ub[j2] << 16), __uint_as_float(ub[j2] & 0xffff0000u), wb.x, wb.y, n0, n1);
-                                ub[j2] = pack_bf16x2(n0, n1);
-                                rope_rotate(__uint_as_float(ub[j2 + 1] << 16), __uint_as_float(ub[j2 + 1] & 0xffff0000u), wb.z, wb.w, n0, n1);
-                                ub[j2 + 1] = pack_bf16x2(n0, n1);
-                            }
-                        }
-                        *pa = va; *pb = vb;
-                    }
-                }
-                fence_proxy_async();                 // generic-proxy stores -> visible to the MMA's reads
-                mbar_arrive(&bars[BAR_Q_ROT]);
             }
             if (!(ok = mbar_wait_warp(&bars[BAR_S_FULL + st], (c.g >> 1) & 1))) break;
             tc_fence_after();
@@ -671,6 +618,64 @@ __global__ void __launch_bounds__(kTcThreads, 2) prefill_tc_kernel(const __grid_
     if (warp == kMmaWarp) tmem_dealloc(tb, kTmemCols);
 }
 
+// ---- rotation of Q for sp_superpose_prefill_rope -----------------------------------------
+// Rotates the rows of every tile from q into out, where the attention kernel then reads its query tiles: an item's tile
+// is in shared memory long before its epilogue overwrites those rows (one head's columns of one tile's rows belong to one
+// item), so no other buffer is needed and q stays as it is.  One read and one write of Q at HBM speed.  The rotation inside
+// the attention kernel that this replaced (on the softmax warps, from a per-token table) cost 1.2 ms of a 2.9 ms launch at
+// 236 000 tokens x 32 heads; this pass costs 0.6.  Rows that belong to no segment are left alone.
+constexpr int kRopeRows = 4;          // rows per block iteration: 256 angles, one per thread
+struct RopeRows {
+    const __nv_bfloat16 *q;
+    __nv_bfloat16 *out;
+    const float *pos;
+    const TcHeader *hdr;
+    const TcTile *tiles;
+    int n_heads, half_split;
+    double inv_freq[kHD / 2];
+};
+__global__ void __launch_bounds__(256, 8) rope_rows_kernel(const __grid_constant__ RopeRows a)
+{
+    __shared__ float2 cs[kRopeRows][kHD / 2];
+    const uint32_t n_groups = a.hdr->n_tiles * (kBM / kRopeRows);
+    for (uint32_t g = blockIdx.x; g < n_groups; g += gridDim.x) {
+        const TcTile t = a.tiles[g / (kBM / kRopeRows)];
+        const int r0 = (int)(g % (kBM / kRopeRows)) * kRopeRows, n = min(kRopeRows, t.n_rows - r0);
+        if (n <= 0) continue;
+        const int64_t row = t.q_row + r0;
+        __syncthreads();
+        const int r = threadIdx.x >> 6, m = threadIdx.x & 63;
+        if (r < n) {
+            double sn, cn;
+            sincos((double)a.pos[row + r] * a.inv_freq[m], &sn, &cn);
+            cs[r][m] = make_float2((float)cn, (float)sn);
+        }
+        __syncthreads();
+        // 16 elements of a head per thread: a piece of each half (half-split) or two neighbouring pieces
+        for (int i = threadIdx.x; i < n * a.n_heads * 8; i += 256) {
+            const int rr = i / (a.n_heads * 8), j = i & 7;
+            const int64_t at = (row + rr) * a.n_heads * kHD + (int64_t)(i - rr * a.n_heads * 8 >> 3) * kHD + (a.half_split ? j * 8 : j * 16);
+            float x[8], y[8];
+            Vec<__nv_bfloat16>::load(a.q + at, x);
+            Vec<__nv_bfloat16>::load(a.q + at + (a.half_split ? kHD / 2 : 8), y);
+            if (a.half_split) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) rope_rotate(x[e], y[e], cs[rr][j * 8 + e].x, cs[rr][j * 8 + e].y, x[e], y[e]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; e += 2) {
+                    const float2 wx = cs[rr][j * 8 + e / 2], wy = cs[rr][j * 8 + 4 + e / 2];
+                    rope_rotate(x[e], x[e + 1], wx.x, wx.y, x[e], x[e + 1]);
+                    rope_rotate(y[e], y[e + 1], wy.x, wy.y, y[e], y[e + 1]);
+                }
+            }
+            uint4 *dst = reinterpret_cast<uint4 *>(a.out + at);
+            dst[0] = make_uint4(pack_bf16x2(x[0], x[1]), pack_bf16x2(x[2], x[3]), pack_bf16x2(x[4], x[5]), pack_bf16x2(x[6], x[7]));
+            dst[a.half_split ? kHD / 16 : 1] = make_uint4(pack_bf16x2(y[0], y[1]), pack_bf16x2(y[2], y[3]), pack_bf16x2(y[4], y[5]), pack_bf16x2(y[6], y[7]));
+        }
+    }
+}
+
 // ---- host side ---------------------------------------------------------------------------
 // Failure-detection test hook (host-injected, no GPU fault): while set, the producer loads no
 // tile, every bounded wait expires, the blocks unwind and the call reports SP_ERR_TIMEOUT
@@ -730,17 +735,18 @@ size_t prefill_tc_workspace_bytes(int n_prompts, int n_paths, int max_pre_len, i
 }
 
 static int launch_tc(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
-                     const float *slopes, const float2 *rope_cs, int rope_pairing, int n_heads, int n_kv_heads,
+                     const float *slopes, const RopeRows *rope, int n_heads, int n_kv_heads,
                      float scale, int rows, void *out, float *lse, void *ws, cudaStream_t st);
 
 int launch_prefill_tc(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
                       const float *slopes, int n_heads, int n_kv_heads, float scale, int rows, void *out,
                       float *lse, void *ws, size_t, cudaStream_t st)
 {
-    return launch_tc(q, k, v, lay, pos, slopes, nullptr, 0, n_heads, n_kv_heads, scale, rows, out, lse, ws, st);
+    return launch_tc(q, k, v, lay, pos, slopes, nullptr, n_heads, n_kv_heads, scale, rows, out, lse, ws, st);
 }
 
-// The (cos, sin) table of the ROPE variant sits behind the tile list and the pair list.
+// sp_superpose_prefill_rope.  The size leaves room for 512 bytes per token behind the tile list: the interface has asked
+// for it since its first version (a table of angles), and callers have sized their workspaces by it.
 size_t prefill_tc_rope_workspace_bytes(int n_prompts, int n_paths, int max_pre_len, int max_path_len, int64_t total_tokens)
 {
     return prefill_tc_workspace_bytes(n_prompts, n_paths, max_pre_len, max_path_len, 0) +
@@ -751,14 +757,15 @@ int launch_prefill_tc_rope(const void *q, const void *k, const void *v, const sp
                            int pairing, int n_heads, int n_kv_heads, float scale, void *out, float *lse, void *ws,
                            cudaStream_t st)
 {
-    float2 *table = reinterpret_cast<float2 *>(static_cast<char *>(ws) + prefill_tc_workspace_bytes(
-                        lay->n_prompts, lay->n_paths, lay->max_pre_len, lay->max_path_len, 0));
-    if (int rc = launch_rope_table(pos, lay->total_tokens, kHD, base, table, st)) return rc;
-    return launch_tc(q, k, v, lay, nullptr, nullptr, table, pairing, n_heads, n_kv_heads, scale, SP_ROWS_ALL, out, lse, ws, st);
+    RopeRows r;
+    r.q = static_cast<const __nv_bfloat16 *>(q); r.out = static_cast<__nv_bfloat16 *>(out); r.pos = pos;
+    r.n_heads = n_heads; r.half_split = pairing == SP_ROPE_HALF_SPLIT;
+    for (int m = 0; m < kHD / 2; ++m) r.inv_freq[m] = std::pow(base, -2.0 * m / kHD);
+    return launch_tc(out, k, v, lay, nullptr, nullptr, &r, n_heads, n_kv_heads, scale, SP_ROWS_ALL, out, lse, ws, st);
 }
 
 static int launch_tc(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
-                     const float *slopes, const float2 *rope_cs, int rope_pairing, int n_heads, int n_kv_heads,
+                     const float *slopes, const RopeRows *rope, int n_heads, int n_kv_heads,
                      float scale, int rows, void *out, float *lse, void *ws, cudaStream_t st)
 {
     {
@@ -766,7 +773,7 @@ static int launch_tc(const void *q, const void *k, const void *v, const sp_layou
         // Parity-green and slower than this kernel on every workload measured, so it is off unless
         // SP_B200_PREFILL_PAIR=1 is set when the library is first used.
         static const bool use_pair = [] { const char *e = std::getenv("SP_B200_PREFILL_PAIR"); return e && e[0] == '1'; }();
-        if (use_pair && rows == SP_ROWS_ALL && !rope_cs)
+        if (use_pair && rows == SP_ROWS_ALL && !rope)
             return launch_prefill_pair(q, k, v, lay, pos, slopes, n_heads, n_kv_heads, scale, out, lse, ws, st);
     }
     static EncodeTiledFn enc = nullptr;
@@ -801,28 +808,31 @@ static int launch_tc(const void *q, const void *k, const void *v, const sp_layou
     pa.hdr = hdr; pa.tiles = tiles;
     prefill_plan_kernel<<<1, 1024, 0, st>>>(pa);
     SP_CUDA(cudaGetLastError());
+    if (rope) {
+        RopeRows r = *rope;
+        r.hdr = hdr; r.tiles = tiles;
+        const int64_t groups = pa.max_tiles * (kBM / kRopeRows);
+        rope_rows_kernel<<<(int)std::min<int64_t>(groups, (int64_t)num_sms() * 16), 256, 0, st>>>(r);
+        SP_CUDA(cudaGetLastError());
+    }
 
     p.hdr = hdr; p.tiles = tiles; p.status = &hdr->status;
     p.out = static_cast<__nv_bfloat16 *>(out); p.lse = lse;
     p.n_heads = n_heads; p.kv_group = n_heads / n_kv_heads;
     p.total_tokens = lay->total_tokens; p.scale_log2e = scale * kLog2eT;
     p.pos = pos; p.slopes = slopes;
-    p.rope_cs = rope_cs; p.rope_pairing = rope_pairing;
     p.stall_producer = g_stall_producer ? 1 : 0;      // test hook, see sp_test_stall_producer below
 
     const int64_t items = max_tiles(lay->n_prompts, lay->n_paths, lay->max_pre_len, lay->max_path_len) * n_heads;
     if (items == 0) return SP_OK;
     const int grid = (int)std::min<int64_t>(items, 2 * num_sms());
     const int smem = kQBytes + 4 * kKVBytes + 4 * 2048 + 1024;
-    if (rope_cs) {
-        SP_CUDA(cudaFuncSetAttribute(prefill_tc_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        prefill_tc_kernel<false, true><<<grid, kTcThreads, smem, st>>>(p);
-    } else if (pos) {
-        SP_CUDA(cudaFuncSetAttribute(prefill_tc_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        prefill_tc_kernel<true, false><<<grid, kTcThreads, smem, st>>>(p);
+    if (pos) {
+        SP_CUDA(cudaFuncSetAttribute(prefill_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        prefill_tc_kernel<true><<<grid, kTcThreads, smem, st>>>(p);
     } else {
-        SP_CUDA(cudaFuncSetAttribute(prefill_tc_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        prefill_tc_kernel<false, false><<<grid, kTcThreads, smem, st>>>(p);
+        SP_CUDA(cudaFuncSetAttribute(prefill_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        prefill_tc_kernel<false><<<grid, kTcThreads, smem, st>>>(p);
     }
     SP_CUDA(cudaGetLastError());
     return SP_OK;

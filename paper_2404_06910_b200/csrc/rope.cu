@@ -187,33 +187,6 @@ static int rope_entry(const char *name, void *x, int64_t ld_token, int n_heads, 
                : launch_rope<__nv_bfloat16>(x, x1, pos, n_tokens, ld_token, ld_token1, n_heads, n_heads1, head_dim, rot_dim, pairing, fr, st);
 }
 
-// The (cos, sin) of every (token, pair) as a table in device memory, for kernels that rotate tiles on the fly:
-// the same fp64 evaluation as above, so a tile rotated from the table equals one rotated by rope_kernel.
-__global__ void __launch_bounds__(256) rope_table_kernel(const float *__restrict__ pos, int64_t n_tokens, int half,
-                                                          float2 *__restrict__ out, const __grid_constant__ RopeFreq fr)
-{
-    const int64_t n = n_tokens * half;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t t = i / half;
-        const int m = (int)(i - t * half);
-        double s, c;
-        sincos((double)pos[t] * fr.inv_freq[m], &s, &c);
-        out[i] = make_float2((float)c, (float)s);
-    }
-}
-
-int launch_rope_table(const float *pos, int64_t n_tokens, int rot_dim, double base, float2 *out, cudaStream_t st)
-{
-    if (n_tokens <= 0) return SP_OK;
-    RopeFreq fr;
-    for (int m = 0; m < rot_dim / 2; ++m) fr.inv_freq[m] = std::pow(base, -2.0 * m / rot_dim);
-    const int64_t n = n_tokens * (rot_dim / 2);
-    const int grid = (int)std::min<int64_t>((n + 255) / 256, (int64_t)num_sms() * 16);
-    rope_table_kernel<<<grid, 256, 0, st>>>(pos, n_tokens, rot_dim / 2, out, fr);
-    SP_CUDA(cudaGetLastError());
-    return SP_OK;
-}
-
 }  // namespace sp
 
 extern "C" int sp_rope_apply(void *x, const float *pos, int64_t n_tokens, int64_t ld_token,
