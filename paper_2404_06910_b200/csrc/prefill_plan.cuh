@@ -15,15 +15,21 @@ struct TcTile {                       // one query tile (shared by all heads)
     int32_t pad0, pad1;
 };
 
-struct PairRec {                      // up to two consecutive query tiles of one segment
-    int32_t tile0;                    // index of the first one in the tile list
-    int32_t n;                        // 1 or 2
+constexpr int kPairKeys = 64;         // keys per key tile of a pair
+struct TcPair {                       // one or two consecutive query tiles of a segment (shared by all heads)
+    // Keys of the segment are numbered u: its fully visible prefix (the prompt's preamble, may be empty) at [0, pre_len),
+    // its own rows from p16 = pre_len rounded up to 16.
+    int32_t own_base;                 // packed row of own key u is own_base + u
+    int32_t q_u;                      // key number of tile A's first row
+    int32_t pre_row, pre_len, p16;
+    int32_t rows_ab;                  // rows of tile A | rows of tile B, which follows it, << 16 (0: no tile B)
+    int32_t steps_a, steps;           // key tiles: of tile A, of the item
 };
+static_assert(sizeof(TcPair) == sizeof(TcTile), "both lists use the same slots of the workspace");
 
 struct TcHeader {                     // start of the workspace
     uint32_t status;
-    uint32_t n_tiles;
-    uint32_t n_pairs;
+    uint32_t n_tiles;                 // entries of the list: tiles, or pairs of tiles
 };
 
 // ---- plan: ragged layout -> tile list ---------------------------------------------------
@@ -35,8 +41,7 @@ struct PlanArgs {
     int64_t total_tokens;             // T: every segment must lie inside [0, T)
     int64_t max_tiles;                // capacity of the tile list
     TcHeader *hdr;
-    TcTile *tiles;
-    PairRec *pairs = nullptr;         // optional: the tiles grouped two by two per segment
+    void *list;                       // TcTile or TcPair
 };
 
 // What the host cannot check, the plan kernel does: a segment whose device-side numbers
@@ -44,11 +49,16 @@ struct PlanArgs {
 // and the status word reports it, so nothing outside the caller's tensors is ever touched and
 // the tile list cannot outgrow the workspace that was sized from those scalars.
 
+// PAIRS: the tiles of a segment two by two from its end (an odd one stands alone at the front, where it has the
+// fewest keys).  A segment that needs n tiles gets tiles of equal height, rounded up to the 32 rows of a warp:
+// 184 rows as 96 + 88 instead of 128 + 56, which leaves tile A 32 keys less to look at.
+template <bool PAIRS>
 static __global__ void __launch_bounds__(1024) prefill_plan_kernel(const PlanArgs a)
 {
-    __shared__ int warp_tot[32], warp_tot2[32];
-    __shared__ int running, running2;
-    if (threadIdx.x == 0) { running = 0; running2 = 0; }
+    __shared__ int warp_tot[32];
+    __shared__ int running;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // a dependent kernel may set itself up meanwhile
+    if (threadIdx.x == 0) { running = 0; a.hdr->status = STATUS_OK; }
     __syncthreads();
     const int n_seq = a.n_prompts + a.n_paths;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -86,46 +96,52 @@ static __global__ void __launch_bounds__(1024) prefill_plan_kernel(const PlanArg
             rows = bad ? 0 : dl + ql - first;
         }
         if (bad) a.hdr->status = STATUS_BAD_LAYOUT;
-        const int nt = (rows + a.tile_rows - 1) / a.tile_rows;
-        const int np = (nt + 1) / 2;
-        int incl = nt, incl2 = np;
+        int nt = (rows + a.tile_rows - 1) / a.tile_rows, height = a.tile_rows;
+        if (PAIRS && nt > 1) {
+            height = min(a.tile_rows, ((rows + nt - 1) / nt + 31) & ~31);
+            nt = (rows + height - 1) / height;
+        }
+        const int n_rec = PAIRS ? (nt + 1) / 2 : nt;
+        int incl = n_rec;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int v = __shfl_up_sync(0xffffffffu, incl, o);
-            const int v2 = __shfl_up_sync(0xffffffffu, incl2, o);
-            if (lane >= o) { incl += v; incl2 += v2; }
+            if (lane >= o) incl += v;
         }
-        if (lane == 31) { warp_tot[warp] = incl; warp_tot2[warp] = incl2; }
+        if (lane == 31) warp_tot[warp] = incl;
         __syncthreads();
-        int before = running, before2 = running2;
-        for (int w = 0; w < warp; ++w) { before += warp_tot[w]; before2 += warp_tot2[w]; }
-        int off = before + incl - nt;
-        if (a.pairs) {
-            const int off2 = before2 + incl2 - np;
-            for (int t = 0; t < np && off + 2 * t < a.max_tiles; ++t) {
-                PairRec pr;
-                pr.tile0 = off + 2 * t;
-                pr.n = (2 * t + 1 < nt && off + 2 * t + 1 < a.max_tiles) ? 2 : 1;
-                a.pairs[off2 + t] = pr;
+        int before = running;
+        for (int w = 0; w < warp; ++w) before += warp_tot[w];
+        const int off = before + incl - n_rec;
+        for (int t = 0; t < n_rec && off + t < a.max_tiles; ++t) {
+            if (PAIRS) {
+                const int t0 = max(2 * t - (nt & 1), 0);          // first tile of the record
+                const bool two = !((nt & 1) && t == 0);
+                const int rows_a = min(height, rows - t0 * height), rows_b = two ? min(height, rows - (t0 + 1) * height) : 0;
+                TcPair pr;
+                pr.p16 = (pre_n + 15) & ~15;
+                pr.own_base = own_row - pr.p16;
+                pr.q_u = pr.p16 + first + t0 * height;
+                pr.pre_row = pre_row; pr.pre_len = pre_n;
+                pr.rows_ab = rows_a | rows_b << 16;
+                pr.steps_a = (pr.q_u + rows_a + kPairKeys - 1) / kPairKeys;
+                pr.steps = (pr.q_u + rows_a + rows_b + kPairKeys - 1) / kPairKeys;
+                static_cast<TcPair *>(a.list)[off + t] = pr;
+            } else {
+                TcTile tl;
+                tl.q_off = first + t * height;
+                tl.q_row = own_row + tl.q_off;
+                tl.n_rows = min(height, rows - t * height);
+                tl.own_row = own_row;
+                tl.pre_row = pre_row; tl.pre_len = pre_n; tl.pad0 = 0; tl.pad1 = 0;
+                static_cast<TcTile *>(a.list)[off + t] = tl;
             }
         }
-        for (int t = 0; t < nt && off + t < a.max_tiles; ++t) {
-            TcTile tl;
-            tl.q_off = first + t * a.tile_rows;
-            tl.q_row = own_row + tl.q_off;
-            tl.n_rows = min(a.tile_rows, rows - t * a.tile_rows);
-            tl.own_row = own_row;
-            tl.pre_row = pre_row; tl.pre_len = pre_n; tl.pad0 = 0; tl.pad1 = 0;
-            a.tiles[off + t] = tl;
-        }
         __syncthreads();
-        if (threadIdx.x == 1023) { running = before + incl; running2 = before2 + incl2; }
+        if (threadIdx.x == 1023) running = before + incl;
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        a.hdr->n_tiles = (uint32_t)min((int64_t)running, a.max_tiles);
-        a.hdr->n_pairs = (uint32_t)min((int64_t)running2, a.max_tiles);
-    }
+    if (threadIdx.x == 0) a.hdr->n_tiles = (uint32_t)min((int64_t)running, a.max_tiles);
 }
 
 static inline int64_t plan_max_tiles(int n_prompts, int n_paths, int max_pre_len, int max_path_len, int tile_rows)

@@ -1,8 +1,7 @@
 // Fork-join prefill attention, fp32 SIMT variant (Section 3.2: a row attends to its
 // prompt's preamble and, causally, to its own path).
 //
-// Used where the tensor-core kernel does not apply: fp32 storage (tight tolerance rules
-// out reduced-precision products) and head_dim 64.  One warp owns one (row, head): the
+// Used for fp32 storage (the tight tolerance rules out reduced-precision products).  One warp owns one (row, head): the
 // head dimension is spread over the lanes, scores are warp-reduced, softmax is online
 // with exact exp2f.  Masked keys are never visited: the loop runs over the row's key
 // ranges only.
@@ -34,15 +33,6 @@ template <> struct LaneVec<float, 4> {
     __device__ static void load(const float *p, float (&f)[4]) { const float4 w = *reinterpret_cast<const float4 *>(p); f[0] = w.x; f[1] = w.y; f[2] = w.z; f[3] = w.w; }
     __device__ static void store(float *p, const float (&f)[4]) { *reinterpret_cast<float4 *>(p) = make_float4(f[0], f[1], f[2], f[3]); }
 };
-template <> struct LaneVec<__nv_bfloat16, 2> {
-    __device__ static void load(const __nv_bfloat16 *p, float (&f)[2]) { const uint32_t w = *reinterpret_cast<const uint32_t *>(p); f[0] = bf16_lo(w); f[1] = bf16_hi(w); }
-    __device__ static void store(__nv_bfloat16 *p, const float (&f)[2]) { *reinterpret_cast<uint32_t *>(p) = pack_bf16x2(f[0], f[1]); }
-};
-template <> struct LaneVec<__nv_bfloat16, 4> {
-    __device__ static void load(const __nv_bfloat16 *p, float (&f)[4]) { const uint2 w = *reinterpret_cast<const uint2 *>(p); f[0] = bf16_lo(w.x); f[1] = bf16_hi(w.x); f[2] = bf16_lo(w.y); f[3] = bf16_hi(w.y); }
-    __device__ static void store(__nv_bfloat16 *p, const float (&f)[4]) { *reinterpret_cast<uint2 *>(p) = make_uint2(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3])); }
-};
-
 // grid: x = sequence (prompt preambles first, then paths), y = head.
 template <typename T, int D>
 __global__ void __launch_bounds__(kSimtWarps * 32)
@@ -119,7 +109,7 @@ prefill_simt_kernel(const __grid_constant__ PrefillSimtArgs a)
 
 int launch_prefill_simt(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
                         const float *slopes, int n_heads, int n_kv_heads, int head_dim, float scale, int rows,
-                        void *out, float *lse, int dtype, cudaStream_t st)
+                        void *out, float *lse, cudaStream_t st)
 {
     PrefillSimtArgs a;
     a.q = q; a.k = k; a.v = v; a.out = out; a.lse = lse;
@@ -130,13 +120,8 @@ int launch_prefill_simt(const void *q, const void *k, const void *v, const sp_la
     a.pos = pos; a.slopes = slopes;
     const dim3 grid(lay->n_prompts + lay->n_paths, n_heads);
     const int threads = kSimtWarps * 32;
-    if (dtype == SP_F32) {
-        if (head_dim == 64) prefill_simt_kernel<float, 64><<<grid, threads, 0, st>>>(a);
-        else                prefill_simt_kernel<float, 128><<<grid, threads, 0, st>>>(a);
-    } else {
-        if (head_dim == 64) prefill_simt_kernel<__nv_bfloat16, 64><<<grid, threads, 0, st>>>(a);
-        else                prefill_simt_kernel<__nv_bfloat16, 128><<<grid, threads, 0, st>>>(a);
-    }
+    if (head_dim == 64) prefill_simt_kernel<float, 64><<<grid, threads, 0, st>>>(a);
+    else                prefill_simt_kernel<float, 128><<<grid, threads, 0, st>>>(a);
     SP_CUDA(cudaGetLastError());
     return SP_OK;
 }
