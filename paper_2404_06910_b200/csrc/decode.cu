@@ -295,38 +295,27 @@ struct DecodeRope {
     double inv_freq[64];      // base^(-2m/D), m < D/2 <= 64
 };
 
-// MINB: resident blocks per SM the register budget is sized for.  Split launches want 8 (a whole
-// launch in one wave, clusters of 2^n blocks pack evenly); an unsplit launch over a large batch
-// runs faster with the few registers more that 7 leave (nothing spills).
-template <typename T, int D, int GRP, bool ALIBI, bool ROPE, int MINB>
-__global__ void __launch_bounds__(kDecThreads, MINB)
-decode_cluster_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ DecodeRope rope, int rope_pairing)
+// Segment table of a block in shared memory: logical start, K row, V row and positions of each segment.
+template <typename T> struct DecodeSmem {
+    int *lo;                                 // [n_seg + 1]
+    const T **k, **v;
+    const float **pos;                       // ALiBi only
+    float *end;
+    __device__ __forceinline__ DecodeSmem(unsigned char *raw, int n_seg)
+    {
+        lo = reinterpret_cast<int *>(raw);
+        k = reinterpret_cast<const T **>(raw + round_up((n_seg + 1) * sizeof(int), 16));
+        v = k + n_seg;
+        pos = reinterpret_cast<const float **>(v + n_seg);
+        end = reinterpret_cast<float *>(pos + n_seg);
+    }
+};
+static size_t decode_table_bytes(int n_seg) { return round_up((n_seg + 1) * sizeof(int), 16) + 3 * n_seg * sizeof(void *); }
+
+// Segments of prompt b: 0 = preamble, 1..k = kept paths, k+1 = tail; lengths land in lo[s+1].
+template <typename T, bool ALIBI>
+__device__ __forceinline__ void decode_segments(const DecodeArgs &a, const DecodeSmem<T> &sm, int n_seg, int b, int hk, int D, int64_t row_elems)
 {
-    namespace cg = cooperative_groups;
-    constexpr int N = Vec<T>::N;            // elements per 16-byte load
-    constexpr int LPK = D / N;              // lanes that share one key row
-    constexpr int G = kDecThreads / LPK;    // key groups per block
-    constexpr int PS = D + 2;               // one partial: D outputs, max, sum
-    static_assert(LPK <= 32 && (32 % LPK) == 0, "a key row must fit in one warp");
-
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int n_seg = a.k + 2;
-    int *seg_lo = reinterpret_cast<int *>(smem_raw);                        // [n_seg+1]
-    const T **seg_k = reinterpret_cast<const T **>(smem_raw + round_up((n_seg + 1) * sizeof(int), 16));
-    const T **seg_v = seg_k + n_seg;
-    const float **seg_pos = reinterpret_cast<const float **>(seg_v + n_seg);       // [n_seg], ALiBi only
-    float *red = reinterpret_cast<float *>(seg_pos + n_seg);                // [G][GRP][PS]
-    float *part = red + G * GRP * PS;                                       // [GRP][PS], read by the cluster's first block
-    float2 *cs = reinterpret_cast<float2 *>(part + GRP * PS);               // [D/2] (cos, sin), ROPE only
-
-    const int split = blockIdx.x, b = blockIdx.z;
-    const int group = a.n_heads / a.n_kv_heads;                 // query heads per KV head
-    const int per_kv = group / GRP;                             // blocks (in y) per KV head
-    const int hk = blockIdx.y / per_kv;
-    const int h0 = hk * group + (blockIdx.y - hk * per_kv) * GRP;   // first query head of this block
-    const int64_t row_elems = (int64_t)a.n_kv_heads * D;
-
-    // segments: 0 = preamble, 1..k = kept paths, k+1 = tail; lengths land in seg_lo[s+1]
     for (int sgm = threadIdx.x; sgm < n_seg; sgm += kDecThreads) {
         const T *kc = static_cast<const T *>(a.k_cache) + (int64_t)hk * D;
         const T *vc = static_cast<const T *>(a.v_cache) + (int64_t)hk * D;
@@ -347,38 +336,114 @@ decode_cluster_kernel(const __grid_constant__ DecodeArgs a, const __grid_constan
         }
         // a cache segment that the device-side layout puts outside the tensors is not read at all
         if (sgm <= a.k && (len < 0 || row < 0 || row + len > a.total_tokens)) { len = 0; row = 0; }
-        seg_k[sgm] = kc + row * row_elems;
-        seg_v[sgm] = vc + row * row_elems;
-        if (ALIBI) seg_pos[sgm] = (sgm == a.k + 1 && len ? a.tail_pos : a.cache_pos) + row;
-        seg_lo[sgm + 1] = len;
+        sm.k[sgm] = kc + row * row_elems;
+        sm.v[sgm] = vc + row * row_elems;
+        if (ALIBI) sm.pos[sgm] = (sgm == a.k + 1 && len ? a.tail_pos : a.cache_pos) + row;
+        sm.lo[sgm + 1] = len;
     }
-    if (ROPE && threadIdx.x < D / 2) {
-        // The angle is formed in fp64 at the real-valued position and brought into [-pi, pi] there
-        // (two fused steps with a split 2 pi); the small remainder goes through the fp32 sine and
-        // cosine, whose error is then far below one rounding of the rotated values.
-        const double ang = (double)a.q_pos[b] * rope.inv_freq[threadIdx.x];
-        const double turns = rint(ang * 0.15915494309189535);
-        const double r = fma(-turns, 2.4492935982947064e-16, fma(-turns, 6.283185307179586, ang));
-        float sn, cn;
-        sincosf((float)r, &sn, &cn);
-        cs[threadIdx.x] = make_float2(cn, sn);
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {                 // prefix sum of the lengths, 32 segments per round
-        int carry = 0;
-        if (threadIdx.x == 0) seg_lo[0] = 0;
-        for (int base = 0; base < n_seg; base += 32) {
-            const int sgm = base + (int)threadIdx.x;
-            int v = sgm < n_seg ? seg_lo[sgm + 1] : 0;
+}
+
+// Prefix sum of the lengths by the first warp, 32 segments per round.
+template <typename T> __device__ __forceinline__ void decode_scan(const DecodeSmem<T> &sm, int n_seg)
+{
+    if (threadIdx.x >= 32) return;
+    int carry = 0;
+    if (threadIdx.x == 0) sm.lo[0] = 0;
+    for (int base = 0; base < n_seg; base += 32) {
+        const int sgm = base + (int)threadIdx.x;
+        int v = sgm < n_seg ? sm.lo[sgm + 1] : 0;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int up = __shfl_up_sync(0xffffffffu, v, o);
-                if ((int)threadIdx.x >= o) v += up;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int up = __shfl_up_sync(0xffffffffu, v, o);
+            if ((int)threadIdx.x >= o) v += up;
+        }
+        if (sgm < n_seg) sm.lo[sgm + 1] = carry + v;
+        carry += __shfl_sync(0xffffffffu, v, 31);
+    }
+}
+
+// (cos, sin) of prompt b's position.  The angle is formed in fp64 at the real-valued position and brought into [-pi, pi]
+// there (two fused steps with a split 2 pi); the small remainder goes through the fp32 sine and cosine, whose error is then
+// far below one rounding of the rotated values.
+template <int D> __device__ __forceinline__ void decode_angles(const DecodeArgs &a, const DecodeRope &rope, int b, float2 *cs)
+{
+    if (threadIdx.x >= D / 2) return;
+    const double ang = (double)a.q_pos[b] * rope.inv_freq[threadIdx.x];
+    const double turns = rint(ang * 0.15915494309189535);
+    const double r = fma(-turns, 2.4492935982947064e-16, fma(-turns, 6.283185307179586, ang));
+    float sn, cn;
+    sincosf((float)r, &sn, &cn);
+    cs[threadIdx.x] = make_float2(cn, sn);
+}
+
+// Element d of one (prompt, head): maximum bm (log2 units), sum bl and unnormalised output bo -> out, lse.
+template <typename T>
+__device__ __forceinline__ void decode_store(const DecodeArgs &a, int64_t bh, int D, int d, float bm, float bl, float bo)
+{
+    store_val(static_cast<T *>(a.out) + bh * D + d, bo * (bl > 0.f ? 1.f / bl : 0.f));
+    if (d == 0 && a.lse) a.lse[bh] = bl > 0.f ? (bm + log2f(bl)) * kLn2D : -INFINITY;
+}
+
+// Merges the blocks' partials [heads][D + 2] through the cluster's shared memory, in split order, and stores them: element d of
+// heads r0, r0 + dr, ..; r0 < 0: this thread has none.
+template <typename T, int D>
+__device__ __forceinline__ void decode_cluster_merge(const DecodeArgs &a, float *part, int split, int n_heads, int d, int r0, int dr, int64_t bh0)
+{
+    namespace cg = cooperative_groups;
+    constexpr int PS = D + 2;
+    cg::cluster_group cluster = cg::this_cluster();
+    cluster.sync();
+    if (split == 0 && r0 >= 0) {
+        for (int r = r0; r < n_heads; r += dr) {
+            float M = -INFINITY;
+            for (int i = 0; i < a.n_splits; ++i) M = fmaxf(M, cluster.map_shared_rank(part, i)[r * PS + D]);
+            float L = 0.f, O = 0.f;
+            for (int i = 0; i < a.n_splits; ++i) {
+                const float *rp = cluster.map_shared_rank(part, i) + r * PS;
+                const float w = (rp[D] == -INFINITY) ? 0.f : ex2f(rp[D] - M);
+                L += rp[D + 1] * w;
+                O += rp[d] * w;
             }
-            if (sgm < n_seg) seg_lo[sgm + 1] = carry + v;
-            carry += __shfl_sync(0xffffffffu, v, 31);
+            decode_store<T>(a, bh0 + r, D, d, M, L, O);
         }
     }
+    cluster.sync();                     // the others' shared memory stays alive until it has been read
+}
+
+// MINB: resident blocks per SM the register budget is sized for.  Split launches want 8 (a whole
+// launch in one wave, clusters of 2^n blocks pack evenly); an unsplit launch over a large batch
+// runs faster with the few registers more that 7 leave (nothing spills).
+template <typename T, int D, int GRP, bool ALIBI, bool ROPE, int MINB>
+__global__ void __launch_bounds__(kDecThreads, MINB)
+decode_cluster_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ DecodeRope rope, int rope_pairing)
+{
+    constexpr int N = Vec<T>::N;            // elements per 16-byte load
+    constexpr int LPK = D / N;              // lanes that share one key row
+    constexpr int G = kDecThreads / LPK;    // key groups per block
+    constexpr int PS = D + 2;               // one partial: D outputs, max, sum
+    static_assert(LPK <= 32 && (32 % LPK) == 0, "a key row must fit in one warp");
+
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int n_seg = a.k + 2;
+    const DecodeSmem<T> sm(smem_raw, n_seg);
+    int *seg_lo = sm.lo;
+    const T **seg_k = sm.k, **seg_v = sm.v;
+    const float **seg_pos = sm.pos;
+    float *red = sm.end;                                                    // [G][GRP][PS]
+    float *part = red + G * GRP * PS;                                       // [GRP][PS], read by the cluster's first block
+    float2 *cs = reinterpret_cast<float2 *>(part + GRP * PS);               // [D/2] (cos, sin), ROPE only
+
+    const int split = blockIdx.x, b = blockIdx.z;
+    const int group = a.n_heads / a.n_kv_heads;                 // query heads per KV head
+    const int per_kv = group / GRP;                             // blocks (in y) per KV head
+    const int hk = blockIdx.y / per_kv;
+    const int h0 = hk * group + (blockIdx.y - hk * per_kv) * GRP;   // first query head of this block
+    const int64_t row_elems = (int64_t)a.n_kv_heads * D;
+
+    decode_segments<T, ALIBI>(a, sm, n_seg, b, hk, D, row_elems);
+    if (ROPE) decode_angles<D>(a, rope, b, cs);
+    __syncthreads();
+    decode_scan(sm, n_seg);
     __syncthreads();
 
     const int total = seg_lo[n_seg];
@@ -566,8 +631,6 @@ decode_cluster_kernel(const __grid_constant__ DecodeArgs a, const __grid_constan
     }
 
     if (a.n_splits > 1) {
-        // ---- merge the splits through the cluster's shared memory, in split order ---------
-        cg::cluster_group cluster = cg::this_cluster();
         if (threadIdx.x < D) {
 #pragma unroll
             for (int r = 0; r < GRP; ++r) {
@@ -575,63 +638,35 @@ decode_cluster_kernel(const __grid_constant__ DecodeArgs a, const __grid_constan
                 if (threadIdx.x == 0) { part[r * PS + D] = bm[r]; part[r * PS + D + 1] = bl[r]; }
             }
         }
-        cluster.sync();
-        if (split == 0 && threadIdx.x < D) {
+        decode_cluster_merge<T, D>(a, part, split, GRP, threadIdx.x, threadIdx.x < D ? 0 : -1, 1, (int64_t)b * a.n_heads + h0);
+    } else if (threadIdx.x < D) {
 #pragma unroll
-            for (int r = 0; r < GRP; ++r) {
-                float M = -INFINITY;
-                for (int i = 0; i < a.n_splits; ++i) M = fmaxf(M, cluster.map_shared_rank(part, i)[r * PS + D]);
-                float L = 0.f, O = 0.f;
-                for (int i = 0; i < a.n_splits; ++i) {
-                    const float *rp = cluster.map_shared_rank(part, i) + r * PS;
-                    const float w = (rp[D] == -INFINITY) ? 0.f : ex2f(rp[D] - M);
-                    L += rp[D + 1] * w;
-                    O += rp[threadIdx.x] * w;
-                }
-                bm[r] = M; bl[r] = L; bo[r] = O;
-            }
-        }
-        cluster.sync();                     // the others' shared memory stays alive until it has been read
-        if (split != 0) return;
-    }
-    if (threadIdx.x < D) {
-#pragma unroll
-        for (int r = 0; r < GRP; ++r) {
-            const int64_t bh = (int64_t)b * a.n_heads + h0 + r;
-            const float inv = bl[r] > 0.f ? 1.f / bl[r] : 0.f;
-            store_val(static_cast<T *>(a.out) + bh * D + threadIdx.x, bo[r] * inv);
-            if (threadIdx.x == 0 && a.lse) a.lse[bh] = bl[r] > 0.f ? (bm[r] + log2f(bl[r])) * kLn2D : -INFINITY;
-        }
+        for (int r = 0; r < GRP; ++r) decode_store<T>(a, (int64_t)b * a.n_heads + h0 + r, D, threadIdx.x, bm[r], bl[r], bo[r]);
     }
 }
 
+}  // namespace sp
+
+#include "decode_mma.cuh"
+
+namespace sp {
+
 // Splits of a launch: a power of two (cluster size), at most 16, such that one launch stays
-// within about one resident wave and a split keeps at least 32 keys.
-static int cluster_splits(int n_prompts, int blocks_y, int64_t max_keys, int blocks_per_sm)
+// within about one resident wave and a split keeps at least min_keys keys.
+static int cluster_splits(int n_prompts, int blocks_y, int64_t max_keys, int min_keys, int blocks_per_sm)
 {
     const int64_t by = std::max<int64_t>(1, (int64_t)n_prompts * blocks_y);
-    const int64_t want = std::min<int64_t>(((int64_t)blocks_per_sm * num_sms()) / by, (max_keys + 31) / 32);
+    const int64_t want = std::min<int64_t>(((int64_t)blocks_per_sm * num_sms()) / by, (max_keys + min_keys - 1) / min_keys);
     int n = 1;
     while (n * 2 <= want && n < 16) n *= 2;
     return n;
 }
 
-template <typename T, int D, int GRP, bool ALIBI, bool ROPE>
-static int launch_decode_cluster(DecodeArgs a, const DecodeRope &rope, int pairing, int n_prompts, int64_t max_keys,
+template <typename K>
+static int launch_cluster_kernel(K kern, const DecodeArgs &a, const DecodeRope &rope, int pairing, int blocks_y, int n_prompts, size_t smem,
                                  cudaStream_t st)
 {
-    constexpr int G = kDecThreads / (D / Vec<T>::N);
-    constexpr int PS = D + 2;
-    const int group = a.n_heads / a.n_kv_heads;
-    const int blocks_y = a.n_kv_heads * (group / GRP);
-    constexpr int kMinB = GRP == 1 ? 8 : (GRP == 2 ? 5 : 3);
-    a.n_splits = cluster_splits(n_prompts, blocks_y, max_keys, kMinB);
-    const int n_seg = a.k + 2;
-    const size_t smem = round_up((n_seg + 1) * sizeof(int), 16) + 3 * n_seg * sizeof(void *) +
-                        (size_t)(G + 1) * GRP * PS * sizeof(float) + (D / 2) * sizeof(float2);
     SP_REQUIRE(smem <= 200 * 1024, SP_ERR_UNSUPPORTED, "sp_pruned_decode: k = %d needs too much shared memory", a.k);
-    auto kern = (GRP == 1 && a.n_splits == 1) ? decode_cluster_kernel<T, D, GRP, ALIBI, ROPE, kMinB - (GRP == 1 ? 1 : 0)>
-                                              : decode_cluster_kernel<T, D, GRP, ALIBI, ROPE, kMinB>;
     if (smem > 48 * 1024)
         SP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (a.n_splits > 8)
@@ -650,15 +685,45 @@ static int launch_decode_cluster(DecodeArgs a, const DecodeRope &rope, int pairi
     return SP_OK;
 }
 
+template <int D, bool ALIBI, bool ROPE>
+static int launch_decode_mma(DecodeArgs a, const DecodeRope &rope, int pairing, int n_prompts, int64_t max_keys, cudaStream_t st)
+{
+    constexpr int W = kDecThreads / 32;
+    const int group = a.n_heads / a.n_kv_heads, blocks_y = a.n_kv_heads * ((group + kMmaHeads - 1) / kMmaHeads);
+    a.n_splits = cluster_splits(n_prompts, blocks_y, max_keys, W * kMmaKeys, kMmaBlocks);
+    const size_t smem = decode_table_bytes(a.k + 2) + (size_t)(W + 1) * kMmaHeads * (D + 2) * sizeof(float) + (D / 2) * sizeof(float2);
+    return launch_cluster_kernel(decode_mma_kernel<D, ALIBI, ROPE>, a, rope, pairing, blocks_y, n_prompts, smem, st);
+}
+
+template <typename T, int D, int GRP, bool ALIBI, bool ROPE>
+static int launch_decode_cluster(DecodeArgs a, const DecodeRope &rope, int pairing, int n_prompts, int64_t max_keys,
+                                 cudaStream_t st)
+{
+    constexpr int G = kDecThreads / (D / Vec<T>::N);
+    constexpr int PS = D + 2;
+    const int group = a.n_heads / a.n_kv_heads;
+    const int blocks_y = a.n_kv_heads * (group / GRP);
+    constexpr int kMinB = GRP == 1 ? 8 : (GRP == 2 ? 5 : 3);
+    a.n_splits = cluster_splits(n_prompts, blocks_y, max_keys, 32, kMinB);
+    const size_t smem = decode_table_bytes(a.k + 2) + (size_t)(G + 1) * GRP * PS * sizeof(float) + (D / 2) * sizeof(float2);
+    auto kern = (GRP == 1 && a.n_splits == 1) ? decode_cluster_kernel<T, D, GRP, ALIBI, ROPE, kMinB - (GRP == 1 ? 1 : 0)>
+                                              : decode_cluster_kernel<T, D, GRP, ALIBI, ROPE, kMinB>;
+    return launch_cluster_kernel(kern, a, rope, pairing, blocks_y, n_prompts, smem, st);
+}
+
 template <typename T, int D, bool ALIBI, bool ROPE>
 static int launch_decode_grp(const DecodeArgs &a, const DecodeRope &rope, int pairing, int n_prompts, int64_t max_keys,
                              cudaStream_t st)
 {
-    // query heads per block: the largest of 4, 2, 1 that divides the group, so grouped heads share
-    // one pass over their K and V rows
     const int group = a.n_heads / a.n_kv_heads;
-    if (group % 4 == 0) return launch_decode_cluster<T, D, 4, ALIBI, ROPE>(a, rope, pairing, n_prompts, max_keys, st);
-    if (group % 2 == 0) return launch_decode_cluster<T, D, 2, ALIBI, ROPE>(a, rope, pairing, n_prompts, max_keys, st);
+    if constexpr (sizeof(T) == 2) {
+        if (group > 1) return launch_decode_mma<D, ALIBI, ROPE>(a, rope, pairing, n_prompts, max_keys, st);
+    } else {
+        // query heads per block: the largest of 4, 2, 1 that divides the group, so grouped heads share
+        // one pass over their K and V rows
+        if (group % 4 == 0) return launch_decode_cluster<T, D, 4, ALIBI, ROPE>(a, rope, pairing, n_prompts, max_keys, st);
+        if (group % 2 == 0) return launch_decode_cluster<T, D, 2, ALIBI, ROPE>(a, rope, pairing, n_prompts, max_keys, st);
+    }
     return launch_decode_cluster<T, D, 1, ALIBI, ROPE>(a, rope, pairing, n_prompts, max_keys, st);
 }
 
