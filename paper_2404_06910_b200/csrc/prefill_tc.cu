@@ -244,7 +244,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
             // A tile lands as [half][64 (Q: 128) rows][128 bytes], swizzled.  A whole tile of one segment is one box; otherwise
             // 32- and 16-row boxes per half, so that a key tile may hold the end of the preamble and the start of the own rows
             // and ragged ends pull in at most 15 rows nobody needs.
-            if (lane == 0 && !p.stall_producer) {
+            if (!p.stall_producer) {
+                const uint32_t lead = elect_one();
                 const bool is_q = warp == WARP_Q;
                 const int kind = warp - WARP_K, slots = is_q ? C::NQ : C::NKV, tile_rows = is_q ? kBM : kBN;
                 uint64_t *full = &bars[is_q ? C::BAR_Q_FULL : (kind ? C::BAR_V_FULL : C::BAR_K_FULL)];
@@ -260,7 +261,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                     const int head = (is_q ? w.h : w.h / p.kv_group) * C::HALVES, units = is_q ? w.n_q() : w.t.steps;
 #pragma unroll 1
                     for (int j = 0; j < units; ++j) {
-                        if (!(ok = mbar_wait(empty + slot, ph))) break;
+                        if (!(ok = mbar_wait_warp(empty + slot, ph))) break;
                         // rows [u0, u1) of the segment's key numbering; a query tile is part of its own rows
                         const int u0 = is_q ? w.t.q_u + (j ? w.rows_a() : 0) : j * kBN;
                         const int have = is_q ? (j ? w.rows_b() : w.rows_a()) : min(kBN, w.end() - u0);
@@ -270,7 +271,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                         last = (last & ~(0xffu << (8 * slot))) | (uint32_t)to << (8 * slot);
                         fills ^= 1u << to;
                         unsigned char *dst = base + slot * (tile_rows * D * 2);
-                        mbar_expect_tx(bar, (uint32_t)(u1 - u0) * (D * 2));
+                        if (lead) mbar_expect_tx(bar, (uint32_t)(u1 - u0) * (D * 2));
+                        __syncwarp();
 #pragma unroll 1
                         for (int u = u0; u < u1;) {
                             const bool pre = u < split;                         // preamble part, then own part
@@ -278,10 +280,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                             const int box = left == tile_rows ? 0 : (left >= 32 ? 1 : 2);
 #pragma unroll 1
                             for (int hh = 0; hh < (box ? C::HALVES : 1); ++hh)
-                                tma_load_3d_hint(dst + hh * (tile_rows * 128) + (u - u0) * 128, maps + box, 0, row, head + hh, bar, pol);
+                                tma_load_3d_hint(lead, dst + hh * (tile_rows * 128) + (u - u0) * 128, maps + box, 0, row, head + hh, bar, pol);
                             u += box == 0 ? tile_rows : (box == 1 ? 32 : 16);
                         }
-                        if (!is_q && w.one_lane(j)) mbar_arrive(empty + slot);      // for the lane that has no use for it
+                        if (lead && !is_q && w.one_lane(j)) mbar_arrive(empty + slot);      // for the lane that has no use for it
                         ++n;
                         if (++slot == slots) { slot = 0; ph ^= 1; }
                     }
@@ -290,7 +292,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                 if (!ok)
                     for (int i = 0; i < slots && i < (int)n; ++i) {
                         const uint32_t to = last >> (8 * i) & 0xff;
-                        mbar_wait(full + to, (fills >> to & 1) ^ 1);
+                        mbar_wait_warp(full + to, (fills >> to & 1) ^ 1);
                     }
             }
         } else if (ALIBI) {
@@ -335,7 +337,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
             uint32_t kv_ph = 0, q_ph = 0;                   // parity of the lane's own barriers, a bit per slot (V: 8 bits up)
             uint32_t g_s = 0, g_o = 0, tiles = 0, skip = 0; // S and O += P V issued so far
             // The (at most two) steps whose O += P V is still to be issued, oldest in the low half: 16-key steps, V stage (<< 3),
-            // first (<< 8) / last (<< 9) of its tile, parity of its tile number (<< 10), not the lane's first tile (<< 11)
+            // first of its tile (<< 8), parity of its tile number (<< 10), not the lane's first tile (<< 11)
             uint32_t pending = 0;
             Walk w(p);
             LaneTile t = {};
@@ -356,66 +358,69 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                     skip = w.t.steps - t.steps;
                     if (t.steps) ++tiles;
                 }
-                const uint32_t n_pending = g_s - g_o;
+                // What the next S needs is looked at before the wait for P, so that in the steady state (two steps pending) a turn
+                // is: wait for P(g), issue O += P V (g), issue S (g+2).
                 uint64_t *k_bar = own_kv + C::BAR_K_READY + k.i, *q_bar = own_q + C::BAR_Q_FULL + q_slot;
-                // S of the next tile as soon as a buffer is free and its operands are there.  With P V pending there is no waiting for
-                // them: they may lie behind tiles of the other lane that need the V stages still held here.
-                bool go = more && n_pending < 2;
-                if (go && n_pending)
-                    go = __all_sync(0xffffffffu, mbar_test(k_bar, kv_ph >> k.i & 1) && (j > 0 || mbar_test(q_bar, q_ph >> q_slot & 1)));
-                if (go) {
-                    if (n_pending == 0) {
-                        if (!(ok = mbar_wait_warp(k_bar, kv_ph >> k.i & 1))) break;
-                        if (j == 0 && !(ok = mbar_wait_warp(q_bar, q_ph >> q_slot & 1))) break;
-                    }
-                    kv_ph ^= 1u << k.i;
-                    if (j == 0) q_ph ^= 1u << q_slot;
+                auto look = [&]() { return more && __all_sync(0xffffffffu, mbar_test(k_bar, kv_ph >> k.i & 1) && (j > 0 || mbar_test(q_bar, q_ph >> q_slot & 1))); };
+                const int n_mma = (min(kBN, t.end - j * kBN) + 15) & ~15;
+                const uint64_t qd = d_hi | uniform(q_lo + q_slot * (C::Q_BYTES >> 4)), kd = d_hi | uniform(k_lo + k.i * (C::KV_BYTES >> 4));
+                const uint32_t id_s = uniform(idesc_bf16(kBM, 0, 0, 0) | ((uint32_t)(n_mma >> 3) << 17)), d_s = uniform(s_col + (g_s & 1) * kBN);
+                bool ready = look();
+                if (g_s - g_o == 2 || (g_s != g_o && !ready)) {
+                    const uint32_t vs = pending >> 3 & 3, buf = g_o & 1;
+                    const uint32_t n = uniform(pending & 7), fresh = uniform(pending & 256u), a = uniform(s_col + buf * kBN);
+                    const uint64_t vd = d_hi | uniform(v_lo + vs * (C::KV_BYTES >> 4));
+                    if (!(ok = mbar_wait_warp(own_kv + C::BAR_V_READY + vs, kv_ph >> (8 + vs) & 1))) break;
+                    kv_ph ^= 256u << vs;
+                    // the first O = P V of a tile overwrites O: the lane's previous tile must have been read out
+                    if ((pending & (256u | 2048u)) == (256u | 2048u) && !(ok = mbar_wait_warp(own2 + C::BAR_O_FREE, pending >> 10 & 1))) break;
+                    if (!(ok = mbar_wait_warp(own_buf + C::BAR_P + buf, g_o >> 1 & 1))) break;
                     tc_fence_after();
-                    const int n_mma = (min(kBN, t.end - j * kBN) + 15) & ~15;
-                    const uint32_t buf = g_s & 1;
-                    const uint64_t qd = d_hi | uniform(q_lo + q_slot * (C::Q_BYTES >> 4)), kd = d_hi | uniform(k_lo + k.i * (C::KV_BYTES >> 4));
-                    const uint32_t id_s = uniform(idesc_bf16(kBM, 0, 0, 0) | ((uint32_t)(n_mma >> 3) << 17)), d = uniform(s_col + buf * kBN);
 #pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk)             // contraction over head_dim
-                        umma_ss(lead, d, qd + (kk >> 2) * ((kBM * 128) >> 4) + (kk & 3) * 2, kd + (kk >> 2) * ((kBN * 128) >> 4) + (kk & 3) * 2,
-                                id_s, kk > 0 ? 1u : 0u);
-                    const bool last = j == t.steps - 1;
+                    for (int kk = 0; kk < kBN / 16; ++kk)           // contraction over keys
+                        if (kk < n) {
+                            const uint32_t at = a + (C::SPLIT_P ? (kk >> 1) * 32 + (kk & 1) * 8 : kk * 8);
+                            umma_ts(lead, o_col, at, vd + kk * (2048 >> 4), id_o, kk > 0 || !fresh ? 1u : 0u);
+                            if (C::SPLIT_P) umma_ts(lead, o_col, at + 16, vd + kk * (2048 >> 4), id_o, 1u);
+                        }
                     if (lead) {
-                        umma_commit(own_buf + C::BAR_S_FULL + buf);
-                        umma_commit(bars + C::BAR_K_EMPTY + k.i);
-                        if (last) umma_commit(bars + C::BAR_Q_EMPTY + q_slot);
+                        umma_commit(own_buf + C::BAR_O_DONE + buf);
+                        umma_commit(bars + C::BAR_V_EMPTY + vs);
                     }
                     __syncwarp();
-                    const uint32_t info = (uint32_t)(n_mma >> 4) | k.i << 3 | (j == 0 ? 256u : 0u) | (last ? 512u : 0u) | (tiles & 1) << 10 | (tiles > 1 ? 2048u : 0u);
-                    pending |= info << (16 * n_pending);
-                    ++j; ++g_s;
-                    k.next();
+                    pending >>= 16;
+                    ++g_o;
+                    if (!ready) ready = look();
+                }
+                if (!more) {
+                    if (g_s == g_o) break;
                     continue;
                 }
-                if (n_pending == 0) break;
-                const uint32_t vs = pending >> 3 & 3, buf = g_o & 1;
-                if (!(ok = mbar_wait_warp(own_kv + C::BAR_V_READY + vs, kv_ph >> (8 + vs) & 1))) break;
-                kv_ph ^= 256u << vs;
-                // the first O = P V of a tile overwrites O: the lane's previous tile must have been read out
-                if ((pending & (256u | 2048u)) == (256u | 2048u) && !(ok = mbar_wait_warp(own2 + C::BAR_O_FREE, pending >> 10 & 1))) break;
-                if (!(ok = mbar_wait_warp(own_buf + C::BAR_P + buf, g_o >> 1 & 1))) break;
+                if (!ready) {
+                    // With a step pending there is no waiting for K or Q: they may lie behind tiles of the other lane that need
+                    // the V stages still held here.
+                    if (g_s != g_o) continue;
+                    if (!(ok = mbar_wait_warp(k_bar, kv_ph >> k.i & 1))) break;
+                    if (j == 0 && !(ok = mbar_wait_warp(q_bar, q_ph >> q_slot & 1))) break;
+                }
                 tc_fence_after();
-                const uint32_t n = uniform(pending & 7), fresh = uniform(pending & 256u), a = uniform(s_col + buf * kBN);
-                const uint64_t vd = d_hi | uniform(v_lo + vs * (C::KV_BYTES >> 4));
 #pragma unroll
-                for (int kk = 0; kk < kBN / 16; ++kk)               // contraction over keys
-                    if (kk < n) {
-                        const uint32_t at = a + (C::SPLIT_P ? (kk >> 1) * 32 + (kk & 1) * 8 : kk * 8);
-                        umma_ts(lead, o_col, at, vd + kk * (2048 >> 4), id_o, kk > 0 || !fresh ? 1u : 0u);
-                        if (C::SPLIT_P) umma_ts(lead, o_col, at + 16, vd + kk * (2048 >> 4), id_o, 1u);
-                    }
+                for (int kk = 0; kk < D / 16; ++kk)                 // contraction over head_dim
+                    umma_ss(lead, d_s, qd + (kk >> 2) * ((kBM * 128) >> 4) + (kk & 3) * 2, kd + (kk >> 2) * ((kBN * 128) >> 4) + (kk & 3) * 2,
+                            id_s, kk > 0 ? 1u : 0u);
+                const bool last = j == t.steps - 1;
                 if (lead) {
-                    umma_commit(own_buf + C::BAR_O_DONE + buf);
-                    umma_commit(bars + C::BAR_V_EMPTY + vs);
+                    umma_commit(own_buf + C::BAR_S_FULL + (g_s & 1));
+                    umma_commit(bars + C::BAR_K_EMPTY + k.i);
+                    if (last) umma_commit(bars + C::BAR_Q_EMPTY + q_slot);
                 }
                 __syncwarp();
-                pending >>= 16;
-                ++g_o;
+                kv_ph ^= 1u << k.i;
+                if (j == 0) q_ph ^= 1u << q_slot;
+                const uint32_t info = (uint32_t)(n_mma >> 4) | k.i << 3 | (j == 0 ? 256u : 0u) | (tiles & 1) << 10 | (tiles > 1 ? 2048u : 0u);
+                pending |= info << (16 * (g_s - g_o));
+                ++j; ++g_s;
+                k.next();
             }
             if (!ok) {
                 // a wait ran out: every MMA of this lane must finish (bounded) before its tensor memory is freed

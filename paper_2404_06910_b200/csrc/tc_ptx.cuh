@@ -81,7 +81,7 @@ __device__ __forceinline__ void prefetch_tmap(const CUtensorMap *m)
 }
 // L2 eviction-priority policies (first: data that is read once), and the 3-D tile load that carries one: coordinates
 // (x, y, z) from the innermost dimension outwards, completion counted in bytes on `bar`.  x is in elements and must keep the
-// copy 16-byte aligned.
+// copy 16-byte aligned.  Executed by the thread with `lead` set; the whole warp runs through it.
 __device__ __forceinline__ uint64_t l2_policy_evict_first()
 {
     uint64_t pol;
@@ -94,11 +94,12 @@ __device__ __forceinline__ uint64_t l2_policy_evict_normal()
     asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
     return pol;
 }
-__device__ __forceinline__ void tma_load_3d_hint(void *dst, const CUtensorMap *m, int x, int y, int z, uint64_t *bar, uint64_t pol)
+__device__ __forceinline__ void tma_load_3d_hint(uint32_t lead, void *dst, const CUtensorMap *m, int x, int y, int z, uint64_t *bar, uint64_t pol)
 {
     asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;"
-        ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)), "l"(pol) : "memory");
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %7, 0;\n\t"
+        "@q cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;\n\t}"
+        ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)), "l"(pol), "r"(lead) : "memory");
 }
 
 // ---- TMEM ------------------------------------------------------------------------------
