@@ -6,7 +6,7 @@
 namespace sp {
 int launch_prefill_simt(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
                         const float *slopes, int n_heads, int n_kv_heads, int head_dim, float scale, int rows,
-                        void *out, float *lse, cudaStream_t st);
+                        void *out, float *lse, void *ws, cudaStream_t st);
 size_t prefill_tc_workspace_bytes(int n_prompts, int n_paths, int max_pre_len, int max_path_len, int n_heads);
 int launch_prefill_tc(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
                       const float *slopes, int n_heads, int n_kv_heads, int head_dim, float scale, int rows, void *out,
@@ -60,8 +60,7 @@ static int prefill_entry(const void *q, const void *k, const void *v, const sp_l
     // SIMT kernel, which served it before, took 9.4 ms)
     if (dtype == SP_BF16)
         return launch_prefill_tc(q, k, v, lay, pos, slopes, n_heads, n_kv_heads, head_dim, scale, rows, out, lse, ws, st);
-    SP_CUDA(cudaMemsetAsync(ws, 0, 256, st));
-    return launch_prefill_simt(q, k, v, lay, pos, slopes, n_heads, n_kv_heads, head_dim, scale, rows, out, lse, st);
+    return launch_prefill_simt(q, k, v, lay, pos, slopes, n_heads, n_kv_heads, head_dim, scale, rows, out, lse, ws, st);
 }
 }  // namespace sp
 

@@ -1,46 +1,47 @@
 // Fork-join prefill attention, fp32 SIMT variant (Section 3.2: a row attends to its
 // prompt's preamble and, causally, to its own path).
 //
-// Used for fp32 storage (the tight tolerance rules out reduced-precision products).  One warp owns one (row, head): the
-// head dimension is spread over the lanes, scores are warp-reduced, softmax is online
-// with exact exp2f.  Masked keys are never visited: the loop runs over the row's key
-// ranges only.
+// Used for fp32 storage (the tight tolerance rules out reduced-precision products).  A block owns 16 query rows of one
+// segment and one head and walks their keys (the preamble's rows, then the segment's own up to its last row) in tiles
+// staged in shared memory; masked tiles are never visited.  Half a warp shares two query rows: a thread holds their scores
+// against every 16th key of the tile, reduces maxima and sums over the half warp (online softmax, exact exp2f), and then
+// owns 2 x D / 16 outputs.  One tile of the small problems this path serves is a handful of dependent memory
+// latencies; the warp-per-row loop before it took one per key (176 tokens x 4 heads x 64: 43 us, now 5.6).
 #include "common.cuh"
 
 namespace sp {
 
-constexpr int kSimtWarps = 8;
+constexpr int kSimtThreads = 128;
+constexpr int kSimtRows = 16;        // query rows per block
 constexpr float kLog2eP = 1.4426950408889634f;
 constexpr float kLn2P = 0.6931471805599453f;
 
 struct PrefillSimtArgs {
-    const void *q, *k, *v;
-    void *out;
-    float *lse;
+    const float *q, *k, *v;
+    float *out, *lse;
     const int32_t *ppo, *pre_start, *pre_len, *path_start, *doc_len, *qry_len;
+    uint32_t *status;            // workspace status word: this kernel has nothing to report and clears it
     int n_prompts, n_paths, n_heads, n_kv_heads, rows_mode;
     int64_t total_tokens;
     float scale_log2e;
     const float *pos, *slopes;   // ALiBi: token positions [T] and head slopes [H]; NULL = no bias
 };
 
-template <typename T, int EPL> struct LaneVec;     // EPL contiguous elements of one lane
-template <> struct LaneVec<float, 2> {
-    __device__ static void load(const float *p, float (&f)[2]) { const float2 w = *reinterpret_cast<const float2 *>(p); f[0] = w.x; f[1] = w.y; }
-    __device__ static void store(float *p, const float (&f)[2]) { *reinterpret_cast<float2 *>(p) = make_float2(f[0], f[1]); }
-};
-template <> struct LaneVec<float, 4> {
-    __device__ static void load(const float *p, float (&f)[4]) { const float4 w = *reinterpret_cast<const float4 *>(p); f[0] = w.x; f[1] = w.y; f[2] = w.z; f[3] = w.w; }
-    __device__ static void store(float *p, const float (&f)[4]) { *reinterpret_cast<float4 *>(p) = make_float4(f[0], f[1], f[2], f[3]); }
-};
-// grid: x = sequence (prompt preambles first, then paths), y = head.
-template <typename T, int D>
-__global__ void __launch_bounds__(kSimtWarps * 32)
+// grid: x = row tile x sequences (prompt preambles first, then paths), y = head.
+template <int D>
+__global__ void __launch_bounds__(kSimtThreads)
 prefill_simt_kernel(const __grid_constant__ PrefillSimtArgs a)
 {
-    constexpr int EPL = D / 32;
-    const int seq = blockIdx.x, h = blockIdx.y;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int BN = 4096 / D;             // keys per tile: 32 KB of K and V
+    constexpr int KPT = BN / 16;             // keys per thread
+    constexpr int CPT = D / 64;              // float4 output columns per thread and row
+    constexpr int KS = D + 4;                // padded K row: 16 lanes reading 16 rows hit different banks
+    __shared__ __align__(16) float sq[kSimtRows][D], sk[BN][KS], sv[BN][D], sp_[kSimtRows][BN];
+    __shared__ float s_pos[BN];
+
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *a.status = STATUS_OK;
+    const int n_seq = a.n_prompts + a.n_paths;
+    const int tile = blockIdx.x / n_seq, seq = blockIdx.x - tile * n_seq, h = blockIdx.y;
     const int hk = h / (a.n_heads / a.n_kv_heads);
 
     // key ranges of this sequence: [pre_lo, pre_lo+pre_n) fully visible, own rows causal
@@ -60,68 +61,135 @@ prefill_simt_kernel(const __grid_constant__ PrefillSimtArgs a)
         own_lo = a.path_start[i]; own_n = a.doc_len[i] + a.qry_len[i];
         first_row = a.rows_mode == SP_ROWS_QUERY_ONLY ? a.doc_len[i] : 0;
     }
+    const int r0 = first_row + tile * kSimtRows;    // first row of the tile, counted in the segment
+    const int n_rows = min(kSimtRows, own_n - r0);
+    if (n_rows <= 0) return;
+    const int n_keys = pre_n + r0 + n_rows;
 
-    const T *Q = static_cast<const T *>(a.q);
-    const T *K = static_cast<const T *>(a.k) + (int64_t)hk * D + lane * EPL;
-    const T *V = static_cast<const T *>(a.v) + (int64_t)hk * D + lane * EPL;
-    const int64_t kv_stride = (int64_t)a.n_kv_heads * D;
+    for (int i = threadIdx.x; i < kSimtRows * (D / 4); i += kSimtThreads) {
+        const int r = i / (D / 4), c = i % (D / 4);
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < n_rows) x = *reinterpret_cast<const float4 *>(a.q + ((int64_t)(own_lo + r0 + r) * a.n_heads + h) * D + c * 4);
+        *reinterpret_cast<float4 *>(&sq[r][c * 4]) = make_float4(x.x * a.scale_log2e, x.y * a.scale_log2e, x.z * a.scale_log2e, x.w * a.scale_log2e);
+    }
 
-    for (int j = first_row + warp; j < own_n; j += kSimtWarps) {
-        const int64_t r = own_lo + j;
-        float qf[EPL], acc[EPL];
-        LaneVec<T, EPL>::load(Q + (r * a.n_heads + h) * D + lane * EPL, qf);
+    const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15, row = 2 * ty;
+    float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f}, pq[2] = {0.f, 0.f};
+    float4 o[2][CPT];
 #pragma unroll
-        for (int e = 0; e < EPL; ++e) { qf[e] *= a.scale_log2e; acc[e] = 0.f; }
-        float m = -INFINITY, l = 0.f;
-        const float pq = a.pos ? a.pos[r] : 0.f;
-        const float slope_l2 = a.pos ? a.slopes[h] * kLog2eP : 0.f;
+    for (int r = 0; r < 2; ++r) {
+#pragma unroll
+        for (int c = 0; c < CPT; ++c) o[r][c] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (a.pos && row + r < n_rows) pq[r] = a.pos[own_lo + r0 + row + r];
+    }
+    const float slope_l2 = a.pos ? a.slopes[h] * kLog2eP : 0.f;
 
-        const int n_keys = pre_n + j + 1;
-        for (int c = 0; c < n_keys; ++c) {
-            const int64_t kr = c < pre_n ? (int64_t)pre_lo + c : (int64_t)own_lo + (c - pre_n);
-            float kf[EPL], vf[EPL];
-            LaneVec<T, EPL>::load(K + kr * kv_stride, kf);
-            LaneVec<T, EPL>::load(V + kr * kv_stride, vf);
-            float s = 0.f;
-#pragma unroll
-            for (int e = 0; e < EPL; ++e) s = fmaf(qf[e], kf[e], s);
-            s = warp_sum(s);
-            if (a.pos) s -= slope_l2 * fabsf(pq - a.pos[kr]);     // ALiBi: linear distance penalty
-            if (s > m) {
-                const float rs = exp2f(m - s);
-                l *= rs;
-#pragma unroll
-                for (int e = 0; e < EPL; ++e) acc[e] *= rs;
-                m = s;
+    for (int base = 0; base < n_keys; base += BN) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < BN * (D / 4); i += kSimtThreads) {
+            const int key = i / (D / 4), c = i % (D / 4), j = base + key;
+            float4 kx = make_float4(0.f, 0.f, 0.f, 0.f), vx = kx;
+            if (j < n_keys) {
+                const int64_t at = ((int64_t)(j < pre_n ? pre_lo + j : own_lo + j - pre_n) * a.n_kv_heads + hk) * D + c * 4;
+                kx = *reinterpret_cast<const float4 *>(a.k + at);
+                vx = *reinterpret_cast<const float4 *>(a.v + at);
             }
-            const float p = exp2f(s - m);
-            l += p;
-#pragma unroll
-            for (int e = 0; e < EPL; ++e) acc[e] = fmaf(p, vf[e], acc[e]);
+            *reinterpret_cast<float4 *>(&sk[key][c * 4]) = kx;
+            *reinterpret_cast<float4 *>(&sv[key][c * 4]) = vx;
         }
-        const float inv = 1.f / l;
+        if (a.pos && threadIdx.x < BN) {
+            const int j = base + (int)threadIdx.x;
+            s_pos[threadIdx.x] = j < n_keys ? a.pos[j < pre_n ? pre_lo + j : own_lo + j - pre_n] : 0.f;
+        }
+        __syncthreads();
+
+        float s[2][KPT];
 #pragma unroll
-        for (int e = 0; e < EPL; ++e) acc[e] *= inv;
-        LaneVec<T, EPL>::store(static_cast<T *>(a.out) + (r * a.n_heads + h) * D + lane * EPL, acc);
-        if (a.lse && lane == 0) a.lse[(int64_t)h * a.total_tokens + r] = (m + log2f(l)) * kLn2P;
+        for (int i = 0; i < KPT; ++i) s[0][i] = s[1][i] = 0.f;
+#pragma unroll 4
+        for (int d = 0; d < D; d += 4) {
+            const float4 q0 = *reinterpret_cast<const float4 *>(&sq[row][d]), q1 = *reinterpret_cast<const float4 *>(&sq[row + 1][d]);
+#pragma unroll
+            for (int i = 0; i < KPT; ++i) {
+                const float4 kx = *reinterpret_cast<const float4 *>(&sk[tx + 16 * i][d]);
+                s[0][i] = fmaf(q0.x, kx.x, fmaf(q0.y, kx.y, fmaf(q0.z, kx.z, fmaf(q0.w, kx.w, s[0][i]))));
+                s[1][i] = fmaf(q1.x, kx.x, fmaf(q1.y, kx.y, fmaf(q1.z, kx.z, fmaf(q1.w, kx.w, s[1][i]))));
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int lim = pre_n + r0 + row + r + 1 - base;         // keys of the tile this row may see
+            float mx = -INFINITY;
+#pragma unroll
+            for (int i = 0; i < KPT; ++i) {
+                if (a.pos) s[r][i] -= slope_l2 * fabsf(pq[r] - s_pos[tx + 16 * i]);     // ALiBi: linear distance penalty
+                if (tx + 16 * i >= lim) s[r][i] = -INFINITY;
+                mx = fmaxf(mx, s[r][i]);
+            }
+#pragma unroll
+            for (int d = 8; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
+            if (mx > m[r]) {                                          // the same in the whole half warp
+                const float rs = exp2f(m[r] - mx);
+                l[r] *= rs;
+#pragma unroll
+                for (int c = 0; c < CPT; ++c) { o[r][c].x *= rs; o[r][c].y *= rs; o[r][c].z *= rs; o[r][c].w *= rs; }
+                m[r] = mx;
+            }
+#pragma unroll
+            for (int i = 0; i < KPT; ++i) {
+                const float p = s[r][i] == -INFINITY ? 0.f : exp2f(s[r][i] - m[r]);
+                l[r] += p;                                            // this thread's keys; summed over the half warp at the end
+                sp_[row + r][tx + 16 * i] = p;
+            }
+        }
+        __syncwarp();
+        const int n = min(BN, n_keys - base);
+#pragma unroll 4
+        for (int key = 0; key < n; ++key) {
+            const float p0 = sp_[row][key], p1 = sp_[row + 1][key];
+#pragma unroll
+            for (int c = 0; c < CPT; ++c) {
+                const float4 vx = *reinterpret_cast<const float4 *>(&sv[key][c * 64 + tx * 4]);
+                o[0][c].x = fmaf(p0, vx.x, o[0][c].x); o[0][c].y = fmaf(p0, vx.y, o[0][c].y);
+                o[0][c].z = fmaf(p0, vx.z, o[0][c].z); o[0][c].w = fmaf(p0, vx.w, o[0][c].w);
+                o[1][c].x = fmaf(p1, vx.x, o[1][c].x); o[1][c].y = fmaf(p1, vx.y, o[1][c].y);
+                o[1][c].z = fmaf(p1, vx.z, o[1][c].z); o[1][c].w = fmaf(p1, vx.w, o[1][c].w);
+            }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+#pragma unroll
+        for (int d = 8; d > 0; d >>= 1) l[r] += __shfl_xor_sync(0xffffffffu, l[r], d);
+        if (row + r >= n_rows) continue;
+        const int64_t at = own_lo + r0 + row + r;
+        const float inv = 1.f / l[r];
+#pragma unroll
+        for (int c = 0; c < CPT; ++c)
+            *reinterpret_cast<float4 *>(a.out + (at * a.n_heads + h) * D + c * 64 + tx * 4) =
+                make_float4(o[r][c].x * inv, o[r][c].y * inv, o[r][c].z * inv, o[r][c].w * inv);
+        if (a.lse && tx == 0) a.lse[(int64_t)h * a.total_tokens + at] = (m[r] + log2f(l[r])) * kLn2P;
     }
 }
 
 int launch_prefill_simt(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
                         const float *slopes, int n_heads, int n_kv_heads, int head_dim, float scale, int rows,
-                        void *out, float *lse, cudaStream_t st)
+                        void *out, float *lse, void *ws, cudaStream_t st)
 {
     PrefillSimtArgs a;
-    a.q = q; a.k = k; a.v = v; a.out = out; a.lse = lse;
+    a.q = static_cast<const float *>(q); a.k = static_cast<const float *>(k); a.v = static_cast<const float *>(v);
+    a.out = static_cast<float *>(out); a.lse = lse; a.status = static_cast<uint32_t *>(ws);
     a.ppo = lay->prompt_path_off; a.pre_start = lay->pre_start; a.pre_len = lay->pre_len;
     a.path_start = lay->path_start; a.doc_len = lay->doc_len; a.qry_len = lay->qry_len;
     a.n_prompts = lay->n_prompts; a.n_paths = lay->n_paths; a.n_heads = n_heads; a.n_kv_heads = n_kv_heads;
     a.rows_mode = rows; a.total_tokens = lay->total_tokens; a.scale_log2e = scale * kLog2eP;
     a.pos = pos; a.slopes = slopes;
-    const dim3 grid(lay->n_prompts + lay->n_paths, n_heads);
-    const int threads = kSimtWarps * 32;
-    if (head_dim == 64) prefill_simt_kernel<float, 64><<<grid, threads, 0, st>>>(a);
-    else                prefill_simt_kernel<float, 128><<<grid, threads, 0, st>>>(a);
+    const int64_t tiles = (std::max(lay->max_pre_len, lay->max_path_len) + kSimtRows - 1) / kSimtRows;
+    const int64_t blocks = std::max<int64_t>(1, tiles) * (lay->n_prompts + lay->n_paths);
+    SP_REQUIRE(blocks < (int64_t)INT32_MAX, SP_ERR_UNSUPPORTED, "sp_superpose_prefill: %lld row tiles", (long long)blocks);
+    const dim3 grid((unsigned)blocks, n_heads);
+    if (head_dim == 64) prefill_simt_kernel<64><<<grid, kSimtThreads, 0, st>>>(a);
+    else                prefill_simt_kernel<128><<<grid, kSimtThreads, 0, st>>>(a);
     SP_CUDA(cudaGetLastError());
     return SP_OK;
 }
