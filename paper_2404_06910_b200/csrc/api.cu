@@ -64,30 +64,52 @@ int check_layout(const sp_layout *lay)
     if (NP > 0) SP_REQUIRE(m.path_start && m.doc_len && m.qry_len, SP_ERR_INVALID_ARG, "layout: host mirror of the per-path arrays is NULL");
     if (B > 0) SP_REQUIRE(m.prompt_path_off[0] == 0 && m.prompt_path_off[B] == NP, SP_ERR_INVALID_ARG,
                           "layout: prompt_path_off must run from 0 to n_paths");
-    std::vector<std::pair<int64_t, int64_t>> seg;          // (first row, one past the last row)
-    seg.reserve((size_t)B + NP);
+    // One pass over the arrays, in packed order: when every segment starts at or behind the end of the one before, none
+    // overlap.  (Sorting all segments took 30 us of every call at 800 paths, more than a decode step's kernel.)
+    int64_t end = 0;
+    bool ascending = true;
+    auto place = [&](int64_t row, int64_t n) {
+        ascending &= n == 0 || row >= end;
+        end = n ? row + n : end;
+    };
     for (int b = 0; b < B; ++b) {
         SP_REQUIRE(m.prompt_path_off[b] <= m.prompt_path_off[b + 1], SP_ERR_INVALID_ARG, "layout: prompt_path_off decreases at prompt %d", b);
         SP_REQUIRE(m.pre_len[b] >= 0 && m.pre_len[b] <= lay->max_pre_len, SP_ERR_INVALID_ARG,
                    "layout: pre_len[%d] = %d outside [0, max_pre_len = %d]", b, m.pre_len[b], lay->max_pre_len);
         SP_REQUIRE(m.pre_start[b] >= 0 && (int64_t)m.pre_start[b] + m.pre_len[b] <= T, SP_ERR_INVALID_ARG,
                    "layout: preamble of prompt %d leaves [0, total_tokens)", b);
+    }
+    for (int b = 0; b < B; ++b) {
+        place(m.pre_start[b], m.pre_len[b]);
+        for (int i = m.prompt_path_off[b]; i < m.prompt_path_off[b + 1]; ++i) {
+            const int64_t n = (int64_t)m.doc_len[i] + m.qry_len[i];
+            SP_REQUIRE(m.doc_len[i] >= 0 && m.qry_len[i] >= 0 && n <= lay->max_path_len,
+                       SP_ERR_INVALID_ARG, "layout: path %d has lengths (%d, %d) outside [0, max_path_len = %d]", i, m.doc_len[i],
+                       m.qry_len[i], lay->max_path_len);
+            SP_REQUIRE(m.path_start[i] >= 0 && m.path_start[i] + n <= T, SP_ERR_INVALID_ARG,
+                       "layout: path %d leaves [0, total_tokens)", i);
+            place(m.path_start[i], n);
+        }
+    }
+    if (ascending) return SP_OK;
+    std::vector<std::pair<int64_t, int64_t>> seg;          // (first row, one past the last row)
+    seg.reserve((size_t)B + NP);
+    for (int b = 0; b < B; ++b)
         if (m.pre_len[b]) seg.emplace_back(m.pre_start[b], (int64_t)m.pre_start[b] + m.pre_len[b]);
-    }
-    for (int i = 0; i < NP; ++i) {
-        SP_REQUIRE(m.doc_len[i] >= 0 && m.qry_len[i] >= 0 && (int64_t)m.doc_len[i] + m.qry_len[i] <= lay->max_path_len,
-                   SP_ERR_INVALID_ARG, "layout: path %d has lengths (%d, %d) outside [0, max_path_len = %d]", i, m.doc_len[i],
-                   m.qry_len[i], lay->max_path_len);
-        const int64_t n = (int64_t)m.doc_len[i] + m.qry_len[i];
-        SP_REQUIRE(m.path_start[i] >= 0 && m.path_start[i] + n <= T, SP_ERR_INVALID_ARG,
-                   "layout: path %d leaves [0, total_tokens)", i);
-        if (n) seg.emplace_back(m.path_start[i], m.path_start[i] + n);
-    }
+    for (int i = 0; i < NP; ++i)
+        if (m.doc_len[i] + m.qry_len[i]) seg.emplace_back(m.path_start[i], (int64_t)m.path_start[i] + m.doc_len[i] + m.qry_len[i]);
     std::sort(seg.begin(), seg.end());
     for (size_t i = 1; i < seg.size(); ++i)
         SP_REQUIRE(seg[i].first >= seg[i - 1].second, SP_ERR_INVALID_ARG,
                    "layout: the segments starting at rows %lld and %lld overlap", (long long)seg[i - 1].first, (long long)seg[i].first);
     return SP_OK;
+}
+
+// base^(-2m / rot_dim) for m < rot_dim / 2: one logarithm and an exponential each (std::pow, 64 times, was 2.5 us of a call).
+void rope_inv_freq(double base, int rot_dim, double *out)
+{
+    const double step = -2.0 * std::log(base) / rot_dim;
+    for (int m = 0; m < rot_dim / 2; ++m) out[m] = std::exp(step * m);
 }
 
 }  // namespace sp

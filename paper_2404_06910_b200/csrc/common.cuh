@@ -37,6 +37,7 @@ inline int elt_bytes(int dtype) { return dtype == SP_F32 ? 4 : 2; }
 __host__ __device__ constexpr size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 int check_layout(const sp_layout *lay);     // host-visible fields only (api.cu)
+void rope_inv_freq(double base, int rot_dim, double *out);   // [rot_dim / 2] (api.cu)
 
 // Device status word codes (first 4 bytes of a workspace).
 enum : uint32_t { STATUS_OK = 0, STATUS_TIMEOUT = 1, STATUS_BAD_LAYOUT = 2 };

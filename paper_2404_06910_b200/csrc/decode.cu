@@ -801,7 +801,7 @@ static int decode_with_workspace(const void *q, const void *k_cache, const void 
         const int group = n_heads / n_kv_heads;
         SP_REQUIRE(group == 1 || group == 2 || group == 4, SP_ERR_UNSUPPORTED,
                    "sp_pruned_decode_rope: %d query heads per KV head (1, 2 or 4 supported: one block must own the new key)", group);
-        for (int m = 0; m < head_dim / 2; ++m) rope.inv_freq[m] = std::pow(rope_base, -2.0 * m / head_dim);
+        rope_inv_freq(rope_base, head_dim, rope.inv_freq);
         return launch_decode_any<false, true>(a, rope, pairing, lay->n_prompts, max_keys, head_dim, dtype, st);
     }
     return slopes ? launch_decode_any<true, false>(a, rope, 0, lay->n_prompts, max_keys, head_dim, dtype, st)

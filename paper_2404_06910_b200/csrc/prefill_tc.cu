@@ -851,7 +851,7 @@ int launch_prefill_tc_rope(const void *q, const void *k, const void *v, const sp
     RopeRows r;
     r.q = static_cast<const __nv_bfloat16 *>(q); r.out = static_cast<__nv_bfloat16 *>(out); r.pos = pos;
     r.n_heads = n_heads; r.half_split = pairing == SP_ROPE_HALF_SPLIT;
-    for (int m = 0; m < 64; ++m) r.inv_freq[m] = std::pow(base, -2.0 * m / 128);
+    rope_inv_freq(base, 128, r.inv_freq);
     return launch_tc(out, k, v, lay, nullptr, nullptr, &r, n_heads, n_kv_heads, 128, scale, SP_ROWS_ALL, out, lse, ws, st);
 }
 

@@ -180,7 +180,7 @@ static int rope_entry(const char *name, void *x, int64_t ld_token, int n_heads, 
                SP_ERR_INVALID_ARG, "%s: x is not aligned to its element size", name);
 
     RopeFreq fr;
-    for (int m = 0; m < rot_dim / 2; ++m) fr.inv_freq[m] = std::pow(base, -2.0 * m / rot_dim);
+    rope_inv_freq(base, rot_dim, fr.inv_freq);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     return dtype == SP_F32
                ? launch_rope<float>(x, x1, pos, n_tokens, ld_token, ld_token1, n_heads, n_heads1, head_dim, rot_dim, pairing, fr, st)
