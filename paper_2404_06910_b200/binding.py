@@ -13,6 +13,8 @@ from dataclasses import dataclass
 import numpy as np
 import torch
 
+from . import _marshal
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 # SP_B200_DEBUG_BOUNDS=1 selects the twin built with -DSP_DEBUG_BOUNDS (extra device-side layout checks)
 LIB_PATH = os.path.join(_HERE, "libsp_b200_debug.so" if os.environ.get("SP_B200_DEBUG_BOUNDS") == "1" else "libsp_b200.so")
@@ -103,9 +105,35 @@ def _load() -> ctypes.CDLL:
 
 lib = _load()
 
+# The launching entry points go through the native marshalling module: its case number (the order here) and the kind of every
+# argument, t / r contiguous / strided tensor or None, a address, i integer, d floating point.
+_KINDS = (
+    ("sp_rope_apply", "rriiiiidiia"),
+    ("sp_rope_apply_pair", "riiriiriiidiia"),
+    ("sp_superpose_prefill", "tttaiiidittti" "ia"),
+    ("sp_superpose_prefill_alibi", "tttattiiidittti" "ia"),
+    ("sp_superpose_prefill_rope", "tttatdiiiidttti" "ia"),
+    ("sp_path_scores", "rittiiitttttiia"),
+    ("sp_prune_topk", "ttiitta"),
+    ("sp_pruned_decode", "tttatitttiiiiidttti" "ia"),
+    ("sp_pruned_decode_alibi", "tttatitttiittttiiidttti" "ia"),
+    ("sp_pruned_decode_rope", "tttatitttiitdiiiidttia"),
+    ("sp_pruned_decode_static", "tttatitttiiiiidttia"),
+)
+for _i, (_name, _kinds) in enumerate(_KINDS):
+    _marshal.bind(_i, ctypes.cast(getattr(lib, _name), ctypes.c_void_p).value, _kinds)
+(_ROPE, _ROPE_PAIR, _PREFILL, _PREFILL_ALIBI, _PREFILL_ROPE, _SCORES, _TOPK, _DECODE, _DECODE_ALIBI, _DECODE_ROPE,
+ _DECODE_STATIC) = range(len(_KINDS))
+
 
 def _check(rc: int):
     if rc != SP_OK:
+        raise SpError(rc, lib.sp_last_error().decode())
+
+
+def _call(*args):
+    rc = _marshal.call(*args)
+    if rc:
         raise SpError(rc, lib.sp_last_error().decode())
 
 
@@ -134,7 +162,7 @@ def _stream(stream=None):
     if stream is not None:
         return stream.cuda_stream
     # the current stream's handle without a Stream object around it (1.5 us of every call)
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 @dataclass
@@ -187,9 +215,8 @@ def sp_rope_apply(x: torch.Tensor, pos: torch.Tensor, n_heads: int, head_dim: in
     """In place on x ([n_tokens, n_heads, head_dim] with token stride ld_token elements)."""
     n = pos.numel() if n_tokens is None else n_tokens
     ld = n_heads * head_dim if ld_token is None else ld_token
-    _check(lib.sp_rope_apply(x.data_ptr(), pos.data_ptr(), n, ld, n_heads, head_dim,
-                             head_dim if rot_dim is None else rot_dim, base, pairing, dtype_code(x),
-                             _stream(stream)))
+    _call(_ROPE, x, pos, n, ld, n_heads, head_dim, head_dim if rot_dim is None else rot_dim, base, pairing,
+          dtype_code(x), _stream(stream))
 
 
 def sp_rope_apply_pair(xq: torch.Tensor, n_heads_q: int, xk: torch.Tensor, n_heads_k: int, pos: torch.Tensor,
@@ -197,10 +224,9 @@ def sp_rope_apply_pair(xq: torch.Tensor, n_heads_q: int, xk: torch.Tensor, n_hea
                        pairing: int = SP_ROPE_HALF_SPLIT, stream=None):
     """sp_rope_apply on a step's queries and keys (same positions) in one launch, in place."""
     n = pos.numel() if n_tokens is None else n_tokens
-    _check(lib.sp_rope_apply_pair(xq.data_ptr(), n_heads_q * head_dim if ld_q is None else ld_q, n_heads_q,
-                                  xk.data_ptr(), n_heads_k * head_dim if ld_k is None else ld_k, n_heads_k,
-                                  pos.data_ptr(), n, head_dim, head_dim if rot_dim is None else rot_dim, base,
-                                  pairing, dtype_code(xq), _stream(stream)))
+    _call(_ROPE_PAIR, xq, n_heads_q * head_dim if ld_q is None else ld_q, n_heads_q, xk, n_heads_k * head_dim if
+          ld_k is None else ld_k, n_heads_k, pos, n, head_dim, head_dim if rot_dim is None else rot_dim, base,
+          pairing, dtype_code(xq), _stream(stream))
 
 
 def sp_prefill_workspace_bytes(lay: DeviceLayout, n_heads: int, head_dim: int, dtype: int) -> int:
@@ -212,8 +238,8 @@ def sp_superpose_prefill(q, k, v, lay: DeviceLayout, scale: float, out, lse=None
                          rows: int = SP_ROWS_ALL, stream=None):
     T, H, D = q.shape
     Hkv = k.shape[1]
-    _check(lib.sp_superpose_prefill(_ptr(q), _ptr(k), _ptr(v), ctypes.byref(lay.c), H, Hkv, D, scale, rows,
-                                    _ptr(out), _ptr(lse), _ptr(ws), _nbytes(ws), dtype_code(q), _stream(stream)))
+    _call(_PREFILL, q, k, v, ctypes.addressof(lay.c), H, Hkv, D, scale, rows, out, lse, ws, _nbytes(ws),
+          dtype_code(q), _stream(stream))
 
 
 def sp_superpose_prefill_alibi(q, k, v, lay: DeviceLayout, pos, slopes, scale: float, out, lse=None, ws=None,
@@ -221,9 +247,8 @@ def sp_superpose_prefill_alibi(q, k, v, lay: DeviceLayout, pos, slopes, scale: f
     """sp_superpose_prefill with the ALiBi bias -slopes[h] * |pos[q] - pos[k]| (pos fp32 [T], slopes fp32 [H])."""
     T, H, D = q.shape
     Hkv = k.shape[1]
-    _check(lib.sp_superpose_prefill_alibi(_ptr(q), _ptr(k), _ptr(v), ctypes.byref(lay.c), _ptr(pos), _ptr(slopes), H,
-                                          Hkv, D, scale, rows, _ptr(out), _ptr(lse), _ptr(ws), _nbytes(ws),
-                                          dtype_code(q), _stream(stream)))
+    _call(_PREFILL_ALIBI, q, k, v, ctypes.addressof(lay.c), pos, slopes, H, Hkv, D, scale, rows, out, lse, ws,
+          _nbytes(ws), dtype_code(q), _stream(stream))
 
 
 def sp_prefill_rope_workspace_bytes(lay: DeviceLayout, n_heads: int, head_dim: int, dtype: int) -> int:
@@ -236,9 +261,8 @@ def sp_superpose_prefill_rope(q, k, v, lay: DeviceLayout, pos, base: float, pair
     """sp_superpose_prefill over all rows with the rotation of the (unrotated) q folded in; k already rotated."""
     T, H, D = q.shape
     Hkv = k.shape[1]
-    _check(lib.sp_superpose_prefill_rope(_ptr(q), _ptr(k), _ptr(v), ctypes.byref(lay.c), _ptr(pos), base, pairing, H,
-                                         Hkv, D, scale, _ptr(out), _ptr(lse), _ptr(ws), _nbytes(ws), dtype_code(q),
-                                         _stream(stream)))
+    _call(_PREFILL_ROPE, q, k, v, ctypes.addressof(lay.c), pos, base, pairing, H, Hkv, D, scale, out, lse, ws,
+          _nbytes(ws), dtype_code(q), _stream(stream))
 
 
 def sp_path_scores_workspace_bytes(n_rows: int) -> int:
@@ -248,14 +272,12 @@ def sp_path_scores_workspace_bytes(n_rows: int) -> int:
 def sp_path_scores(logits, targets, row_off, scores, prior=None, weight=None, row_logp=None, ws=None,
                    stream=None):
     R, V = logits.shape
-    _check(lib.sp_path_scores(logits.data_ptr(), logits.stride(0) if R else V, _ptr(targets), _ptr(row_off), R,
-                              row_off.numel() - 1, V, _ptr(prior), _ptr(weight), _ptr(scores), _ptr(row_logp),
-                              _ptr(ws), _nbytes(ws), dtype_code(logits), _stream(stream)))
+    _call(_SCORES, logits, logits.stride(0) if R else V, targets, row_off, R, row_off.numel() - 1, V, prior,
+          weight, scores, row_logp, ws, _nbytes(ws), dtype_code(logits), _stream(stream))
 
 
 def sp_prune_topk(scores, prompt_path_off, k: int, kept_idx, kept_post=None, stream=None):
-    _check(lib.sp_prune_topk(_ptr(scores), _ptr(prompt_path_off), prompt_path_off.numel() - 1, k,
-                             _ptr(kept_idx), _ptr(kept_post), _stream(stream)))
+    _call(_TOPK, scores, prompt_path_off, prompt_path_off.numel() - 1, k, kept_idx, kept_post, _stream(stream))
 
 
 def sp_decode_workspace_bytes(n_prompts: int, n_heads: int, head_dim: int) -> int:
@@ -266,9 +288,8 @@ def sp_pruned_decode(q, k_cache, v_cache, lay: DeviceLayout, kept_idx, k: int, t
                      tail_cap: int, scale: float, out, lse=None, ws=None, max_keys: int = 0, stream=None):
     B, H, D = q.shape
     Hkv = k_cache.shape[1]
-    _check(lib.sp_pruned_decode(_ptr(q), _ptr(k_cache), _ptr(v_cache), ctypes.byref(lay.c), _ptr(kept_idx), k,
-                                _ptr(tail_k), _ptr(tail_v), _ptr(tail_len), tail_cap, max_keys, H, Hkv, D, scale,
-                                _ptr(out), _ptr(lse), _ptr(ws), _nbytes(ws), dtype_code(q), _stream(stream)))
+    _call(_DECODE, q, k_cache, v_cache, ctypes.addressof(lay.c), kept_idx, k, tail_k, tail_v, tail_len,
+          tail_cap, max_keys, H, Hkv, D, scale, out, lse, ws, _nbytes(ws), dtype_code(q), _stream(stream))
 
 
 def sp_pruned_decode_alibi(q, k_cache, v_cache, lay: DeviceLayout, kept_idx, k: int, tail_k, tail_v, tail_len,
@@ -278,10 +299,9 @@ def sp_pruned_decode_alibi(q, k_cache, v_cache, lay: DeviceLayout, kept_idx, k: 
     slopes fp32 [H]."""
     B, H, D = q.shape
     Hkv = k_cache.shape[1]
-    _check(lib.sp_pruned_decode_alibi(_ptr(q), _ptr(k_cache), _ptr(v_cache), ctypes.byref(lay.c), _ptr(kept_idx), k,
-                                      _ptr(tail_k), _ptr(tail_v), _ptr(tail_len), tail_cap, max_keys, _ptr(q_pos),
-                                      _ptr(cache_pos), _ptr(tail_pos), _ptr(slopes), H, Hkv, D, scale, _ptr(out),
-                                      _ptr(lse), _ptr(ws), _nbytes(ws), dtype_code(q), _stream(stream)))
+    _call(_DECODE_ALIBI, q, k_cache, v_cache, ctypes.addressof(lay.c), kept_idx, k, tail_k, tail_v, tail_len,
+          tail_cap, max_keys, q_pos, cache_pos, tail_pos, slopes, H, Hkv, D, scale, out, lse, ws, _nbytes(ws),
+          dtype_code(q), _stream(stream))
 
 
 def sp_pruned_decode_rope(q, k_cache, v_cache, lay: DeviceLayout, kept_idx, k: int, tail_k, tail_v, tail_len,
@@ -291,10 +311,8 @@ def sp_pruned_decode_rope(q, k_cache, v_cache, lay: DeviceLayout, kept_idx, k: i
     unrotated and are rotated at q_pos (fp32 [B]); the key row is written back rotated."""
     B, H, D = q.shape
     Hkv = k_cache.shape[1]
-    _check(lib.sp_pruned_decode_rope(_ptr(q), _ptr(k_cache), _ptr(v_cache), ctypes.byref(lay.c), _ptr(kept_idx), k,
-                                     _ptr(tail_k), _ptr(tail_v), _ptr(tail_len), tail_cap, max_keys, _ptr(q_pos),
-                                     base, pairing, H, Hkv, D, scale, _ptr(out), _ptr(lse), dtype_code(q),
-                                     _stream(stream)))
+    _call(_DECODE_ROPE, q, k_cache, v_cache, ctypes.addressof(lay.c), kept_idx, k, tail_k, tail_v, tail_len,
+          tail_cap, max_keys, q_pos, base, pairing, H, Hkv, D, scale, out, lse, dtype_code(q), _stream(stream))
 
 
 def sp_pruned_decode_static_max_bytes() -> int:
@@ -307,9 +325,8 @@ def sp_pruned_decode_static(q, k_cache, v_cache, lay: DeviceLayout, kept_idx, k:
     fixed array inside the library (see include/sp.h for its limit and sharing rules)."""
     B, H, D = q.shape
     Hkv = k_cache.shape[1]
-    _check(lib.sp_pruned_decode_static(_ptr(q), _ptr(k_cache), _ptr(v_cache), ctypes.byref(lay.c), _ptr(kept_idx),
-                                       k, _ptr(tail_k), _ptr(tail_v), _ptr(tail_len), tail_cap, max_keys, H, Hkv,
-                                       D, scale, _ptr(out), _ptr(lse), dtype_code(q), _stream(stream)))
+    _call(_DECODE_STATIC, q, k_cache, v_cache, ctypes.addressof(lay.c), kept_idx, k, tail_k, tail_v, tail_len,
+          tail_cap, max_keys, H, Hkv, D, scale, out, lse, dtype_code(q), _stream(stream))
 
 
 def sp_check_status(ws, stream=None) -> None:

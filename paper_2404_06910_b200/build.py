@@ -1,10 +1,12 @@
 """Builds the CUDA library in-tree: every csrc/*.cu -> libsp_b200.so (sm_100a only), and the same
-sources with -DSP_DEBUG_BOUNDS (extra device-side layout checks) -> libsp_b200_debug.so."""
+sources with -DSP_DEBUG_BOUNDS (extra device-side layout checks) -> libsp_b200_debug.so; and the Python argument
+marshalling, csrc/marshal.c -> _marshal.so."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -13,6 +15,7 @@ OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libsp_b200.so")
 OBJ_DEBUG = os.path.join(HERE, "_build_debug")
 LIB_DEBUG = os.path.join(HERE, "libsp_b200_debug.so")
+MARSHAL = os.path.join(HERE, "_marshal.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -59,8 +62,18 @@ def _build_one(lib: str, obj_dir: str, extra, force: bool, verbose: bool) -> str
     return lib
 
 
+def _build_marshal(force: bool) -> None:
+    src = os.path.join(CSRC, "marshal.c")
+    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= os.path.getmtime(src):
+        return
+    tmp = MARSHAL + f".tmp{os.getpid()}"
+    subprocess.check_call(["gcc", "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], src, "-o", tmp])
+    os.replace(tmp, MARSHAL)
+
+
 def build(force: bool = False, verbose: bool = False, debug: bool = True) -> str:
     """Builds the library and (debug=True) its bounds-checking twin; returns the library's path."""
+    _build_marshal(force)
     lib = _build_one(LIB, OBJ, (), force, verbose)
     if debug:
         _build_one(LIB_DEBUG, OBJ_DEBUG, ("-DSP_DEBUG_BOUNDS",), force, verbose)
