@@ -53,6 +53,37 @@ __device__ __forceinline__ void rope_rotate(float a, float b, float c, float s, 
 #endif
 int num_sms();                              // multiprocessors of the current device (api.cu)
 
+// ---- programmatic dependent launch -------------------------------------------------
+// Every kernel of the library is launched as a programmatic dependent of what precedes it in the stream: its blocks may be
+// scheduled, and set themselves up, while the last blocks of the kernel before are still running, which takes launch latency
+// and ramp-up off every boundary of a chain of short kernels.  In return every thread of every kernel calls
+// pdl_wait() before it touches global memory; after it, everything earlier in the stream is complete and visible.
+// pdl_trigger() lets the next kernel's blocks in as soon as all blocks of this one have started.  One prompt of 20 documents,
+// whole step: 93 -> 83 us; 4 documents in fp32: 39 -> 29.
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+int launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, unsigned cluster_x, A &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster_x; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster_x > 1 ? 2 : 1;
+    SP_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
+    return SP_OK;
+}
+#endif
+
 // ---- device helpers ----------------------------------------------------------------
 #ifdef __CUDACC__
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }

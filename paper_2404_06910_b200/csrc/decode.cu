@@ -95,6 +95,7 @@ decode_kernel(const __grid_constant__ DecodeArgs a)
     float *red = reinterpret_cast<float *>(seg_v + n_seg);                  // [G][D+2]
     const float **seg_pos = reinterpret_cast<const float **>(red + G * (D + 2));   // [n_seg], ALiBi only
     __shared__ unsigned int s_ticket;
+    pdl_wait();
 
     const int split = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
     const int hk = h / (a.n_heads / a.n_kv_heads);
@@ -271,9 +272,7 @@ static int launch_decode_v(const DecodeArgs &a, int n_prompts, cudaStream_t st)
     if (smem > 48 * 1024)
         SP_CUDA(cudaFuncSetAttribute(decode_kernel<T, D, ALIBI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     dim3 grid(a.n_splits, a.n_heads, n_prompts);
-    decode_kernel<T, D, ALIBI><<<grid, kDecThreads, smem, st>>>(a);
-    SP_CUDA(cudaGetLastError());
-    return SP_OK;
+    return launch(decode_kernel<T, D, ALIBI>, grid, kDecThreads, smem, st, 1, a);
 }
 template <typename T, int D>
 static int launch_decode(const DecodeArgs &a, int n_prompts, cudaStream_t st)
@@ -440,6 +439,9 @@ decode_cluster_kernel(const __grid_constant__ DecodeArgs a, const __grid_constan
     const int h0 = hk * group + (blockIdx.y - hk * per_kv) * GRP;   // first query head of this block
     const int64_t row_elems = (int64_t)a.n_kv_heads * D;
 
+    // No pdl_trigger(): letting the next launch's clusters in early makes them wait in slots and slows both (2 prompts x 400
+    // documents, us per step: 24.6 without, 30.2 with a trigger behind the key loop, 34.8 with one here).
+    pdl_wait();
     decode_segments<T, ALIBI>(a, sm, n_seg, b, hk, D, row_elems);
     if (ROPE) decode_angles<D>(a, rope, b, cs);
     __syncthreads();
@@ -671,18 +673,7 @@ static int launch_cluster_kernel(K kern, const DecodeArgs &a, const DecodeRope &
         SP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (a.n_splits > 8)
         SP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.n_splits, blocks_y, n_prompts);
-    cfg.blockDim = dim3(kDecThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = a.n_splits; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = a.n_splits > 1 ? 1 : 0;      // one block per (prompt, KV head group): a plain launch
-    SP_CUDA(cudaLaunchKernelEx(&cfg, kern, a, rope, pairing));
-    return SP_OK;
+    return launch(kern, dim3(a.n_splits, blocks_y, n_prompts), kDecThreads, smem, st, a.n_splits, a, rope, pairing);
 }
 
 template <int D, bool ALIBI, bool ROPE>

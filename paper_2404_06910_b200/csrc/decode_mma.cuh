@@ -48,6 +48,7 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
     const int h0 = hk * group + sub_group * kMmaHeads, nh = min(kMmaHeads, group - sub_group * kMmaHeads);
     const int64_t row_elems = (int64_t)a.n_kv_heads * D;
 
+    pdl_wait();
     decode_segments<T, ALIBI>(a, sm, n_seg, b, hk, D, row_elems);
     if (ROPE) decode_angles<D>(a, rope, b, cs);
     __syncthreads();

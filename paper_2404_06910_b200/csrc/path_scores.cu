@@ -49,6 +49,8 @@ __global__ void __launch_bounds__(kScoreThreads)
 row_logp_kernel(const T *__restrict__ logits, int64_t ld, const int32_t *__restrict__ targets,
                 int vocab, float *__restrict__ row_logp)
 {
+    pdl_wait();
+    pdl_trigger();
     const int64_t t = blockIdx.x;
     const int32_t y = targets[t];
     if (y < 0 || y >= vocab) {           // no target: contributes nothing, row is not read
@@ -122,6 +124,8 @@ path_sum_kernel(const float *__restrict__ row_logp, const int32_t *__restrict__ 
                 const float *__restrict__ prior, const float *__restrict__ weight,
                 float *__restrict__ scores)
 {
+    pdl_wait();
+    pdl_trigger();
     const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (i >= n_paths) return;
     const int lane = threadIdx.x & 31;
@@ -169,19 +173,16 @@ extern "C" int sp_path_scores(const void *logits, int64_t ld_logits, const int32
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (n_rows > 0) {
         const bool vec = aligned16(logits) && ((ld_logits * elt_bytes(dtype)) % 16 == 0);
-        const unsigned grid = (unsigned)n_rows;
+        auto go = [&](auto kern, auto *p) { return launch(kern, (unsigned)n_rows, kScoreThreads, 0, st, 1, p, ld_logits, targets, vocab, rows_out); };
+        int rc;
         if (dtype == SP_BF16) {
             auto *p = static_cast<const __nv_bfloat16 *>(logits);
-            if (vec) row_logp_kernel<__nv_bfloat16, true><<<grid, kScoreThreads, 0, st>>>(p, ld_logits, targets, vocab, rows_out);
-            else     row_logp_kernel<__nv_bfloat16, false><<<grid, kScoreThreads, 0, st>>>(p, ld_logits, targets, vocab, rows_out);
+            rc = vec ? go(row_logp_kernel<__nv_bfloat16, true>, p) : go(row_logp_kernel<__nv_bfloat16, false>, p);
         } else {
             auto *p = static_cast<const float *>(logits);
-            if (vec) row_logp_kernel<float, true><<<grid, kScoreThreads, 0, st>>>(p, ld_logits, targets, vocab, rows_out);
-            else     row_logp_kernel<float, false><<<grid, kScoreThreads, 0, st>>>(p, ld_logits, targets, vocab, rows_out);
+            rc = vec ? go(row_logp_kernel<float, true>, p) : go(row_logp_kernel<float, false>, p);
         }
-        SP_CUDA(cudaGetLastError());
+        if (rc) return rc;
     }
-    path_sum_kernel<<<(n_paths + 7) / 8, 256, 0, st>>>(rows_out, row_off, n_paths, prior, weight, scores);
-    SP_CUDA(cudaGetLastError());
-    return SP_OK;
+    return launch(path_sum_kernel, (n_paths + 7) / 8, 256, 0, st, 1, rows_out, row_off, n_paths, prior, weight, scores);
 }

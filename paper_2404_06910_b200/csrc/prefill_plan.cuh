@@ -57,7 +57,8 @@ static __global__ void __launch_bounds__(1024) prefill_plan_kernel(const PlanArg
 {
     __shared__ int warp_tot[32];
     __shared__ int running;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // a dependent kernel may set itself up meanwhile
+    pdl_trigger();                    // the attention kernel sets itself up meanwhile
+    pdl_wait();
     if (threadIdx.x == 0) { running = 0; a.hdr->status = STATUS_OK; }
     __syncthreads();
     const int n_seq = a.n_prompts + a.n_paths;

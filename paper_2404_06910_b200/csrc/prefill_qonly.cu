@@ -156,6 +156,8 @@ __global__ void __launch_bounds__(kQThreads, kQBlocksPerSM) prefill_qonly_kernel
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gid = lane >> 2, tig = lane & 3;
+    pdl_wait();
+    pdl_trigger();
     const uint32_t n_items = p.hdr->n_tiles * (uint32_t)p.n_heads;
     const int64_t q_pitch = (int64_t)p.n_heads * kRowB, kv_pitch = (int64_t)p.n_kv_heads * kRowB;
 
@@ -347,8 +349,7 @@ int launch_prefill_qonly(const void *q, const void *k, const void *v, const sp_l
     pa.max_pre_len = lay->max_pre_len; pa.max_path_len = lay->max_path_len; pa.total_tokens = lay->total_tokens;
     pa.max_tiles = plan_max_tiles(lay->n_prompts, lay->n_paths, lay->max_pre_len, lay->max_path_len, kQM);
     pa.hdr = hdr; pa.list = tiles;
-    prefill_plan_kernel<false><<<1, 1024, 0, st>>>(pa);
-    SP_CUDA(cudaGetLastError());
+    if (int rc = launch(prefill_plan_kernel<false>, 1, 1024, 0, st, 1, pa)) return rc;
 
     const int64_t items = plan_max_tiles(0, lay->n_paths, 0, lay->max_path_len, kQM) * n_heads;
     if (items == 0) return SP_OK;
@@ -363,13 +364,11 @@ int launch_prefill_qonly(const void *q, const void *k, const void *v, const sp_l
     const int grid = (int)std::min<int64_t>(items, (int64_t)kQBlocksPerSM * num_sms());
     if (pos) {
         SP_CUDA(cudaFuncSetAttribute(prefill_qonly_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        prefill_qonly_kernel<true><<<grid, kQThreads, smem, st>>>(p);
+        return launch(prefill_qonly_kernel<true>, grid, kQThreads, smem, st, 1, p);
     } else {
         SP_CUDA(cudaFuncSetAttribute(prefill_qonly_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        prefill_qonly_kernel<false><<<grid, kQThreads, smem, st>>>(p);
+        return launch(prefill_qonly_kernel<false>, grid, kQThreads, smem, st, 1, p);
     }
-    SP_CUDA(cudaGetLastError());
-    return SP_OK;
 }
 
 }  // namespace sp

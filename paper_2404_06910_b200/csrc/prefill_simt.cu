@@ -39,6 +39,8 @@ prefill_simt_kernel(const __grid_constant__ PrefillSimtArgs a)
     __shared__ __align__(16) float sq[kSimtRows][D], sk[BN][KS], sv[BN][D], sp_[kSimtRows][BN];
     __shared__ float s_pos[BN];
 
+    pdl_wait();
+    pdl_trigger();
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *a.status = STATUS_OK;
     const int n_seq = a.n_prompts + a.n_paths;
     const int tile = blockIdx.x / n_seq, seq = blockIdx.x - tile * n_seq, h = blockIdx.y;
@@ -188,10 +190,8 @@ int launch_prefill_simt(const void *q, const void *k, const void *v, const sp_la
     const int64_t blocks = std::max<int64_t>(1, tiles) * (lay->n_prompts + lay->n_paths);
     SP_REQUIRE(blocks < (int64_t)INT32_MAX, SP_ERR_UNSUPPORTED, "sp_superpose_prefill: %lld row tiles", (long long)blocks);
     const dim3 grid((unsigned)blocks, n_heads);
-    if (head_dim == 64) prefill_simt_kernel<64><<<grid, kSimtThreads, 0, st>>>(a);
-    else                prefill_simt_kernel<128><<<grid, kSimtThreads, 0, st>>>(a);
-    SP_CUDA(cudaGetLastError());
-    return SP_OK;
+    return head_dim == 64 ? launch(prefill_simt_kernel<64>, grid, kSimtThreads, 0, st, 1, a)
+                          : launch(prefill_simt_kernel<128>, grid, kSimtThreads, 0, st, 1, a);
 }
 
 }  // namespace sp

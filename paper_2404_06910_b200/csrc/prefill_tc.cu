@@ -231,7 +231,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    grid_dependency_wait();           // the tile list and everything before it in the stream
+    pdl_trigger();
+    pdl_wait();                       // the tile list and everything before it in the stream
     const uint32_t tb = *tmem_base_s;
     bool ok = (smem_u32(smem) & 1023u) == 0;      // the swizzle atoms need it; reported like an expired wait
 
@@ -675,6 +676,8 @@ struct RopeRows {
 __global__ void __launch_bounds__(256, 8) rope_rows_kernel(const __grid_constant__ RopeRows a)
 {
     __shared__ float2 cs[kRopeRows][64];
+    pdl_wait();
+    pdl_trigger();
     constexpr uint32_t kGroups = 2 * kBM / kRopeRows;          // of an item
     const uint32_t n_groups = a.hdr->n_tiles * kGroups;
     for (uint32_t g = blockIdx.x; g < n_groups; g += gridDim.x) {
@@ -758,19 +761,7 @@ template <int D, bool ALIBI> static int launch_kernel(const TcParams &p, int gri
 {
     using C = TcConfig<D, ALIBI>;
     SP_CUDA(cudaFuncSetAttribute(prefill_tc_kernel<D, ALIBI>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kTcThreads);
-    cfg.dynamicSmemBytes = C::SMEM;
-    cfg.stream = st;
-    // The kernel sets itself up while the plan kernel still runs and waits for it on the device.
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    SP_CUDA(cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D, ALIBI>, p));
-    return SP_OK;
+    return launch(prefill_tc_kernel<D, ALIBI>, grid, kTcThreads, C::SMEM, st, 1, p);
 }
 
 static int launch_tc(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
@@ -804,14 +795,12 @@ static int launch_tc(const void *q, const void *k, const void *v, const sp_layou
     pa.max_pre_len = lay->max_pre_len; pa.max_path_len = lay->max_path_len; pa.total_tokens = lay->total_tokens;
     pa.max_tiles = max_tiles(lay->n_prompts, lay->n_paths, lay->max_pre_len, lay->max_path_len);
     pa.hdr = hdr; pa.list = pairs;
-    prefill_plan_kernel<true><<<1, 1024, 0, st>>>(pa);
-    SP_CUDA(cudaGetLastError());
+    if (int rc = launch(prefill_plan_kernel<true>, 1, 1024, 0, st, 1, pa)) return rc;
     if (rope) {
         RopeRows r = *rope;
         r.hdr = hdr; r.pairs = pairs;
         const int64_t groups = pa.max_tiles * (kBM / kRopeRows);
-        rope_rows_kernel<<<(int)std::min<int64_t>(groups, (int64_t)num_sms() * 16), 256, 0, st>>>(r);
-        SP_CUDA(cudaGetLastError());
+        if (int rc = launch(rope_rows_kernel, (unsigned)std::min<int64_t>(groups, (int64_t)num_sms() * 16), 256, 0, st, 1, r)) return rc;
     }
 
     p.hdr = hdr; p.pairs = pairs; p.status = &hdr->status;

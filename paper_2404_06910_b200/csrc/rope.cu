@@ -109,6 +109,8 @@ rope_kernel(T *__restrict__ x, T *__restrict__ x1, const float *__restrict__ pos
             const __grid_constant__ RopeFreq fr)
 {
     __shared__ float2 cs[kRopeTokens][128];   // (cos, sin) per (token, pair)
+    pdl_wait();
+    pdl_trigger();
     const int half = rot_dim >> 1;
     const int64_t n_groups = (n_tokens + kRopeTokens - 1) / kRopeTokens;
 
@@ -147,15 +149,12 @@ static int launch_rope(void *x, void *x1, const float *pos, int64_t n_tokens, in
     const int64_t n_groups = (n_tokens + kRopeTokens - 1) / kRopeTokens;
     const int grid = (int)std::min<int64_t>(n_groups, (int64_t)num_sms() * 16);
     auto go = [&](auto kern) {
-        kern<<<grid, kRopeThreads, 0, st>>>((T *)x, (T *)x1, pos, n_tokens, ld_token, ld_token1, n_heads, n_heads1,
-                                            head_dim, rot_dim, pairing, fr);
+        return launch(kern, grid, kRopeThreads, 0, st, 1, (T *)x, (T *)x1, pos, n_tokens, ld_token, ld_token1, n_heads, n_heads1,
+                      head_dim, rot_dim, pairing, fr);
     };
-    if (v0 && v1) go(rope_kernel<T, true, true>);
-    else if (v0) go(rope_kernel<T, true, false>);
-    else if (v1) go(rope_kernel<T, false, true>);
-    else go(rope_kernel<T, false, false>);
-    SP_CUDA(cudaGetLastError());
-    return SP_OK;
+    if (v0 && v1) return go(rope_kernel<T, true, true>);
+    if (v0) return go(rope_kernel<T, true, false>);
+    return v1 ? go(rope_kernel<T, false, true>) : go(rope_kernel<T, false, false>);
 }
 
 static int rope_entry(const char *name, void *x, int64_t ld_token, int n_heads, void *x1, int64_t ld_token1, int n_heads1,

@@ -206,8 +206,6 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
           "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
           "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]) : "memory");
 }
-// Waits until the grids this one was launched behind (programmatic dependent launch) are complete and visible.
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // 32 bytes to a 32-byte aligned global address, one full sector per thread; the line is not kept in L1.
 __device__ __forceinline__ void st_global_32b(void *p, const uint32_t (&r)[8])
 {

@@ -33,6 +33,8 @@ __global__ void __launch_bounds__(128)
 prune_topk_kernel(const float *__restrict__ scores, const int32_t *__restrict__ ppo, int n_prompts,
                   int k, int32_t *__restrict__ kept_idx, float *__restrict__ kept_post)
 {
+    pdl_wait();
+    pdl_trigger();
     const int b = blockIdx.x * 4 + (threadIdx.x >> 5);
     if (b >= n_prompts) return;
     const int lane = threadIdx.x & 31;
@@ -91,8 +93,6 @@ extern "C" int sp_prune_topk(const float *scores, const int32_t *prompt_path_off
     SP_REQUIRE(n_prompts >= 0, SP_ERR_INVALID_ARG, "sp_prune_topk: n_prompts < 0");
     if (n_prompts == 0) return SP_OK;
     SP_REQUIRE(scores && prompt_path_off && kept_idx, SP_ERR_INVALID_ARG, "sp_prune_topk: NULL pointer");
-    prune_topk_kernel<<<(n_prompts + 3) / 4, 128, 0, static_cast<cudaStream_t>(stream)>>>(
-        scores, prompt_path_off, n_prompts, k, kept_idx, kept_post);
-    SP_CUDA(cudaGetLastError());
-    return SP_OK;
+    return launch(prune_topk_kernel, (n_prompts + 3) / 4, 128, 0, static_cast<cudaStream_t>(stream), 1, scores, prompt_path_off,
+                  n_prompts, k, kept_idx, kept_post);
 }
