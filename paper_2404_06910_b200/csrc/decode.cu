@@ -62,6 +62,7 @@ __device__ __forceinline__ uint4 ld_stream16(const void *p)
                  : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w) : "l"(p));
     return w;
 }
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 template <typename T> struct Raw16;
 template <> struct Raw16<__nv_bfloat16> {
     __device__ __forceinline__ static void unpack(const uint4 &w, float (&f)[8]) {
@@ -315,7 +316,7 @@ static size_t decode_table_bytes(int n_seg) { return round_up((n_seg + 1) * size
 template <typename T, bool ALIBI>
 __device__ __forceinline__ void decode_segments(const DecodeArgs &a, const DecodeSmem<T> &sm, int n_seg, int b, int hk, int D, int64_t row_elems)
 {
-    for (int sgm = threadIdx.x; sgm < n_seg; sgm += kDecThreads) {
+    for (int sgm = threadIdx.x; sgm < n_seg; sgm += blockDim.x) {
         const T *kc = static_cast<const T *>(a.k_cache) + (int64_t)hk * D;
         const T *vc = static_cast<const T *>(a.v_cache) + (int64_t)hk * D;
         int len = 0;
@@ -366,13 +367,14 @@ template <typename T> __device__ __forceinline__ void decode_scan(const DecodeSm
 // far below one rounding of the rotated values.
 template <int D> __device__ __forceinline__ void decode_angles(const DecodeArgs &a, const DecodeRope &rope, int b, float2 *cs)
 {
-    if (threadIdx.x >= D / 2) return;
-    const double ang = (double)a.q_pos[b] * rope.inv_freq[threadIdx.x];
-    const double turns = rint(ang * 0.15915494309189535);
-    const double r = fma(-turns, 2.4492935982947064e-16, fma(-turns, 6.283185307179586, ang));
-    float sn, cn;
-    sincosf((float)r, &sn, &cn);
-    cs[threadIdx.x] = make_float2(cn, sn);
+    for (int m = threadIdx.x; m < D / 2; m += blockDim.x) {
+        const double ang = (double)a.q_pos[b] * rope.inv_freq[m];
+        const double turns = rint(ang * 0.15915494309189535);
+        const double r = fma(-turns, 2.4492935982947064e-16, fma(-turns, 6.283185307179586, ang));
+        float sn, cn;
+        sincosf((float)r, &sn, &cn);
+        cs[m] = make_float2(cn, sn);
+    }
 }
 
 // Element d of one (prompt, head): maximum bm (log2 units), sum bl and unnormalised output bo -> out, lse.
@@ -383,30 +385,42 @@ __device__ __forceinline__ void decode_store(const DecodeArgs &a, int64_t bh, in
     if (d == 0 && a.lse) a.lse[bh] = bl > 0.f ? (bm + log2f(bl)) * kLn2D : -INFINITY;
 }
 
-// Merges the blocks' partials [heads][D + 2] through the cluster's shared memory, in split order, and stores them: element d of
-// heads r0, r0 + dr, ..; r0 < 0: this thread has none.
-template <typename T, int D>
-__device__ __forceinline__ void decode_cluster_merge(const DecodeArgs &a, float *part, int split, int n_heads, int d, int r0, int dr, int64_t bh0)
+// The merge over the blocks of a cluster: every block writes its partials into the first block's shared memory and leaves;
+// the first one waits and merges what has arrived, in split order.  decode_cluster_begin() at the start of the kernel and
+// decode_cluster_target() before the writes see to it that the first block is there to be written to.
+__device__ __forceinline__ void decode_cluster_begin(const DecodeArgs &a)
 {
-    namespace cg = cooperative_groups;
+    if (a.n_splits > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+// This block's slot of `floats` numbers in the first block's array.
+__device__ __forceinline__ float *decode_cluster_target(const DecodeArgs &a, float *part, int floats)
+{
+    if (a.n_splits == 1) return part;
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    return cooperative_groups::this_cluster().map_shared_rank(part, 0) + blockIdx.x * floats;
+}
+// After the writes: merges [n_splits][n_heads][D + 2] and stores the heads bh0 .. ; element index idx = head * D + d.
+template <typename T, int D>
+__device__ __forceinline__ void decode_cluster_merge(const DecodeArgs &a, const float *part, int n_heads, int64_t bh0)
+{
     constexpr int PS = D + 2;
-    cg::cluster_group cluster = cg::this_cluster();
-    cluster.sync();
-    if (split == 0 && r0 >= 0) {
-        for (int r = r0; r < n_heads; r += dr) {
-            float M = -INFINITY;
-            for (int i = 0; i < a.n_splits; ++i) M = fmaxf(M, cluster.map_shared_rank(part, i)[r * PS + D]);
-            float L = 0.f, O = 0.f;
-            for (int i = 0; i < a.n_splits; ++i) {
-                const float *rp = cluster.map_shared_rank(part, i) + r * PS;
-                const float w = (rp[D] == -INFINITY) ? 0.f : ex2f(rp[D] - M);
-                L += rp[D + 1] * w;
-                O += rp[d] * w;
-            }
-            decode_store<T>(a, bh0 + r, D, d, M, L, O);
+    if (a.n_splits == 1) return;            // stored already
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    if (blockIdx.x != 0) return;
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    for (int idx = threadIdx.x; idx < n_heads * D; idx += blockDim.x) {
+        const int r = idx / D, d = idx & (D - 1);
+        float M = -INFINITY;
+        for (int i = 0; i < a.n_splits; ++i) M = fmaxf(M, part[(i * n_heads + r) * PS + D]);
+        float L = 0.f, O = 0.f;
+        for (int i = 0; i < a.n_splits; ++i) {
+            const float *rp = part + (i * n_heads + r) * PS;
+            const float w = (rp[D] == -INFINITY) ? 0.f : ex2f(rp[D] - M);
+            L += rp[D + 1] * w;
+            O += rp[d] * w;
         }
+        decode_store<T>(a, bh0 + r, D, d, M, L, O);
     }
-    cluster.sync();                     // the others' shared memory stays alive until it has been read
 }
 
 // MINB: resident blocks per SM the register budget is sized for.  Split launches want 8 (a whole
@@ -429,8 +443,8 @@ decode_cluster_kernel(const __grid_constant__ DecodeArgs a, const __grid_constan
     const T **seg_k = sm.k, **seg_v = sm.v;
     const float **seg_pos = sm.pos;
     float *red = sm.end;                                                    // [G][GRP][PS]
-    float *part = red + G * GRP * PS;                                       // [GRP][PS], read by the cluster's first block
-    float2 *cs = reinterpret_cast<float2 *>(part + GRP * PS);               // [D/2] (cos, sin), ROPE only
+    float2 *cs = reinterpret_cast<float2 *>(red + G * GRP * PS);            // [D/2] (cos, sin), ROPE only
+    float *part = reinterpret_cast<float *>(cs + D / 2);                    // first block: [n_splits][GRP][PS]
 
     const int split = blockIdx.x, b = blockIdx.z;
     const int group = a.n_heads / a.n_kv_heads;                 // query heads per KV head
@@ -441,7 +455,13 @@ decode_cluster_kernel(const __grid_constant__ DecodeArgs a, const __grid_constan
 
     // No pdl_trigger(): letting the next launch's clusters in early makes them wait in slots and slows both (2 prompts x 400
     // documents, us per step: 24.6 without, 30.2 with a trigger behind the key loop, 34.8 with one here).
+    decode_cluster_begin(a);
     pdl_wait();
+    const int g = threadIdx.x / LPK, sub = threadIdx.x % LPK;
+    float qf[GRP][N];                       // on their way while the table is built
+#pragma unroll
+    for (int r = 0; r < GRP; ++r)
+        Vec<T>::load(static_cast<const T *>(a.q) + ((int64_t)b * a.n_heads + h0 + r) * D + sub * N, qf[r]);
     decode_segments<T, ALIBI>(a, sm, n_seg, b, hk, D, row_elems);
     if (ROPE) decode_angles<D>(a, rope, b, cs);
     __syncthreads();
@@ -456,7 +476,6 @@ decode_cluster_kernel(const __grid_constant__ DecodeArgs a, const __grid_constan
     const bool owns_new = j_new >= lo && j_new < hi;                 // block-uniform; j_new is then hi - 1
     const int hi_loop = owns_new ? hi - 1 : hi;                        // the new key is handled after the loop
 
-    const int g = threadIdx.x / LPK, sub = threadIdx.x % LPK;
     // rotates the N elements this lane holds of a D-vector spread over LPK lanes
     auto rotate = [&](float (&f)[N]) {
         if (rope_pairing == SP_ROPE_HALF_SPLIT) {
@@ -479,10 +498,8 @@ decode_cluster_kernel(const __grid_constant__ DecodeArgs a, const __grid_constan
         }
     };
 
-    float qf[GRP][N];
 #pragma unroll
     for (int r = 0; r < GRP; ++r) {
-        Vec<T>::load(static_cast<const T *>(a.q) + ((int64_t)b * a.n_heads + h0 + r) * D + sub * N, qf[r]);
         if (ROPE) {
             rotate(qf[r]);
 #pragma unroll
@@ -503,6 +520,11 @@ decode_cluster_kernel(const __grid_constant__ DecodeArgs a, const __grid_constan
     float slope_l2[GRP];
 #pragma unroll
     for (int r = 0; r < GRP; ++r) slope_l2[r] = ALIBI ? a.slopes[h0 + r] * kLog2eD : 0.f;
+
+    if (ROPE && owns_new && threadIdx.x < 2 * LPK) {     // the newest key's rows, asked into L2 ahead of their use
+        const int64_t off = (int64_t)(j_new - seg_lo[n_seg - 1]) * row_elems + sub * N;
+        prefetch_l2((threadIdx.x < LPK ? seg_k : seg_v)[n_seg - 1] + off);
+    }
 
     int seg = 0;
     for (int base = lo; base < hi_loop; base += G * kDecUnroll) {   // trip count is block-uniform
@@ -569,9 +591,8 @@ decode_cluster_kernel(const __grid_constant__ DecodeArgs a, const __grid_constan
     }
 
     if (ROPE && owns_new && threadIdx.x < 32) {
-        // The newest key, outside the streaming loop: warp 0 loads the unrotated row (every key
-        // group of the warp holds a copy), rotates it, group 0 writes it back for the later steps
-        // and takes it into its running softmax like any other key.
+        // The newest key, outside the streaming loop: rotated, written back by group 0 for the later steps and taken into
+        // its running softmax like any other key.
         const int64_t off = (int64_t)(j_new - seg_lo[n_seg - 1]) * row_elems + sub * N;
         T *krow = const_cast<T *>(seg_k[n_seg - 1]) + off;
         float kf[N], vf[N];
@@ -617,34 +638,27 @@ decode_cluster_kernel(const __grid_constant__ DecodeArgs a, const __grid_constan
     }
     __syncthreads();
 
-    float bm[GRP], bl[GRP], bo[GRP];
+    float *mine = decode_cluster_target(a, part, GRP * PS);
+    if (threadIdx.x < D) {
 #pragma unroll
-    for (int r = 0; r < GRP; ++r) {
-        bm[r] = -INFINITY; bl[r] = 0.f; bo[r] = 0.f;
-        for (int i = 0; i < G; ++i) bm[r] = fmaxf(bm[r], red[(i * GRP + r) * PS + D]);
-        if (threadIdx.x < D) {
+        for (int r = 0; r < GRP; ++r) {
+            float bm = -INFINITY, bl = 0.f, bo = 0.f;
+            for (int i = 0; i < G; ++i) bm = fmaxf(bm, red[(i * GRP + r) * PS + D]);
             for (int i = 0; i < G; ++i) {
                 const float gm = red[(i * GRP + r) * PS + D];
-                const float w = (gm == -INFINITY) ? 0.f : ex2f(gm - bm[r]);
-                bl[r] += red[(i * GRP + r) * PS + D + 1] * w;
-                bo[r] += red[(i * GRP + r) * PS + threadIdx.x] * w;
+                const float w = (gm == -INFINITY) ? 0.f : ex2f(gm - bm);
+                bl += red[(i * GRP + r) * PS + D + 1] * w;
+                bo += red[(i * GRP + r) * PS + threadIdx.x] * w;
+            }
+            if (a.n_splits == 1) {
+                decode_store<T>(a, (int64_t)b * a.n_heads + h0 + r, D, threadIdx.x, bm, bl, bo);
+            } else {
+                mine[r * PS + threadIdx.x] = bo;
+                if (threadIdx.x == 0) { mine[r * PS + D] = bm; mine[r * PS + D + 1] = bl; }
             }
         }
     }
-
-    if (a.n_splits > 1) {
-        if (threadIdx.x < D) {
-#pragma unroll
-            for (int r = 0; r < GRP; ++r) {
-                part[r * PS + threadIdx.x] = bo[r];
-                if (threadIdx.x == 0) { part[r * PS + D] = bm[r]; part[r * PS + D + 1] = bl[r]; }
-            }
-        }
-        decode_cluster_merge<T, D>(a, part, split, GRP, threadIdx.x, threadIdx.x < D ? 0 : -1, 1, (int64_t)b * a.n_heads + h0);
-    } else if (threadIdx.x < D) {
-#pragma unroll
-        for (int r = 0; r < GRP; ++r) decode_store<T>(a, (int64_t)b * a.n_heads + h0 + r, D, threadIdx.x, bm[r], bl[r], bo[r]);
-    }
+    decode_cluster_merge<T, D>(a, part, GRP, (int64_t)b * a.n_heads + h0);
 }
 
 }  // namespace sp
@@ -665,25 +679,31 @@ static int cluster_splits(int n_prompts, int blocks_y, int64_t max_keys, int min
 }
 
 template <typename K>
-static int launch_cluster_kernel(K kern, const DecodeArgs &a, const DecodeRope &rope, int pairing, int blocks_y, int n_prompts, size_t smem,
-                                 cudaStream_t st)
+static int launch_cluster_kernel(K kern, const DecodeArgs &a, const DecodeRope &rope, int pairing, int blocks_y, int n_prompts, int threads,
+                                 size_t smem, cudaStream_t st)
 {
     SP_REQUIRE(smem <= 200 * 1024, SP_ERR_UNSUPPORTED, "sp_pruned_decode: k = %d needs too much shared memory", a.k);
     if (smem > 48 * 1024)
         SP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (a.n_splits > 8)
         SP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    return launch(kern, dim3(a.n_splits, blocks_y, n_prompts), kDecThreads, smem, st, a.n_splits, a, rope, pairing);
+    return launch(kern, dim3(a.n_splits, blocks_y, n_prompts), threads, smem, st, a.n_splits, a, rope, pairing);
 }
 
 template <int D, bool ALIBI, bool ROPE>
 static int launch_decode_mma(DecodeArgs a, const DecodeRope &rope, int pairing, int n_prompts, int64_t max_keys, cudaStream_t st)
 {
-    constexpr int W = kDecThreads / 32;
     const int group = a.n_heads / a.n_kv_heads, blocks_y = a.n_kv_heads * ((group + kMmaHeads - 1) / kMmaHeads);
-    a.n_splits = cluster_splits(n_prompts, blocks_y, max_keys, W * kMmaKeys, kMmaBlocks);
-    const size_t smem = decode_table_bytes(a.k + 2) + (size_t)(W + 1) * kMmaHeads * (D + 2) * sizeof(float) + (D / 2) * sizeof(float2);
-    return launch_cluster_kernel(decode_mma_kernel<D, ALIBI, ROPE>, a, rope, pairing, blocks_y, n_prompts, smem, st);
+    const int warps = kMmaWarpsPerSM * num_sms();
+    const int64_t units = (int64_t)n_prompts * blocks_y;
+    a.n_splits = cluster_splits(n_prompts, blocks_y, max_keys, kMmaMaxWarps * kMmaKeys, kMmaWarpsPerSM / kMmaMaxWarps);
+    // Unsplit launches take as many warps a block as still leave every block resident at once: 64 prompts x 8 KV heads fit with
+    // three (30 us a step); blocks of four need a second wave (33).
+    int w = kMmaMaxWarps;
+    if (a.n_splits == 1) w = (int)std::max<int64_t>(1, std::min<int64_t>(w, warps / units));
+    const size_t smem = decode_table_bytes(a.k + 2) + (size_t)(w + a.n_splits) * std::min(group, kMmaHeads) * (D + 2) * sizeof(float) +
+                        (D / 2) * sizeof(float2);
+    return launch_cluster_kernel(decode_mma_kernel<D, ALIBI, ROPE>, a, rope, pairing, blocks_y, n_prompts, 32 * w, smem, st);
 }
 
 template <typename T, int D, int GRP, bool ALIBI, bool ROPE>
@@ -696,10 +716,10 @@ static int launch_decode_cluster(DecodeArgs a, const DecodeRope &rope, int pairi
     const int blocks_y = a.n_kv_heads * (group / GRP);
     constexpr int kMinB = GRP == 1 ? 8 : (GRP == 2 ? 5 : 3);
     a.n_splits = cluster_splits(n_prompts, blocks_y, max_keys, 32, kMinB);
-    const size_t smem = decode_table_bytes(a.k + 2) + (size_t)(G + 1) * GRP * PS * sizeof(float) + (D / 2) * sizeof(float2);
+    const size_t smem = decode_table_bytes(a.k + 2) + (size_t)(G + a.n_splits) * GRP * PS * sizeof(float) + (D / 2) * sizeof(float2);
     auto kern = (GRP == 1 && a.n_splits == 1) ? decode_cluster_kernel<T, D, GRP, ALIBI, ROPE, kMinB - (GRP == 1 ? 1 : 0)>
                                               : decode_cluster_kernel<T, D, GRP, ALIBI, ROPE, kMinB>;
-    return launch_cluster_kernel(kern, a, rope, pairing, blocks_y, n_prompts, smem, st);
+    return launch_cluster_kernel(kern, a, rope, pairing, blocks_y, n_prompts, kDecThreads, smem, st);
 }
 
 template <typename T, int D, bool ALIBI, bool ROPE>

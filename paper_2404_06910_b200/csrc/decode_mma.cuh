@@ -15,7 +15,8 @@ namespace sp {
 
 constexpr int kMmaHeads = 8;         // query heads per block at most
 constexpr int kMmaKeys = 16;         // keys per warp and turn
-constexpr int kMmaBlocks = 3;        // resident blocks per SM
+constexpr int kMmaMaxWarps = 4;      // warps per block at most
+constexpr int kMmaWarpsPerSM = 12;   // resident, with the 168 registers that a warp's loads and accumulators take
 
 __device__ __forceinline__ void mma_16n8k16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
 {
@@ -25,7 +26,7 @@ __device__ __forceinline__ void mma_16n8k16(float (&d)[4], uint32_t a0, uint32_t
 
 // Grid (n_splits, KV heads x blocks of up to 8 query heads, prompts); the n_splits blocks of a (prompt, y) are a cluster.
 template <int D, bool ALIBI, bool ROPE>
-__global__ void __launch_bounds__(kDecThreads, kMmaBlocks)
+__global__ void __launch_bounds__(32 * kMmaMaxWarps, kMmaWarpsPerSM / kMmaMaxWarps)
 decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ DecodeRope rope, int rope_pairing)
 {
     using T = __nv_bfloat16;
@@ -33,22 +34,30 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
     constexpr int NV = D / 64;              // 16-byte pieces of a V row per thread (pieces gid + 8 c)
     constexpr int NM = D / 16;              // 16-row tiles of O^T
     constexpr int PS = D + 2;               // one partial: D outputs, max, sum
-    constexpr int W = kDecThreads / 32;
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n_seg = a.k + 2;
     const DecodeSmem<T> sm(smem_raw, n_seg);
-    float *red = sm.end;                                        // [W][heads][PS]
-    float *part = red + W * kMmaHeads * PS;                     // [heads][PS], read by the cluster's first block
-    float2 *cs = reinterpret_cast<float2 *>(part + kMmaHeads * PS);     // [D/2] (cos, sin), ROPE only
-
     const int split = blockIdx.x, b = blockIdx.z;
     const int group = a.n_heads / a.n_kv_heads, per_kv = (group + kMmaHeads - 1) / kMmaHeads;
     const int hk = blockIdx.y / per_kv, sub_group = blockIdx.y - hk * per_kv;
     const int h0 = hk * group + sub_group * kMmaHeads, nh = min(kMmaHeads, group - sub_group * kMmaHeads);
     const int64_t row_elems = (int64_t)a.n_kv_heads * D;
+    const int W = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
+    float2 *cs = reinterpret_cast<float2 *>(sm.end);            // [D/2] (cos, sin), ROPE only
+    float *red = reinterpret_cast<float *>(cs + D / 2);         // [W][nh][PS]
+    float *part = red + W * nh * PS;                            // first block of the cluster: [n_splits][nh][PS]
 
+    decode_cluster_begin(a);
     pdl_wait();
+    uint4 qf[NC];                            // query head h0 + gid, unscaled bf16; on its way while the table is built
+#pragma unroll
+    for (int c = 0; c < NC; ++c) qf[c] = make_uint4(0u, 0u, 0u, 0u);
+    if (gid < nh) {
+        const uint4 *src = reinterpret_cast<const uint4 *>(static_cast<const T *>(a.q) + ((int64_t)b * a.n_heads + h0 + gid) * D);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) qf[c] = __ldg(src + tig + 4 * c);
+    }
     decode_segments<T, ALIBI>(a, sm, n_seg, b, hk, D, row_elems);
     if (ROPE) decode_angles<D>(a, rope, b, cs);
     __syncthreads();
@@ -63,7 +72,6 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
     const bool owns_new = j_new >= lo && j_new < hi;                 // block-uniform; j_new is then hi - 1
     const int hi_loop = owns_new ? hi - 1 : hi;                      // the new key is handled after the loop
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
     // rotates this thread's pieces tig + 4 c of a row: elements 8 (tig + 4 c) .. + 7
     auto rotate = [&](uint4 (&x)[NC]) {
         if (rope_pairing == SP_ROPE_HALF_SPLIT) {
@@ -95,14 +103,6 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
         }
     };
 
-    uint4 qf[NC];                            // query head h0 + gid, unscaled bf16
-#pragma unroll
-    for (int c = 0; c < NC; ++c) qf[c] = make_uint4(0u, 0u, 0u, 0u);
-    if (gid < nh) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(static_cast<const T *>(a.q) + ((int64_t)b * a.n_heads + h0 + gid) * D);
-#pragma unroll
-        for (int c = 0; c < NC; ++c) qf[c] = __ldg(src + tig + 4 * c);
-    }
     if (ROPE) rotate(qf);
 
     float m = -INFINITY, l = 0.f, o[NM][4];  // head gid: maximum, this thread's share of the sum; O^T rows, heads 2 tig, + 1
@@ -161,6 +161,11 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
         }
     };
 
+    const bool mine_new = ROPE && owns_new && warp == 0;
+    const int64_t new_off = mine_new ? (int64_t)(j_new - sm.lo[n_seg - 1]) * row_elems : 0;
+    if (mine_new && lane < 4)              // asked into L2 ahead of its use
+        prefetch_l2((lane < 2 ? sm.k : sm.v)[n_seg - 1] + new_off + (lane & 1) * (D / 2));
+
     int seg = 0;
     for (int base = lo + warp * kMmaKeys; base < hi_loop; base += W * kMmaKeys) {
         const int n = min(kMmaKeys, hi_loop - base);
@@ -186,14 +191,15 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
         attend(kr, vr, n, kpos);
     }
 
-    if (ROPE && owns_new && warp == 0) {
+    if (mine_new) {
         // The newest key: rotated, rounded and written back for the later steps, then one more turn with one key.
-        const int64_t off = (int64_t)(j_new - sm.lo[n_seg - 1]) * row_elems;
-        uint4 *krow = reinterpret_cast<uint4 *>(const_cast<T *>(sm.k[n_seg - 1]) + off);
-        const uint4 *vrow = reinterpret_cast<const uint4 *>(sm.v[n_seg - 1] + off);
+        uint4 *krow = reinterpret_cast<uint4 *>(const_cast<T *>(sm.k[n_seg - 1]) + new_off);
+        const uint4 *vrow = reinterpret_cast<const uint4 *>(sm.v[n_seg - 1] + new_off);
         uint4 kr[2][NC], vr[4][NV];
 #pragma unroll
         for (int c = 0; c < NC; ++c) kr[0][c] = krow[tig + 4 * c];
+#pragma unroll
+        for (int c = 0; c < NV; ++c) vr[0][c] = vr[1][c] = vr[2][c] = vr[3][c] = vrow[gid + 8 * c];
         rotate(kr[0]);
         __syncwarp();
 #pragma unroll
@@ -201,8 +207,6 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
             if (gid == 0) krow[tig + 4 * c] = kr[0][c];
             kr[1][c] = kr[0][c];
         }
-#pragma unroll
-        for (int c = 0; c < NV; ++c) vr[0][c] = vr[1][c] = vr[2][c] = vr[3][c] = vrow[gid + 8 * c];
         attend(kr, vr, 1, 0.f);
     }
 
@@ -212,20 +216,20 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
 #pragma unroll
     for (int r = 0; r < 2; ++r)
         if (2 * tig + r < nh) {
-            float *mine = red + (warp * kMmaHeads + 2 * tig + r) * PS + 8 * gid;
+            float *mine = red + (warp * nh + 2 * tig + r) * PS + 8 * gid;
 #pragma unroll
             for (int i = 0; i < NM; ++i) { mine[i] = o[i][r]; mine[D == 128 ? i + 64 : i + 4] = o[i][2 + r]; }
         }
-    if (tig == 0 && gid < nh) { red[(warp * kMmaHeads + gid) * PS + D] = m; red[(warp * kMmaHeads + gid) * PS + D + 1] = l; }
+    if (tig == 0 && gid < nh) { red[(warp * nh + gid) * PS + D] = m; red[(warp * nh + gid) * PS + D + 1] = l; }
     __syncthreads();
 
-    // thread: element d of heads r0, r0 + kDecThreads / D, ...
-    const int d = threadIdx.x & (D - 1);
-    for (int r = threadIdx.x / D; r < nh; r += kDecThreads / D) {
+    float *mine = decode_cluster_target(a, part, nh * PS);
+    for (int idx = threadIdx.x; idx < nh * D; idx += blockDim.x) {
+        const int r = idx / D, d = idx & (D - 1);
         float bm = -INFINITY, bl = 0.f, bo = 0.f;
-        for (int i = 0; i < W; ++i) bm = fmaxf(bm, red[(i * kMmaHeads + r) * PS + D]);
+        for (int i = 0; i < W; ++i) bm = fmaxf(bm, red[(i * nh + r) * PS + D]);
         for (int i = 0; i < W; ++i) {
-            const float *rp = red + (i * kMmaHeads + r) * PS;
+            const float *rp = red + (i * nh + r) * PS;
             const float wgt = rp[D] == -INFINITY ? 0.f : ex2f(rp[D] - bm);
             bl += rp[D + 1] * wgt;
             bo += rp[d] * wgt;
@@ -233,12 +237,11 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
         if (a.n_splits == 1) {
             decode_store<T>(a, (int64_t)b * a.n_heads + h0 + r, D, d, bm, bl, bo);
         } else {
-            part[r * PS + d] = bo;
-            if (d == 0) { part[r * PS + D] = bm; part[r * PS + D + 1] = bl; }
+            mine[r * PS + d] = bo;
+            if (d == 0) { mine[r * PS + D] = bm; mine[r * PS + D + 1] = bl; }
         }
     }
-    if (a.n_splits == 1) return;
-    decode_cluster_merge<T, D>(a, part, split, nh, d, threadIdx.x / D, kDecThreads / D, (int64_t)b * a.n_heads + h0);
+    decode_cluster_merge<T, D>(a, part, nh, (int64_t)b * a.n_heads + h0);
 }
 
 }  // namespace sp
