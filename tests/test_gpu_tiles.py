@@ -1,0 +1,106 @@
+"""The prefill and decode kernels at the sizes where their tiling can go wrong: edges of query tiles, tile pairs, key tiles
+and of the preamble's padding, the smallest and largest of each range, and both sides of every dispatch rule, against the
+oracle with the tolerances of the parity suite (bf16: rel-L2 1e-2, from one rounding of probabilities and output; per row
+twice that; fp32: 1e-5)."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2404_06910_b200 as sp
+from helpers import dev, f32, rel_l2, workspace
+from workloads import build_layout
+
+pytestmark = pytest.mark.gpu
+
+TOL = {torch.bfloat16: 1e-2, torch.float32: 1e-5}
+
+
+def _randn(shape, seed, dtype=torch.bfloat16):
+    return torch.randn(*shape, generator=torch.Generator().manual_seed(seed)).to(dtype)
+
+
+def _prefill(lay, H, Hkv, D, dtype=torch.bfloat16, rows=sp.SP_ROWS_ALL, alibi=False, shift=0):
+    """Runs and checks one prefill; shift: elements by which the output's address misses 32-byte alignment."""
+    T = lay.total_tokens
+    q, k, v = _randn((T, H, D), 1, dtype), _randn((T, Hkv, D), 2, dtype), _randn((T, Hkv, D), 3, dtype)
+    pos = torch.rand(T, generator=torch.Generator().manual_seed(4)).mul(300).float() if alibi else None
+    slopes = np.array([2.0 ** (-8.0 * (h + 1) / H) for h in range(H)], np.float32)
+    bias = dict(pos=pos.numpy(), slopes=slopes) if alibi else {}
+    ref_o, ref_l = oracle.prefill(f32(q), f32(k), f32(v), lay, 1 / math.sqrt(D), **bias)
+    dl = sp.DeviceLayout.from_host(lay)
+    out = torch.full((T * H * D + shift,), float("nan"), dtype=dtype, device="cuda")[shift:].view(T, H, D)
+    lse = torch.full((H, T), float("nan"), device="cuda")
+    ws = workspace(sp.sp_prefill_workspace_bytes(dl, H, D, sp.dtype_code(q)))
+    if alibi:
+        sp.sp_superpose_prefill_alibi(dev(q), dev(k), dev(v), dl, dev(pos), dev(slopes), 1 / math.sqrt(D), out, lse, ws, rows=rows)
+    else:
+        sp.sp_superpose_prefill(dev(q), dev(k), dev(v), dl, 1 / math.sqrt(D), out, lse, ws, rows=rows)
+    sp.sp_check_status(ws)
+    sel = np.ones(T, bool)
+    if rows == sp.SP_ROWS_QUERY_ONLY:
+        sel[:] = False
+        for s, d, n in zip(lay.path_start, lay.doc_len, lay.qry_len):
+            sel[s + d:s + d + n] = True
+    got, got_l = f32(out), lse.cpu().numpy()
+    assert not np.isnan(got[sel]).any() and np.isnan(got[~sel]).all()
+    assert rel_l2(got[sel], ref_o[sel]) <= TOL[dtype]
+    num = np.linalg.norm((got - ref_o)[sel].reshape(int(sel.sum()), -1), axis=1)
+    assert (num / (np.linalg.norm(ref_o[sel].reshape(int(sel.sum()), -1), axis=1) + 1e-6)).max() <= 2 * TOL[dtype]
+    np.testing.assert_allclose(got_l[:, sel], ref_l[:, sel], atol=2e-5 if dtype == torch.float32 else 2e-2)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("alibi", [False, True])
+@pytest.mark.parametrize("pre", [0, 1, 16, 63, 65, 130])
+def test_prefill_segment_lengths(D, alibi, pre):
+    """One, two and three query tiles and one row on either side of each; preambles around the 16-row padding and the key tile."""
+    lens = [1, 31, 33, 127, 128, 129, 191, 255, 256, 257, 385]
+    lay = build_layout([pre, 17], [[n - 1 for n in lens], [64, 300]], [[1] * len(lens), [9, 20]])
+    _prefill(lay, 4, 2, D, alibi=alibi)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_prefill_output_aligned_to_16_bytes_only(D):
+    _prefill(build_layout([20], [[100, 150]], [[24, 24]]), 2, 2, D, shift=8)
+
+
+@pytest.mark.parametrize("pre,alibi", [(64, True), (65, True), (384, False), (385, False)])
+def test_prefill_query_only_either_kernel(pre, alibi):
+    _prefill(build_layout([pre, 5], [[40, 130], [9, 0]], [[32, 7], [33, 100]]), 4, 2, 128, rows=sp.SP_ROWS_QUERY_ONLY, alibi=alibi)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("alibi", [False, True])
+def test_prefill_f32_tiles(D, alibi):
+    lay = build_layout([0, 33], [[1, 14, 15, 62], [64, 130]], [[1, 2, 1, 3], [5, 40]])
+    _prefill(lay, 4, 2, D, torch.float32, alibi=alibi)
+    _prefill(lay, 4, 2, D, torch.float32, rows=sp.SP_ROWS_QUERY_ONLY, alibi=alibi)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("H,Hkv", [(5, 1), (8, 1), (9, 1), (16, 1), (64, 32), (24, 8)])
+@pytest.mark.parametrize("n_prompts", [1, 60])
+def test_decode_group_sizes(D, H, Hkv, n_prompts):
+    """Query heads per KV head up to, at and above a block's eight; split over a cluster and unsplit with one to four warps;
+    key counts around the 16 keys of a warp's turn."""
+    rng = np.random.default_rng(3)
+    lay = build_layout([int(x) for x in rng.integers(0, 40, n_prompts)], [[int(x) for x in rng.integers(0, 70, 3)] for _ in range(n_prompts)],
+                       [[int(x) for x in rng.integers(1, 9, 3)] for _ in range(n_prompts)])
+    T, cap, k = lay.total_tokens, 5, 2
+    q, kc, vc = _randn((n_prompts, H, D), 1), _randn((T, Hkv, D), 2), _randn((T, Hkv, D), 3)
+    tk, tv = _randn((n_prompts, cap, Hkv, D), 4), _randn((n_prompts, cap, Hkv, D), 5)
+    kept = np.stack([lay.prompt_path_off[b] + rng.permutation(3)[:k] for b in range(n_prompts)]).astype(np.int32)
+    tl = rng.integers(0, cap + 1, n_prompts).astype(np.int32)
+    tl[0] = cap
+    ref_o, ref_l = oracle.pruned_decode(f32(q), f32(kc), f32(vc), lay, kept, f32(tk), f32(tv), tl, 1 / math.sqrt(D))
+    out = torch.full((n_prompts, H, D), float("nan"), dtype=torch.bfloat16, device="cuda")
+    lse = torch.full((n_prompts, H), float("nan"), device="cuda")
+    sp.sp_pruned_decode(dev(q), dev(kc), dev(vc), sp.DeviceLayout.from_host(lay), dev(kept), k, dev(tk), dev(tv), dev(tl), cap,
+                        1 / math.sqrt(D), out, lse, workspace(sp.sp_decode_workspace_bytes(n_prompts, H, D)))
+    assert rel_l2(f32(out), ref_o) <= TOL[torch.bfloat16]
+    fin = np.isfinite(ref_l)
+    np.testing.assert_allclose(lse.cpu().numpy()[fin], ref_l[fin], atol=2e-2)
+    np.testing.assert_array_equal(lse.cpu().numpy()[~fin], ref_l[~fin])
