@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
         reg_alloc<C::R_SOFT>();
         const int ln = warp >> 2, quad = warp & 3, row = quad * 32 + lane;
         const uint32_t s_base = tb + ln * kLaneCols + ((uint32_t)(quad * 32) << 16);
-        const float sc = p.scale_log2e, sc_exp = ALIBI ? 1.f : sc;   // ALiBi scores are scaled when the bias is added
+        const float sc = p.scale_log2e;
         uint64_t *own2 = bars + ln, *own_buf = bars + 2 * ln;
         uint32_t g = 0, tiles = 0, pos_ph = 0;
         Ring<C::NKV> v;
@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
             float pq = 0.f, neg_slope = 0.f;
             if (ALIBI && t.steps) {
                 pq = row < t.rows ? __ldg(p.pos + w.t.own_base + t.q_u + row) : 0.f;
-                neg_slope = -p.slopes[w.h] * kLog2eT;
+                neg_slope = -p.slopes[w.h] * (kLog2eT / sc);     // in units of the unscaled score: one scaling serves both
             }
             // counted from the key tile's first key: the first one this row may not see, the padding behind the preamble
             int lim = min(t.q_u + row + 1, t.end), g0 = w.t.pre_len, g1 = w.t.p16;
@@ -499,8 +499,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
                         if (c == 1 && see <= 32) break;
-                        if (ALIBI) {              // score * scale - slope * |distance|; key positions are broadcast reads
-                            const uint64_t sc2 = pack_f32x2(sc, sc), pq2 = pack_f32x2(-pq, -pq), ns2 = pack_f32x2(neg_slope, neg_slope);
+                        if (ALIBI) {              // score - slope * |distance|; key positions are broadcast reads
+                            const uint64_t pq2 = pack_f32x2(-pq, -pq), ns2 = pack_f32x2(neg_slope, neg_slope);
 #pragma unroll
                             for (int i = 0; i < 32; i += 4) {
                                 const ulonglong2 kp = *reinterpret_cast<const ulonglong2 *>(s_pos + v.i * kBN + c * 32 + i);
@@ -508,7 +508,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                                 for (int e = 0; e < 4; e += 2) {
                                     const uint64_t d = add_f32x2(e ? kp.y : kp.x, pq2) & 0x7fffffff7fffffffull;
                                     float x0, x1;
-                                    unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[c][i + e]), __uint_as_float(r[c][i + e + 1])), sc2, mul_f32x2(d, ns2)), x0, x1);
+                                    unpack_f32x2(fma_f32x2(d, ns2, pack_f32x2(__uint_as_float(r[c][i + e]), __uint_as_float(r[c][i + e + 1]))), x0, x1);
                                     r[c][i + e] = __float_as_uint(x0); r[c][i + e + 1] = __float_as_uint(x1);
                                 }
                             }
@@ -522,7 +522,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
 #pragma unroll
                         for (int i = 0; i < 32; i += 2) mx[(i >> 1) & 3] = fmax3(mx[(i >> 1) & 3], __uint_as_float(r[c][i]), __uint_as_float(r[c][i + 1]));
                     }
-                    const float m_tile = fmaxf(fmax3(mx[0], mx[1], mx[2]), mx[3]) * sc_exp;
+                    const float m_tile = fmaxf(fmax3(mx[0], mx[1], mx[2]), mx[3]) * sc;
                     const bool grow = j > 0 && m_tile > m_ref + kRescaleThreshold;
                     if (__any_sync(0xffffffffu, grow)) {      // rare: bring O and l to the new reference
                         // needs the lane's previous O += P V complete
@@ -542,7 +542,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                     }
                     if (j == 0 || grow) m_ref = m_tile;
                     // P = exp2(score - reference) as bf16
-                    const uint64_t sc2 = pack_f32x2(sc_exp, sc_exp), nm2 = pack_f32x2(-m_ref, -m_ref);
+                    const uint64_t sc2 = pack_f32x2(sc, sc), nm2 = pack_f32x2(-m_ref, -m_ref);
                     uint64_t sum[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
