@@ -104,3 +104,21 @@ def test_decode_group_sizes(D, H, Hkv, n_prompts):
     fin = np.isfinite(ref_l)
     np.testing.assert_allclose(lse.cpu().numpy()[fin], ref_l[fin], atol=2e-2)
     np.testing.assert_array_equal(lse.cpu().numpy()[~fin], ref_l[~fin])
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("vocab,pad", [(1, 0), (7, 0), (8, 0), (9, 4), (129, 0), (2051, 3)])
+@pytest.mark.parametrize("n_paths,qry", [(3, 5), (900, 4)])
+def test_path_scores_row_alignments(dtype, vocab, pad, n_paths, qry):
+    """Rows that start at every offset from a 16-byte boundary, shorter than a vector and longer; few rows (256 threads a row)
+    and many (128).  Tolerance: 1e-3 per row as in the parity suite."""
+    rows = n_paths * qry
+    logits = _randn((rows, vocab + pad), 7, dtype) * 3
+    tgt = torch.randint(0, vocab, (rows,), generator=torch.Generator().manual_seed(8), dtype=torch.int32)
+    tgt[qry - 1::qry] = -1
+    off = np.arange(0, rows + 1, qry, dtype=np.int32)
+    ref_s, ref_r = oracle.path_scores(f32(logits[:, :vocab].contiguous()), tgt.numpy(), off, None, None)
+    scores, row_logp = torch.empty(n_paths, device="cuda"), torch.empty(rows, device="cuda")
+    sp.sp_path_scores(dev(logits)[:, :vocab], dev(tgt), dev(off), scores, None, None, row_logp)
+    np.testing.assert_allclose(row_logp.cpu().numpy(), ref_r, atol=1e-3)
+    np.testing.assert_allclose(scores.cpu().numpy(), ref_s, atol=1e-3 * qry)
