@@ -58,8 +58,11 @@ static int prefill_entry(const void *q, const void *k, const void *v, const sp_l
     // while a path's keys are mostly its own; behind a long preamble the smaller tiles of the warp-level kernel win.  us at 8
     // prompts x 100 documents, 32 query rows, tcgen05 / warp-level: preamble 48: 615 / 654, 256: 950 / 955, about 1 250: 2522 /
     // 2368; ALiBi, whose bias a lone softmax warp feels more: 48: 749 / 747, 128: 879 / 868, 256: 1255 / 1113.  More than 32
-    // query rows per path would speak for tcgen05 at any length (48 rows behind 1 000: 997 / 1859) but are not known here.
-    if (dtype == SP_BF16 && head_dim == 128 && rows == SP_ROWS_QUERY_ONLY && lay->max_pre_len > (pos ? 64 : 384))
+    // query rows per path would speak for tcgen05 at any length (48 rows behind 1 000: 997 / 1859) but are not known here.  With
+    // an even number of query heads to a KV head the tcgen05 tiles hold the rows of several heads and win everywhere: preamble
+    // 1 250, 40 documents: 618 / 1128 (two heads), 360 / 1123 (four); ALiBi behind 500: 449 / 672, 254 / 657.
+    if (dtype == SP_BF16 && head_dim == 128 && rows == SP_ROWS_QUERY_ONLY && lay->max_pre_len > (pos ? 64 : 384) &&
+        n_heads / n_kv_heads % 2)
         return launch_prefill_qonly(q, k, v, lay, pos, slopes, n_heads, n_kv_heads, scale, out, lse, ws, st);
     // bf16 goes to the tensor cores for both head sizes (head_dim 64, 8 prompts x 20 documents, 32 heads: 0.17 ms; the fp32
     // SIMT kernel, which served it before, took 9.4 ms)

@@ -1,7 +1,9 @@
 // Fork-join prefill attention on the Blackwell tensor cores (bf16, head_dim 64 and 128).
 // Section 3.2: a row attends to its prompt's preamble and, causally, to its own path.
 //
-// Work unit ("item"): one or two consecutive query tiles (up to 128 rows each) of one segment, for one head.  Its keys are
+// Work unit ("item"): one or two consecutive query tiles of one segment, for one head; with grouped query heads a tile's 128
+// rows are 128 / G rows of the segment for each of G = 2, 4 or 8 heads that share a KV head, so that K and V are loaded once for
+// all of them and a tile's rows lie closer to the diagonal.  Its keys are
 // the preamble's rows (all visible) followed by the segment's own rows up to the diagonal, as one sequence cut into tiles
 // of 64 (the preamble is padded to a multiple of 16 in front of the own rows, so one tile may hold both); key tiles that the
 // fork-join mask excludes are never loaded or multiplied.  Per query tile and key tile:
@@ -130,7 +132,8 @@ struct TcParams {
     uint32_t *status;
     __nv_bfloat16 *out;
     float *lse;
-    int n_heads, kv_group;
+    int n_heads;
+    int log_rows, n_units, units_per_kv;   // rows of a head in a tile (log2); units of G heads in all and per KV head
     int64_t total_tokens;
     float scale_log2e;
     int wide_stores;                  // out is 32-byte aligned
@@ -144,21 +147,21 @@ struct TcParams {
 struct Walk {
     const TcPair *pairs;
     uint32_t pair, n_pairs, item_no;
-    int h, n_heads, dp, dh;
+    int h, n_units, dp, dh;           // h: unit of G heads
     TcPair t;
     __device__ __forceinline__ explicit Walk(const TcParams &p)
     {
-        pairs = p.pairs; n_pairs = p.hdr->n_tiles; n_heads = p.n_heads; item_no = 0xffffffffu;
-        dp = gridDim.x / n_heads; dh = gridDim.x - dp * n_heads;
-        pair = blockIdx.x / n_heads; h = blockIdx.x - pair * n_heads;
+        pairs = p.pairs; n_pairs = p.hdr->n_tiles; n_units = p.n_units; item_no = 0xffffffffu;
+        dp = gridDim.x / n_units; dh = gridDim.x - dp * n_units;
+        pair = blockIdx.x / n_units; h = blockIdx.x - pair * n_units;
         // one step back: next() comes before every item, the first one included, so that its code exists once per role
         h -= dh; pair -= dp;
-        if (h < 0) { h += n_heads; --pair; }
+        if (h < 0) { h += n_units; --pair; }
     }
     __device__ __forceinline__ bool next()
     {
         ++item_no; pair += dp; h += dh;
-        if (h >= n_heads) { h -= n_heads; ++pair; }
+        if (h >= n_units) { h -= n_units; ++pair; }
         if (pair >= n_pairs) return false;
         const int4 *src = reinterpret_cast<const int4 *>(pairs + pair);
         const int4 a = __ldg(src), b = __ldg(src + 1);
@@ -205,10 +208,13 @@ template <int N> __device__ __forceinline__ void reg_dealloc() { asm volatile("s
 
 // ALIBI: scores get -slope_h * |pos_q - pos_k| before the softmax (Section 3.2.2: real-valued positions are no obstacle
 // for ALiBi).
-template <int D, bool ALIBI>
+// GROUPED: tiles of several heads.  A kernel of its own: the index arithmetic costs a launch of single heads 1.5 % (32 query rows of
+// 800 paths, 621 against 630 us).
+template <int D, bool ALIBI, bool GROUPED>
 __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_constant__ TcParams p)
 {
     using C = TcConfig<D, ALIBI>;
+    const int log_rows = GROUPED ? p.log_rows : 7;
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char *sQ = smem, *sK = smem + C::NQ * C::Q_BYTES, *sV = sK + C::NKV * C::KV_BYTES;
     float *x_l = reinterpret_cast<float *>(smem + C::X_OFF);                            // [lane][row] row sums
@@ -255,11 +261,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                 const CUtensorMap *maps = p.maps[kind];
                 uint64_t pol;                         // query tiles are read once: leave L2 to the K / V rows
                 if (is_q) pol = l2_policy_evict_first(); else pol = l2_policy_evict_normal();
+                const int log_g = 7 - log_rows, heads = is_q ? 1 << log_g : 1;       // heads in a tile of this kind
                 int slot = 0;
                 uint32_t ph = 1, n = 0, last = 0, fills = 0;      // per slot: barrier of its last fill; per barrier: parity of the next one
 #pragma unroll 1
                 for (Walk w(p); ok && w.next();) {
-                    const int head = (is_q ? w.h : w.h / p.kv_group) * C::HALVES, units = is_q ? w.n_q() : w.t.steps;
+                    const int head = (is_q ? w.h << log_g : w.h / p.units_per_kv) * C::HALVES, units = is_q ? w.n_q() : w.t.steps;
 #pragma unroll 1
                     for (int j = 0; j < units; ++j) {
                         if (!(ok = mbar_wait_warp(empty + slot, ph))) break;
@@ -272,17 +279,22 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                         last = (last & ~(0xffu << (8 * slot))) | (uint32_t)to << (8 * slot);
                         fills ^= 1u << to;
                         unsigned char *dst = base + slot * (tile_rows * D * 2);
-                        if (lead) mbar_expect_tx(bar, (uint32_t)(u1 - u0) * (D * 2));
+                        if (lead) mbar_expect_tx(bar, (uint32_t)((u1 - u0) * heads) * (D * 2));
                         __syncwarp();
 #pragma unroll 1
-                        for (int u = u0; u < u1;) {
-                            const bool pre = u < split;                         // preamble part, then own part
-                            const int left = (pre ? split : u1) - u, row = u + (pre ? w.t.pre_row : w.t.own_base);
-                            const int box = left == tile_rows ? 0 : (left >= 32 ? 1 : 2);
+                        for (int hq = 0; hq < heads; ++hq) {
+                            unsigned char *to_rows = dst + (hq << log_rows) * 128;
 #pragma unroll 1
-                            for (int hh = 0; hh < (box ? C::HALVES : 1); ++hh)
-                                tma_load_3d_hint(lead, dst + hh * (tile_rows * 128) + (u - u0) * 128, maps + box, 0, row, head + hh, bar, pol);
-                            u += box == 0 ? tile_rows : (box == 1 ? 32 : 16);
+                            for (int u = u0; u < u1;) {
+                                const bool pre = u < split;                         // preamble part, then own part
+                                const int left = (pre ? split : u1) - u, row = u + (pre ? w.t.pre_row : w.t.own_base);
+                                const int box = left == tile_rows ? 0 : (left >= 32 ? 1 : 2);
+#pragma unroll 1
+                                for (int hh = 0; hh < (box ? C::HALVES : 1); ++hh)
+                                    tma_load_3d_hint(lead, to_rows + hh * (tile_rows * 128) + (u - u0) * 128, maps + box, 0, row,
+                                                     head + hq * C::HALVES + hh, bar, pol);
+                                u += box == 0 ? tile_rows : (box == 1 ? 32 : 16);
+                            }
                         }
                         if (lead && !is_q && w.one_lane(j)) mbar_arrive(empty + slot);      // for the lane that has no use for it
                         ++n;
@@ -466,6 +478,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
         // -------------------------------------------------------------------- softmax, one thread per query row
         reg_alloc<C::R_SOFT>();
         const int ln = warp >> 2, quad = warp & 3, row = quad * 32 + lane;
+        const int rows_per_head = 1 << log_rows, hr = row & (rows_per_head - 1);            // row of the tile, for head row >> log_rows
+        const int hr0 = quad * 32 & (rows_per_head - 1), hr1 = hr0 + min(32, rows_per_head);  // ... of the warp
         const uint32_t s_base = tb + ln * kLaneCols + ((uint32_t)(quad * 32) << 16);
         const float sc = p.scale_log2e;
         uint64_t *own2 = bars + ln, *own_buf = bars + 2 * ln;
@@ -474,16 +488,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
 #pragma unroll 1
         for (Walk w(p); ok && w.next();) {
             const LaneTile t(w, ln);
-            const bool live_w = quad * 32 < t.rows;      // rows past the tile's last one take part in barriers only
+            const bool live_w = hr0 < t.rows;            // rows past the tile's last one take part in barriers only
+            const int head = (w.h << (7 - log_rows)) + (row >> log_rows);
             float m_ref = -INFINITY, l = 0.f;            // reference maximum (log2 units) and row sum
             float pq = 0.f, neg_slope = 0.f;
             if (ALIBI && t.steps) {
-                pq = row < t.rows ? __ldg(p.pos + w.t.own_base + t.q_u + row) : 0.f;
-                neg_slope = -p.slopes[w.h] * (kLog2eT / sc);     // in units of the unscaled score: one scaling serves both
+                pq = hr < t.rows ? __ldg(p.pos + w.t.own_base + t.q_u + hr) : 0.f;
+                neg_slope = -p.slopes[head] * (kLog2eT / sc);     // in units of the unscaled score: one scaling serves both
             }
             // counted from the key tile's first key: the first one this row may not see, the padding behind the preamble
-            int lim = min(t.q_u + row + 1, t.end), g0 = w.t.pre_len, g1 = w.t.p16;
-            int see = live_w ? min(t.q_u + quad * 32 + 32, t.end) : 0;      // keys some row of the warp may see
+            int lim = min(t.q_u + hr + 1, t.end), g0 = w.t.pre_len, g1 = w.t.p16;
+            int see = live_w ? min(t.q_u + hr1, t.end) : 0;      // keys some row of the warp may see
 #pragma unroll 1
             for (int j = 0; j < t.steps; ++j, ++g, lim -= kBN, g0 -= kBN, g1 -= kBN, see -= kBN) {
                 const uint32_t buf = g & 1, s_addr = s_base + buf * kBN;
@@ -587,7 +602,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
             __syncwarp();
             if (lane == 0) mbar_arrive(own2 + C::BAR_L_READY);
             ++tiles;
-            if (p.lse && row < t.rows) p.lse[(int64_t)w.h * p.total_tokens + w.t.own_base + t.q_u + row] = (m_ref + log2f(l)) * kLn2T;
+            if (p.lse && hr < t.rows) p.lse[(int64_t)head * p.total_tokens + w.t.own_base + t.q_u + hr] = (m_ref + log2f(l)) * kLn2T;
         }
     } else {
         // -------------------------------------------------------------------- epilogue
@@ -595,6 +610,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
         // the accumulator is handed back before the last 64 columns are stored.
         reg_dealloc<C::R_EPI>();
         const int quad = warp - WARP_EPI, row = quad * 32 + lane;
+        const int hr = row & ((1 << log_rows) - 1), hr0 = quad * 32 & ((1 << log_rows) - 1);
         uint32_t ph = 0, g[2] = {0, 0};                  // tiles so far, mod 2, a bit per lane; key tiles so far
 #pragma unroll 1
         for (Walk w(p); ok && w.next();) {
@@ -614,11 +630,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                 const uint32_t o_addr = tb + ln * kLaneCols + kOCol + ((uint32_t)(quad * 32) << 16);
                 const uint64_t inv2 = pack_f32x2(inv, inv);
                 unsigned char *dst = reinterpret_cast<unsigned char *>(p.out) +
-                                     ((int64_t)(w.t.own_base + t.q_u + row) * p.n_heads + w.h) * (D * 2);
+                                     ((int64_t)(w.t.own_base + t.q_u + hr) * p.n_heads + (w.h << (7 - log_rows)) + (row >> log_rows)) * (D * 2);
 #pragma unroll 1
                 for (int cc = 0; cc < C::HALVES; ++cc) {       // 64 columns
                     uint32_t o[32];
-                    if (quad * 32 < t.rows) {
+                    if (hr0 < t.rows) {
                         uint32_t r0[32], r1[32];
                         tmem_ld32(o_addr + cc * 64, r0);
                         tmem_ld32(o_addr + cc * 64 + 32, r1);
@@ -636,7 +652,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&bars[C::BAR_O_FREE + ln]);
                     }
-                    if (row < t.rows) {
+                    if (hr < t.rows) {
                         if (p.wide_stores) {
 #pragma unroll
                             for (int i = 0; i < 4; ++i) st_global_32b(dst + cc * 128 + i * 32, *reinterpret_cast<const uint32_t (*)[8]>(&o[i * 8]));
@@ -671,6 +687,7 @@ struct RopeRows {
     const TcHeader *hdr;
     const TcPair *pairs;
     int n_heads, half_split;
+    uint32_t item_groups;             // of kRopeRows rows, in an item at most
     double inv_freq[64];
 };
 __global__ void __launch_bounds__(256, 8) rope_rows_kernel(const __grid_constant__ RopeRows a)
@@ -678,11 +695,10 @@ __global__ void __launch_bounds__(256, 8) rope_rows_kernel(const __grid_constant
     __shared__ float2 cs[kRopeRows][64];
     pdl_wait();
     pdl_trigger();
-    constexpr uint32_t kGroups = 2 * kBM / kRopeRows;          // of an item
-    const uint32_t n_groups = a.hdr->n_tiles * kGroups;
+    const uint32_t n_groups = a.hdr->n_tiles * a.item_groups;
     for (uint32_t g = blockIdx.x; g < n_groups; g += gridDim.x) {
-        const TcPair t = a.pairs[g / kGroups];
-        const int r0 = (int)(g % kGroups) * kRopeRows, n = min(kRopeRows, (t.rows_ab & 0xffff) + (t.rows_ab >> 16) - r0);
+        const TcPair t = a.pairs[g / a.item_groups];
+        const int r0 = (int)(g % a.item_groups) * kRopeRows, n = min(kRopeRows, (t.rows_ab & 0xffff) + (t.rows_ab >> 16) - r0);
         if (n <= 0) continue;
         const int64_t row = t.own_base + t.q_u + r0;
         __syncthreads();
@@ -745,23 +761,18 @@ static int encode_rows_map(EncodeTiledFn enc, CUtensorMap *m, const void *base, 
     return SP_OK;
 }
 
-static int64_t max_tiles(int n_prompts, int n_paths, int max_pre_len, int max_path_len)
-{
-    return plan_max_tiles(n_prompts, n_paths, max_pre_len, max_path_len, kBM);
-}
-
 size_t prefill_tc_workspace_bytes(int n_prompts, int n_paths, int max_pre_len, int max_path_len, int)
 {
     if (n_prompts < 0 || n_paths < 0 || max_pre_len < 0 || max_path_len < 0) return 256;
-    const size_t cap = (size_t)max_tiles(n_prompts, n_paths, max_pre_len, max_path_len);
-    return 256 + round_up(cap * sizeof(TcPair), 256);
+    // the head counts are not known yet: items of 2 x 16 rows, those of eight heads in a tile
+    return 256 + round_up((size_t)plan_max_tiles(n_prompts, n_paths, max_pre_len, max_path_len, 32) * sizeof(TcPair), 256);
 }
 
-template <int D, bool ALIBI> static int launch_kernel(const TcParams &p, int grid, cudaStream_t st)
+template <int D, bool ALIBI, bool GROUPED> static int launch_kernel(const TcParams &p, int grid, cudaStream_t st)
 {
     using C = TcConfig<D, ALIBI>;
-    SP_CUDA(cudaFuncSetAttribute(prefill_tc_kernel<D, ALIBI>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-    return launch(prefill_tc_kernel<D, ALIBI>, grid, kTcThreads, C::SMEM, st, 1, p);
+    SP_CUDA(cudaFuncSetAttribute(prefill_tc_kernel<D, ALIBI, GROUPED>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
+    return launch(prefill_tc_kernel<D, ALIBI, GROUPED>, grid, kTcThreads, C::SMEM, st, 1, p);
 }
 
 static int launch_tc(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
@@ -791,31 +802,41 @@ static int launch_tc(const void *q, const void *k, const void *v, const sp_layou
     PlanArgs pa;
     pa.ppo = lay->prompt_path_off; pa.pre_start = lay->pre_start; pa.pre_len = lay->pre_len;
     pa.path_start = lay->path_start; pa.doc_len = lay->doc_len; pa.qry_len = lay->qry_len;
-    pa.n_prompts = lay->n_prompts; pa.n_paths = lay->n_paths; pa.rows_mode = rows; pa.tile_rows = kBM;
+    // Heads that share a tile: the largest of 8, 4, 2, 1 that divides the group; 16-row boxes rule out more.  Less of a tile is
+    // empty (segments of a few hundred rows, queries of 8 to 48) and its rows lie closer to the diagonal.  us with one head a
+    // tile / this, 32 heads over 8: 2 prompts x 400 documents of 128-512 rows 2376 / 1972, 64 x 20 of 100-200 rows 1399 / 1054, 32
+    // query rows only of 8 x 100 552 / 190, head_dim 64 163 / 127.
+    const int group = n_heads / n_kv_heads, log_g = group % 8 == 0 ? 3 : (group % 4 == 0 ? 2 : (group % 2 == 0 ? 1 : 0));
+    pa.n_prompts = lay->n_prompts; pa.n_paths = lay->n_paths; pa.rows_mode = rows; pa.tile_rows = kBM >> log_g;
     pa.max_pre_len = lay->max_pre_len; pa.max_path_len = lay->max_path_len; pa.total_tokens = lay->total_tokens;
-    pa.max_tiles = max_tiles(lay->n_prompts, lay->n_paths, lay->max_pre_len, lay->max_path_len);
+    pa.max_tiles = plan_max_tiles(lay->n_prompts, lay->n_paths, lay->max_pre_len, lay->max_path_len, 2 * pa.tile_rows);
     pa.hdr = hdr; pa.list = pairs;
     if (int rc = launch(prefill_plan_kernel<true>, 1, 1024, 0, st, 1, pa)) return rc;
     if (rope) {
         RopeRows r = *rope;
-        r.hdr = hdr; r.pairs = pairs;
-        const int64_t groups = pa.max_tiles * (kBM / kRopeRows);
+        r.hdr = hdr; r.pairs = pairs; r.item_groups = 2 * pa.tile_rows / kRopeRows;
+        const int64_t groups = pa.max_tiles * r.item_groups;
         if (int rc = launch(rope_rows_kernel, (unsigned)std::min<int64_t>(groups, (int64_t)num_sms() * 16), 256, 0, st, 1, r)) return rc;
     }
 
     p.hdr = hdr; p.pairs = pairs; p.status = &hdr->status;
     p.out = static_cast<__nv_bfloat16 *>(out); p.lse = lse;
-    p.n_heads = n_heads; p.kv_group = n_heads / n_kv_heads;
+    p.n_heads = n_heads; p.log_rows = 7 - log_g; p.n_units = n_heads >> log_g; p.units_per_kv = group >> log_g;
     p.total_tokens = lay->total_tokens; p.scale_log2e = scale * kLog2eT;
     p.wide_stores = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
     p.pos = pos; p.slopes = slopes;
     p.stall_producer = g_stall_producer ? 1 : 0;      // test hook, see sp_test_stall_producer below
 
-    const int64_t items = pa.max_tiles * n_heads;
+    const int64_t items = pa.max_tiles * p.n_units;
     if (items == 0) return SP_OK;
     const int grid = (int)std::min<int64_t>(items, num_sms());
-    if (head_dim == 64) return pos ? launch_kernel<64, true>(p, grid, st) : launch_kernel<64, false>(p, grid, st);
-    return pos ? launch_kernel<128, true>(p, grid, st) : launch_kernel<128, false>(p, grid, st);
+    using Launch = int (*)(const TcParams &, int, cudaStream_t);
+    const auto run = [&](Launch single, Launch grouped) { return (log_g ? grouped : single)(p, grid, st); };
+    if (head_dim == 64)
+        return pos ? run(launch_kernel<64, true, false>, launch_kernel<64, true, true>)
+                   : run(launch_kernel<64, false, false>, launch_kernel<64, false, true>);
+    return pos ? run(launch_kernel<128, true, false>, launch_kernel<128, true, true>)
+               : run(launch_kernel<128, false, false>, launch_kernel<128, false, true>);
 }
 
 int launch_prefill_tc(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,

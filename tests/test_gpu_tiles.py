@@ -63,13 +63,23 @@ def test_prefill_segment_lengths(D, alibi, pre):
 
 
 @pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("H,Hkv", [(3, 1), (6, 1), (4, 1), (12, 1), (16, 2), (16, 1)])
+@pytest.mark.parametrize("rows,alibi", [(sp.SP_ROWS_ALL, False), (sp.SP_ROWS_ALL, True), (sp.SP_ROWS_QUERY_ONLY, False)])
+def test_prefill_heads_sharing_a_tile(D, H, Hkv, rows, alibi):
+    """1, 2, 4 and 8 heads in a tile (128, 64, 32 and 16 rows of each); segments around the tiles' and pairs' edges."""
+    lens = [1, 15, 16, 17, 31, 32, 33, 63, 64, 65, 96, 127, 129, 257]
+    lay = build_layout([21, 70], [[n - min(n, 33) for n in lens], [40, 150]], [[min(n, 33) for n in lens], [16, 17]])
+    _prefill(lay, H, Hkv, D, rows=rows, alibi=alibi)
+
+
+@pytest.mark.parametrize("D", [64, 128])
 def test_prefill_output_aligned_to_16_bytes_only(D):
     _prefill(build_layout([20], [[100, 150]], [[24, 24]]), 2, 2, D, shift=8)
 
 
 @pytest.mark.parametrize("pre,alibi", [(64, True), (65, True), (384, False), (385, False)])
 def test_prefill_query_only_either_kernel(pre, alibi):
-    _prefill(build_layout([pre, 5], [[40, 130], [9, 0]], [[32, 7], [33, 100]]), 4, 2, 128, rows=sp.SP_ROWS_QUERY_ONLY, alibi=alibi)
+    _prefill(build_layout([pre, 5], [[40, 130], [9, 0]], [[32, 7], [33, 100]]), 6, 2, 128, rows=sp.SP_ROWS_QUERY_ONLY, alibi=alibi)
 
 
 @pytest.mark.parametrize("D", [64, 128])
