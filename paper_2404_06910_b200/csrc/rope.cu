@@ -13,7 +13,6 @@ struct RopeFreq {
 };
 
 constexpr int kRopeThreads = 256;
-constexpr int kRopeTokens = 4;   // tokens per block iteration
 
 template <typename T> struct Pack;
 template <> struct Pack<__nv_bfloat16> {
@@ -102,21 +101,22 @@ __device__ __forceinline__ void rotate_tokens(T *__restrict__ x, const float2 (*
 
 // One launch may rotate two tensors that share their positions (a step's Q and K): x1 == NULL
 // rotates x alone.  VEC / VEC1: whether the 16-byte path applies to x / x1.
-template <typename T, bool VEC, bool VEC1>
+// GROUP: tokens per block iteration.
+template <typename T, bool VEC, bool VEC1, int GROUP>
 __global__ void __launch_bounds__(kRopeThreads, 8)   // 32 registers: full occupancy for the streaming pass
 rope_kernel(T *__restrict__ x, T *__restrict__ x1, const float *__restrict__ pos, int64_t n_tokens, int64_t ld_token,
             int64_t ld_token1, int n_heads, int n_heads1, int head_dim, int rot_dim, int pairing,
             const __grid_constant__ RopeFreq fr)
 {
-    __shared__ float2 cs[kRopeTokens][128];   // (cos, sin) per (token, pair)
+    __shared__ float2 cs[GROUP][128];   // (cos, sin) per (token, pair)
     pdl_wait();
     pdl_trigger();
     const int half = rot_dim >> 1;
-    const int64_t n_groups = (n_tokens + kRopeTokens - 1) / kRopeTokens;
+    const int64_t n_groups = (n_tokens + GROUP - 1) / GROUP;
 
     for (int64_t g = blockIdx.x; g < n_groups; g += gridDim.x) {
-        const int64_t t0 = g * kRopeTokens;
-        const int nt = (int)min((int64_t)kRopeTokens, n_tokens - t0);
+        const int64_t t0 = g * GROUP;
+        const int nt = (int)min((int64_t)GROUP, n_tokens - t0);
         __syncthreads();
         for (int i = threadIdx.x; i < nt * half; i += kRopeThreads) {
             const int t = i / half, m = i - t * half;
@@ -146,15 +146,24 @@ static int launch_rope(void *x, void *x1, const float *pos, int64_t n_tokens, in
 {
     const bool v0 = rope_vec_ok<T>(x, ld_token, head_dim, rot_dim, pairing);
     const bool v1 = x1 == nullptr || rope_vec_ok<T>(x1, ld_token1, head_dim, rot_dim, pairing);
-    const int64_t n_groups = (n_tokens + kRopeTokens - 1) / kRopeTokens;
+    // Tokens per block iteration (GROUP).  The angles of four tokens keep every thread of a block busy and pay off in the long pass, but
+    // a launch of few tokens wants its blocks small: the chain position -> angle -> data is run through once, and blocks of a
+    // last wave should be many.  us with 4 / 2 / 1 tokens at 32 heads of 128: 300 tokens 3.9 / 3.3 / 2.9, 3 060 14.2 / 10.8 / 10.3,
+    // 6 000 19.7 / 19.0 / 19.4, 9 000 26.7 / 26.7 / 27.7, 60 000 155 / 159 / 173; with few heads one token leaves threads idle (8
+    // heads, 4 000 tokens: 6.1 / 5.9 / 7.3).
+    const int64_t wave = (int64_t)num_sms() * 8;
+    const int vecs = n_heads * (rot_dim / 2) / Pack<T>::N;               // per token, of either half
+    const int group = n_tokens > 8 * wave || !v0 || !v1 ? 4 : (n_tokens <= 3 * wave && vecs >= kRopeThreads ? 1 : 2);
+    const int64_t n_groups = (n_tokens + group - 1) / group;
     const int grid = (int)std::min<int64_t>(n_groups, (int64_t)num_sms() * 16);
     auto go = [&](auto kern) {
         return launch(kern, grid, kRopeThreads, 0, st, 1, (T *)x, (T *)x1, pos, n_tokens, ld_token, ld_token1, n_heads, n_heads1,
                       head_dim, rot_dim, pairing, fr);
     };
-    if (v0 && v1) return go(rope_kernel<T, true, true>);
-    if (v0) return go(rope_kernel<T, true, false>);
-    return v1 ? go(rope_kernel<T, false, true>) : go(rope_kernel<T, false, false>);
+    if (v0 && v1)
+        return group == 4 ? go(rope_kernel<T, true, true, 4>) : (group == 2 ? go(rope_kernel<T, true, true, 2>) : go(rope_kernel<T, true, true, 1>));
+    if (v0) return go(rope_kernel<T, true, false, 4>);
+    return v1 ? go(rope_kernel<T, false, true, 4>) : go(rope_kernel<T, false, false, 4>);
 }
 
 static int rope_entry(const char *name, void *x, int64_t ld_token, int n_heads, void *x1, int64_t ld_token1, int n_heads1,

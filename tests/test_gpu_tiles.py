@@ -132,3 +132,23 @@ def test_path_scores_row_alignments(dtype, vocab, pad, n_paths, qry):
     sp.sp_path_scores(dev(logits)[:, :vocab], dev(tgt), dev(off), scores, None, None, row_logp)
     np.testing.assert_allclose(row_logp.cpu().numpy(), ref_r, atol=1e-3)
     np.testing.assert_allclose(scores.cpu().numpy(), ref_s, atol=1e-3 * qry)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("H,D", [(2, 64), (64, 64)])
+@pytest.mark.parametrize("waves", [0, 3, 8])
+@pytest.mark.parametrize("more", [0, 1])
+def test_rope_tokens_per_block(dtype, H, D, waves, more):
+    """One, two and four tokens to a block: both sides of each limit (waves of 8 blocks per SM), a last block that is not full.
+    Tolerances of the parity suite (fp32: a few roundings of values up to 5; bf16: one rounding more, up to 2^-8 of the value)."""
+    T = waves * 8 * torch.cuda.get_device_properties(0).multi_processor_count + more + (1 if waves == 0 else 0)
+    x = _randn((T, H, D), 1, dtype)
+    pos = torch.rand(T, generator=torch.Generator().manual_seed(2)).mul(700).float()
+    got = dev(x)
+    sp.sp_rope_apply(got, dev(pos), H, D)
+    at = np.unique(np.concatenate([np.arange(min(T, 5)), np.arange(max(T - 5, 0), T), np.arange(0, T, 97)]))
+    ref = oracle.rope(f32(x)[at], pos.numpy()[at])
+    got = f32(got)
+    assert np.isfinite(got).all()
+    bound = 4e-6 if dtype == torch.float32 else np.abs(ref) * 2.0 ** -8 * 1.02 + 1e-6
+    assert (np.abs(got[at] - ref) <= bound).all()
