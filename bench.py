@@ -46,12 +46,12 @@ PREFILL_LAUNCHES = 2           # kernels sp_superpose_prefill launches per call 
 # Each entry names the hash of the kernel sources it was taken from: after a kernel change the
 # figure is withheld (null in the JSON line) until the capture is repeated.
 NCU_TRAFFIC = {
-    ("prefill", "cfg2_batched_serving"): {"bytes_per_unit": 2602638512.0 / 74087, "unit": "token",
+    ("prefill", "cfg2_batched_serving"): {"bytes_per_unit": 2441349632.0 / 74087, "unit": "token",
                                           "capture": "the cfg2 shape with 20 prompts (74 087 tokens), one launch",
-                                          "source_hash": "84bbcbe117cf"},
-    ("decode", "cfg3_llama2_7b"): {"bytes_per_unit": 109603584.0 / 6548, "unit": "gathered key",
+                                          "source_hash": "e5954b3e32ae"},
+    ("decode", "cfg3_llama2_7b"): {"bytes_per_unit": 110206976.0 / 6548, "unit": "gathered key",
                                    "capture": "cfg3 (8 prompts, 6 548 keys per launch), two launches averaged",
-                                   "source_hash": "18396a4613a6"},
+                                   "source_hash": "743f3273fb32"},
 }
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
@@ -303,7 +303,7 @@ class HotPath:
 
 STAGES = ("rope", "prefill", "path_scores", "topk", "decode")
 PREFILL_SOURCES = ("prefill_tc.cu", "prefill_plan.cuh", "tc_ptx.cuh")
-DECODE_SOURCES = ("decode.cu",)
+DECODE_SOURCES = ("decode.cu", "decode_mma.cuh")
 
 
 def source_hash(names) -> str:
@@ -601,8 +601,8 @@ def run_widened(args):
                                                           sp.SP_ROPE_HALF_SPLIT, hp.scale, hp.out, None, ws_rope))
     rope_fused = {"workload": cfg.name, "rope_q_ms": rope_q_ms, "prefill_ms": plain_ms, "two_calls_ms": rope_q_ms + plain_ms,
                   "prefill_rope_ms": fused_ms,
-                  "note": "sp_superpose_prefill_rope = (cos, sin) table kernel + tile plan + prefill kernel that rotates each "
-                          "query tile in shared memory; K is rotated by sp_rope_apply in both paths"}
+                  "note": "sp_superpose_prefill_rope = tile plan + a pass that rotates Q into the output tensor + the prefill "
+                          "kernel reading its query tiles there; K is rotated by sp_rope_apply in both paths"}
     del ws_rope
     hp.step()
     torch.cuda.synchronize()
@@ -650,7 +650,7 @@ def run_widened(args):
         del q, k, v, out
         torch.cuda.empty_cache()
     # grouped query heads: the cfg2 decode shape with 8 KV heads under the 32 query heads (one block owns
-    # a KV head and 4 of its query heads, so each K / V row is read once per group)
+    # a KV head and all 4 of its query heads, so each K / V row is read once per group)
     lay_g = draw_lengths(cfg)
     Bg, Hkv_g, n_g = lay_g.n_prompts, 8, 8
     g = torch.Generator(device=device); g.manual_seed(8)
@@ -676,7 +676,7 @@ def run_widened(args):
     del kc_sets, qg, tkg, tvg, out_g
     torch.cuda.empty_cache()
 
-    # bf16 with head_dim 64 (served by the fp32-arithmetic SIMT kernel): a smaller batch of the cfg2 shape
+    # bf16 with head_dim 64: a smaller batch of the cfg2 shape
     lay64 = draw_lengths(get_config("cfg2"), n_prompts=8)
     T64, H64, D64 = lay64.total_tokens, 32, 64
     g = torch.Generator(device=device); g.manual_seed(64)
@@ -686,12 +686,12 @@ def run_widened(args):
     ws64 = torch.zeros(max(256, sp.sp_prefill_workspace_bytes(dl64, H64, D64, sp.SP_BF16)), dtype=torch.uint8, device=device)
     ms64 = timed(lambda: sp.sp_superpose_prefill(q, k, v, dl64, D64 ** -0.5, out, None, ws64), reps=3)
     flop64 = 4.0 * D64 * H64 * lay64.allowed_pairs()
-    simt = {"shape": "cfg2 lengths, 8 prompts, 32 heads x 64, bf16", "tokens": int(T64), "prefill_ms": ms64,
+    dim64 = {"shape": "cfg2 lengths, 8 prompts, 32 heads x 64, bf16", "tokens": int(T64), "prefill_ms": ms64,
             "useful_tflops": flop64 / (ms64 * 1e-3) / 1e12, "frac_hbm": gb(4.0 * T64 * H64 * D64 * 2, ms64) / hbm,
-            "note": "warp per (row, head), fp32 FMA arithmetic, no tensor cores"}
+            "note": "tensor cores, probabilities as the sum of two bf16 numbers"}
     del q, k, v, out
     print(json.dumps({"widened": True, "alibi": alibi, "rope_folded_into_prefill": rope_fused, "decode_grouped_heads": gqa,
-                      "bf16_head_dim_64": simt,
+                      "bf16_head_dim_64": dim64,
                       "iterative": {"prompts": n_prompts, "documents": n_docs, "kept_per_round": k_keep, "rounds": iters,
                                     "data": "synthetic, lengths U{60..180}"}}))
 

@@ -4,9 +4,14 @@
 // HBM-bound: every kept K and V row is read exactly once.  Pruning is an index list --
 // the kernel walks [preamble | kept path ranges | tail] as one logical key sequence and
 // never copies KV.  The sequence is split across blocks (split-KV) so that small batches
-// still fill the machine; each block keeps an online softmax per key group, writes one
-// partial (max, sum, unnormalised output), and the last block to finish a (prompt, head)
-// merges the partials in split order, so results do not depend on scheduling.
+// still fill the machine.  The blocks of a (prompt, KV head) are one thread-block cluster: each
+// keeps an online softmax per key group and writes one partial (max, sum, unnormalised output)
+// per head into the shared memory of the cluster's first block, which merges them in split
+// order, so results do not depend on scheduling.  sp_pruned_decode_static merges through global
+// memory instead.  bf16 with several query heads to a KV head: decode_mma.cuh.
+// Measured, 2 prompts x 32 heads, 8 kept of 400 paths of 160-544 rows, 95 MB: 24.6 us (26.6 with
+// partials fetched by the first block and without programmatic dependent launch), 14.5 at the
+// copy bandwidth; what is left is launch, index loads and one wave's ramp.
 #include <cooperative_groups.h>
 
 #include "common.cuh"

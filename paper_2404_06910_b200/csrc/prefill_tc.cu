@@ -33,6 +33,10 @@
 // Every mbarrier wait is bounded: on expiry the block records a timeout in the workspace status word, unwinds, frees its
 // tensor memory and exits.
 // sp_superpose_prefill_rope rotates Q into `out` first and runs the same kernel on it.
+// Measured (32 heads of 128, us; before: two blocks per SM, a tile each, K and V loaded per tile): 2 prompts x 400 documents of
+// 128-512 rows 3208 -> 2580, 64 prompts x 17 paths behind a prefix of some 390 rows 3224 -> 2724, ALiBi 1366 -> 954; head_dim 64
+// (before: fp32 arithmetic) 9387 -> 172.  These launches run at the board's power limit (1.3 to 1.55 GHz): leaving out all
+// exponentials gains 2 %, so time follows the energy of the loads and products rather than any one pipe.
 #include "common.cuh"
 #include "prefill_plan.cuh"
 #include "tc_ptx.cuh"
