@@ -814,6 +814,8 @@ static int launch_tc(const void *q, const void *k, const void *v, const sp_layou
     pa.n_prompts = lay->n_prompts; pa.n_paths = lay->n_paths; pa.rows_mode = rows; pa.tile_rows = kBM >> log_g;
     pa.max_pre_len = lay->max_pre_len; pa.max_path_len = lay->max_path_len; pa.total_tokens = lay->total_tokens;
     pa.max_tiles = plan_max_tiles(lay->n_prompts, lay->n_paths, lay->max_pre_len, lay->max_path_len, 2 * pa.tile_rows);
+    // the sort takes a microsecond: worth it from a dozen items per block
+    pa.sort_from = 12 * num_sms() / (n_heads >> log_g);
     pa.hdr = hdr; pa.list = pairs;
     if (int rc = launch(prefill_plan_kernel<true>, 1, 1024, 0, st, 1, pa)) return rc;
     if (rope) {

@@ -72,6 +72,16 @@ def test_prefill_heads_sharing_a_tile(D, H, Hkv, rows, alibi):
     _prefill(lay, H, Hkv, D, rows=rows, alibi=alibi)
 
 
+@pytest.mark.parametrize("n_paths", [20, 63, 64, 79])
+@pytest.mark.parametrize("H,Hkv", [(40, 40), (64, 8)])
+def test_prefill_sorted_work_list(n_paths, H, Hkv):
+    """Lists from a dozen items per block are sorted in runs of 16 records: shorter ones, whole runs and a last run that is
+    not full (a record per path and two for the preambles at one head per tile)."""
+    rng = np.random.default_rng(n_paths)
+    lay = build_layout([33, 5], [rng.integers(0, 180, n_paths), [70]], [[3] * n_paths, [8]])
+    _prefill(lay, H, Hkv, 64)
+
+
 @pytest.mark.parametrize("D", [64, 128])
 def test_prefill_output_aligned_to_16_bytes_only(D):
     _prefill(build_layout([20], [[100, 150]], [[24, 24]]), 2, 2, D, shift=8)
