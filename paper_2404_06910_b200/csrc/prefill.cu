@@ -56,11 +56,13 @@ static int prefill_entry(const void *q, const void *k, const void *v, const sp_l
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // Query rows only: the tcgen05 kernel has a quarter of its tile's rows at work but loads keys with TMA and is the faster one
     // while a path's keys are mostly its own; behind a long preamble the smaller tiles of the warp-level kernel win.  us at 8
-    // prompts x 100 documents, 32 query rows, tcgen05 / warp-level: preamble 48: 615 / 654, 256: 950 / 955, about 1 250: 2522 /
-    // 2368; ALiBi, whose bias a lone softmax warp feels more: 48: 749 / 747, 128: 879 / 868, 256: 1255 / 1113.  More than 32
-    // query rows per path would speak for tcgen05 at any length (48 rows behind 1 000: 997 / 1859) but are not known here.  With
-    // an even number of query heads to a KV head the tcgen05 tiles hold the rows of several heads and win everywhere: preamble
-    // 1 250, 40 documents: 618 / 1128 (two heads), 360 / 1123 (four); ALiBi behind 500: 449 / 672, 254 / 657.
+    // prompts x 100 documents of 64-256 rows, 32 query rows, tcgen05 / warp-level: preamble 16: 530 / 552, 64: 600 / 605, 128:
+    // 701 / 715, 256: 959 / 936, 400: 1295 / 1214, 600: 1752 / 1553, 1 200: 3112 / 2607; 2 x 40 documents: 128: 82 / 88, 400: 143 /
+    // 145, 1 200: 333 / 302; ALiBi, whose bias a lone softmax warp feels more: 16: 630 / 694, 64: 755 / 748, 96: 890 / 805, 256:
+    // 1343 / 1110.  The line lies above the crossing (about 200 rows, ALiBi 64) because the number of query rows is not known
+    // here: from 33 rows per path the warp-level kernel reads every key twice (48 rows behind 48 rows: 666 / 1216, behind 600:
+    // 1825 / 3114).  With an even number of query heads to a KV head the tcgen05 tiles hold the rows of several heads and win
+    // everywhere: behind 1 200 rows, 4 x 20 documents: 193 / 302 (two heads), 114 / 303 (four); ALiBi 257 / 347, 155 / 343.
     if (dtype == SP_BF16 && head_dim == 128 && rows == SP_ROWS_QUERY_ONLY && lay->max_pre_len > (pos ? 64 : 384) &&
         n_heads / n_kv_heads % 2)
         return launch_prefill_qonly(q, k, v, lay, pos, slopes, n_heads, n_kv_heads, scale, out, lse, ws, st);

@@ -56,10 +56,13 @@ constexpr float kRescaleThreshold = 8.f;   // log2 units: rescale O only when th
 
 enum { WARP_EPI = 8, WARP_K = 12, WARP_V, WARP_Q, WARP_POS, WARP_MMA, WARP_PASS = WARP_MMA + 2 };
 
-// SPLIT_P (head_dim 64): P is carried as the sum of two bf16 numbers (16 bits of mantissa), so that this path is as
-// precise as fp32 arithmetic; the second product then runs twice, which its short rows leave time for.
-template <int D, bool ALIBI> struct TcConfig {
-    static constexpr bool SPLIT_P = D == 64;
+// SPLIT_P: P is carried as the sum of two bf16 numbers (16 bits of mantissa) and the second product runs twice.  Set for
+// head_dim 64, which is then as precise as fp32 arithmetic, and for query rows only: relative to the maximum over a first
+// key tile, P in one bf16 number was less exact there (2.27e-3 of the norm from 64-bit results, 8 prompts x 100 documents)
+// than relative to the running maximum of prefill_qonly.cu (2.13e-3); as two it is 1.66e-3, the rounding of the output.  Cost
+// there: 514 -> 584 us.
+template <int D, bool ALIBI, bool SPLIT> struct TcConfig {
+    static constexpr bool SPLIT_P = SPLIT;
     static constexpr int HALVES = D / 64;                       // 64-column halves of a row (one 128-byte swizzle atom each)
     static constexpr int Q_BYTES = kBM * D * 2, KV_BYTES = kBN * D * 2;
     static constexpr int NQ = D == 64 ? 4 : 3;                  // query slots
@@ -81,7 +84,7 @@ template <int D, bool ALIBI> struct TcConfig {
     static_assert(2 * R_SOFT + R_EPI + R_LOAD + R_MMA <= kTcThreads / 128 * R_LAUNCH, "registers of a block");
     static_assert(R_SOFT >= R_LAUNCH && R_EPI <= R_LAUNCH && R_LOAD <= R_LAUNCH && R_MMA <= R_LAUNCH, "direction of setmaxnreg");
 };
-static_assert(TcConfig<128, false>::SMEM <= 232448 && TcConfig<128, true>::SMEM <= 232448, "one block's shared memory");
+static_assert(TcConfig<128, false, false>::SMEM <= 232448 && TcConfig<128, true, false>::SMEM <= 232448, "one block's shared memory");
 
 // The instruction stream of the softmax warps is what paces a lane: three-input maxima and two-lane fp32 forms.
 __device__ __forceinline__ float fmax3(float a, float b, float c)
@@ -214,10 +217,10 @@ template <int N> __device__ __forceinline__ void reg_dealloc() { asm volatile("s
 // for ALiBi).
 // GROUPED: tiles of several heads.  A kernel of its own: the index arithmetic costs a launch of single heads 1.5 % (32 query rows of
 // 800 paths, 621 against 630 us).
-template <int D, bool ALIBI, bool GROUPED>
+template <int D, bool ALIBI, bool GROUPED, bool SPLIT>
 __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_constant__ TcParams p)
 {
-    using C = TcConfig<D, ALIBI>;
+    using C = TcConfig<D, ALIBI, SPLIT>;
     const int log_rows = GROUPED ? p.log_rows : 7;
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char *sQ = smem, *sK = smem + C::NQ * C::Q_BYTES, *sV = sK + C::NKV * C::KV_BYTES;
@@ -772,11 +775,11 @@ size_t prefill_tc_workspace_bytes(int n_prompts, int n_paths, int max_pre_len, i
     return 256 + round_up((size_t)plan_max_tiles(n_prompts, n_paths, max_pre_len, max_path_len, 32) * sizeof(TcPair), 256);
 }
 
-template <int D, bool ALIBI, bool GROUPED> static int launch_kernel(const TcParams &p, int grid, cudaStream_t st)
+template <int D, bool ALIBI, bool GROUPED, bool SPLIT> static int launch_kernel(const TcParams &p, int grid, cudaStream_t st)
 {
-    using C = TcConfig<D, ALIBI>;
-    SP_CUDA(cudaFuncSetAttribute(prefill_tc_kernel<D, ALIBI, GROUPED>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-    return launch(prefill_tc_kernel<D, ALIBI, GROUPED>, grid, kTcThreads, C::SMEM, st, 1, p);
+    using C = TcConfig<D, ALIBI, SPLIT>;
+    SP_CUDA(cudaFuncSetAttribute(prefill_tc_kernel<D, ALIBI, GROUPED, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
+    return launch(prefill_tc_kernel<D, ALIBI, GROUPED, SPLIT>, grid, kTcThreads, C::SMEM, st, 1, p);
 }
 
 static int launch_tc(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
@@ -839,10 +842,13 @@ static int launch_tc(const void *q, const void *k, const void *v, const sp_layou
     using Launch = int (*)(const TcParams &, int, cudaStream_t);
     const auto run = [&](Launch single, Launch grouped) { return (log_g ? grouped : single)(p, grid, st); };
     if (head_dim == 64)
-        return pos ? run(launch_kernel<64, true, false>, launch_kernel<64, true, true>)
-                   : run(launch_kernel<64, false, false>, launch_kernel<64, false, true>);
-    return pos ? run(launch_kernel<128, true, false>, launch_kernel<128, true, true>)
-               : run(launch_kernel<128, false, false>, launch_kernel<128, false, true>);
+        return pos ? run(launch_kernel<64, true, false, true>, launch_kernel<64, true, true, true>)
+                   : run(launch_kernel<64, false, false, true>, launch_kernel<64, false, true, true>);
+    if (rows == SP_ROWS_QUERY_ONLY)               // P as two bf16 numbers, see TcConfig
+        return pos ? run(launch_kernel<128, true, false, true>, launch_kernel<128, true, true, true>)
+                   : run(launch_kernel<128, false, false, true>, launch_kernel<128, false, true, true>);
+    return pos ? run(launch_kernel<128, true, false, false>, launch_kernel<128, true, true, false>)
+               : run(launch_kernel<128, false, false, false>, launch_kernel<128, false, true, false>);
 }
 
 int launch_prefill_tc(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,

@@ -92,6 +92,29 @@ def test_prefill_query_only_either_kernel(pre, alibi):
     _prefill(build_layout([pre, 5], [[40, 130], [9, 0]], [[32, 7], [33, 100]]), 6, 2, 128, rows=sp.SP_ROWS_QUERY_ONLY, alibi=alibi)
 
 
+@pytest.mark.parametrize("H,Hkv,pre,alibi,bound", [(6, 6, 48, False, 1.8e-3), (6, 2, 64, True, 1.8e-3), (8, 2, 400, False, 1.8e-3),
+                                                   (6, 6, 400, False, 2.4e-3)])
+def test_prefill_query_only_precision(H, Hkv, pre, alibi, bound):
+    """Distance of the query rows to 64-bit results.  Rounding the output to bf16 alone is 1.66e-3 of its norm for values spread
+    over binades (2^-8 / sqrt 3 over a root-mean-square mantissa of 1.36); probabilities carried to 16 bits add 1e-5, rounded to
+    bf16 relative to the running maximum (the kernel behind long preambles) they add 1.4e-3 in quadrature: 2.2e-3."""
+    lay = build_layout([pre] * 4, [[150, 90, 200, 64]] * 4, [[32, 24, 9, 31]] * 4)
+    T, D = lay.total_tokens, 128
+    q, k, v = _randn((T, H, D), 1), _randn((T, Hkv, D), 2), _randn((T, Hkv, D), 3)
+    pos = torch.rand(T, generator=torch.Generator().manual_seed(4)).mul(300).float()
+    slopes = np.array([2.0 ** (-8.0 * (h + 1) / H) for h in range(H)], np.float32)
+    dl = sp.DeviceLayout.from_host(lay)
+    out, ws = torch.zeros((T, H, D), dtype=torch.bfloat16, device="cuda"), workspace(sp.sp_prefill_workspace_bytes(dl, H, D, sp.SP_BF16))
+    args = (dev(q), dev(k), dev(v), dl)
+    if alibi:
+        sp.sp_superpose_prefill_alibi(*args, dev(pos), dev(slopes), D ** -0.5, out, None, ws, rows=sp.SP_ROWS_QUERY_ONLY)
+    else:
+        sp.sp_superpose_prefill(*args, D ** -0.5, out, None, ws, rows=sp.SP_ROWS_QUERY_ONLY)
+    ref, _ = oracle.prefill(f32(q), f32(k), f32(v), lay, D ** -0.5, **(dict(pos=pos.numpy(), slopes=slopes) if alibi else {}))
+    rows = np.concatenate([np.arange(s + d, s + d + n) for s, d, n in zip(lay.path_start, lay.doc_len, lay.qry_len)])
+    assert rel_l2(f32(out)[rows], ref[rows]) <= bound
+
+
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("alibi", [False, True])
 def test_prefill_f32_tiles(D, alibi):
