@@ -158,7 +158,7 @@ int sp_superpose_prefill(const void *q, const void *k, const void *v, const sp_l
  *   scores[i]   = weight[i] * sum_{t in [row_off[i], row_off[i+1])} row_logp[t] + prior[i].
  * The cross-entropy is "shifted": row t is scored against the segment's token t+1 and the
  * last row has target -1.  logits: [R, vocab], row stride ld_logits elements, rows
- * path-major, finite values; targets: int32 [R] in [-1, vocab); row_off: int32
+ * path-major, finite values or -inf (a masked logit; not the target's); targets: int32 [R] in [-1, vocab); row_off: int32
  * [n_paths+1]; prior / weight: fp32 [n_paths] or NULL (0 / 1).  scores: fp32 [n_paths];
  * row_logp: fp32 [R] or NULL (then the workspace holds it).  n_rows = R (host scalar).
  * Targets outside [-1, vocab) score as -1.  One pass over the logits; sums run in a fixed

@@ -168,6 +168,35 @@ def test_path_scores_row_alignments(dtype, vocab, pad, n_paths, qry):
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("vocab,pad", [(8, 0), (129, 0), (2051, 3), (2048, 0), (50257, 0)])
+@pytest.mark.parametrize("n_paths,qry", [(3, 5), (900, 4)])
+@pytest.mark.parametrize("lowest", [False, True])
+def test_path_scores_masked_logits(dtype, vocab, pad, n_paths, qry, lowest):
+    """Logits of -inf or the type's lowest value at the head of a row, at its end, over a whole range, in every vector of some
+    threads, and everywhere but at the target.  Tolerance: 1e-3 per row as in the parity suite."""
+    if vocab == 50257 and n_paths == 900:
+        n_paths = 300                                        # 1 200 rows suffice where rows are long
+    rows = n_paths * qry
+    mask = torch.finfo(dtype).min if lowest else float("-inf")
+    logits = _randn((rows, vocab + pad), 7, dtype) * 3
+    tgt = torch.randint(0, vocab, (rows,), generator=torch.Generator().manual_seed(8), dtype=torch.int32)
+    tgt[qry - 1::qry] = -1
+    at = torch.arange(vocab + pad)
+    banned = [at < 1, at >= vocab - 1, at >= vocab // 2, at // 8 % 256 == 3, at >= 0]
+    for r in range(rows):
+        keep = logits[r, max(int(tgt[r]), 0)].clone()
+        logits[r, banned[r % 5]] = mask
+        logits[r, max(int(tgt[r]), 0)] = keep
+    off = np.arange(0, rows + 1, qry, dtype=np.int32)
+    ref_s, ref_r = oracle.path_scores(f32(logits[:, :vocab].contiguous()), tgt.numpy(), off, None, None)
+    assert np.isfinite(ref_r).all()
+    scores, row_logp = torch.empty(n_paths, device="cuda"), torch.empty(rows, device="cuda")
+    sp.sp_path_scores(dev(logits)[:, :vocab], dev(tgt), dev(off), scores, None, None, row_logp)
+    np.testing.assert_allclose(row_logp.cpu().numpy(), ref_r, atol=1e-3)
+    np.testing.assert_allclose(scores.cpu().numpy(), ref_s, atol=1e-3 * qry)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("H,D", [(2, 64), (64, 64)])
 @pytest.mark.parametrize("waves", [0, 3, 8])
 @pytest.mark.parametrize("more", [0, 1])
