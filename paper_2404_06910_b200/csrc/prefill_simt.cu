@@ -145,15 +145,26 @@ prefill_simt_kernel(const __grid_constant__ PrefillSimtArgs a)
             }
         }
         __syncwarp();
-        const int n = min(BN, n_keys - base);
+        // V rows hidden from both rows of the pair are not touched, and the key that only the second row sees has no part in the
+        // first: 0 x Inf or 0 x NaN would reach the rows in front of it
+        const int n = min(BN, n_keys - base), last = pre_n + r0 + row + 1 - base;
 #pragma unroll 4
-        for (int key = 0; key < n; ++key) {
+        for (int key = 0; key < min(n, last); ++key) {
             const float p0 = sp_[row][key], p1 = sp_[row + 1][key];
 #pragma unroll
             for (int c = 0; c < CPT; ++c) {
                 const float4 vx = *reinterpret_cast<const float4 *>(&sv[key][c * 64 + tx * 4]);
                 o[0][c].x = fmaf(p0, vx.x, o[0][c].x); o[0][c].y = fmaf(p0, vx.y, o[0][c].y);
                 o[0][c].z = fmaf(p0, vx.z, o[0][c].z); o[0][c].w = fmaf(p0, vx.w, o[0][c].w);
+                o[1][c].x = fmaf(p1, vx.x, o[1][c].x); o[1][c].y = fmaf(p1, vx.y, o[1][c].y);
+                o[1][c].z = fmaf(p1, vx.z, o[1][c].z); o[1][c].w = fmaf(p1, vx.w, o[1][c].w);
+            }
+        }
+        if (last >= 0 && last < n) {
+            const float p1 = sp_[row + 1][last];
+#pragma unroll
+            for (int c = 0; c < CPT; ++c) {
+                const float4 vx = *reinterpret_cast<const float4 *>(&sv[last][c * 64 + tx * 4]);
                 o[1][c].x = fmaf(p1, vx.x, o[1][c].x); o[1][c].y = fmaf(p1, vx.y, o[1][c].y);
                 o[1][c].z = fmaf(p1, vx.z, o[1][c].z); o[1][c].w = fmaf(p1, vx.w, o[1][c].w);
             }

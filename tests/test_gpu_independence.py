@@ -93,6 +93,31 @@ def test_prefill_ignores_rows_outside_every_segment():
     assert torch.equal(out0[used], out1[used]) and torch.equal(lse0[:, used], lse1[:, used])
 
 
+@pytest.mark.parametrize("dtype,D", [("f32", 64), ("f32", 128)])
+@pytest.mark.parametrize("rows", [sp.SP_ROWS_ALL, sp.SP_ROWS_QUERY_ONLY])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_prefill_rows_in_front_of_a_key_do_not_see_it(dtype, D, rows, bad):
+    """Causality with a value that is not finite: the rows in front of it keep their bits, the rows behind it have it in its
+    column and keep the others (probabilities of a few hundred keys do not underflow)."""
+    lay = _layout()
+    T, H, Hkv = lay.total_tokens, 4, 2
+    q, k, v = _randn((T, H, D), dtype, 930), _randn((T, Hkv, D), dtype, 931), _randn((T, Hkv, D), dtype, 932)
+    out0, lse0 = _run_prefill(q, k, v, lay, rows)
+    own = _path_rows(lay, 1)                              # 137 rows, the last seven are query rows
+    for at in (0, 1, 62, 63, 64, 127, 131, 135, 136):
+        v2 = v.clone()
+        v2[own[at], :, 5] = bad
+        out1, lse1 = _run_prefill(q, k, v2, lay, rows)
+        behind = own[at:] if rows == sp.SP_ROWS_ALL else own[max(at, 130):]
+        keep = torch.ones(T, dtype=torch.bool)
+        keep[torch.from_numpy(behind)] = False
+        cols = torch.arange(D) != 5
+        assert torch.equal(out0[keep], out1[keep]) and torch.equal(lse0, lse1), at
+        assert torch.equal(out0[behind][..., cols], out1[behind][..., cols]), at
+        got = out1[behind][..., 5]
+        assert bool(torch.isnan(got).all() if bad != bad else (got == bad).all()), at
+
+
 @pytest.mark.parametrize("dtype,D", [("bf16", 128), ("f32", 64)])
 @pytest.mark.parametrize("kind", ["finite", "non_finite"])
 def test_decode_sees_only_kept_paths(dtype, D, kind):
