@@ -20,14 +20,40 @@ struct PrefillSimtArgs {
     const float *q, *k, *v;
     float *out, *lse;
     const int32_t *ppo, *pre_start, *pre_len, *path_start, *doc_len, *qry_len;
-    uint32_t *status;            // workspace status word: this kernel has nothing to report and clears it
+    uint32_t *status;            // workspace status word
     int n_prompts, n_paths, n_heads, n_kv_heads, rows_mode;
+    int max_pre_len, max_path_len;               // the host's bounds on the lengths (they sized the grid)
     int64_t total_tokens;
     float scale_log2e;
     const float *pos, *slopes;   // ALiBi: token positions [T] and head slopes [H]; NULL = no bias
 };
 
-// grid: x = row tile x sequences (prompt preambles first, then paths), y = head.
+// Sequence seq (prompt preambles first, then paths): its key ranges [pre_lo, pre_lo + pre_n), fully visible, and [own_lo,
+// own_lo + own_n), causal, and the first row to compute.  False where the device arrays contradict the host scalars (negative or
+// oversized length, rows outside [0, T)), as in the plan of the tensor-core kernels: such a segment is skipped and reported.
+struct SimtSegment { int pre_lo, pre_n, own_lo, own_n, first_row; };
+__device__ __forceinline__ bool simt_segment(const PrefillSimtArgs &a, int seq, SimtSegment &g)
+{
+    auto inside = [&](int row, int n) { return n >= 0 && row >= 0 && (int64_t)row + n <= a.total_tokens; };
+    if (seq < a.n_prompts) {
+        g = {0, 0, a.pre_start[seq], a.pre_len[seq], 0};
+        const bool ok = inside(g.own_lo, g.own_n) && g.own_n <= a.max_pre_len;
+        if (a.rows_mode == SP_ROWS_QUERY_ONLY) g.own_n = 0;
+        return ok;
+    }
+    const int i = seq - a.n_prompts;
+    int lo = 0, hi = a.n_prompts - 1;           // prompt owning path i
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (a.ppo[mid] <= i) lo = mid; else hi = mid - 1;
+    }
+    const int dl = a.doc_len[i], ql = a.qry_len[i];
+    g = {a.pre_start[lo], a.pre_len[lo], a.path_start[i], dl + ql, a.rows_mode == SP_ROWS_QUERY_ONLY ? dl : 0};
+    return dl >= 0 && ql >= 0 && (int64_t)dl + ql <= a.max_path_len && inside(g.own_lo, g.own_n) && inside(g.pre_lo, g.pre_n) &&
+           g.pre_n <= a.max_pre_len;
+}
+
+// grid: x = row tile x sequences, and one block more that reports on the layout; y = head.
 template <int D>
 __global__ void __launch_bounds__(kSimtThreads)
 prefill_simt_kernel(const __grid_constant__ PrefillSimtArgs a)
@@ -41,28 +67,20 @@ prefill_simt_kernel(const __grid_constant__ PrefillSimtArgs a)
 
     pdl_wait();
     pdl_trigger();
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *a.status = STATUS_OK;
     const int n_seq = a.n_prompts + a.n_paths;
+    if (blockIdx.x == gridDim.x - 1) {          // a block of its own: nobody waits for it, and the word has one writer
+        if (blockIdx.y) return;
+        bool bad = false;
+        for (int s = threadIdx.x; s < n_seq; s += kSimtThreads) { SimtSegment g; bad |= !simt_segment(a, s, g); }
+        bad = __syncthreads_or(bad);
+        if (threadIdx.x == 0) *a.status = bad ? STATUS_BAD_LAYOUT : STATUS_OK;
+        return;
+    }
     const int tile = blockIdx.x / n_seq, seq = blockIdx.x - tile * n_seq, h = blockIdx.y;
     const int hk = h / (a.n_heads / a.n_kv_heads);
-
-    // key ranges of this sequence: [pre_lo, pre_lo+pre_n) fully visible, own rows causal
-    int pre_lo, pre_n, own_lo, own_n, first_row;
-    if (seq < a.n_prompts) {
-        if (a.rows_mode == SP_ROWS_QUERY_ONLY) return;
-        pre_lo = 0; pre_n = 0;
-        own_lo = a.pre_start[seq]; own_n = a.pre_len[seq]; first_row = 0;
-    } else {
-        const int i = seq - a.n_prompts;
-        int lo = 0, hi = a.n_prompts - 1;           // prompt owning path i
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (a.ppo[mid] <= i) lo = mid; else hi = mid - 1;
-        }
-        pre_lo = a.pre_start[lo]; pre_n = a.pre_len[lo];
-        own_lo = a.path_start[i]; own_n = a.doc_len[i] + a.qry_len[i];
-        first_row = a.rows_mode == SP_ROWS_QUERY_ONLY ? a.doc_len[i] : 0;
-    }
+    SimtSegment g;
+    if (!simt_segment(a, seq, g)) return;
+    const int pre_lo = g.pre_lo, pre_n = g.pre_n, own_lo = g.own_lo, own_n = g.own_n, first_row = g.first_row;
     const int r0 = first_row + tile * kSimtRows;    // first row of the tile, counted in the segment
     const int n_rows = min(kSimtRows, own_n - r0);
     if (n_rows <= 0) return;
@@ -195,12 +213,13 @@ int launch_prefill_simt(const void *q, const void *k, const void *v, const sp_la
     a.ppo = lay->prompt_path_off; a.pre_start = lay->pre_start; a.pre_len = lay->pre_len;
     a.path_start = lay->path_start; a.doc_len = lay->doc_len; a.qry_len = lay->qry_len;
     a.n_prompts = lay->n_prompts; a.n_paths = lay->n_paths; a.n_heads = n_heads; a.n_kv_heads = n_kv_heads;
+    a.max_pre_len = lay->max_pre_len; a.max_path_len = lay->max_path_len;
     a.rows_mode = rows; a.total_tokens = lay->total_tokens; a.scale_log2e = scale * kLog2eP;
     a.pos = pos; a.slopes = slopes;
     const int64_t tiles = (std::max(lay->max_pre_len, lay->max_path_len) + kSimtRows - 1) / kSimtRows;
     const int64_t blocks = std::max<int64_t>(1, tiles) * (lay->n_prompts + lay->n_paths);
     SP_REQUIRE(blocks < (int64_t)INT32_MAX, SP_ERR_UNSUPPORTED, "sp_superpose_prefill: %lld row tiles", (long long)blocks);
-    const dim3 grid((unsigned)blocks, n_heads);
+    const dim3 grid((unsigned)blocks + 1, n_heads);
     return head_dim == 64 ? launch(prefill_simt_kernel<64>, grid, kSimtThreads, 0, st, 1, a)
                           : launch(prefill_simt_kernel<128>, grid, kSimtThreads, 0, st, 1, a);
 }

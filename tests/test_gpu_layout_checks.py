@@ -64,12 +64,13 @@ def test_host_mirror_refuses_inconsistent_layouts(name):
 
 @pytest.mark.parametrize("rows", [sp.SP_ROWS_ALL, sp.SP_ROWS_QUERY_ONLY])
 @pytest.mark.parametrize("name", ["start_beyond_T", "length_over_max", "negative_length"])
-def test_device_checks_skip_and_report_without_a_mirror(name, rows):
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_device_checks_skip_and_report_without_a_mirror(name, rows, dtype):
     base, bad = _bad_layouts()
     T = base.total_tokens
-    q, k, v = _tensors(T)
+    q, k, v = (t.to(dtype) for t in _tensors(T))
     good_dl = sp.DeviceLayout.from_host(base, mirror=False)
-    ws = workspace(sp.sp_prefill_workspace_bytes(good_dl, H, D, sp.SP_BF16))
+    ws = workspace(sp.sp_prefill_workspace_bytes(good_dl, H, D, sp.dtype_code(q)))
     ref = torch.full_like(q, 7.0)
     sp.sp_superpose_prefill(q, k, v, good_dl, 1 / math.sqrt(D), ref, None, ws, rows=rows)
     sp.sp_check_status(ws)
