@@ -22,7 +22,8 @@ struct PrefillSimtArgs {
     const int32_t *ppo, *pre_start, *pre_len, *path_start, *doc_len, *qry_len;
     uint32_t *status;            // workspace status word
     int n_prompts, n_paths, n_heads, n_kv_heads, rows_mode;
-    int max_pre_len, max_path_len;               // the host's bounds on the lengths (they sized the grid)
+    int max_pre_len, max_path_len;               // the host's bounds on the lengths
+    int pre_tiles, path_tiles, pre_z, path_z;    // row tiles a preamble / a path can have, and blocks that share them
     int64_t total_tokens;
     float scale_log2e;
     const float *pos, *slopes;   // ALiBi: token positions [T] and head slopes [H]; NULL = no bias
@@ -53,10 +54,8 @@ __device__ __forceinline__ bool simt_segment(const PrefillSimtArgs &a, int seq, 
            g.pre_n <= a.max_pre_len;
 }
 
-// grid: x = row tile x sequences, and one block more that reports on the layout; y = head.
-template <int D>
-__global__ void __launch_bounds__(kSimtThreads)
-prefill_simt_kernel(const __grid_constant__ PrefillSimtArgs a)
+// Row tile `tile` of sequence `seq` for the head of the block; the whole block takes part.
+template <int D> __device__ __forceinline__ void simt_tile(const PrefillSimtArgs &a, int seq, int tile)
 {
     constexpr int BN = 4096 / D;             // keys per tile: 32 KB of K and V
     constexpr int KPT = BN / 16;             // keys per thread
@@ -64,20 +63,7 @@ prefill_simt_kernel(const __grid_constant__ PrefillSimtArgs a)
     constexpr int KS = D + 4;                // padded K row: 16 lanes reading 16 rows hit different banks
     __shared__ __align__(16) float sq[kSimtRows][D], sk[BN][KS], sv[BN][D], sp_[kSimtRows][BN];
     __shared__ float s_pos[BN];
-
-    pdl_wait();
-    pdl_trigger();
-    const int n_seq = a.n_prompts + a.n_paths;
-    if (blockIdx.x == gridDim.x - 1) {          // a block of its own: nobody waits for it, and the word has one writer
-        if (blockIdx.y) return;
-        bool bad = false;
-        for (int s = threadIdx.x; s < n_seq; s += kSimtThreads) { SimtSegment g; bad |= !simt_segment(a, s, g); }
-        bad = __syncthreads_or(bad);
-        if (threadIdx.x == 0) *a.status = bad ? STATUS_BAD_LAYOUT : STATUS_OK;
-        return;
-    }
-    const int tile = blockIdx.x / n_seq, seq = blockIdx.x - tile * n_seq, h = blockIdx.y;
-    const int hk = h / (a.n_heads / a.n_kv_heads);
+    const int h = blockIdx.y, hk = h / (a.n_heads / a.n_kv_heads);
     SimtSegment g;
     if (!simt_segment(a, seq, g)) return;
     const int pre_lo = g.pre_lo, pre_n = g.pre_n, own_lo = g.own_lo, own_n = g.own_n, first_row = g.first_row;
@@ -86,6 +72,7 @@ prefill_simt_kernel(const __grid_constant__ PrefillSimtArgs a)
     if (n_rows <= 0) return;
     const int n_keys = pre_n + r0 + n_rows;
 
+    __syncthreads();                                // the block's previous tile is done with the query rows
     for (int i = threadIdx.x; i < kSimtRows * (D / 4); i += kSimtThreads) {
         const int r = i / (D / 4), c = i % (D / 4);
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -203,6 +190,28 @@ prefill_simt_kernel(const __grid_constant__ PrefillSimtArgs a)
     }
 }
 
+// grid: x = blocks of the preambles, blocks of the paths, and one block more that reports on the layout; y = head.
+template <int D>
+__global__ void __launch_bounds__(kSimtThreads)
+prefill_simt_kernel(const __grid_constant__ PrefillSimtArgs a)
+{
+    pdl_wait();
+    pdl_trigger();
+    const int n_seq = a.n_prompts + a.n_paths;
+    if (blockIdx.x == gridDim.x - 1) {          // a block of its own: nobody waits for it, and the word has one writer
+        if (blockIdx.y) return;
+        bool bad = false;
+        for (int s = threadIdx.x; s < n_seq; s += kSimtThreads) { SimtSegment g; bad |= !simt_segment(a, s, g); }
+        bad = __syncthreads_or(bad);
+        if (threadIdx.x == 0) *a.status = bad ? STATUS_BAD_LAYOUT : STATUS_OK;
+        return;
+    }
+    const int x = blockIdx.x, n_pre = a.n_prompts * a.pre_z;
+    const bool pre = x < n_pre;
+    const int first = pre ? x / a.n_prompts : (x - n_pre) / a.n_paths, seq = pre ? x - first * a.n_prompts : a.n_prompts + (x - n_pre - first * a.n_paths);
+    for (int tile = first; tile < (pre ? a.pre_tiles : a.path_tiles); tile += pre ? a.pre_z : a.path_z) simt_tile<D>(a, seq, tile);
+}
+
 int launch_prefill_simt(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
                         const float *slopes, int n_heads, int n_kv_heads, int head_dim, float scale, int rows,
                         void *out, float *lse, void *ws, cudaStream_t st)
@@ -216,10 +225,16 @@ int launch_prefill_simt(const void *q, const void *k, const void *v, const sp_la
     a.max_pre_len = lay->max_pre_len; a.max_path_len = lay->max_path_len;
     a.rows_mode = rows; a.total_tokens = lay->total_tokens; a.scale_log2e = scale * kLog2eP;
     a.pos = pos; a.slopes = slopes;
-    const int64_t tiles = (std::max(lay->max_pre_len, lay->max_path_len) + kSimtRows - 1) / kSimtRows;
-    const int64_t blocks = std::max<int64_t>(1, tiles) * (lay->n_prompts + lay->n_paths);
-    SP_REQUIRE(blocks < (int64_t)INT32_MAX, SP_ERR_UNSUPPORTED, "sp_superpose_prefill: %lld row tiles", (long long)blocks);
-    const dim3 grid((unsigned)blocks + 1, n_heads);
+    // No segment is longer than T, however loose the bounds; preambles and paths have a range of their own (one prefix of 1 000
+    // rows beside hundreds of short paths: 63 tiles for every path otherwise).  Beyond 2^16 blocks a sequence's tiles share some.
+    const auto tiles = [&](int64_t n) { return (int)((std::min<int64_t>(n, lay->total_tokens) + kSimtRows - 1) / kSimtRows); };
+    const auto share = [](int n_tiles, int n) { return std::min(n_tiles, std::max(1, (1 << 16) / std::max(n, 1))); };
+    a.pre_tiles = rows == SP_ROWS_ALL ? tiles(lay->max_pre_len) : 0;
+    a.path_tiles = tiles(lay->max_path_len);
+    a.pre_z = share(a.pre_tiles, lay->n_prompts); a.path_z = share(a.path_tiles, lay->n_paths);
+    const int64_t blocks = (int64_t)lay->n_prompts * a.pre_z + (int64_t)lay->n_paths * a.path_z + 1;
+    SP_REQUIRE(blocks < (int64_t)INT32_MAX, SP_ERR_UNSUPPORTED, "sp_superpose_prefill: %d prompts and %d paths", lay->n_prompts, lay->n_paths);
+    const dim3 grid((unsigned)blocks, n_heads);
     return head_dim == 64 ? launch(prefill_simt_kernel<64>, grid, kSimtThreads, 0, st, 1, a)
                           : launch(prefill_simt_kernel<128>, grid, kSimtThreads, 0, st, 1, a);
 }

@@ -123,6 +123,25 @@ def test_prefill_f32_tiles(D, alibi):
     _prefill(lay, 4, 2, D, torch.float32, rows=sp.SP_ROWS_QUERY_ONLY, alibi=alibi)
 
 
+@pytest.mark.parametrize("mirror", [False, True])
+@pytest.mark.parametrize("H,more", [(4, 0), (1, 600000)])
+def test_prefill_f32_loose_bounds(mirror, H, more):
+    """max_pre_len / max_path_len are upper bounds: however large, every row is computed and no launch grows with them (with 600 000
+    more rows in the tensors the blocks of a path walk its row tiles: four paths share 2^16 blocks)."""
+    lay = build_layout([40, 3], [[1, 70, 15], [33]], [[4, 1, 2], [9]])
+    lay.total_tokens += more
+    T, D = lay.total_tokens, 64
+    q, k, v = (torch.randn((T, H, D), device="cuda", generator=torch.Generator("cuda").manual_seed(i)) for i in (1, 2, 3))
+    dl, ws, out = sp.DeviceLayout.from_host(lay, mirror=mirror), workspace(256), []
+    for pre, path in ((lay.max_pre_len, lay.max_path_len), (2 ** 31 - 1, 2 ** 31 - 1)):
+        dl.c.max_pre_len, dl.c.max_path_len = pre, path
+        for rows in (sp.SP_ROWS_ALL, sp.SP_ROWS_QUERY_ONLY):
+            out.append(torch.zeros_like(q))
+            sp.sp_superpose_prefill(q, k, v, dl, 0.125, out[-1], None, ws, rows=rows)
+            sp.sp_check_status(ws)
+    assert torch.equal(out[0], out[2]) and torch.equal(out[1], out[3])
+
+
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("H,Hkv", [(5, 1), (8, 1), (9, 1), (16, 1), (64, 32), (24, 8)])
 @pytest.mark.parametrize("n_prompts", [1, 60])
