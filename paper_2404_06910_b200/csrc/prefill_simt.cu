@@ -13,6 +13,7 @@ namespace sp {
 
 constexpr int kSimtThreads = 128;
 constexpr int kSimtRows = 16;        // query rows per block
+constexpr int64_t kSimtMaxBlocks = 1 << 17;      // in a launch, per head
 constexpr float kLog2eP = 1.4426950408889634f;
 constexpr float kLn2P = 0.6931471805599453f;
 
@@ -23,7 +24,7 @@ struct PrefillSimtArgs {
     uint32_t *status;            // workspace status word
     int n_prompts, n_paths, n_heads, n_kv_heads, rows_mode;
     int max_pre_len, max_path_len;               // the host's bounds on the lengths
-    int pre_tiles, path_tiles, pre_z, path_z;    // row tiles a preamble / a path can have, and blocks that share them
+    int n_pre_blocks, tile0;                     // blocks of the preambles (those of the paths follow), first row tile of the launch
     int64_t total_tokens;
     float scale_log2e;
     const float *pos, *slopes;   // ALiBi: token positions [T] and head slopes [H]; NULL = no bias
@@ -35,27 +36,44 @@ struct PrefillSimtArgs {
 struct SimtSegment { int pre_lo, pre_n, own_lo, own_n, first_row; };
 __device__ __forceinline__ bool simt_segment(const PrefillSimtArgs &a, int seq, SimtSegment &g)
 {
-    auto inside = [&](int row, int n) { return n >= 0 && row >= 0 && (int64_t)row + n <= a.total_tokens; };
+    int dl = 0, ql, most;
     if (seq < a.n_prompts) {
-        g = {0, 0, a.pre_start[seq], a.pre_len[seq], 0};
-        const bool ok = inside(g.own_lo, g.own_n) && g.own_n <= a.max_pre_len;
-        if (a.rows_mode == SP_ROWS_QUERY_ONLY) g.own_n = 0;
-        return ok;
+        g.pre_lo = 0; g.pre_n = 0;
+        g.own_lo = a.pre_start[seq]; ql = a.pre_len[seq]; most = a.max_pre_len;
+    } else {
+        const int i = seq - a.n_prompts;
+        int lo = 0, hi = a.n_prompts - 1;           // prompt owning path i
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (a.ppo[mid] <= i) lo = mid; else hi = mid - 1;
+        }
+        g.pre_lo = a.pre_start[lo]; g.pre_n = a.pre_len[lo];
+        g.own_lo = a.path_start[i]; dl = a.doc_len[i]; ql = a.qry_len[i]; most = a.max_path_len;
     }
-    const int i = seq - a.n_prompts;
-    int lo = 0, hi = a.n_prompts - 1;           // prompt owning path i
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (a.ppo[mid] <= i) lo = mid; else hi = mid - 1;
-    }
-    const int dl = a.doc_len[i], ql = a.qry_len[i];
-    g = {a.pre_start[lo], a.pre_len[lo], a.path_start[i], dl + ql, a.rows_mode == SP_ROWS_QUERY_ONLY ? dl : 0};
-    return dl >= 0 && ql >= 0 && (int64_t)dl + ql <= a.max_path_len && inside(g.own_lo, g.own_n) && inside(g.pre_lo, g.pre_n) &&
-           g.pre_n <= a.max_pre_len;
+    g.own_n = dl + ql;
+    g.first_row = a.rows_mode == SP_ROWS_QUERY_ONLY ? (seq < a.n_prompts ? ql : dl) : 0;
+    // all below 2^31 once none is negative: sums of two fit 32 bits
+    const uint32_t T = (uint32_t)a.total_tokens;
+    return (g.pre_lo | g.pre_n | g.own_lo | dl | ql) >= 0 && (uint32_t)dl + ql <= (uint32_t)most && (uint32_t)g.own_lo + g.own_n <= T &&
+           (uint32_t)g.pre_lo + g.pre_n <= T && g.pre_n <= a.max_pre_len;
 }
 
-// Row tile `tile` of sequence `seq` for the head of the block; the whole block takes part.
-template <int D> __device__ __forceinline__ void simt_tile(const PrefillSimtArgs &a, int seq, int tile)
+// The status word, written by one block that computes nothing; a function of its own, so that the other blocks, whose time goes
+// by the code they have to fetch, do not carry it.
+static __device__ __noinline__ void simt_report(const PrefillSimtArgs &a)
+{
+    bool bad = false;
+    for (int s = threadIdx.x; s < a.n_prompts + a.n_paths; s += kSimtThreads) { SimtSegment g; bad |= !simt_segment(a, s, g); }
+    bad = __syncthreads_or(bad);
+    if (threadIdx.x == 0) *a.status = bad ? STATUS_BAD_LAYOUT : STATUS_OK;
+}
+
+// grid: x = row tiles of the preambles, row tiles of the paths, and one block more that reports on the layout; y = head.
+// head_dim 64: registers for four blocks per SM, as shared memory would let five in (32 query-row tiles of 4 prompts: 44.2 us with
+// five, whose SMs then have unequal shares, 41.6 with four; head_dim 128 is 4 % slower with this bound).
+template <int D>
+__global__ void __launch_bounds__(kSimtThreads, D == 64 ? 4 : 5)
+prefill_simt_kernel(const __grid_constant__ PrefillSimtArgs a)
 {
     constexpr int BN = 4096 / D;             // keys per tile: 32 KB of K and V
     constexpr int KPT = BN / 16;             // keys per thread
@@ -63,16 +81,25 @@ template <int D> __device__ __forceinline__ void simt_tile(const PrefillSimtArgs
     constexpr int KS = D + 4;                // padded K row: 16 lanes reading 16 rows hit different banks
     __shared__ __align__(16) float sq[kSimtRows][D], sk[BN][KS], sv[BN][D], sp_[kSimtRows][BN];
     __shared__ float s_pos[BN];
+
+    pdl_wait();
+    pdl_trigger();
     const int h = blockIdx.y, hk = h / (a.n_heads / a.n_kv_heads);
+    const bool pre = (int)blockIdx.x < a.n_pre_blocks;
+    const int x = pre ? blockIdx.x : blockIdx.x - a.n_pre_blocks, n = pre ? a.n_prompts : a.n_paths;
+    if (blockIdx.x == gridDim.x - 1) {
+        if (h == 0) simt_report(a);
+        return;
+    }
+    const int tile = x / n, seq = x - tile * n + (pre ? 0 : a.n_prompts);
     SimtSegment g;
     if (!simt_segment(a, seq, g)) return;
     const int pre_lo = g.pre_lo, pre_n = g.pre_n, own_lo = g.own_lo, own_n = g.own_n, first_row = g.first_row;
-    const int r0 = first_row + tile * kSimtRows;    // first row of the tile, counted in the segment
+    const int r0 = first_row + (a.tile0 + tile) * kSimtRows;    // first row of the tile, counted in the segment
     const int n_rows = min(kSimtRows, own_n - r0);
     if (n_rows <= 0) return;
     const int n_keys = pre_n + r0 + n_rows;
 
-    __syncthreads();                                // the block's previous tile is done with the query rows
     for (int i = threadIdx.x; i < kSimtRows * (D / 4); i += kSimtThreads) {
         const int r = i / (D / 4), c = i % (D / 4);
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -152,9 +179,9 @@ template <int D> __device__ __forceinline__ void simt_tile(const PrefillSimtArgs
         __syncwarp();
         // V rows hidden from both rows of the pair are not touched, and the key that only the second row sees has no part in the
         // first: 0 x Inf or 0 x NaN would reach the rows in front of it
-        const int n = min(BN, n_keys - base), last = pre_n + r0 + row + 1 - base;
+        const int n_here = min(BN, n_keys - base), last = pre_n + r0 + row + 1 - base;
 #pragma unroll 4
-        for (int key = 0; key < min(n, last); ++key) {
+        for (int key = 0; key < min(n_here, last); ++key) {
             const float p0 = sp_[row][key], p1 = sp_[row + 1][key];
 #pragma unroll
             for (int c = 0; c < CPT; ++c) {
@@ -165,7 +192,7 @@ template <int D> __device__ __forceinline__ void simt_tile(const PrefillSimtArgs
                 o[1][c].z = fmaf(p1, vx.z, o[1][c].z); o[1][c].w = fmaf(p1, vx.w, o[1][c].w);
             }
         }
-        if (last >= 0 && last < n) {
+        if (last >= 0 && last < n_here) {
             const float p1 = sp_[row + 1][last];
 #pragma unroll
             for (int c = 0; c < CPT; ++c) {
@@ -190,28 +217,6 @@ template <int D> __device__ __forceinline__ void simt_tile(const PrefillSimtArgs
     }
 }
 
-// grid: x = blocks of the preambles, blocks of the paths, and one block more that reports on the layout; y = head.
-template <int D>
-__global__ void __launch_bounds__(kSimtThreads)
-prefill_simt_kernel(const __grid_constant__ PrefillSimtArgs a)
-{
-    pdl_wait();
-    pdl_trigger();
-    const int n_seq = a.n_prompts + a.n_paths;
-    if (blockIdx.x == gridDim.x - 1) {          // a block of its own: nobody waits for it, and the word has one writer
-        if (blockIdx.y) return;
-        bool bad = false;
-        for (int s = threadIdx.x; s < n_seq; s += kSimtThreads) { SimtSegment g; bad |= !simt_segment(a, s, g); }
-        bad = __syncthreads_or(bad);
-        if (threadIdx.x == 0) *a.status = bad ? STATUS_BAD_LAYOUT : STATUS_OK;
-        return;
-    }
-    const int x = blockIdx.x, n_pre = a.n_prompts * a.pre_z;
-    const bool pre = x < n_pre;
-    const int first = pre ? x / a.n_prompts : (x - n_pre) / a.n_paths, seq = pre ? x - first * a.n_prompts : a.n_prompts + (x - n_pre - first * a.n_paths);
-    for (int tile = first; tile < (pre ? a.pre_tiles : a.path_tiles); tile += pre ? a.pre_z : a.path_z) simt_tile<D>(a, seq, tile);
-}
-
 int launch_prefill_simt(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
                         const float *slopes, int n_heads, int n_kv_heads, int head_dim, float scale, int rows,
                         void *out, float *lse, void *ws, cudaStream_t st)
@@ -226,17 +231,19 @@ int launch_prefill_simt(const void *q, const void *k, const void *v, const sp_la
     a.rows_mode = rows; a.total_tokens = lay->total_tokens; a.scale_log2e = scale * kLog2eP;
     a.pos = pos; a.slopes = slopes;
     // No segment is longer than T, however loose the bounds; preambles and paths have a range of their own (one prefix of 1 000
-    // rows beside hundreds of short paths: 63 tiles for every path otherwise).  Beyond 2^16 blocks a sequence's tiles share some.
-    const auto tiles = [&](int64_t n) { return (int)((std::min<int64_t>(n, lay->total_tokens) + kSimtRows - 1) / kSimtRows); };
-    const auto share = [](int n_tiles, int n) { return std::min(n_tiles, std::max(1, (1 << 16) / std::max(n, 1))); };
-    a.pre_tiles = rows == SP_ROWS_ALL ? tiles(lay->max_pre_len) : 0;
-    a.path_tiles = tiles(lay->max_path_len);
-    a.pre_z = share(a.pre_tiles, lay->n_prompts); a.path_z = share(a.path_tiles, lay->n_paths);
-    const int64_t blocks = (int64_t)lay->n_prompts * a.pre_z + (int64_t)lay->n_paths * a.path_z + 1;
-    SP_REQUIRE(blocks < (int64_t)INT32_MAX, SP_ERR_UNSUPPORTED, "sp_superpose_prefill: %d prompts and %d paths", lay->n_prompts, lay->n_paths);
-    const dim3 grid((unsigned)blocks, n_heads);
-    return head_dim == 64 ? launch(prefill_simt_kernel<64>, grid, kSimtThreads, 0, st, 1, a)
-                          : launch(prefill_simt_kernel<128>, grid, kSimtThreads, 0, st, 1, a);
+    // rows beside hundreds of short paths: 63 tiles for every path otherwise).  What is too much for one grid takes several.
+    const auto tiles = [&](int64_t n) { return (std::min<int64_t>(n, lay->total_tokens) + kSimtRows - 1) / kSimtRows; };
+    const int64_t pre_tiles = rows == SP_ROWS_ALL ? tiles(lay->max_pre_len) : 0, path_tiles = tiles(lay->max_path_len);
+    const int64_t step = std::max<int64_t>(1, kSimtMaxBlocks / ((int64_t)lay->n_prompts + lay->n_paths));
+    for (int64_t t = 0; t == 0 || t < std::max(pre_tiles, path_tiles); t += step) {
+        const int64_t n_pre = lay->n_prompts * std::clamp<int64_t>(pre_tiles - t, 0, step), n_path = lay->n_paths * std::clamp<int64_t>(path_tiles - t, 0, step);
+        a.tile0 = (int)t; a.n_pre_blocks = (int)n_pre;
+        const dim3 grid((unsigned)(n_pre + n_path + 1), n_heads);
+        const int rc = head_dim == 64 ? launch(prefill_simt_kernel<64>, grid, kSimtThreads, 0, st, 1, a)
+                                      : launch(prefill_simt_kernel<128>, grid, kSimtThreads, 0, st, 1, a);
+        if (rc) return rc;
+    }
+    return SP_OK;
 }
 
 }  // namespace sp

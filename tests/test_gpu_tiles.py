@@ -127,7 +127,7 @@ def test_prefill_f32_tiles(D, alibi):
 @pytest.mark.parametrize("H,more", [(4, 0), (1, 600000)])
 def test_prefill_f32_loose_bounds(mirror, H, more):
     """max_pre_len / max_path_len are upper bounds: however large, every row is computed and no launch grows with them (with 600 000
-    more rows in the tensors the blocks of a path walk its row tiles: four paths share 2^16 blocks)."""
+    more rows in the tensors the tiles of six segments take two launches of up to 2^17 blocks)."""
     lay = build_layout([40, 3], [[1, 70, 15], [33]], [[4, 1, 2], [9]])
     lay.total_tokens += more
     T, D = lay.total_tokens, 64
