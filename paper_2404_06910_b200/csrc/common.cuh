@@ -117,6 +117,15 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     return *reinterpret_cast<uint32_t *>(&t);
 }
 
+// Two probabilities as sums of two bf16 numbers each: hi is p cut off behind 8 bits, lo the rest (16 bits in all).  lo is never
+// negative, and the 2^-23 p in it, less than p's own rounding, keeps it above zero where p is: the products with an Inf in V
+// are then infinities of one sign, as that of p would be, and not NaN.
+__device__ __forceinline__ void split_bf16(float p0, float p1, uint32_t &hi, uint32_t &lo) {
+    const uint32_t a = __float_as_uint(p0) & 0xffff0000u, b = __float_as_uint(p1) & 0xffff0000u;
+    hi = __byte_perm(a, b, 0x7632);
+    lo = pack_bf16x2(fmaf(p0, 1.f + 0x1p-23f, -__uint_as_float(a)), fmaf(p1, 1.f + 0x1p-23f, -__uint_as_float(b)));
+}
+
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));

@@ -58,11 +58,11 @@ enum { WARP_EPI = 8, WARP_K = 12, WARP_V, WARP_Q, WARP_POS, WARP_MMA, WARP_PASS 
 
 // SPLIT_P: P is carried as the sum of two bf16 numbers (16 bits of mantissa) and the second product runs twice.  Set for
 // head_dim 64, which is then as precise as fp32 arithmetic, and for query rows only: relative to the maximum over a first
-// key tile, P in one bf16 number was less exact there (2.27e-3 of the norm from 64-bit results, 8 prompts x 100 documents)
+// key tile, P in one bf16 number is less exact there (2.27e-3 of the norm from 64-bit results, 8 prompts x 100 documents)
 // than relative to the running maximum of prefill_qonly.cu (2.13e-3); as two it is 1.66e-3, the rounding of the output.  Cost
-// there: 514 -> 584 us.
+// there: 8 prompts x 100 documents, two heads to a KV head, 326 -> 341 us; four, 197 -> 217.
 template <int D, bool ALIBI, bool SPLIT> struct TcConfig {
-    static constexpr bool SPLIT_P = SPLIT;
+    static constexpr bool SPLIT_P = SPLIT, EXACT = D == 64;
     static constexpr int HALVES = D / 64;                       // 64-column halves of a row (one 128-byte swizzle atom each)
     static constexpr int Q_BYTES = kBM * D * 2, KV_BYTES = kBN * D * 2;
     static constexpr int NQ = D == 64 ? 4 : 3;                  // query slots
@@ -139,7 +139,8 @@ struct TcParams {
     uint32_t *status;
     __nv_bfloat16 *out;
     float *lse;
-    int n_heads;
+    const __nv_bfloat16 *q, *k, *v;
+    int n_heads, n_kv_heads;
     int log_rows, n_units, units_per_kv;   // rows of a head in a tile (log2); units of G heads in all and per KV head
     int64_t total_tokens;
     float scale_log2e;
@@ -209,6 +210,70 @@ template <int N> struct Ring {        // stage and parity of a ring of N barrier
     }
     __device__ __forceinline__ void next() { skip(1); }
 };
+
+// One row (key number `last`, 64 columns; o: bf16 pairs) in fp32 arithmetic over exactly the keys it sees: its values that are not
+// finite are replaced.
+template <bool ALIBI>
+__device__ __forceinline__ void exact_row64(const TcParams &p, const TcPair &t, int head, int kv_head, int last, uint32_t (&o)[32])
+{
+    const int64_t own = t.own_base + last;
+    const uint4 *q = reinterpret_cast<const uint4 *>(p.q + (own * p.n_heads + head) * 64);
+    const float pq = ALIBI ? p.pos[own] : 0.f, slope = ALIBI ? p.slopes[head] * kLog2eT : 0.f;
+    auto packed_row = [&](int u) { return (int64_t)u + (u < t.pre_len ? t.pre_row : t.own_base); };
+    auto score = [&](int64_t row) {
+        const uint4 *k = reinterpret_cast<const uint4 *>(p.k + (row * p.n_kv_heads + kv_head) * 64);
+        float s = 0.f;
+#pragma unroll 1
+        for (int c = 0; c < 8; ++c) {
+            const uint4 x = q[c], y = k[c];
+            s = fmaf(bf16_lo(x.x), bf16_lo(y.x), s); s = fmaf(bf16_hi(x.x), bf16_hi(y.x), s);
+            s = fmaf(bf16_lo(x.y), bf16_lo(y.y), s); s = fmaf(bf16_hi(x.y), bf16_hi(y.y), s);
+            s = fmaf(bf16_lo(x.z), bf16_lo(y.z), s); s = fmaf(bf16_hi(x.z), bf16_hi(y.z), s);
+            s = fmaf(bf16_lo(x.w), bf16_lo(y.w), s); s = fmaf(bf16_hi(x.w), bf16_hi(y.w), s);
+        }
+        s *= p.scale_log2e;
+        return ALIBI ? s - slope * fabsf(pq - p.pos[row]) : s;
+    };
+    float m = -INFINITY, l = 0.f;
+#pragma unroll 1
+    for (int u = 0; u <= last; ++u) {
+        if (u >= t.pre_len && u < t.p16) continue;
+        const float s = score(packed_row(u));
+        if (s > m) { l *= ex2(m - s); m = s; }
+        l += ex2(s - m);
+    }
+    const float inv = 1.f / l;
+#pragma unroll
+    for (int part = 0; part < 4; ++part) {               // 16 columns at a time
+        float acc[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) acc[i] = 0.f;
+#pragma unroll 1
+        for (int u = 0; u <= last; ++u) {
+            if (u >= t.pre_len && u < t.p16) continue;
+            const int64_t row = packed_row(u);
+            const float w = ex2(score(row) - m);
+            const uint4 *v = reinterpret_cast<const uint4 *>(p.v + (row * p.n_kv_heads + kv_head) * 64) + 2 * part;
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const uint4 y = v[c];
+                const uint32_t wd[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    acc[8 * c + 2 * e] = fmaf(w, bf16_lo(wd[e]), acc[8 * c + 2 * e]);
+                    acc[8 * c + 2 * e + 1] = fmaf(w, bf16_hi(wd[e]), acc[8 * c + 2 * e + 1]);
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {                    // the finite ones are right as they are
+            const uint32_t x = pack_bf16x2(acc[2 * i] * inv, acc[2 * i + 1] * inv);
+            uint32_t &y = o[8 * part + i];
+            if ((y & 0x7f80u) == 0x7f80u) y = (y & 0xffff0000u) | (x & 0xffffu);
+            if ((y & 0x7f800000u) == 0x7f800000u) y = (y & 0xffffu) | (x & 0xffff0000u);
+        }
+    }
+}
 
 template <int N> __device__ __forceinline__ void reg_alloc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
 template <int N> __device__ __forceinline__ void reg_dealloc() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
@@ -576,8 +641,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                                 unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[c][i]), __uint_as_float(r[c][i + 1])), sc2, nm2), x0, x1);
                                 const float p0 = ex2(x0), p1 = ex2(x1);
                                 sum[(i >> 1) & 3] = add_f32x2(sum[(i >> 1) & 3], pack_f32x2(p0, p1));
-                                hi[i >> 1] = pack_bf16x2(p0, p1);
-                                if (C::SPLIT_P) lo[C::SPLIT_P ? i >> 1 : 0] = pack_bf16x2(p0 - bf16_lo(hi[i >> 1]), p1 - bf16_hi(hi[i >> 1]));
+                                if (C::SPLIT_P) split_bf16(p0, p1, hi[i >> 1], lo[C::SPLIT_P ? i >> 1 : 0]);
+                                else hi[i >> 1] = pack_bf16x2(p0, p1);
                             }
                         } else {                                     // no row of this warp sees these keys
 #pragma unroll
@@ -658,6 +723,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&bars[C::BAR_O_FREE + ln]);
+                    }
+                    if (C::EXACT && hr < t.rows) {
+                        // Hidden keys have a P of exactly zero, but 0 x Inf and 0 x NaN reach O: a row with a value that is not
+                        // finite is computed again over its own keys, as the fp32 kernel that served head_dim 64 before would
+                        // have.  The look at the row costs nothing that shows; looking through the V tiles instead cost the
+                        // ALiBi variant 14 % (one more warp on the SM partition of two softmax warps).
+                        uint32_t nan = 0u;
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) asm("fma.rn.bf16x2 %0, %1, %2, %0;" : "+r"(nan) : "r"(o[i]), "r"(0u));
+                        if (nan & 0x7fff7fffu)
+                            exact_row64<ALIBI>(p, w.t, (w.h << (7 - log_rows)) + (row >> log_rows), w.h / p.units_per_kv, t.q_u + hr, o);
                     }
                     if (hr < t.rows) {
                         if (p.wide_stores) {
@@ -830,6 +906,8 @@ static int launch_tc(const void *q, const void *k, const void *v, const sp_layou
 
     p.hdr = hdr; p.pairs = pairs; p.status = &hdr->status;
     p.out = static_cast<__nv_bfloat16 *>(out); p.lse = lse;
+    p.q = static_cast<const __nv_bfloat16 *>(q); p.k = static_cast<const __nv_bfloat16 *>(k); p.v = static_cast<const __nv_bfloat16 *>(v);
+    p.n_kv_heads = n_kv_heads;
     p.n_heads = n_heads; p.log_rows = 7 - log_g; p.n_units = n_heads >> log_g; p.units_per_kv = group >> log_g;
     p.total_tokens = lay->total_tokens; p.scale_log2e = scale * kLog2eT;
     p.wide_stores = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;

@@ -93,12 +93,14 @@ def test_prefill_ignores_rows_outside_every_segment():
     assert torch.equal(out0[used], out1[used]) and torch.equal(lse0[:, used], lse1[:, used])
 
 
-@pytest.mark.parametrize("dtype,D", [("f32", 64), ("f32", 128)])
-@pytest.mark.parametrize("rows", [sp.SP_ROWS_ALL, sp.SP_ROWS_QUERY_ONLY])
-@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("dtype,D,rows", [("f32", 64, sp.SP_ROWS_ALL), ("f32", 64, sp.SP_ROWS_QUERY_ONLY), ("f32", 128, sp.SP_ROWS_ALL),
+                                          ("f32", 128, sp.SP_ROWS_QUERY_ONLY), ("bf16", 64, sp.SP_ROWS_ALL),
+                                          ("bf16", 64, sp.SP_ROWS_QUERY_ONLY)])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), float("-inf")])
 def test_prefill_rows_in_front_of_a_key_do_not_see_it(dtype, D, rows, bad):
-    """Causality with a value that is not finite: the rows in front of it keep their bits, the rows behind it have it in its
-    column and keep the others (probabilities of a few hundred keys do not underflow)."""
+    """Causality with a value that is not finite: the rows in front of it keep theirs, the rows behind it have it in its column
+    and keep the other columns (probabilities of a few hundred keys do not underflow).  Bit for bit, except that bf16 may have
+    computed the column of the rows in front another way: one rounding of the output."""
     lay = _layout()
     T, H, Hkv = lay.total_tokens, 4, 2
     q, k, v = _randn((T, H, D), dtype, 930), _randn((T, Hkv, D), dtype, 931), _randn((T, Hkv, D), dtype, 932)
@@ -112,7 +114,10 @@ def test_prefill_rows_in_front_of_a_key_do_not_see_it(dtype, D, rows, bad):
         keep = torch.ones(T, dtype=torch.bool)
         keep[torch.from_numpy(behind)] = False
         cols = torch.arange(D) != 5
-        assert torch.equal(out0[keep], out1[keep]) and torch.equal(lse0, lse1), at
+        front0, front1 = out0[keep].float(), out1[keep].float()
+        assert torch.equal(front0[..., cols], front1[..., cols]) and torch.equal(lse0, lse1), at
+        off = (front0[..., 5] - front1[..., 5]).abs()
+        assert bool((off <= (0.0 if dtype == "f32" else 2.0 ** -7 * front0[..., 5].abs() + 1e-6)).all()), at
         assert torch.equal(out0[behind][..., cols], out1[behind][..., cols]), at
         got = out1[behind][..., 5]
         assert bool(torch.isnan(got).all() if bad != bad else (got == bad).all()), at
