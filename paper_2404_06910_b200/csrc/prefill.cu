@@ -31,6 +31,29 @@ extern "C" size_t sp_prefill_workspace_bytes(int n_prompts, int n_paths, int max
 }
 
 namespace sp {
+// Query rows only, head_dim 128: which of two kernels.  The tcgen05 kernel has a quarter of its tile's rows at work (32 of 128) and
+// carries P as two bf16 numbers; the warp-level kernel (prefill_qonly.cu) works on 32 rows at a time.
+//  - An even number of query heads to a KV head: tcgen05, whose tiles then hold the rows of several heads.  us, tcgen05 /
+//    warp-level, 4 x 20 documents behind 1 200 rows: 193 / 302 (two heads), 114 / 303 (four); ALiBi 257 / 347, 155 / 343.
+//  - Few items (a path's query rows and a head each): tcgen05; the warp-level kernel has too few warps to hide its latency.  1
+//    prompt x 20 documents of 64-256 rows, 32 heads: 23.3 / 24.1 behind 32 rows, 43.4 / 52.6 behind 384; 2 prompts: 47 / 54
+//    behind 128, 175 / 181 behind 1 200; ALiBi 61 / 66 behind 128, 83 / 83 behind 256, 110 / 105 behind 400.
+//  - More than 32 query rows in a path: tcgen05; the warp-level kernel reads every key again for each 32 rows.  48 rows, 8 x 100
+//    documents: 666 / 1216 behind 48 rows, 1825 / 3114 behind 600.
+//  - Otherwise warp-level: 8 x 100 documents, back to back: 622 / 600 behind 16 rows, 689 / 655 behind 48, 839 / 769 behind 128,
+//    1430 / 1202 behind 384; ALiBi 722 / 696 behind 16, 841 / 758 behind 64.
+// The number of query rows is known from the host mirror only; without one tcgen05 up to the preamble behind which it loses
+// less than the warp-level kernel does with 33 rows and more.
+static bool query_rows_warp_level(const sp_layout *lay, bool alibi, int n_heads, int n_kv_heads)
+{
+    if (n_heads / n_kv_heads % 2 == 0) return false;
+    if ((int64_t)lay->n_paths * n_heads <= 9 * (int64_t)num_sms() && (!alibi || lay->max_pre_len <= 256)) return false;
+    if (!lay->host_mirror) return lay->max_pre_len > (alibi ? 64 : 384);
+    int longest = 0;
+    for (int i = 0; i < lay->n_paths; ++i) longest = std::max(longest, lay->host_mirror->qry_len[i]);
+    return longest <= 32;
+}
+
 static int prefill_entry(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
                          const float *slopes, int n_heads, int n_kv_heads, int head_dim, float scale, int rows,
                          void *out, float *lse, void *ws, size_t ws_bytes, int dtype, void *stream)
@@ -54,17 +77,7 @@ static int prefill_entry(const void *q, const void *k, const void *v, const sp_l
                "sp_superpose_prefill: workspace of %zu bytes (256-byte aligned) required", need);
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // Query rows only: the tcgen05 kernel has a quarter of its tile's rows at work but loads keys with TMA and is the faster one
-    // while a path's keys are mostly its own; behind a long preamble the smaller tiles of the warp-level kernel win.  us at 8
-    // prompts x 100 documents of 64-256 rows, 32 query rows, tcgen05 / warp-level: preamble 16: 530 / 552, 64: 600 / 605, 128:
-    // 701 / 715, 256: 959 / 936, 400: 1295 / 1214, 600: 1752 / 1553, 1 200: 3112 / 2607; 2 x 40 documents: 128: 82 / 88, 400: 143 /
-    // 145, 1 200: 333 / 302; ALiBi, whose bias a lone softmax warp feels more: 16: 630 / 694, 64: 755 / 748, 96: 890 / 805, 256:
-    // 1343 / 1110.  The line lies above the crossing (about 200 rows, ALiBi 64) because the number of query rows is not known
-    // here: from 33 rows per path the warp-level kernel reads every key twice (48 rows behind 48 rows: 666 / 1216, behind 600:
-    // 1825 / 3114).  With an even number of query heads to a KV head the tcgen05 tiles hold the rows of several heads and win
-    // everywhere: behind 1 200 rows, 4 x 20 documents: 193 / 302 (two heads), 114 / 303 (four); ALiBi 257 / 347, 155 / 343.
-    if (dtype == SP_BF16 && head_dim == 128 && rows == SP_ROWS_QUERY_ONLY && lay->max_pre_len > (pos ? 64 : 384) &&
-        n_heads / n_kv_heads % 2)
+    if (dtype == SP_BF16 && head_dim == 128 && rows == SP_ROWS_QUERY_ONLY && query_rows_warp_level(lay, pos != nullptr, n_heads, n_kv_heads))
         return launch_prefill_qonly(q, k, v, lay, pos, slopes, n_heads, n_kv_heads, scale, out, lse, ws, st);
     // bf16 goes to the tensor cores for both head sizes (head_dim 64, 8 prompts x 20 documents, 32 heads: 0.17 ms; the fp32
     // SIMT kernel, which served it before, took 9.4 ms)

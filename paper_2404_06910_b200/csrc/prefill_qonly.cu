@@ -11,8 +11,8 @@
 // tcgen05 tile, 32 rows fill a quarter of one, and the tensor pipe is idle either way at this
 // intensity; small warp-level tiles keep many independent items in flight per SM instead.
 // The grid is persistent with the head as the fastest index, like the full prefill.
-// It serves long preambles with an odd number of query heads to a KV head; elsewhere the tcgen05 kernel is the faster one (the
-// rule and both sides' times: prefill.cu).
+// It serves up to 32 query rows per path with an odd number of query heads to a KV head, but for small launches; elsewhere the
+// tcgen05 kernel is the faster one (the rule and both sides' times: prefill.cu).
 #include "common.cuh"
 #include "prefill_plan.cuh"
 

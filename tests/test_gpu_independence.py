@@ -46,7 +46,7 @@ def _run_prefill(q, k, v, lay, rows):
     return out.cpu(), lse.cpu()
 
 
-# tensor-core kernel (bf16, 128), query-only kernel (bf16, 128, query rows), SIMT kernel (the rest)
+# tcgen05 kernel (bf16), SIMT kernel (fp32); the warp-level kernel for query rows has a test of its own below
 @pytest.mark.parametrize("dtype,D,rows", [("bf16", 128, sp.SP_ROWS_ALL), ("bf16", 128, sp.SP_ROWS_QUERY_ONLY),
                                           ("f32", 64, sp.SP_ROWS_ALL), ("bf16", 64, sp.SP_ROWS_ALL)])
 @pytest.mark.parametrize("kind", ["finite", "non_finite"])
@@ -69,6 +69,27 @@ def test_prefill_paths_do_not_see_each_other(dtype, D, rows, kind):
         keep[r.numpy()] = False
         assert torch.equal(out0[keep], out1[keep]), f"path {j} ({kind}) leaked into another path's output"
         assert torch.equal(lse0[:, keep], lse1[:, keep])
+
+
+@pytest.mark.parametrize("kind", ["finite", "non_finite"])
+def test_query_rows_on_the_warp_level_kernel_do_not_see_other_paths(kind):
+    """Query rows, an odd number of heads and more than 9 items per SM: the warp-level kernel."""
+    rng = np.random.default_rng(7)
+    lay = build_layout([21, 400], [[int(x) for x in rng.integers(0, 60, n)] for n in (50, 45)],
+                       [[int(x) for x in rng.integers(1, 33, n)] for n in (50, 45)])
+    T, H, D = lay.total_tokens, 15, 128
+    q, k, v = _randn((T, H, D), "bf16", 940), _randn((T, H, D), "bf16", 941), _randn((T, H, D), "bf16", 942)
+    out0, lse0 = _run_prefill(q, k, v, lay, sp.SP_ROWS_QUERY_ONLY)
+    rows = np.concatenate([_path_rows(lay, j) for j in range(0, lay.n_paths, 3)])
+    r = torch.from_numpy(rows)
+    if kind == "finite":
+        q[r], k[r], v[r] = q[r] * -1.5 + 0.25, k[r] * 2.0 - 0.5, v[r] * -3.0 + 1.0
+    else:
+        q[r], k[r], v[r] = float("nan"), float("inf"), float("nan")
+    out1, lse1 = _run_prefill(q, k, v, lay, sp.SP_ROWS_QUERY_ONLY)
+    keep = np.ones(T, dtype=bool)
+    keep[rows] = False
+    assert torch.equal(out0[keep], out1[keep]) and torch.equal(lse0[:, keep], lse1[:, keep])
 
 
 def test_prefill_ignores_rows_outside_every_segment():

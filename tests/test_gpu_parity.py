@@ -209,9 +209,9 @@ def _query_row_mask(lay):
 
 @pytest.mark.parametrize("case", ["ragged", "long_queries", "no_preamble_short", "many_paths"])
 def test_prefill_query_only_ragged(case):
-    """Query rows only (bf16, head_dim 128): query lengths around and beyond the 32-row item,
-    empty documents and preambles, items of one or two key tiles behind longer ones, grouped
-    heads; per-row check, untouched non-query rows, and bit-identical repeats."""
+    """Query rows only (bf16, head_dim 128; all of these run on the tcgen05 kernel): query lengths
+    around and beyond 32 rows, empty documents and preambles, items of one or two key tiles behind
+    longer ones, grouped heads; per-row check, untouched non-query rows, and bit-identical repeats."""
     rng = np.random.default_rng(11)
     if case == "ragged":
         lay = build_layout([0, 5, 40, 130], [[1, 15, 16, 31], [17, 127, 0], [128, 129], [300, 2, 64]],
