@@ -120,24 +120,18 @@ row_logp_kernel(const T *__restrict__ logits, int64_t ld, const int32_t *__restr
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (lane == 0) { sm[warp] = m; ss[warp] = s; }
     __syncthreads();
-    float top = sm[0];
-    for (int w = 1; w < kScoreThreads / 32; ++w) top = fmaxf(top, sm[w]);
-    if (fabsf(top) > 1e38f && top > -INFINITY) {          // block-uniform
+    if (warp > 0) return;
+    m = sm[0]; s = ss[0];
+    for (int w = 1; w < kScoreThreads / 32; ++w) merge_ms(m, s, sm[w], ss[w]);
+    if (fabsf(m) > 1e38f && m > -INFINITY) {              // the same in all lanes
         s = 0.f;
-        for (int c = threadIdx.x; c < vocab; c += kScoreThreads) {
+        for (int c = lane; c < vocab; c += 32) {
             const float xv = to_float(row[c]);
-            if (xv != -INFINITY) s += fast_exp2((xv - top) * kLog2e);
+            if (xv != -INFINITY) s += fast_exp2((xv - m) * kLog2e);
         }
         s = warp_sum(s);
-        __syncthreads();
-        if (lane == 0) { sm[warp] = top; ss[warp] = s; }
-        __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        m = sm[0]; s = ss[0];
-        for (int w = 1; w < kScoreThreads / 32; ++w) merge_ms(m, s, sm[w], ss[w]);
-        row_logp[t] = picked - (m + logf(s));
-    }
+    if (lane == 0) row_logp[t] = picked - (m + logf(s));
 }
 
 // scores[i] = weight[i] * sum_t row_logp[t] + prior[i]; one warp per path, fixed order.
