@@ -63,7 +63,7 @@ static int decode_split_cap(int n_prompts, int n_heads)
 __device__ __forceinline__ uint4 ld_stream16(const void *p)
 {
     uint4 w;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w) : "l"(p));
     return w;
 }

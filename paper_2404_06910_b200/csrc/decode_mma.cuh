@@ -56,7 +56,7 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
     if (gid < nh) {
         const uint4 *src = reinterpret_cast<const uint4 *>(static_cast<const T *>(a.q) + ((int64_t)b * a.n_heads + h0 + gid) * D);
 #pragma unroll
-        for (int c = 0; c < NC; ++c) qf[c] = __ldg(src + tig + 4 * c);
+        for (int c = 0; c < NC; ++c) qf[c] = src[tig + 4 * c];
     }
     decode_segments<T, ALIBI>(a, sm, n_seg, b, hk, D, row_elems);
     if (ROPE) decode_angles<D>(a, rope, b, cs);

@@ -33,17 +33,23 @@ __device__ __forceinline__ void merge_ms(float &m, float &s, float m2, float s2)
     m = mn;
 }
 
+__device__ __forceinline__ uint4 ld_evict_first(const void *p)
+{
+    uint4 w;
+    asm volatile("ld.global.cs.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w) : "l"(p));
+    return w;
+}
 template <typename T> __device__ __forceinline__ void load_stream(const T *p, float (&f)[Vec<T>::N]);
 template <> __device__ __forceinline__ void load_stream<__nv_bfloat16>(const __nv_bfloat16 *p, float (&f)[8])
 {
-    const uint4 w = __ldcs(reinterpret_cast<const uint4 *>(p));
+    const uint4 w = ld_evict_first(p);
     f[0] = bf16_lo(w.x); f[1] = bf16_hi(w.x); f[2] = bf16_lo(w.y); f[3] = bf16_hi(w.y);
     f[4] = bf16_lo(w.z); f[5] = bf16_hi(w.z); f[6] = bf16_lo(w.w); f[7] = bf16_hi(w.w);
 }
 template <> __device__ __forceinline__ void load_stream<float>(const float *p, float (&f)[4])
 {
-    const float4 w = __ldcs(reinterpret_cast<const float4 *>(p));
-    f[0] = w.x; f[1] = w.y; f[2] = w.z; f[3] = w.w;
+    const uint4 w = ld_evict_first(p);
+    f[0] = __uint_as_float(w.x); f[1] = __uint_as_float(w.y); f[2] = __uint_as_float(w.z); f[3] = __uint_as_float(w.w);
 }
 
 // Rows start at any element (ld is the vocabulary size, which is rarely a multiple of 8): up to one vector's worth of elements
@@ -54,8 +60,7 @@ template <> __device__ __forceinline__ void load_stream<float>(const float *p, f
 // whose maximum itself is that large is summed again (a test of the maximum inside the loop: 508 us where this takes 500).
 template <typename T, int kScoreThreads>
 __global__ void __launch_bounds__(kScoreThreads)
-row_logp_kernel(const T *__restrict__ logits, int64_t ld, const int32_t *__restrict__ targets,
-                int vocab, float *__restrict__ row_logp)
+row_logp_kernel(const T *logits, int64_t ld, const int32_t *targets, int vocab, float *row_logp)
 {
     pdl_wait();
     pdl_trigger();
@@ -136,9 +141,7 @@ row_logp_kernel(const T *__restrict__ logits, int64_t ld, const int32_t *__restr
 
 // scores[i] = weight[i] * sum_t row_logp[t] + prior[i]; one warp per path, fixed order.
 __global__ void __launch_bounds__(256)
-path_sum_kernel(const float *__restrict__ row_logp, const int32_t *__restrict__ row_off, int n_paths,
-                const float *__restrict__ prior, const float *__restrict__ weight,
-                float *__restrict__ scores)
+path_sum_kernel(const float *row_logp, const int32_t *row_off, int n_paths, const float *prior, const float *weight, float *scores)
 {
     pdl_wait();
     pdl_trigger();

@@ -172,7 +172,7 @@ struct Walk {
         if (h >= n_units) { h -= n_units; ++pair; }
         if (pair >= n_pairs) return false;
         const int4 *src = reinterpret_cast<const int4 *>(pairs + pair);
-        const int4 a = __ldg(src), b = __ldg(src + 1);
+        const int4 a = src[0], b = src[1];
         t.own_base = a.x; t.q_u = a.y; t.pre_row = a.z; t.pre_len = a.w;
         t.p16 = b.x; t.rows_ab = b.y; t.steps_a = b.z; t.steps = b.w;
         return true;
@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
 #pragma unroll
                     for (int i = 0; i < kBN / 32; ++i) {
                         const int u = j * kBN + i * 32 + lane;
-                        x[i] = u < w.t.pre_len || (u >= w.t.p16 && u < end) ? __ldg(p.pos + u + (u < w.t.pre_len ? w.t.pre_row : w.t.own_base)) : 0.f;
+                        x[i] = u < w.t.pre_len || (u >= w.t.p16 && u < end) ? p.pos[u + (u < w.t.pre_len ? w.t.pre_row : w.t.own_base)] : 0.f;
                     }
                     if (!(ok = mbar_wait_warp(&bars[C::BAR_V_EMPTY + v.i], v.ph ^ 1))) break;
 #pragma unroll
@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
             float m_ref = -INFINITY, l = 0.f;            // reference maximum (log2 units) and row sum
             float pq = 0.f, neg_slope = 0.f;
             if (ALIBI && t.steps) {
-                pq = hr < t.rows ? __ldg(p.pos + w.t.own_base + t.q_u + hr) : 0.f;
+                pq = hr < t.rows ? p.pos[w.t.own_base + t.q_u + hr] : 0.f;
                 neg_slope = -p.slopes[head] * (kLog2eT / sc);     // in units of the unscaled score: one scaling serves both
             }
             // counted from the key tile's first key: the first one this row may not see, the padding behind the preamble

@@ -36,7 +36,7 @@ template <> struct Pack<float> {
 // Rotates nt tokens (starting at t0) of one tensor with the (cos, sin) table of the group.
 // VEC: 16-byte accesses (requires alignment and divisibility, checked by the host).
 template <typename T, bool VEC>
-__device__ __forceinline__ void rotate_tokens(T *__restrict__ x, const float2 (*cs)[128], int64_t t0, int nt,
+__device__ __forceinline__ void rotate_tokens(T *x, const float2 (*cs)[128], int64_t t0, int nt,
                                               int64_t ld_token, int n_heads, int head_dim, int rot_dim, int pairing)
 {
     const int half = rot_dim >> 1;
@@ -104,7 +104,7 @@ __device__ __forceinline__ void rotate_tokens(T *__restrict__ x, const float2 (*
 // GROUP: tokens per block iteration.
 template <typename T, bool VEC, bool VEC1, int GROUP>
 __global__ void __launch_bounds__(kRopeThreads, 8)   // 32 registers: full occupancy for the streaming pass
-rope_kernel(T *__restrict__ x, T *__restrict__ x1, const float *__restrict__ pos, int64_t n_tokens, int64_t ld_token,
+rope_kernel(T *x, T *x1, const float *pos, int64_t n_tokens, int64_t ld_token,
             int64_t ld_token1, int n_heads, int n_heads1, int head_dim, int rot_dim, int pairing,
             const __grid_constant__ RopeFreq fr)
 {

@@ -30,8 +30,7 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
 }
 
 __global__ void __launch_bounds__(128)
-prune_topk_kernel(const float *__restrict__ scores, const int32_t *__restrict__ ppo, int n_prompts,
-                  int k, int32_t *__restrict__ kept_idx, float *__restrict__ kept_post)
+prune_topk_kernel(const float *scores, const int32_t *ppo, int n_prompts, int k, int32_t *kept_idx, float *kept_post)
 {
     pdl_wait();
     pdl_trigger();

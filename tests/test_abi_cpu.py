@@ -120,3 +120,13 @@ def test_next_round_layout_moves_kept_documents_into_the_prefix():
     assert list(nxt.doc_len) == [20, 5] and list(nxt.qry_len) == [4, 2]
     assert list(nxt.prompt_path_off) == [0, 1, 2]
     assert nxt.total_tokens == 43 + 24 + 6 + 7
+
+
+def test_kernels_read_coherently():
+    """Every kernel may start while the one before it still writes (programmatic dependent launch), so none may read through the
+    non-coherent path or promise the compiler that its pointers do not alias: such loads are not ordered by the wait."""
+    src = os.path.join(os.path.dirname(sp.LIB_PATH), "csrc")
+    for name in sorted(os.listdir(src)):
+        text = re.sub(r"//[^\n]*|/\*.*?\*/", "", open(os.path.join(src, name)).read(), flags=re.S)
+        found = re.findall(r"__ldg|__restrict__|ld\.global\.nc|__ldcs", text)
+        assert not found, (name, found)

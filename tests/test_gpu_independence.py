@@ -177,3 +177,75 @@ def test_decode_sees_only_kept_paths(dtype, D, kind):
             k2[r], v2[r] = float("inf"), float("nan")
         out1, lse1 = run(k2, v2)
         assert torch.equal(out0, out1) and torch.equal(lse0, lse1), f"pruned path {j} ({kind}) reached the decode output"
+
+
+@pytest.mark.parametrize("D,Hkv", [(128, 4), (128, 2), (64, 4)])
+def test_prefills_in_a_row_through_one_workspace(D, Hkv):
+    """Launches may start before the one in front of them has finished: each reads the work list of its own layout.  Layouts of
+    different lengths through one workspace, nothing waited for in between, against runs on their own."""
+    lays = [build_layout([21, 40], [[37, 130, 9, 77], [150, 3, 61]], [[5, 7, 3, 11], [9, 2, 6]]),
+            build_layout([300], [[400, 20]], [[30, 1]]),
+            build_layout([0, 5, 16] * 8, [[60, 1], [200, 31, 8], [90]] * 8, [[8, 2], [32, 1, 9], [40]] * 8)]
+    H, runs = 4, []
+    for n, lay in enumerate(lays):
+        q, k, v = (dev(_randn((lay.total_tokens, h, D), "bf16", 950 + 3 * n + i)) for i, h in enumerate((H, Hkv, Hkv)))
+        runs.append((sp.DeviceLayout.from_host(lay), q, k, v, torch.arange(lay.total_tokens, device="cuda", dtype=torch.float32)))
+    size = sp.sp_prefill_rope_workspace_bytes if D == 128 else sp.sp_prefill_workspace_bytes
+    ws = workspace(max(size(r[0], H, D, sp.SP_BF16) for r in runs))
+
+    def call(r, form):
+        dl, q, k, v, pos = r
+        out = torch.zeros_like(q)
+        if form == 2 and D == 128:
+            sp.sp_superpose_prefill_rope(q, k, v, dl, pos, 10000.0, sp.SP_ROPE_HALF_SPLIT, D ** -0.5, out, None, ws)
+        else:
+            sp.sp_superpose_prefill(q, k, v, dl, D ** -0.5, out, None, ws, rows=sp.SP_ROWS_QUERY_ONLY if form == 1 else sp.SP_ROWS_ALL)
+        return out
+
+    alone = []
+    for r in runs:
+        for form in range(3):
+            alone.append(call(r, form))
+            torch.cuda.synchronize()
+    order = np.random.default_rng(1).integers(0, len(alone), 120)
+    got = [call(runs[i // 3], i % 3) for i in order]
+    sp.sp_check_status(ws)
+    for i, o in zip(order, got):
+        assert torch.equal(o, alone[i]), (i // 3, i % 3)
+
+
+@pytest.mark.parametrize("H,Hkv", [(4, 4), (8, 2)])
+def test_a_chain_reads_what_the_call_before_wrote(H, Hkv):
+    """Rotation -> decode on inputs that change from step to step, scores -> top-k -> decode: what one kernel writes the next one
+    reads, nothing waited for in between, against the same steps one by one."""
+    lay, D, V, k, steps = _layout(), 128, 600, 2, 24
+    dl = sp.DeviceLayout.from_host(lay)
+    B, T, R = lay.n_prompts, lay.total_tokens, int(lay.qry_len.sum())
+    off = dev(np.concatenate([[0], np.cumsum(lay.qry_len)]).astype(np.int32))
+    kc, vc = dev(_randn((T, Hkv, D), "bf16", 960)), dev(_randn((T, Hkv, D), "bf16", 961))
+    tk, tv = dev(_randn((steps, B, 1, Hkv, D), "bf16", 962)), dev(_randn((steps, B, 1, Hkv, D), "bf16", 963))
+    qs, logits = dev(_randn((steps, B, H, D), "bf16", 964)), dev(_randn((steps, R, V), "bf16", 965))
+    tgt = dev(torch.randint(0, V, (R,), generator=torch.Generator().manual_seed(966), dtype=torch.int32))
+    tl, ws, sws = dev(np.ones(B, np.int32)), workspace(sp.sp_decode_workspace_bytes(B, H, D)), workspace(sp.sp_path_scores_workspace_bytes(R))
+    q, key, scores = torch.empty_like(qs[0]), torch.empty_like(tk[0]), torch.empty(lay.n_paths, device="cuda")
+    kept = torch.empty((B, k), dtype=torch.int32, device="cuda")
+
+    def run(wait):
+        outs = []
+        for i in range(steps):
+            pos = torch.full((B,), 100.0 + i, device="cuda")
+            out = torch.empty_like(q)
+            q.copy_(qs[i])
+            key.copy_(tk[i])
+            for f in (lambda: sp.sp_path_scores(logits[i], tgt, off, scores, None, None, None, sws),
+                      lambda: sp.sp_prune_topk(scores, dl.prompt_path_off, k, kept),
+                      lambda: sp.sp_rope_apply_pair(q, H, key, Hkv, pos, D),
+                      lambda: sp.sp_pruned_decode(q, kc, vc, dl, kept, k, key, tv[i], tl, 1, D ** -0.5, out, None, ws)):
+                f()
+                if wait:
+                    torch.cuda.synchronize()
+            outs.append((out, kept.clone()))
+        return outs
+
+    for (a, ka), (b, kb) in zip(run(True), run(False)):
+        assert torch.equal(ka, kb) and torch.equal(a, b)
