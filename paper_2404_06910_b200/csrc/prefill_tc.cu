@@ -78,6 +78,9 @@ template <int D, bool ALIBI, bool SPLIT> struct TcConfig {
                          BAR_L_READY = BAR_P + 4, BAR_X_FREE = BAR_L_READY + 2, BAR_O_FREE = BAR_X_FREE + 2,
                          BAR_COUNT = BAR_O_FREE + 2;
     static constexpr int SMEM = BAR_OFF + BAR_COUNT * 8 + 16;
+    // No other block with operands in shared memory fits on the SM: less than 1 KB of it is left besides the 1 KB that each block
+    // has reserved (and 4 096 registers).
+    static constexpr bool ALONE = SMEM + 3 * 1024 > 228 * 1024;
     // Registers per thread: at launch (what __launch_bounds__ makes of 65 536), and after the split.  The softmax warps take
     // what the others give back, which has to add up; only they grow.
     static constexpr int R_LAUNCH = 96, R_SOFT = 128, R_EPI = 96, R_LOAD = 56, R_MMA = 64;
@@ -85,6 +88,8 @@ template <int D, bool ALIBI, bool SPLIT> struct TcConfig {
     static_assert(R_SOFT >= R_LAUNCH && R_EPI <= R_LAUNCH && R_LOAD <= R_LAUNCH && R_MMA <= R_LAUNCH, "direction of setmaxnreg");
 };
 static_assert(TcConfig<128, false, false>::SMEM <= 232448 && TcConfig<128, true, false>::SMEM <= 232448, "one block's shared memory");
+
+static_assert(TcConfig<128, false, true>::ALONE && TcConfig<128, true, true>::ALONE && !TcConfig<64, true, true>::ALONE, "who shares an SM");
 
 // The instruction stream of the softmax warps is what paces a lane: three-input maxima and two-lane fp32 forms.
 __device__ __forceinline__ float fmax3(float a, float b, float c)
@@ -305,12 +310,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
     } else if (threadIdx.x >= 96 && threadIdx.x < 105) {
         prefetch_tmap(&p.maps[0][0] + (threadIdx.x - 96));
     }
-    if (warp == WARP_MMA) { tmem_alloc(tmem_base_s, kTmemCols); tmem_relinquish(); }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    pdl_trigger();
-    pdl_wait();                       // the tile list and everything before it in the stream
+    auto take_tmem = [&]() {
+        if (warp == WARP_MMA) { tmem_alloc(tmem_base_s, kTmemCols); tmem_relinquish(); }
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        pdl_trigger();
+    };
+    // pdl_wait(): the tile list and everything before it in the stream.  Where another kernel's block fits beside this one, tensor
+    // memory is taken behind the wait and before the next kernel is let in: a block that held it while it waits, or one of a
+    // dependent's that took it first, could keep its neighbour waiting for columns that are freed only after that neighbour has
+    // ended.  Costs 0.2 us of a launch.
+    if (C::ALONE) { take_tmem(); pdl_wait(); } else { pdl_wait(); take_tmem(); }
     const uint32_t tb = *tmem_base_s;
     bool ok = (smem_u32(smem) & 1023u) == 0;      // the swizzle atoms need it; reported like an expired wait
 

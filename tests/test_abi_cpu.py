@@ -130,3 +130,15 @@ def test_kernels_read_coherently():
         text = re.sub(r"//[^\n]*|/\*.*?\*/", "", open(os.path.join(src, name)).read(), flags=re.S)
         found = re.findall(r"__ldg|__restrict__|ld\.global\.nc|__ldcs", text)
         assert not found, (name, found)
+
+
+def test_tensor_memory_is_taken_between_the_wait_and_the_trigger():
+    """A block that holds tensor memory while it waits for the kernel in front of it, or lets the next kernel's blocks in before
+    it has its own, can deadlock with a neighbour on the SM (nothing to run: this is the order of the statements).  Where shared
+    memory leaves no room for a neighbour the order is free."""
+    body = open(os.path.join(os.path.dirname(sp.LIB_PATH), "csrc", "prefill_tc.cu")).read()
+    assert "ALONE = SMEM + 3 * 1024 > 228 * 1024;" in body
+    body = body[body.index(") prefill_tc_kernel("):]
+    assert body.index("tmem_alloc(") < body.index("pdl_trigger();") < body.index("pdl_wait(); take_tmem();")
+    assert "if (C::ALONE) { take_tmem(); pdl_wait(); } else { pdl_wait(); take_tmem(); }" in body
+    assert body.count("tmem_alloc(") == body.count("pdl_trigger();") - 1 == 1          # the rotation of Q has the other trigger
