@@ -908,6 +908,7 @@ static int launch_tc(const void *q, const void *k, const void *v, const sp_layou
     pa.sort_from = 12 * num_sms() / (n_heads >> log_g);
     pa.hdr = hdr; pa.list = pairs;
     if (int rc = launch(prefill_plan_kernel<true>, 1, 1024, 0, st, 1, pa)) return rc;
+    if (pa.max_tiles == 0) return SP_OK;              // no segment can have a row
     if (rope) {
         RopeRows r = *rope;
         r.hdr = hdr; r.pairs = pairs; r.item_groups = 2 * pa.tile_rows / kRopeRows;
@@ -926,7 +927,6 @@ static int launch_tc(const void *q, const void *k, const void *v, const sp_layou
     p.stall_producer = g_stall_producer ? 1 : 0;      // test hook, see sp_test_stall_producer below
 
     const int64_t items = pa.max_tiles * p.n_units;
-    if (items == 0) return SP_OK;
     const int grid = (int)std::min<int64_t>(items, num_sms());
     using Launch = int (*)(const TcParams &, int, cudaStream_t);
     const auto run = [&](Launch single, Launch grouped) { return (log_g ? grouped : single)(p, grid, st); };
@@ -947,8 +947,8 @@ int launch_prefill_tc(const void *q, const void *k, const void *v, const sp_layo
     return launch_tc(q, k, v, lay, pos, slopes, nullptr, n_heads, n_kv_heads, head_dim, scale, rows, out, lse, ws, st);
 }
 
-// sp_superpose_prefill_rope.  The size leaves room for 512 bytes per token behind the tile list: the interface has asked
-// for it since its first version (a table of angles), and callers have sized their workspaces by it.
+// sp_superpose_prefill_rope.  The size has 512 bytes per token behind the tile list that nothing uses any more (a table of angles
+// was there): the entry point has refused less since its first version, and what it refuses is part of the interface.
 size_t prefill_tc_rope_workspace_bytes(int n_prompts, int n_paths, int max_pre_len, int max_path_len, int64_t total_tokens)
 {
     return prefill_tc_workspace_bytes(n_prompts, n_paths, max_pre_len, max_path_len, 0) +

@@ -106,3 +106,17 @@ def test_prefill_rope_rejects_what_it_does_not_serve():
     with pytest.raises(sp.SpError) as e:
         sp.sp_superpose_prefill_rope(q, q, q, dl, pos, 10000.0, 7, 0.1, out, None, workspace(1 << 20))
     assert e.value.code == sp.SP_ERR_INVALID_ARG
+
+
+def test_fused_rope_without_any_segment():
+    """Rows that belong to no segment: nothing to do, no launch of an empty grid, out untouched."""
+    lay = build_layout([0], [[]], [[]])
+    lay.total_tokens = 8
+    dl = sp.DeviceLayout.from_host(lay)
+    q, out = dev(_randn((8, 2, 128), 1)), torch.full((8, 2, 128), 7.0, dtype=torch.bfloat16, device="cuda")
+    ws = workspace(sp.sp_prefill_rope_workspace_bytes(dl, 2, 128, sp.SP_BF16))
+    for rows in (sp.SP_ROWS_ALL, sp.SP_ROWS_QUERY_ONLY):
+        sp.sp_superpose_prefill(q, q, q, dl, 0.1, out, None, ws, rows=rows)
+    sp.sp_superpose_prefill_rope(q, q, q, dl, torch.zeros(8, device="cuda"), 10000.0, 0, 0.1, out, None, ws)
+    sp.sp_check_status(ws)
+    assert bool((out == 7.0).all())
