@@ -8,7 +8,7 @@
 // A contraction may run over its elements in any order and output rows may be any permutation, so every thread loads
 // contiguous 16-byte pieces of K and V rows and uses them as fragments: no shared memory, no ldmatrix.  Only V needs a
 // byte permute to pair two keys.  P is carried as the sum of two bf16 numbers (16 bits of mantissa), so the result is as
-// good as with fp32 products.
+// good as with fp32 products, values that are not finite included.
 #pragma once
 
 namespace sp {
@@ -23,6 +23,8 @@ __device__ __forceinline__ void mma_16n8k16(float (&d)[4], uint32_t a0, uint32_t
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
+
+static __device__ const uint4 g_zero_row[16] = {};
 
 // Grid (n_splits, KV heads x blocks of up to 8 query heads, prompts); the n_splits blocks of a (prompt, y) are a cluster.
 template <int D, bool ALIBI, bool ROPE>
@@ -145,8 +147,9 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
         float p[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) { p[e] = ex2f(x[e] - m); l += p[e]; }
-        const uint32_t ph0 = pack_bf16x2(p[0], p[1]), ph1 = pack_bf16x2(p[2], p[3]);
-        const uint32_t pl0 = pack_bf16x2(p[0] - bf16_lo(ph0), p[1] - bf16_hi(ph0)), pl1 = pack_bf16x2(p[2] - bf16_lo(ph1), p[3] - bf16_hi(ph1));
+        uint32_t ph0, ph1, pl0, pl1;
+        split_bf16(p[0], p[1], ph0, pl0);
+        split_bf16(p[2], p[3], ph1, pl1);
         // row gid of tile i is element 8 gid + i, row gid + 8 is element 8 gid + i + 64 (D = 64: 8 gid + i + 4)
 #pragma unroll
         for (int i = 0; i < NM; ++i) {
@@ -169,12 +172,13 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
     int seg = 0;
     for (int base = lo + warp * kMmaKeys; base < hi_loop; base += W * kMmaKeys) {
         const int n = min(kMmaKeys, hi_loop - base);
-        // lane i (and i + 16) finds key i of the turn; keys that do not exist read the last one and get no weight
+        // lane i (and i + 16) finds key i of the turn; keys that do not exist read the last one's K and get no weight, which is not
+        // enough where V holds an Inf: they read a V row of zeros
         const int j = base + min(lane & 15, n - 1);
         while (j >= sm.lo[seg + 1]) ++seg;                  // keys ascend: segments only advance
         const int64_t off = (int64_t)(j - sm.lo[seg]) * row_elems;
         const float kpos = ALIBI ? sm.pos[seg][j - sm.lo[seg]] : 0.f;
-        const unsigned long long kp = reinterpret_cast<unsigned long long>(sm.k[seg] + off), vp = reinterpret_cast<unsigned long long>(sm.v[seg] + off);
+        const unsigned long long kp = reinterpret_cast<unsigned long long>(sm.k[seg] + off), vp = reinterpret_cast<unsigned long long>((lane & 15) < n ? sm.v[seg] + off : reinterpret_cast<const T *>(g_zero_row));
         uint4 kr[2][NC], vr[4][NV];
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
@@ -199,7 +203,10 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
 #pragma unroll
         for (int c = 0; c < NC; ++c) kr[0][c] = krow[tig + 4 * c];
 #pragma unroll
-        for (int c = 0; c < NV; ++c) vr[0][c] = vr[1][c] = vr[2][c] = vr[3][c] = vrow[gid + 8 * c];
+        for (int c = 0; c < NV; ++c) {                      // the key is number 0, of the threads with tig 0
+            vr[1][c] = vr[2][c] = vr[3][c] = make_uint4(0u, 0u, 0u, 0u);
+            vr[0][c] = tig == 0 ? vrow[gid + 8 * c] : vr[1][c];
+        }
         rotate(kr[0]);
         __syncwarp();
 #pragma unroll

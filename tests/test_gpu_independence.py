@@ -179,6 +179,39 @@ def test_decode_sees_only_kept_paths(dtype, D, kind):
         assert torch.equal(out0, out1) and torch.equal(lse0, lse1), f"pruned path {j} ({kind}) reached the decode output"
 
 
+@pytest.mark.parametrize("dtype,D,Hkv", [("bf16", 128, 1), ("bf16", 128, 2), ("bf16", 128, 4), ("bf16", 64, 1), ("bf16", 64, 2),
+                                         ("f32", 64, 1)])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), float("-inf")])
+@pytest.mark.parametrize("rope", [False, True])
+def test_decode_values_that_are_not_finite_stay_in_their_column(dtype, D, Hkv, bad, rope):
+    """An Inf in V is an Inf of the output and no NaN, in its column alone, wherever the key lies: preamble, kept paths, the last
+    key of a split, the tail's older rows and the newest one.  The other columns keep their bits."""
+    lay = build_layout([21], [[37, 130, 9, 77]], [[5, 7, 3, 11]])
+    T, H, cap, k = lay.total_tokens, 4, 3, 2
+    kc, vc = _randn((T, Hkv, D), dtype, 970), _randn((T, Hkv, D), dtype, 971)
+    q, tk, tv = dev(_randn((1, H, D), dtype, 972)), _randn((1, cap, Hkv, D), dtype, 973), _randn((1, cap, Hkv, D), dtype, 974)
+    dl, kept, tl, pos = sp.DeviceLayout.from_host(lay), dev(np.array([[3, 0]], np.int32)), dev(np.array([3], np.int32)), torch.full((1,), 9.0, device="cuda")
+
+    def run(vc_, tv_):
+        out = torch.zeros((1, H, D), dtype=TDT[dtype], device="cuda")
+        args = (q, dev(kc), dev(vc_), dl, kept, k, dev(tk), dev(tv_), tl, cap)
+        if rope:
+            sp.sp_pruned_decode_rope(*args, pos, D ** -0.5, out)
+        else:
+            sp.sp_pruned_decode(*args, D ** -0.5, out, None, workspace(sp.sp_decode_workspace_bytes(1, H, D)))
+        return out.cpu()
+
+    out0, cols = run(vc, tv), torch.arange(D) != 5
+    rows = [("cache", r) for r in (0, 15, 20, int(_path_rows(lay, 0)[-1]), int(_path_rows(lay, 3)[0]), int(_path_rows(lay, 3)[-1]))]
+    for where, r in rows + [("tail", 0), ("tail", 2)]:
+        v2, t2 = vc.clone(), tv.clone()
+        (v2 if where == "cache" else t2[0])[r, :, 5] = bad
+        out1 = run(v2, t2)
+        assert torch.equal(out0[..., cols], out1[..., cols]), (where, r)
+        got = out1[..., 5].float()
+        assert bool(torch.isnan(got).all() if bad != bad else (got == bad).all()), (where, r, got)
+
+
 @pytest.mark.parametrize("D,Hkv", [(128, 4), (128, 2), (64, 4)])
 def test_prefills_in_a_row_through_one_workspace(D, Hkv):
     """Launches may start before the one in front of them has finished: each reads the work list of its own layout.  Layouts of
