@@ -1,6 +1,6 @@
 """Builds the CUDA library in-tree: every csrc/*.cu -> libsp_b200.so (sm_100a only), and the same
 sources with -DSP_DEBUG_BOUNDS (extra device-side layout checks) -> libsp_b200_debug.so; and the Python argument
-marshalling, csrc/marshal.c -> _marshal.so."""
+marshalling, csrc/marshal.c -> _marshal (with the interpreter's suffix)."""
 from __future__ import annotations
 
 import os
@@ -15,7 +15,9 @@ OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libsp_b200.so")
 OBJ_DEBUG = os.path.join(HERE, "_build_debug")
 LIB_DEBUG = os.path.join(HERE, "libsp_b200_debug.so")
-MARSHAL = os.path.join(HERE, "_marshal.so")
+MARSHAL = os.path.join(HERE, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))     # an interpreter's own
+MARSHAL_FLAGS = ["-O2", "-Wall", "-Werror=int-conversion", "-Werror=incompatible-pointer-types", "-shared", "-fPIC",
+                 "-I", sysconfig.get_paths()["include"]]
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -64,11 +66,11 @@ def _build_one(lib: str, obj_dir: str, extra, force: bool, verbose: bool) -> str
 
 def _build_marshal(force: bool) -> None:
     src = os.path.join(CSRC, "marshal.c")
-    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= os.path.getmtime(src):
-        return
-    tmp = MARSHAL + f".tmp{os.getpid()}"
-    subprocess.check_call(["gcc", "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], src, "-o", tmp])
-    os.replace(tmp, MARSHAL)
+    newest = max(os.path.getmtime(f) for f in (src, os.path.join(HERE, "..", "include", "sp.h"), os.path.abspath(__file__)))
+    if force or not os.path.exists(MARSHAL) or os.path.getmtime(MARSHAL) < newest:
+        tmp = MARSHAL + f".tmp{os.getpid()}"
+        subprocess.check_call(["gcc", *MARSHAL_FLAGS, src, "-o", tmp])
+        os.replace(tmp, MARSHAL)
 
 
 def build(force: bool = False, verbose: bool = False, debug: bool = True) -> str:

@@ -9,11 +9,12 @@
 #include <Python.h>
 #include <stdint.h>
 
+#include "../../include/sp.h"
+
 #define MAX_FN 32
 #define MAX_ARG 28
 
 typedef union { void *p; long long q; double d; } val;
-typedef const void *P;
 
 static struct { void *fn; char kinds[MAX_ARG + 1]; } entry[MAX_FN];
 static PyObject *s_data_ptr, *s_is_contiguous;
@@ -58,50 +59,52 @@ static PyObject *bind(PyObject *self, PyObject *args)
     Py_RETURN_NONE;
 }
 
-/* The order of the cases is the order in which binding.py binds the entry points. */
+/* The order of the cases is the order in which binding.py binds the entry points.  A call goes through the type that sp.h
+ * declares: a changed parameter does not compile (build.py makes the conversions between integers and pointers errors). */
+#define CALL(name) ((__typeof__(&name))f)
 static int invoke(int i, const val *v)
 {
     void *f = entry[i].fn;
     switch (i) {
     case 0:      /* sp_rope_apply */
-        return ((int (*)(P, P, int64_t, int64_t, int, int, int, double, int, int, P))f)(
+        return CALL(sp_rope_apply)(
             v[0].p, v[1].p, v[2].q, v[3].q, (int)v[4].q, (int)v[5].q, (int)v[6].q, v[7].d, (int)v[8].q, (int)v[9].q, v[10].p);
     case 1:      /* sp_rope_apply_pair */
-        return ((int (*)(P, int64_t, int, P, int64_t, int, P, int64_t, int, int, double, int, int, P))f)(
+        return CALL(sp_rope_apply_pair)(
             v[0].p, v[1].q, (int)v[2].q, v[3].p, v[4].q, (int)v[5].q, v[6].p, v[7].q, (int)v[8].q, (int)v[9].q, v[10].d, (int)v[11].q,
             (int)v[12].q, v[13].p);
     case 2:      /* sp_superpose_prefill */
-        return ((int (*)(P, P, P, P, int, int, int, float, int, P, P, P, size_t, int, P))f)(
+        return CALL(sp_superpose_prefill)(
             v[0].p, v[1].p, v[2].p, v[3].p, (int)v[4].q, (int)v[5].q, (int)v[6].q, (float)v[7].d, (int)v[8].q, v[9].p, v[10].p, v[11].p,
             (size_t)v[12].q, (int)v[13].q, v[14].p);
     case 3:      /* sp_superpose_prefill_alibi */
-        return ((int (*)(P, P, P, P, P, P, int, int, int, float, int, P, P, P, size_t, int, P))f)(
+        return CALL(sp_superpose_prefill_alibi)(
             v[0].p, v[1].p, v[2].p, v[3].p, v[4].p, v[5].p, (int)v[6].q, (int)v[7].q, (int)v[8].q, (float)v[9].d, (int)v[10].q, v[11].p,
             v[12].p, v[13].p, (size_t)v[14].q, (int)v[15].q, v[16].p);
     case 4:      /* sp_superpose_prefill_rope */
-        return ((int (*)(P, P, P, P, P, double, int, int, int, int, float, P, P, P, size_t, int, P))f)(
+        return CALL(sp_superpose_prefill_rope)(
             v[0].p, v[1].p, v[2].p, v[3].p, v[4].p, v[5].d, (int)v[6].q, (int)v[7].q, (int)v[8].q, (int)v[9].q, (float)v[10].d, v[11].p,
             v[12].p, v[13].p, (size_t)v[14].q, (int)v[15].q, v[16].p);
     case 5:      /* sp_path_scores */
-        return ((int (*)(P, int64_t, P, P, int64_t, int, int, P, P, P, P, P, size_t, int, P))f)(
+        return CALL(sp_path_scores)(
             v[0].p, v[1].q, v[2].p, v[3].p, v[4].q, (int)v[5].q, (int)v[6].q, v[7].p, v[8].p, v[9].p, v[10].p, v[11].p, (size_t)v[12].q,
             (int)v[13].q, v[14].p);
     case 6:      /* sp_prune_topk */
-        return ((int (*)(P, P, int, int, P, P, P))f)(v[0].p, v[1].p, (int)v[2].q, (int)v[3].q, v[4].p, v[5].p, v[6].p);
+        return CALL(sp_prune_topk)(v[0].p, v[1].p, (int)v[2].q, (int)v[3].q, v[4].p, v[5].p, v[6].p);
     case 7:      /* sp_pruned_decode */
-        return ((int (*)(P, P, P, P, P, int, P, P, P, int, int64_t, int, int, int, float, P, P, P, size_t, int, P))f)(
+        return CALL(sp_pruned_decode)(
             v[0].p, v[1].p, v[2].p, v[3].p, v[4].p, (int)v[5].q, v[6].p, v[7].p, v[8].p, (int)v[9].q, v[10].q, (int)v[11].q, (int)v[12].q,
             (int)v[13].q, (float)v[14].d, v[15].p, v[16].p, v[17].p, (size_t)v[18].q, (int)v[19].q, v[20].p);
     case 8:      /* sp_pruned_decode_alibi */
-        return ((int (*)(P, P, P, P, P, int, P, P, P, int, int64_t, P, P, P, P, int, int, int, float, P, P, P, size_t, int, P))f)(
+        return CALL(sp_pruned_decode_alibi)(
             v[0].p, v[1].p, v[2].p, v[3].p, v[4].p, (int)v[5].q, v[6].p, v[7].p, v[8].p, (int)v[9].q, v[10].q, v[11].p, v[12].p, v[13].p,
             v[14].p, (int)v[15].q, (int)v[16].q, (int)v[17].q, (float)v[18].d, v[19].p, v[20].p, v[21].p, (size_t)v[22].q, (int)v[23].q, v[24].p);
     case 9:      /* sp_pruned_decode_rope */
-        return ((int (*)(P, P, P, P, P, int, P, P, P, int, int64_t, P, double, int, int, int, int, float, P, P, int, P))f)(
+        return CALL(sp_pruned_decode_rope)(
             v[0].p, v[1].p, v[2].p, v[3].p, v[4].p, (int)v[5].q, v[6].p, v[7].p, v[8].p, (int)v[9].q, v[10].q, v[11].p, v[12].d, (int)v[13].q,
             (int)v[14].q, (int)v[15].q, (int)v[16].q, (float)v[17].d, v[18].p, v[19].p, (int)v[20].q, v[21].p);
     case 10:     /* sp_pruned_decode_static */
-        return ((int (*)(P, P, P, P, P, int, P, P, P, int, int64_t, int, int, int, float, P, P, int, P))f)(
+        return CALL(sp_pruned_decode_static)(
             v[0].p, v[1].p, v[2].p, v[3].p, v[4].p, (int)v[5].q, v[6].p, v[7].p, v[8].p, (int)v[9].q, v[10].q, (int)v[11].q, (int)v[12].q,
             (int)v[13].q, (float)v[14].d, v[15].p, v[16].p, (int)v[17].q, v[18].p);
     }

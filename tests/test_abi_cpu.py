@@ -142,3 +142,27 @@ def test_tensor_memory_is_taken_between_the_wait_and_the_trigger():
     assert body.index("tmem_alloc(") < body.index("pdl_trigger();") < body.index("pdl_wait(); take_tmem();")
     assert "if (C::ALONE) { take_tmem(); pdl_wait(); } else { pdl_wait(); take_tmem(); }" in body
     assert body.count("tmem_alloc(") == body.count("pdl_trigger();") - 1 == 1          # the rotation of Q has the other trigger
+
+
+@pytest.mark.parametrize("old,new", [("", ""), ("int k, const void *tail_k", "const int32_t *k, const void *tail_k"),
+                                     ("int n_prompts, int k,\n                  int32_t *kept_idx", "int n_prompts, int32_t *kept_idx"),
+                                     ("float *lse, int dtype", "float *lse, int more, int dtype"),
+                                     ("int64_t ld_token, int n_heads", "const void *ld_token, int n_heads")])
+def test_marshalling_is_compiled_against_the_header(old, new, tmp_path):
+    """A parameter that sp.h declares otherwise than the marshalling passes it does not compile."""
+    import importlib.util
+    import shutil
+    import subprocess
+    pkg = os.path.dirname(sp.LIB_PATH)
+    spec = importlib.util.spec_from_file_location("sp_build", os.path.join(pkg, "build.py"))
+    build = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(build)
+    (tmp_path / "include").mkdir()
+    (tmp_path / "pkg" / "csrc").mkdir(parents=True)
+    text = re.sub(r",\s*", ", ", open(os.path.join(ROOT, "include", "sp.h")).read())
+    old, new = (re.sub(r",\s*", ", ", x) for x in (old, new))
+    assert old in text
+    (tmp_path / "include" / "sp.h").write_text(text.replace(old, new) if old else text)
+    shutil.copy(os.path.join(pkg, "csrc", "marshal.c"), tmp_path / "pkg" / "csrc")
+    rc = subprocess.run(["gcc", *build.MARSHAL_FLAGS, "-fsyntax-only", str(tmp_path / "pkg" / "csrc" / "marshal.c")], capture_output=True).returncode
+    assert (rc == 0) == (old == "")
