@@ -81,9 +81,8 @@ template <> struct Raw16<float> {
     }
 };
 
-// ALIBI: scores get -slope_h * |pos_q - pos_k| (Section 3.2.2: real-valued positions pose no
-// problem for ALiBi); the plain instantiation carries none of that code.
-template <typename T, int D, bool ALIBI>
+// The kernel of sp_pruned_decode_static.
+template <typename T, int D>
 __global__ void __launch_bounds__(kDecThreads, 8)
 decode_kernel(const __grid_constant__ DecodeArgs a)
 {
@@ -99,7 +98,6 @@ decode_kernel(const __grid_constant__ DecodeArgs a)
     const T **seg_k = reinterpret_cast<const T **>(smem_raw + round_up((n_seg + 1) * sizeof(int), 16));
     const T **seg_v = seg_k + n_seg;
     float *red = reinterpret_cast<float *>(seg_v + n_seg);                  // [G][D+2]
-    const float **seg_pos = reinterpret_cast<const float **>(red + G * (D + 2));   // [n_seg], ALiBi only
     __shared__ unsigned int s_ticket;
     pdl_wait();
 
@@ -128,7 +126,6 @@ decode_kernel(const __grid_constant__ DecodeArgs a)
         }
         seg_k[sgm] = kc + row * row_elems;
         seg_v[sgm] = vc + row * row_elems;
-        if (ALIBI) seg_pos[sgm] = (sgm == a.k + 1 && len ? a.tail_pos : a.cache_pos) + row;
         seg_lo[sgm + 1] = len;
     }
     __syncthreads();
@@ -152,13 +149,10 @@ decode_kernel(const __grid_constant__ DecodeArgs a)
     float m = -INFINITY, l = 0.f, acc[N];
 #pragma unroll
     for (int e = 0; e < N; ++e) acc[e] = 0.f;
-    const float q_pos = ALIBI ? a.q_pos[b] : 0.f;
-    const float slope_l2 = ALIBI ? a.slopes[h] * kLog2eD : 0.f;
 
     int seg = 0;
     for (int base = lo; base < hi; base += G * kDecUnroll) {   // trip count is block-uniform
         uint4 kr[kDecUnroll], vr[kDecUnroll];
-        float kpos[kDecUnroll];
         bool live[kDecUnroll];
 #pragma unroll
         for (int u = 0; u < kDecUnroll; ++u) {                  // all loads of the batch first
@@ -169,7 +163,6 @@ decode_kernel(const __grid_constant__ DecodeArgs a)
                 const int64_t off = (int64_t)(j - seg_lo[seg]) * row_elems + sub * N;
                 kr[u] = ld_stream16(seg_k[seg] + off);
                 vr[u] = ld_stream16(seg_v[seg] + off);
-                if (ALIBI) kpos[u] = seg_pos[seg][j - seg_lo[seg]];
             }
         }
         float s[kDecUnroll], cm = -INFINITY;
@@ -184,7 +177,6 @@ decode_kernel(const __grid_constant__ DecodeArgs a)
             }
 #pragma unroll
             for (int o = LPK / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-            if (ALIBI && live[u]) d -= slope_l2 * fabsf(q_pos - kpos[u]);
             s[u] = live[u] ? d : -INFINITY;
             cm = fmaxf(cm, s[u]);
         }
@@ -267,25 +259,18 @@ decode_kernel(const __grid_constant__ DecodeArgs a)
     }
 }
 
-template <typename T, int D, bool ALIBI>
-static int launch_decode_v(const DecodeArgs &a, int n_prompts, cudaStream_t st)
-{
-    constexpr int G = kDecThreads / (D / Vec<T>::N);
-    const int n_seg = a.k + 2;
-    const size_t smem = round_up((n_seg + 1) * sizeof(int), 16) + 2 * n_seg * sizeof(void *) +
-                        (size_t)G * (D + 2) * sizeof(float) + (ALIBI ? n_seg * sizeof(void *) : 0);
-    SP_REQUIRE(smem <= 200 * 1024, SP_ERR_UNSUPPORTED, "sp_pruned_decode: k = %d needs too much shared memory", a.k);
-    if (smem > 48 * 1024)
-        SP_CUDA(cudaFuncSetAttribute(decode_kernel<T, D, ALIBI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    dim3 grid(a.n_splits, a.n_heads, n_prompts);
-    return launch(decode_kernel<T, D, ALIBI>, grid, kDecThreads, smem, st, 1, a);
-}
 template <typename T, int D>
 static int launch_decode(const DecodeArgs &a, int n_prompts, cudaStream_t st)
 {
-    return a.slopes ? launch_decode_v<T, D, true>(a, n_prompts, st) : launch_decode_v<T, D, false>(a, n_prompts, st);
+    constexpr int G = kDecThreads / (D / Vec<T>::N);
+    const int n_seg = a.k + 2;
+    const size_t smem = round_up((n_seg + 1) * sizeof(int), 16) + 2 * n_seg * sizeof(void *) + (size_t)G * (D + 2) * sizeof(float);
+    SP_REQUIRE(smem <= 200 * 1024, SP_ERR_UNSUPPORTED, "sp_pruned_decode: k = %d needs too much shared memory", a.k);
+    if (smem > 48 * 1024)
+        SP_CUDA(cudaFuncSetAttribute(decode_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    dim3 grid(a.n_splits, a.n_heads, n_prompts);
+    return launch(decode_kernel<T, D>, grid, kDecThreads, smem, st, 1, a);
 }
-
 
 // ---------------------------------------------------------------------------------------
 // Cluster variant (the one sp_pruned_decode runs): the blocks that split one (prompt, KV head)
