@@ -684,9 +684,11 @@ template <int D, bool ALIBI, bool ROPE>
 static int launch_decode_mma(DecodeArgs a, const DecodeRope &rope, int pairing, int n_prompts, int64_t max_keys, cudaStream_t st)
 {
     const int group = a.n_heads / a.n_kv_heads, blocks_y = a.n_kv_heads * ((group + kMmaHeads - 1) / kMmaHeads);
-    const int warps = kMmaWarpsPerSM * num_sms();
+    const int warps = mma_warps_per_sm(D) * num_sms();
     const int64_t units = (int64_t)n_prompts * blocks_y;
-    a.n_splits = cluster_splits(n_prompts, blocks_y, max_keys, kMmaMaxWarps * kMmaKeys, kMmaWarpsPerSM / kMmaMaxWarps);
+    // three blocks per SM for both head sizes: with four, 2 prompts x 16 KV heads of 64 become clusters of 16, which the SMs take in
+    // less evenly than clusters of 8 (12.1 us against 8.0)
+    a.n_splits = cluster_splits(n_prompts, blocks_y, max_keys, kMmaMaxWarps * kMmaKeys, mma_warps_per_sm(128) / kMmaMaxWarps);
     // Unsplit launches take as many warps a block as still leave every block resident at once: 64 prompts x 8 KV heads fit with
     // three (30 us a step); blocks of four need a second wave (33).
     int w = kMmaMaxWarps;

@@ -16,7 +16,9 @@ namespace sp {
 constexpr int kMmaHeads = 8;         // query heads per block at most
 constexpr int kMmaKeys = 16;         // keys per warp and turn
 constexpr int kMmaMaxWarps = 4;      // warps per block at most
-constexpr int kMmaWarpsPerSM = 12;   // resident, with the 168 registers that a warp's loads and accumulators take
+// Warps resident per SM, by the registers that a warp's loads and accumulators take: 168 with head_dim 128, less than 128 with 64
+// (64 prompts x 16 KV heads of 64: one warp to a block and 44.8 us with a budget of 12, two and 29.4 with 16).
+constexpr int mma_warps_per_sm(int D) { return D == 64 ? 16 : 12; }
 
 __device__ __forceinline__ void mma_16n8k16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
 {
@@ -28,7 +30,7 @@ static __device__ const uint4 g_zero_row[16] = {};
 
 // Grid (n_splits, KV heads x blocks of up to 8 query heads, prompts); the n_splits blocks of a (prompt, y) are a cluster.
 template <int D, bool ALIBI, bool ROPE>
-__global__ void __launch_bounds__(32 * kMmaMaxWarps, kMmaWarpsPerSM / kMmaMaxWarps)
+__global__ void __launch_bounds__(32 * kMmaMaxWarps, mma_warps_per_sm(D) / kMmaMaxWarps)
 decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ DecodeRope rope, int rope_pairing)
 {
     using T = __nv_bfloat16;
