@@ -19,11 +19,15 @@ constexpr int kPairKeys = 64;         // keys per key tile of a pair
 struct alignas(16) TcPair {                       // one or two consecutive query tiles of a segment (shared by all heads)
     // Keys of the segment are numbered u: its fully visible prefix (the prompt's preamble, may be empty) at [0, pre_len),
     // its own rows from p16 = pre_len rounded up to 16.
+    // Rows of consecutive paths: the "segment" starts with tile A's first path and ends with the last row of the item; what a row
+    // sees of it starts with its own path.  p16 and steps_a follow from the rest there, and two other numbers take their place.
     int32_t own_base;                 // packed row of own key u is own_base + u
     int32_t q_u;                      // key number of tile A's first row
-    int32_t pre_row, pre_len, p16;
+    int32_t pre_row, pre_len;
+    int32_t p16;                      // rows of consecutive paths: index of tile A's first path (-1: one segment after all)
     int32_t rows_ab;                  // rows of tile A | rows of tile B, which follows it, << 16 (0: no tile B)
-    int32_t steps_a, steps;           // key tiles: of tile A, of the item
+    int32_t steps_a;                  // key tiles of tile A; rows of consecutive paths: key number where tile B's first path starts
+    int32_t steps;                    // key tiles of the item
 };
 static_assert(sizeof(TcPair) == sizeof(TcTile), "both lists use the same slots of the workspace");
 
@@ -31,6 +35,13 @@ struct TcHeader {                     // start of the workspace
     uint32_t status;
     uint32_t n_tiles;                 // entries of the list: tiles, or pairs of tiles
 };
+
+// Height of the query tiles of n rows in a row: as many tiles as it takes, of equal height in whole warps.
+__host__ __device__ inline int even_height(int rows, int tile_rows)
+{
+    const int nt = (rows + tile_rows - 1) / tile_rows, even = nt > 1 ? ((rows + nt - 1) / nt + 31) & ~31 : tile_rows;
+    return even < tile_rows ? even : tile_rows;
+}
 
 // ---- plan: ragged layout -> tile list ---------------------------------------------------
 struct PlanArgs {
@@ -41,6 +52,7 @@ struct PlanArgs {
     int64_t total_tokens;             // T: every segment must lie inside [0, T)
     int64_t max_tiles;                // capacity of the tile list
     int sort_from;                    // pairs: lists of at least so many records are sorted
+    int across;                       // pairs: tiles over the rows of consecutive paths
     TcHeader *hdr;
     void *list;                       // TcTile or TcPair
 };
@@ -73,6 +85,25 @@ static __global__ void __launch_bounds__(1024) prefill_plan_kernel(const PlanArg
     __syncthreads();
     const int n_seq = a.n_prompts + a.n_paths;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto prompt_of = [&](int i) {
+        int lo = 0, hi = a.n_prompts - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (a.ppo[mid] <= i) lo = mid; else hi = mid - 1;
+        }
+        return lo;
+    };
+    bool across = PAIRS && a.across;
+    if (across) {                     // what the host saw in its mirror, in the arrays themselves; otherwise segment by segment
+        bool fit = true;
+        for (int i = threadIdx.x; i < a.n_paths && fit; i += 1024) {
+            const int b = prompt_of(i), n = a.doc_len[i] + a.qry_len[i];
+            fit = a.ppo[b] >= 0 && a.ppo[b] <= i && i < a.ppo[b + 1] && a.ppo[b + 1] <= a.n_paths && a.pre_len[b] > 0 && n > 0 && n <= a.max_path_len &&
+                  a.path_start[i] >= 0 && (int64_t)a.path_start[i] + n <= a.total_tokens &&
+                  (i == a.ppo[b] || a.path_start[i] == a.path_start[i - 1] + a.doc_len[i - 1] + a.qry_len[i - 1]);
+        }
+        across = __syncthreads_and(fit);
+    }
     for (int base = 0; base < n_seq; base += 1024) {
         const int s = base + threadIdx.x;
         int first = 0, rows = 0, own_row = 0, pre_row = 0, pre_n = 0;
@@ -82,12 +113,7 @@ static __global__ void __launch_bounds__(1024) prefill_plan_kernel(const PlanArg
             bad = len < 0 || len > a.max_pre_len || row < 0 || (int64_t)row + len > a.total_tokens;
             if (a.rows_mode == SP_ROWS_ALL && !bad) { rows = len; own_row = row; }
         } else if (s < n_seq) {
-            const int i = s - a.n_prompts;
-            int lo = 0, hi = a.n_prompts - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (a.ppo[mid] <= i) lo = mid; else hi = mid - 1;
-            }
+            const int i = s - a.n_prompts, lo = prompt_of(i);
             pre_row = a.pre_start[lo]; pre_n = a.pre_len[lo];
             own_row = a.path_start[i];
             const int dl = a.doc_len[i], ql = a.qry_len[i];
@@ -107,12 +133,19 @@ static __global__ void __launch_bounds__(1024) prefill_plan_kernel(const PlanArg
             rows = bad ? 0 : dl + ql - first;
         }
         if (bad) a.hdr->status = STATUS_BAD_LAYOUT;
-        int nt = (rows + a.tile_rows - 1) / a.tile_rows, height = a.tile_rows;
-        if (PAIRS && nt > 1) {
-            height = min(a.tile_rows, ((rows + nt - 1) / nt + 31) & ~31);
-            nt = (rows + height - 1) / height;
+        // Rows of consecutive paths: a prompt's rows behind its preamble are cut into pairs of tiles from the first to the last, and a
+        // path writes the records of the pairs that start in it.
+        const bool own = !(across && s >= a.n_prompts && rows > 0);
+        int run0 = 0, run = rows, last = 0;                       // rows cut as one run, the first one's number; its last path
+        if (PAIRS && !own) {
+            const int b = prompt_of(s - a.n_prompts);
+            last = a.ppo[b + 1] - 1;
+            run0 = a.path_start[a.ppo[b]];
+            run = a.path_start[last] + a.doc_len[last] + a.qry_len[last] - run0;
         }
-        const int n_rec = PAIRS ? (nt + 1) / 2 : nt;
+        const int height = PAIRS ? even_height(run, a.tile_rows) : a.tile_rows, nt = (rows + height - 1) / height;
+        const int at = own_row - run0, w0 = own ? 0 : (at + 2 * height - 1) / (2 * height);
+        const int n_rec = !PAIRS ? nt : (own ? (nt + 1) / 2 : (at + rows + 2 * height - 1) / (2 * height) - w0);
         int incl = n_rec;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -125,7 +158,24 @@ static __global__ void __launch_bounds__(1024) prefill_plan_kernel(const PlanArg
         for (int w = 0; w < warp; ++w) before += warp_tot[w];
         const int off = before + incl - n_rec;
         for (int t = 0; t < n_rec && off + t < a.max_tiles; ++t) {
-            if (PAIRS) {
+            if (PAIRS && !own) {
+                const int q0 = (w0 + t) * 2 * height, rows_a = min(height, run - q0), rows_b = min(height, run - q0 - rows_a);
+                TcPair pr;
+                const int p16 = (pre_n + 15) & ~15;
+                pr.own_base = own_row - p16;
+                pr.q_u = p16 + q0 - at;
+                pr.pre_row = pre_row; pr.pre_len = pre_n;
+                pr.p16 = s - a.n_prompts;
+                pr.rows_ab = rows_a | rows_b << 16;
+                int lo = s - a.n_prompts, hi = last;              // the path of tile B's first row
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (a.path_start[mid] - run0 <= q0 + rows_a) lo = mid; else hi = mid - 1;
+                }
+                pr.steps_a = a.path_start[lo] - pr.own_base;
+                pr.steps = (pr.q_u + rows_a + rows_b + kPairKeys - 1) / kPairKeys;
+                static_cast<TcPair *>(a.list)[off + t] = pr;
+            } else if (PAIRS) {
                 const int t0 = max(2 * t - (nt & 1), 0);          // first tile of the record
                 const bool two = !((nt & 1) && t == 0);
                 const int rows_a = min(height, rows - t0 * height), rows_b = two ? min(height, rows - (t0 + 1) * height) : 0;
@@ -135,7 +185,8 @@ static __global__ void __launch_bounds__(1024) prefill_plan_kernel(const PlanArg
                 pr.q_u = pr.p16 + first + t0 * height;
                 pr.pre_row = pre_row; pr.pre_len = pre_n;
                 pr.rows_ab = rows_a | rows_b << 16;
-                pr.steps_a = (pr.q_u + rows_a + kPairKeys - 1) / kPairKeys;
+                pr.steps_a = a.across ? 0 : (pr.q_u + rows_a + kPairKeys - 1) / kPairKeys;
+                if (a.across) pr.p16 = -1;
                 pr.steps = (pr.q_u + rows_a + rows_b + kPairKeys - 1) / kPairKeys;
                 static_cast<TcPair *>(a.list)[off + t] = pr;
             } else {

@@ -6,7 +6,9 @@
 // all of them and a tile's rows lie closer to the diagonal.  Its keys are
 // the preamble's rows (all visible) followed by the segment's own rows up to the diagonal, as one sequence cut into tiles
 // of 64 (the preamble is padded to a multiple of 16 in front of the own rows, so one tile may hold both); key tiles that the
-// fork-join mask excludes are never loaded or multiplied.  Per query tile and key tile:
+// fork-join mask excludes are never loaded or multiplied.  Short paths behind a preamble are cut into tiles without regard to where one
+// ends and the next begins (the rule and its figures: across_pays()): a tile's own keys then start with its first path, and
+// every row has a first own key too.  Per query tile and key tile:
 //   S = Q K^T     tcgen05.mma, A and B from TMA-staged 128B-swizzled shared memory, fp32 in tensor memory
 //   P = softmax   4 warps, one thread per query row, the row's 64 scores in registers: maximum, then exp2 with a lazily
 //                 updated reference maximum; P is rounded to bf16 and written over S
@@ -37,6 +39,8 @@
 // 128-512 rows 3208 -> 2580, 64 prompts x 17 paths behind a prefix of some 390 rows 3224 -> 2724, ALiBi 1366 -> 954; head_dim 64
 // (before: fp32 arithmetic) 9387 -> 172.  These launches run at the board's power limit (1.3 to 1.55 GHz): leaving out all
 // exponentials gains 2 %, so time follows the energy of the loads and products rather than any one pipe.
+#include <climits>
+
 #include "common.cuh"
 #include "prefill_plan.cuh"
 #include "tc_ptx.cuh"
@@ -137,6 +141,13 @@ __device__ __forceinline__ uint32_t low_bits(int n)
     return m;
 }
 
+// Which rows make up a tile.
+enum TileRows {
+    SEGMENT_ROWS,                     // of one segment and head
+    HEAD_ROWS,                        // of one segment and several heads of a KV head
+    ACROSS_ROWS                       // of consecutive paths of a prompt and one head
+};
+
 struct TcParams {
     CUtensorMap maps[3][3];           // [K, V, Q][box: a whole tile of a head's rows, 32 rows x 64 columns, 16 rows x 64 columns]
     const TcHeader *hdr;
@@ -151,17 +162,20 @@ struct TcParams {
     float scale_log2e;
     int wide_stores;                  // out is 32-byte aligned
     const float *pos, *slopes;        // ALiBi variant: token positions [T], head slopes [H]
+    const int32_t *path_start;        // ACROSS_ROWS
+    int n_paths;
     int stall_producer;               // test hook: the producers issue no load, so every wait runs out
 };
 
 // Every role walks the block's items in the same grid-stride order; heads vary fastest, so blocks running side by
 // side read neighbouring head slices of the same token rows.
 // Keys are numbered u = 0 .. : the preamble at [0, pre_len), own rows at [p16, ...), p16 = pre_len rounded up to 16.
-struct Walk {
+template <bool ACROSS> struct Walk {
     const TcPair *pairs;
     uint32_t pair, n_pairs, item_no;
     int h, n_units, dp, dh;           // h: unit of G heads
     TcPair t;
+    int first_path, lo_b;             // ACROSS: tile A's first path (-1: one segment), key number where tile B's first one starts
     __device__ __forceinline__ explicit Walk(const TcParams &p)
     {
         pairs = p.pairs; n_pairs = p.hdr->n_tiles; n_units = p.n_units; item_no = 0xffffffffu;
@@ -180,6 +194,11 @@ struct Walk {
         const int4 a = src[0], b = src[1];
         t.own_base = a.x; t.q_u = a.y; t.pre_row = a.z; t.pre_len = a.w;
         t.p16 = b.x; t.rows_ab = b.y; t.steps_a = b.z; t.steps = b.w;
+        if (ACROSS) {
+            first_path = b.x; lo_b = b.z;
+            t.p16 = (t.pre_len + 15) & ~15;
+            t.steps_a = (t.q_u + rows_a() + kBN - 1) / kBN;
+        }
         return true;
     }
     __device__ __forceinline__ int rows_a() const { return t.rows_ab & 0xffff; }
@@ -187,21 +206,28 @@ struct Walk {
     __device__ __forceinline__ int n_q() const { return rows_b() ? 2 : 1; }
     __device__ __forceinline__ int end() const { return t.q_u + rows_a() + rows_b(); }                  // keys of the item
     __device__ __forceinline__ int lane_a() const { return item_no & 1; }                               // tile A's lane
-    __device__ __forceinline__ bool used_by(int lane, int j) const { return lane == lane_a() ? j < t.steps_a : rows_b() > 0; }
-    __device__ __forceinline__ bool one_lane(int j) const { return rows_b() == 0 || j >= t.steps_a; }
+    // ACROSS: tile B has no use for key tiles behind the preamble and in front of its first path (there are more behind them)
+    __device__ __forceinline__ int gap_at() const { return (t.pre_len + kBN - 1) / kBN; }
+    __device__ __forceinline__ int gap() const { return ACROSS ? max(lo_b / kBN - gap_at(), 0) : 0; }
+    __device__ __forceinline__ bool in_gap(int j) const { return ACROSS && (uint32_t)(j - gap_at()) < (uint32_t)gap(); }
+    __device__ __forceinline__ bool used_by(int lane, int j) const { return lane == lane_a() ? j < t.steps_a : rows_b() > 0 && !in_gap(j); }
+    __device__ __forceinline__ bool one_lane(int j) const { return rows_b() == 0 || j >= t.steps_a || in_gap(j); }
 };
 
 // What a lane does in an item: tile A goes to lane item_no & 1, tile B (if any) to the other one.
 struct LaneTile {
     int b, q_u, rows, end, steps;     // b: it is tile B; q_u: key number of its first row; no steps: the lane has none
+    int gap_at, gap;                  // ACROSS: its steps without [gap_at, gap_at + gap)
     LaneTile() = default;
-    __device__ __forceinline__ LaneTile(const Walk &w, int lane)
+    template <bool ACROSS> __device__ __forceinline__ LaneTile(const Walk<ACROSS> &w, int lane)
     {
         b = (w.item_no & 1) ^ lane;
         rows = b ? w.rows_b() : w.rows_a();
         q_u = w.t.q_u + (b ? w.rows_a() : 0);
         end = q_u + rows;
         steps = b ? (rows ? w.t.steps : 0) : w.t.steps_a;
+        gap_at = w.gap_at();
+        gap = b ? w.gap() : 0;
     }
 };
 
@@ -216,20 +242,20 @@ template <int N> struct Ring {        // stage and parity of a ring of N barrier
     __device__ __forceinline__ void next() { skip(1); }
 };
 
-// One row (key number `last`, 64 columns; o: bf16 pairs) in fp32 arithmetic over exactly the keys it sees: its values that are not
-// finite are replaced.
-template <bool ALIBI>
-__device__ __forceinline__ void exact_row64(const TcParams &p, const TcPair &t, int head, int kv_head, int last, uint32_t (&o)[32])
+// One row (key number `last`, own keys from number `from` up; dst: where this thread has stored it) in fp32 arithmetic over exactly the
+// keys it sees: its values that are not finite are replaced.  Rare, so small: 16 bytes at a time.
+template <int D, bool ALIBI>
+__device__ __forceinline__ void exact_row(const TcParams &p, const TcPair &t, int head, int kv_head, int from, int last, unsigned char *dst)
 {
     const int64_t own = t.own_base + last;
-    const uint4 *q = reinterpret_cast<const uint4 *>(p.q + (own * p.n_heads + head) * 64);
+    const uint4 *q = reinterpret_cast<const uint4 *>(p.q + (own * p.n_heads + head) * D);
     const float pq = ALIBI ? p.pos[own] : 0.f, slope = ALIBI ? p.slopes[head] * kLog2eT : 0.f;
     auto packed_row = [&](int u) { return (int64_t)u + (u < t.pre_len ? t.pre_row : t.own_base); };
     auto score = [&](int64_t row) {
-        const uint4 *k = reinterpret_cast<const uint4 *>(p.k + (row * p.n_kv_heads + kv_head) * 64);
+        const uint4 *k = reinterpret_cast<const uint4 *>(p.k + (row * p.n_kv_heads + kv_head) * D);
         float s = 0.f;
 #pragma unroll 1
-        for (int c = 0; c < 8; ++c) {
+        for (int c = 0; c < D / 8; ++c) {
             const uint4 x = q[c], y = k[c];
             s = fmaf(bf16_lo(x.x), bf16_lo(y.x), s); s = fmaf(bf16_hi(x.x), bf16_hi(y.x), s);
             s = fmaf(bf16_lo(x.y), bf16_lo(y.y), s); s = fmaf(bf16_hi(x.y), bf16_hi(y.y), s);
@@ -242,41 +268,34 @@ __device__ __forceinline__ void exact_row64(const TcParams &p, const TcPair &t, 
     float m = -INFINITY, l = 0.f;
 #pragma unroll 1
     for (int u = 0; u <= last; ++u) {
-        if (u >= t.pre_len && u < t.p16) continue;
+        if (u >= t.pre_len && u < from) continue;
         const float s = score(packed_row(u));
         if (s > m) { l *= ex2(m - s); m = s; }
         l += ex2(s - m);
     }
     const float inv = 1.f / l;
-#pragma unroll
-    for (int part = 0; part < 4; ++part) {               // 16 columns at a time
-        float acc[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) acc[i] = 0.f;
+#pragma unroll 1
+    for (int c = 0; c < D / 8; ++c) {
+        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
         for (int u = 0; u <= last; ++u) {
-            if (u >= t.pre_len && u < t.p16) continue;
+            if (u >= t.pre_len && u < from) continue;
             const int64_t row = packed_row(u);
             const float w = ex2(score(row) - m);
-            const uint4 *v = reinterpret_cast<const uint4 *>(p.v + (row * p.n_kv_heads + kv_head) * 64) + 2 * part;
+            float v[8];
+            Vec<__nv_bfloat16>::load(p.v + (row * p.n_kv_heads + kv_head) * D + c * 8, v);
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const uint4 y = v[c];
-                const uint32_t wd[4] = {y.x, y.y, y.z, y.w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    acc[8 * c + 2 * e] = fmaf(w, bf16_lo(wd[e]), acc[8 * c + 2 * e]);
-                    acc[8 * c + 2 * e + 1] = fmaf(w, bf16_hi(wd[e]), acc[8 * c + 2 * e + 1]);
-                }
-            }
+            for (int e = 0; e < 8; ++e) acc[e] = fmaf(w, v[e], acc[e]);
         }
+        uint4 *at = reinterpret_cast<uint4 *>(dst) + c, o = *at;
+        uint32_t *y = reinterpret_cast<uint32_t *>(&o);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {                    // the finite ones are right as they are
+        for (int i = 0; i < 4; ++i) {                    // the finite ones are right as they are
             const uint32_t x = pack_bf16x2(acc[2 * i] * inv, acc[2 * i + 1] * inv);
-            uint32_t &y = o[8 * part + i];
-            if ((y & 0x7f80u) == 0x7f80u) y = (y & 0xffff0000u) | (x & 0xffffu);
-            if ((y & 0x7f800000u) == 0x7f800000u) y = (y & 0xffffu) | (x & 0xffff0000u);
+            if ((y[i] & 0x7f80u) == 0x7f80u) y[i] = (y[i] & 0xffff0000u) | (x & 0xffffu);
+            if ((y[i] & 0x7f800000u) == 0x7f800000u) y[i] = (y[i] & 0xffffu) | (x & 0xffff0000u);
         }
+        *at = o;
     }
 }
 
@@ -287,11 +306,13 @@ template <int N> __device__ __forceinline__ void reg_dealloc() { asm volatile("s
 // for ALiBi).
 // GROUPED: tiles of several heads.  A kernel of its own: the index arithmetic costs a launch of single heads 1.5 % (32 query rows of
 // 800 paths, 621 against 630 us).
-template <int D, bool ALIBI, bool GROUPED, bool SPLIT>
+template <int D, bool ALIBI, TileRows ROWS, bool SPLIT>
 __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_constant__ TcParams p)
 {
+    constexpr bool ACROSS = ROWS == ACROSS_ROWS;
     using C = TcConfig<D, ALIBI, SPLIT>;
-    const int log_rows = GROUPED ? p.log_rows : 7;
+    using Walk = Walk<ACROSS>;
+    const int log_rows = ROWS == HEAD_ROWS ? p.log_rows : 7;
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char *sQ = smem, *sK = smem + C::NQ * C::Q_BYTES, *sV = sK + C::NKV * C::KV_BYTES;
     float *x_l = reinterpret_cast<float *>(smem + C::X_OFF);                            // [lane][row] row sums
@@ -517,6 +538,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                 pending |= info << (16 * (g_s - g_o));
                 ++j; ++g_s;
                 k.next();
+                if (ACROSS && j == t.gap_at) { j += t.gap; k.skip(t.gap); }
             }
             if (!ok) {
                 // a wait ran out: every MMA of this lane must finish (bounded) before its tensor memory is freed
@@ -582,13 +604,38 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
             // counted from the key tile's first key: the first one this row may not see, the padding behind the preamble
             int lim = min(t.q_u + hr + 1, t.end), g0 = w.t.pre_len, g1 = w.t.p16;
             int see = live_w ? min(t.q_u + hr1, t.end) : 0;      // keys some row of the warp may see
+            // ACROSS: path starts from tile A's on, a lane each; looked at where the first own keys come (g0 < kBN), by when they are here
+            const int row_w = w.t.own_base + t.q_u + hr0, start_a = w.t.own_base + w.t.p16;
+            int see_from = 0, start = INT_MAX;
+            if (ACROSS && t.steps && w.first_path >= 0 && w.first_path + lane < p.n_paths) start = p.path_start[w.first_path + lane];
+            bool look = ACROSS && w.first_path >= 0;
 #pragma unroll 1
             for (int j = 0; j < t.steps; ++j, ++g, lim -= kBN, g0 -= kBN, g1 -= kBN, see -= kBN) {
+                if (ACROSS && look && g0 < kBN) {
+                    // the path of the warp's first row, and a bit for each of its rows that is the first of another one
+                    look = false;
+                    int before = start_a;
+                    uint32_t firsts = 0;
+                    for (int base = w.first_path + lane;; ) {
+                        // a row of another prompt's path is none of the item's: those lie in front of its first row or behind its last
+                        const uint32_t at = (uint32_t)(start - row_w);
+                        before = max(before, start <= row_w ? start : INT_MIN);
+                        if (at - 1u < 31u) firsts |= 1u << at;
+                        if (!__shfl_sync(0xffffffffu, start >= start_a && start < row_w + 32, 31)) break;
+                        base += 32;
+                        start = base < p.n_paths ? p.path_start[base] : INT_MAX;
+                    }
+                    before = __reduce_max_sync(0xffffffffu, before);
+                    firsts = __reduce_or_sync(0xffffffffu, firsts) & low_bits(lane + 1);
+                    const int passed = j * kBN + w.t.own_base;
+                    g1 = (firsts ? row_w + 31 - __clz(firsts) : before) - passed;
+                    see_from = before - w.t.own_base;
+                }
                 const uint32_t buf = g & 1, s_addr = s_base + buf * kBN;
                 if (!(ok = mbar_wait_warp(own_buf + C::BAR_S_FULL + buf, g >> 1 & 1))) break;
                 if (ALIBI && !(ok = mbar_wait_warp(&bars[C::BAR_POS + ln * C::NKV + v.i], pos_ph >> v.i & 1))) break;
                 tc_fence_after();
-                if (see > 0) {
+                if (see > 0 && !(ACROSS && g0 <= 0 && see_from - j * kBN >= kBN)) {
                     uint32_t r[2][32];
                     tmem_ld32(s_addr, r[0]);
                     tmem_ld32(s_addr + 32, r[1]);
@@ -675,6 +722,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                 __syncwarp();
                 if (lane == 0) mbar_arrive(own_buf + C::BAR_P + buf);
                 if (ALIBI) { pos_ph ^= 1u << v.i; v.next(); }
+                if (ACROSS && j + 1 == t.gap_at) {
+                    j += t.gap; lim -= t.gap * kBN; g0 -= t.gap * kBN; g1 -= t.gap * kBN; see -= t.gap * kBN;
+                    if (ALIBI) v.skip(t.gap);
+                }
             }
             if (!ok) break;
             if (ALIBI) v.skip(w.t.steps - t.steps);
@@ -705,7 +756,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                 const float inv = __fdividef(1.f, x_l[ln * kBM + row]);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&bars[C::BAR_X_FREE + ln]);
-                const uint32_t g_last = (ln ? g[1] : g[0]) + t.steps - 1;
+                const uint32_t g_last = (ln ? g[1] : g[0]) + t.steps - t.gap - 1;
                 if (ln) g[1] = g_last + 1; else g[0] = g_last + 1;
                 if (!(ok = mbar_wait_warp(&bars[C::BAR_O_DONE + 2 * ln + (g_last & 1)], g_last >> 1 & 1))) break;      // last O += P V
                 ph ^= 1u << ln;
@@ -714,6 +765,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                 const uint64_t inv2 = pack_f32x2(inv, inv);
                 unsigned char *dst = reinterpret_cast<unsigned char *>(p.out) +
                                      ((int64_t)(w.t.own_base + t.q_u + hr) * p.n_heads + (w.h << (7 - log_rows)) + (row >> log_rows)) * (D * 2);
+                uint32_t nan = 0u;
 #pragma unroll 1
                 for (int cc = 0; cc < C::HALVES; ++cc) {       // 64 columns
                     uint32_t o[32];
@@ -735,16 +787,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&bars[C::BAR_O_FREE + ln]);
                     }
-                    if (C::EXACT && hr < t.rows) {
-                        // Hidden keys have a P of exactly zero, but 0 x Inf and 0 x NaN reach O: a row with a value that is not
-                        // finite is computed again over its own keys, as the fp32 kernel that served head_dim 64 before would
-                        // have.  The look at the row costs nothing that shows; looking through the V tiles instead cost the
-                        // ALiBi variant 14 % (one more warp on the SM partition of two softmax warps).
-                        uint32_t nan = 0u;
+                    if (C::EXACT || ACROSS) {
 #pragma unroll
                         for (int i = 0; i < 32; ++i) asm("fma.rn.bf16x2 %0, %1, %2, %0;" : "+r"(nan) : "r"(o[i]), "r"(0u));
-                        if (nan & 0x7fff7fffu)
-                            exact_row64<ALIBI>(p, w.t, (w.h << (7 - log_rows)) + (row >> log_rows), w.h / p.units_per_kv, t.q_u + hr, o);
                     }
                     if (hr < t.rows) {
                         if (p.wide_stores) {
@@ -756,6 +801,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                                 __stcs(reinterpret_cast<uint4 *>(dst + cc * 128) + i, make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]));
                         }
                     }
+                }
+                // Hidden keys have a P of exactly zero, but 0 x Inf and 0 x NaN reach O: with head_dim 64 (as precise as fp32 arithmetic) and
+                // where a tile holds keys of paths that a row does not see, a row with a value that is not finite is computed again over
+                // its own keys.  The look at the row costs nothing that shows; looking through the V tiles instead cost the ALiBi variant
+                // 14 % (one more warp on the SM partition of two softmax warps).
+                if ((C::EXACT || ACROSS) && hr < t.rows && (nan & 0x7fff7fffu)) {
+                    int start = w.t.own_base + w.t.p16;                    // of the row's own path
+                    const int row_p = w.t.own_base + t.q_u + hr;
+                    if (ACROSS && w.first_path >= 0)
+                        for (int i = w.first_path + 1; i < p.n_paths && p.path_start[i] > start && p.path_start[i] <= row_p; ++i) start = p.path_start[i];
+                    exact_row<D, ALIBI>(p, w.t, (w.h << (7 - log_rows)) + (row >> log_rows), w.h / p.units_per_kv, start - w.t.own_base, t.q_u + hr, dst);
                 }
             }
         }
@@ -862,11 +918,52 @@ size_t prefill_tc_workspace_bytes(int n_prompts, int n_paths, int max_pre_len, i
     return 256 + round_up((size_t)plan_max_tiles(n_prompts, n_paths, max_pre_len, max_path_len, 32) * sizeof(TcPair), 256);
 }
 
-template <int D, bool ALIBI, bool GROUPED, bool SPLIT> static int launch_kernel(const TcParams &p, int grid, cudaStream_t st)
+template <int D, bool ALIBI, TileRows ROWS, bool SPLIT> static int launch_kernel(const TcParams &p, int grid, cudaStream_t st)
 {
     using C = TcConfig<D, ALIBI, SPLIT>;
-    SP_CUDA(cudaFuncSetAttribute(prefill_tc_kernel<D, ALIBI, GROUPED, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-    return launch(prefill_tc_kernel<D, ALIBI, GROUPED, SPLIT>, grid, kTcThreads, C::SMEM, st, 1, p);
+    SP_CUDA(cudaFuncSetAttribute(prefill_tc_kernel<D, ALIBI, ROWS, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
+    return launch(prefill_tc_kernel<D, ALIBI, ROWS, SPLIT>, grid, kTcThreads, C::SMEM, st, 1, p);
+}
+
+// Tiles over the rows of consecutive paths (one head to a tile): full ones, and the preamble's keys loaded and multiplied once per pair of
+// tiles instead of once per path, but every tile also meets the keys of all of its paths.  Both ways are counted from the host
+// mirror: key tiles of all query tiles, in the share that the busiest block gets.  A key tile takes up to a tenth longer across (two
+// lanes that agree less about which keys they need), and with less than three items to a block one block's items are a chain too
+// long.  us segment by segment / across, 32 heads of 128, 20 documents to a prompt, about 120 000 rows (key tiles across in
+// proportion): documents of 8-24 rows behind 64 1495 / 716 (0.37), behind 400 3359 / 1191 (0.28); 32-64 behind 64 758 / 691 (0.85),
+// behind 16 645 / 652 (0.99); 60-180 behind 400 1625 / 1375 (0.84), behind 64 715 / 749 (0.97); 64-256 behind 400 1497 / 1436
+// (0.89); 128-512 behind 64 901 / 970 (1.05); ALiBi 60-180 behind 400 2118 / 1855; head_dim 64 1439 / 1231.  One prompt of 20
+// documents of 32-64 rows behind 128 (0.74, one item to a block): 19.6 / 22.8.
+static bool across_pays(const sp_layout *lay, int n_units)
+{
+    const sp_layout_host *m = lay->host_mirror;
+    if (!m) return false;
+    int64_t alone = 0, across = 0, items_alone = 0, items_across = 0;      // key tiles of all query tiles; pairs of them
+    for (int b = 0; b < lay->n_prompts; ++b) {
+        const int i0 = m->prompt_path_off[b], i1 = m->prompt_path_off[b + 1], p16 = (m->pre_len[b] + 15) & ~15;
+        if (i0 == i1) continue;
+        if (m->pre_len[b] == 0) return false;            // every row has to see the first key tile
+        int run = 0;
+        for (int i = i0; i < i1; ++i) {
+            const int n = m->doc_len[i] + m->qry_len[i], h = even_height(n, kBM);
+            if (n == 0 || m->path_start[i] != m->path_start[i0] + run) return false;
+            run += n;
+            for (int r = h; r < n + h; r += h) alone += (p16 + std::min(r, n) + kBN - 1) / kBN;
+            items_alone += (n + 2 * h - 1) / (2 * h);
+        }
+        const int h = even_height(run, kBM), gap_at = (m->pre_len[b] + kBN - 1) / kBN;
+        for (int r = 0, i = i0, start = 0, start_a = 0; r < run; r += h) {
+            for (int n; start + (n = m->doc_len[i] + m->qry_len[i]) <= r; ++i) start += n;
+            const bool is_b = r / h & 1;
+            if (!is_b) { start_a = start; ++items_across; }
+            const int end = p16 + std::min(r + h, run) - start_a;
+            across += (end + kBN - 1) / kBN - (is_b ? std::max((p16 + start - start_a) / kBN - gap_at, 0) : 0);
+        }
+    }
+    if (items_across * n_units < 3 * (int64_t)num_sms()) return false;
+    // what the busiest block gets, at the mean number of key tiles
+    const auto busiest = [&](int64_t steps, int64_t items) { return (double)((items * n_units + num_sms() - 1) / num_sms()) * steps / items; };
+    return busiest(across, items_across) < 0.9 * busiest(alone, items_alone);
 }
 
 static int launch_tc(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
@@ -906,6 +1003,8 @@ static int launch_tc(const void *q, const void *k, const void *v, const sp_layou
     pa.max_tiles = plan_max_tiles(lay->n_prompts, lay->n_paths, lay->max_pre_len, lay->max_path_len, 2 * pa.tile_rows);
     // the sort takes a microsecond: worth it from a dozen items per block
     pa.sort_from = 12 * num_sms() / (n_heads >> log_g);
+    // (not with the rotation folded in: Q is then where the output goes, and a row that has to be computed again would not find it)
+    pa.across = log_g == 0 && rows == SP_ROWS_ALL && !rope && across_pays(lay, n_heads);
     pa.hdr = hdr; pa.list = pairs;
     if (int rc = launch(prefill_plan_kernel<true>, 1, 1024, 0, st, 1, pa)) return rc;
     if (pa.max_tiles == 0) return SP_OK;              // no segment can have a row
@@ -924,20 +1023,21 @@ static int launch_tc(const void *q, const void *k, const void *v, const sp_layou
     p.total_tokens = lay->total_tokens; p.scale_log2e = scale * kLog2eT;
     p.wide_stores = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
     p.pos = pos; p.slopes = slopes;
+    p.path_start = lay->path_start; p.n_paths = lay->n_paths;
     p.stall_producer = g_stall_producer ? 1 : 0;      // test hook, see sp_test_stall_producer below
 
     const int64_t items = pa.max_tiles * p.n_units;
     const int grid = (int)std::min<int64_t>(items, num_sms());
     using Launch = int (*)(const TcParams &, int, cudaStream_t);
-    const auto run = [&](Launch single, Launch grouped) { return (log_g ? grouped : single)(p, grid, st); };
+    const auto run = [&](Launch segment, Launch heads, Launch across) { return (pa.across ? across : (log_g ? heads : segment))(p, grid, st); };
     if (head_dim == 64)
-        return pos ? run(launch_kernel<64, true, false, true>, launch_kernel<64, true, true, true>)
-                   : run(launch_kernel<64, false, false, true>, launch_kernel<64, false, true, true>);
+        return pos ? run(launch_kernel<64, true, SEGMENT_ROWS, true>, launch_kernel<64, true, HEAD_ROWS, true>, launch_kernel<64, true, ACROSS_ROWS, true>)
+                   : run(launch_kernel<64, false, SEGMENT_ROWS, true>, launch_kernel<64, false, HEAD_ROWS, true>, launch_kernel<64, false, ACROSS_ROWS, true>);
     if (rows == SP_ROWS_QUERY_ONLY)               // P as two bf16 numbers, see TcConfig
-        return pos ? run(launch_kernel<128, true, false, true>, launch_kernel<128, true, true, true>)
-                   : run(launch_kernel<128, false, false, true>, launch_kernel<128, false, true, true>);
-    return pos ? run(launch_kernel<128, true, false, false>, launch_kernel<128, true, true, false>)
-               : run(launch_kernel<128, false, false, false>, launch_kernel<128, false, true, false>);
+        return pos ? run(launch_kernel<128, true, SEGMENT_ROWS, true>, launch_kernel<128, true, HEAD_ROWS, true>, nullptr)
+                   : run(launch_kernel<128, false, SEGMENT_ROWS, true>, launch_kernel<128, false, HEAD_ROWS, true>, nullptr);
+    return pos ? run(launch_kernel<128, true, SEGMENT_ROWS, false>, launch_kernel<128, true, HEAD_ROWS, false>, launch_kernel<128, true, ACROSS_ROWS, false>)
+               : run(launch_kernel<128, false, SEGMENT_ROWS, false>, launch_kernel<128, false, HEAD_ROWS, false>, launch_kernel<128, false, ACROSS_ROWS, false>);
 }
 
 int launch_prefill_tc(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,

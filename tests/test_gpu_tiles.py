@@ -263,3 +263,95 @@ def test_rope_tokens_per_block(dtype, H, D, waves, more):
     assert np.isfinite(got).all()
     bound = 4e-6 if dtype == torch.float32 else np.abs(ref) * 2.0 ** -8 * 1.02 + 1e-6
     assert (np.abs(got[at] - ref) <= bound).all()
+
+
+def _short_paths(pre, n_prompts, n, longest, seed=5):
+    """Prompts of many short paths behind a preamble, with paths that fill warps, tiles and pairs of tiles among them."""
+    rng = np.random.default_rng(seed)
+    docs = [[int(x) for x in rng.integers(0, longest, n)] for _ in range(n_prompts)]
+    qry = [[int(x) for x in rng.integers(1, 9, n)] for _ in range(n_prompts)]
+    for b, edge in enumerate((31, 32, 33, 127, 128, 129, 255, 256, 257)):
+        docs[b % n_prompts][b % n], qry[b % n_prompts][b % n] = edge - 1, 1
+    return build_layout([pre] * n_prompts, docs, qry)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("alibi", [False, True])
+@pytest.mark.parametrize("pre,n_prompts,n,longest", [(1, 4, 300, 8), (16, 4, 90, 24), (63, 6, 50, 40), (64, 6, 50, 40), (65, 6, 50, 40),
+                                                     (200, 5, 30, 90), (40, 2, 1030, 3)])
+def test_prefill_tiles_across_paths(D, alibi, pre, n_prompts, n, longest):
+    """Tiles over the rows of consecutive paths: path starts at every row of a warp, more of them than lanes in a tile, preambles
+    around the key tile, a last pair that is not full, more paths than the plan has threads; and bit-identical repeats."""
+    _prefill(_short_paths(pre, n_prompts, n, longest), 20, 20, D, alibi=alibi, repeats=1)
+
+
+@pytest.mark.parametrize("how", ["prompts in reverse", "gaps", "an empty path", "no preamble", "paths swapped on the device"])
+def test_prefill_tiles_across_paths_conditions(how):
+    """What tiles over consecutive paths rest on: other places of the prompts keep it; paths that do not follow each other, one
+    without rows, a prompt without a preamble, or device arrays unlike the mirror go segment by segment."""
+    import copy
+    lay = _short_paths(0 if how == "no preamble" else 40, 4, 90, 24)
+    H, D, T = 20, 64, lay.total_tokens
+    seen = copy.deepcopy(lay)                                     # what the device arrays say
+    if how == "prompts in reverse":
+        spans = [lay.prompt_row_range(b) for b in range(4)]
+        at = 0
+        for b in (3, 2, 1, 0):
+            move, paths = at - spans[b][0], slice(lay.prompt_path_off[b], lay.prompt_path_off[b + 1])
+            seen.pre_start[b] += move
+            seen.path_start[paths] += move
+            at += spans[b][1] - spans[b][0]
+        lay = seen
+    elif how == "gaps":
+        seen.path_start = (lay.path_start + 3 * np.arange(lay.n_paths)).astype(np.int32)
+        seen.pre_start = (lay.pre_start + 3 * lay.prompt_path_off[:-1]).astype(np.int32)
+        T = seen.total_tokens = lay.total_tokens + 3 * lay.n_paths
+        lay = seen
+    elif how == "an empty path":
+        lay.doc_len[17] = lay.qry_len[17] = 0
+        seen = lay
+    elif how == "paths swapped on the device":
+        seen.path_start[100], seen.path_start[101] = lay.path_start[100], lay.path_start[100]
+        seen.path_start[100] += int(lay.doc_len[101] + lay.qry_len[101])
+    q, k, v = (_randn((T, H, D), i) for i in (1, 2, 3))
+    ref, _ = oracle.prefill(f32(q), f32(k), f32(v), seen, 0.125)
+    dl = sp.DeviceLayout.from_host(lay)
+    dl.arrays[3].copy_(torch.from_numpy(seen.path_start))
+    out, ws = torch.zeros((T, H, D), dtype=torch.bfloat16, device="cuda"), workspace(sp.sp_prefill_workspace_bytes(dl, H, D, sp.SP_BF16))
+    sp.sp_superpose_prefill(dev(q), dev(k), dev(v), dl, 0.125, out, None, ws)
+    sp.sp_check_status(ws)
+    rows = np.concatenate([np.arange(s, s + n) for s, n in zip(np.concatenate([seen.pre_start, seen.path_start]),
+                                                               np.concatenate([seen.pre_len, seen.doc_len + seen.qry_len]))])
+    assert rel_l2(f32(out)[rows], ref[rows]) <= TOL[torch.bfloat16]
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("alibi", [False, True])
+def test_prefill_tiles_across_paths_keep_values_to_their_path(D, alibi):
+    """NaN and Inf in one path's K and V: every other row is as it was, up to the fp32 arithmetic that computes it again where the
+    value shares a tile with it (two roundings of a bf16 result, one of them of P: 2^-7 of the largest value)."""
+    lay = _short_paths(40, 4, 90, 24)
+    H, T = 20, lay.total_tokens
+    q, k, v = (_randn((T, H, D), i) for i in (1, 2, 3))
+    pos, slopes = torch.rand(T, generator=torch.Generator().manual_seed(4)).mul(300).float(), torch.linspace(0.01, 0.5, H)
+    dl = sp.DeviceLayout.from_host(lay)
+    ws = workspace(sp.sp_prefill_workspace_bytes(dl, H, D, sp.SP_BF16))
+
+    def run(k, v):
+        out, lse = torch.zeros((T, H, D), dtype=torch.bfloat16, device="cuda"), torch.zeros((H, T), device="cuda")
+        if alibi:
+            sp.sp_superpose_prefill_alibi(dev(q), dev(k), dev(v), dl, dev(pos), dev(slopes), D ** -0.5, out, lse, ws)
+        else:
+            sp.sp_superpose_prefill(dev(q), dev(k), dev(v), dl, D ** -0.5, out, lse, ws)
+        sp.sp_check_status(ws)
+        return f32(out), lse.cpu().numpy()
+
+    out0, lse0 = run(k, v)
+    k2, v2, others = k.clone(), v.clone(), np.ones(T, bool)
+    for i in (5, 120, 200, 355):
+        r = slice(int(lay.path_start[i]), int(lay.path_start[i] + lay.doc_len[i] + lay.qry_len[i]))
+        k2[r], v2[r], others[r] = float("inf"), float("nan"), False
+        v2[r][::2] = float("-inf")
+    out1, lse1 = run(k2, v2)
+    np.testing.assert_array_equal(lse0[:, others], lse1[:, others])
+    assert np.abs(out0[others] - out1[others]).max() <= 2 ** -7 * np.abs(out0).max()
