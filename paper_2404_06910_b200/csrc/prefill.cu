@@ -17,8 +17,8 @@ int launch_prefill_tc_rope(const void *q, const void *k, const void *v, const sp
                            cudaStream_t st);
 size_t prefill_qonly_workspace_bytes(int n_prompts, int n_paths, int max_pre_len, int max_path_len);
 int launch_prefill_qonly(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
-                         const float *slopes, int n_heads, int n_kv_heads, float scale, void *out, float *lse,
-                         void *ws, cudaStream_t st);
+                         const float *slopes, int n_heads, int n_kv_heads, float scale, int longest, bool split, void *out,
+                         float *lse, void *ws, cudaStream_t st);
 }  // namespace sp
 
 extern "C" size_t sp_prefill_workspace_bytes(int n_prompts, int n_paths, int max_pre_len,
@@ -31,27 +31,31 @@ extern "C" size_t sp_prefill_workspace_bytes(int n_prompts, int n_paths, int max
 }
 
 namespace sp {
-// Query rows only, head_dim 128: which of two kernels.  The tcgen05 kernel has a quarter of its tile's rows at work (32 of 128) and
-// carries P as two bf16 numbers; the warp-level kernel (prefill_qonly.cu) works on 32 rows at a time.
-//  - An even number of query heads to a KV head: tcgen05, whose tiles then hold the rows of several heads.  us, tcgen05 /
-//    warp-level, 4 x 20 documents behind 1 200 rows: 193 / 302 (two heads), 114 / 303 (four); ALiBi 257 / 347, 155 / 343.
-//  - Few items (a path's query rows and a head each): tcgen05; the warp-level kernel has too few warps to hide its latency.  1
-//    prompt x 20 documents of 64-256 rows, 32 heads: 23.3 / 24.1 behind 32 rows, 43.4 / 52.6 behind 384; 2 prompts: 47 / 54
-//    behind 128, 175 / 181 behind 1 200; ALiBi 61 / 66 behind 128, 83 / 83 behind 256, 110 / 105 behind 400.
-//  - More than 32 query rows in a path: tcgen05; the warp-level kernel reads every key again for each 32 rows.  48 rows, 8 x 100
-//    documents: 666 / 1216 behind 48 rows, 1825 / 3114 behind 600.
-//  - Otherwise warp-level: 8 x 100 documents, back to back: 622 / 600 behind 16 rows, 689 / 655 behind 48, 839 / 769 behind 128,
-//    1430 / 1202 behind 384; ALiBi 722 / 696 behind 16, 841 / 758 behind 64.
-// The number of query rows is known from the host mirror only; without one tcgen05 up to the preamble behind which it loses
-// less than the warp-level kernel does with 33 rows and more.
-static bool query_rows_warp_level(const sp_layout *lay, bool alibi, int n_heads, int n_kv_heads)
+// Query rows only, head_dim 128: which of two kernels, and how P is carried in the one made for them (prefill_qonly.cu).
+//  - An even number of query heads to a KV head: the kernel for all rows, whose tiles then hold the rows of several heads and load
+//    K and V once for them.  us, that / prefill_qonly.cu, 32 rows of 8 x 100 documents behind 48 rows: 336 / 387 (two heads), 200 /
+//    365 (four).
+//  - More than 48 query rows in a path, which are two items there: the kernel for all rows.  64 rows 704 / 998, behind 400 rows 1521 / 2001.
+//  - Otherwise prefill_qonly.cu.  8 x 100 documents, against what served them before (the tcgen05 kernel for few items and for more
+//    than 32 rows, a warp-level one): 32 rows behind 48 610 / 470, behind 384 1162 / 724, behind 1 200 (4 x 100) 1334 / 860; 8 rows 549 / 416;
+//    48 rows 734 / 553, behind 600 2270 / 1290; ALiBi 32 rows 762 / 480, 48 rows 792 / 718; 1 prompt x 20 documents 22.0 / 17.4.
+// The number of query rows is known from the host mirror only; without one the kernel for all rows, but for many items behind a preamble
+// from which on it loses more than the other one does with more than 48 rows.
+// P as two bf16 numbers, but with many items (path, head) of a few key tiles: there it is one number except for an item's first 32
+// keys, which is as exact as what served them before (2.09e-3 of the norm from 64-bit results at 8 x 100 documents behind 48 rows, 2.13e-3
+// before; two numbers 1.66e-3) and 0 to 3 % faster (documents of 32-64 rows 100.5 / 104.0 us, ALiBi 476 / 480).  With more key tiles
+// the running maximum it needs costs more than the second number (behind 384 rows 836 / 721).
+static int qonly_rows(const sp_layout *lay, bool alibi, int n_heads, int n_kv_heads)      // 0: the kernel for all rows
 {
-    if (n_heads / n_kv_heads % 2 == 0) return false;
-    if ((int64_t)lay->n_paths * n_heads <= 9 * (int64_t)num_sms() && (!alibi || lay->max_pre_len <= 256)) return false;
-    if (!lay->host_mirror) return lay->max_pre_len > (alibi ? 64 : 384);
-    int longest = 0;
+    if (n_heads / n_kv_heads % 2 == 0) return 0;
+    if (!lay->host_mirror) return (int64_t)lay->n_paths * n_heads > 9 * (int64_t)num_sms() && lay->max_pre_len > (alibi ? 64 : 384) ? 48 : 0;
+    int longest = 1;
     for (int i = 0; i < lay->n_paths; ++i) longest = std::max(longest, lay->host_mirror->qry_len[i]);
-    return longest <= 32;
+    return longest <= 48 ? longest : 0;
+}
+static bool qonly_split(const sp_layout *lay, int n_heads)
+{
+    return (int64_t)lay->n_paths * n_heads <= 9 * (int64_t)num_sms() || lay->max_pre_len > 128 || (int64_t)lay->max_pre_len + lay->max_path_len > 640;
 }
 
 static int prefill_entry(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
@@ -77,8 +81,9 @@ static int prefill_entry(const void *q, const void *k, const void *v, const sp_l
                "sp_superpose_prefill: workspace of %zu bytes (256-byte aligned) required", need);
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (dtype == SP_BF16 && head_dim == 128 && rows == SP_ROWS_QUERY_ONLY && query_rows_warp_level(lay, pos != nullptr, n_heads, n_kv_heads))
-        return launch_prefill_qonly(q, k, v, lay, pos, slopes, n_heads, n_kv_heads, scale, out, lse, ws, st);
+    if (dtype == SP_BF16 && head_dim == 128 && rows == SP_ROWS_QUERY_ONLY)
+        if (const int longest = qonly_rows(lay, pos != nullptr, n_heads, n_kv_heads))
+            return launch_prefill_qonly(q, k, v, lay, pos, slopes, n_heads, n_kv_heads, scale, longest, qonly_split(lay, n_heads), out, lse, ws, st);
     // bf16 goes to the tensor cores for both head sizes (head_dim 64, 8 prompts x 20 documents, 32 heads: 0.17 ms; the fp32
     // SIMT kernel, which served it before, took 9.4 ms)
     if (dtype == SP_BF16)

@@ -44,6 +44,7 @@
 #include "common.cuh"
 #include "prefill_plan.cuh"
 #include "tc_ptx.cuh"
+#include "tensor_map.cuh"
 
 namespace sp {
 
@@ -62,9 +63,8 @@ enum { WARP_EPI = 8, WARP_K = 12, WARP_V, WARP_Q, WARP_POS, WARP_MMA, WARP_PASS 
 
 // SPLIT_P: P is carried as the sum of two bf16 numbers (16 bits of mantissa) and the second product runs twice.  Set for
 // head_dim 64, which is then as precise as fp32 arithmetic, and for query rows only: relative to the maximum over a first
-// key tile, P in one bf16 number is less exact there (2.27e-3 of the norm from 64-bit results, 8 prompts x 100 documents)
-// than relative to the running maximum of prefill_qonly.cu (2.13e-3); as two it is 1.66e-3, the rounding of the output.  Cost
-// there: 8 prompts x 100 documents, two heads to a KV head, 326 -> 341 us; four, 197 -> 217.
+// key tile, P in one bf16 number is 2.27e-3 of the norm from 64-bit results there (8 prompts x 100 documents), as two it is
+// 1.66e-3, the rounding of the output.  Cost: 8 prompts x 100 documents, two heads to a KV head, 326 -> 341 us; four, 197 -> 217.
 template <int D, bool ALIBI, bool SPLIT> struct TcConfig {
     static constexpr bool SPLIT_P = SPLIT, EXACT = D == 64;
     static constexpr int HALVES = D / 64;                       // 64-column halves of a row (one 128-byte swizzle atom each)
@@ -100,31 +100,6 @@ __device__ __forceinline__ float fmax3(float a, float b, float c)
 {
     float d;
     asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi)
-{
-    uint64_t d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
-    return d;
-}
-__device__ __forceinline__ void unpack_f32x2(uint64_t v, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c)
-{
-    uint64_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("add.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("mul.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
 __device__ __forceinline__ float ex2(float x)
@@ -889,27 +864,7 @@ __global__ void __launch_bounds__(256, 8) rope_rows_kernel(const __grid_constant
 // tile, every bounded wait expires, the blocks unwind and the call reports SP_ERR_TIMEOUT
 // through the workspace status word.  Set only through sp_test_stall_producer(), a symbol for
 // the test suite that the public header does not declare.
-static bool g_stall_producer = false;
-
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static int encode_rows_map(EncodeTiledFn enc, CUtensorMap *m, const void *base, int64_t rows, int64_t cols, int box_rows, int halves)
-{
-    // [rows, cols] bf16 row-major seen as 3-D (64 columns, rows, cols / 64): a box of box_rows rows and one or all
-    // 64-column halves of a head lands as [half][row][64 columns] with the 128-byte swizzle, the layout the MMA
-    // descriptors expect.
-    cuuint64_t dims[3] = {64, (cuuint64_t)rows, (cuuint64_t)(cols / 64)};
-    cuuint64_t strides[2] = {(cuuint64_t)cols * 2, 128};
-    cuuint32_t box[3] = {64, (cuuint32_t)box_rows, (cuuint32_t)halves};
-    cuuint32_t estr[3] = {1, 1, 1};
-    const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, estr,
-                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    SP_REQUIRE(r == CUDA_SUCCESS, SP_ERR_CUDA, "cuTensorMapEncodeTiled failed with code %d", (int)r);
-    return SP_OK;
-}
+bool g_stall_producer = false;
 
 size_t prefill_tc_workspace_bytes(int n_prompts, int n_paths, int max_pre_len, int max_path_len, int)
 {
@@ -970,22 +925,13 @@ static int launch_tc(const void *q, const void *k, const void *v, const sp_layou
                      const float *slopes, const RopeRows *rope, int n_heads, int n_kv_heads, int head_dim,
                      float scale, int rows, void *out, float *lse, void *ws, cudaStream_t st)
 {
-    static EncodeTiledFn enc = nullptr;
-    if (!enc) {
-        void *fn = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        SP_CUDA(cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres));
-        SP_REQUIRE(fn != nullptr && qres == cudaDriverEntryPointSuccess, SP_ERR_CUDA,
-                   "cuTensorMapEncodeTiled is not available from this driver");
-        enc = reinterpret_cast<EncodeTiledFn>(fn);
-    }
     TcParams p;
     const int halves = head_dim / 64;
     const int64_t q_cols = (int64_t)n_heads * head_dim, kv_cols = (int64_t)n_kv_heads * head_dim;
     const struct { const void *base; int64_t cols; } src[3] = {{k, kv_cols}, {v, kv_cols}, {q, q_cols}};
     for (int i = 0; i < 3; ++i)
         for (int b = 0; b < 3; ++b)
-            if (int rc = encode_rows_map(enc, &p.maps[i][b], src[i].base, lay->total_tokens, src[i].cols,
+            if (int rc = encode_rows_map(&p.maps[i][b], src[i].base, lay->total_tokens, src[i].cols,
                                          b == 0 ? (i == 2 ? kBM : kBN) : (b == 1 ? 32 : 16), b == 0 ? halves : 1)) return rc;
 
     TcHeader *hdr = static_cast<TcHeader *>(ws);

@@ -45,3 +45,32 @@ def test_prefill_bounded_waits_report_timeout_and_context_survives():
     sp.sp_check_status(ws)                      # status word is cleared by the next call
     torch.cuda.synchronize()
     assert torch.equal(good, again)
+
+
+@pytest.mark.parametrize("rows", [32, 48])
+def test_query_rows_bounded_waits_report_timeout_and_context_survives(rows):
+    lay = build_layout([32], [[100, 40]], [[24, rows]])
+    H, D = 2, 128
+    g = torch.Generator().manual_seed(5)
+    qd, kd, vd = (dev(torch.randn(lay.total_tokens, H, D, generator=g).bfloat16()) for _ in range(3))
+    dl = sp.DeviceLayout.from_host(lay)
+    ws = workspace(sp.sp_prefill_workspace_bytes(dl, H, D, sp.SP_BF16))
+
+    def run():
+        out = torch.zeros_like(qd)
+        sp.sp_superpose_prefill(qd, kd, vd, dl, 1 / math.sqrt(D), out, None, ws, rows=sp.SP_ROWS_QUERY_ONLY)
+        return out
+
+    good = run()
+    sp.sp_check_status(ws)
+    sp.lib.sp_test_stall_producer(1)
+    try:
+        run()
+        with pytest.raises(sp.SpError) as e:
+            sp.sp_check_status(ws)
+        assert e.value.code == sp.SP_ERR_TIMEOUT
+    finally:
+        sp.lib.sp_test_stall_producer(0)
+    again = run()
+    sp.sp_check_status(ws)
+    assert torch.equal(good, again)

@@ -355,3 +355,54 @@ def test_prefill_tiles_across_paths_keep_values_to_their_path(D, alibi):
     out1, lse1 = run(k2, v2)
     np.testing.assert_array_equal(lse0[:, others], lse1[:, others])
     assert np.abs(out0[others] - out1[others]).max() <= 2 ** -7 * np.abs(out0).max()
+
+
+QRY_EDGES = [1, 8, 15, 16, 17, 31, 32, 33, 47, 48]
+
+
+@pytest.mark.parametrize("alibi", [False, True])
+@pytest.mark.parametrize("longest", [32, 48])
+@pytest.mark.parametrize("pre", [0, 1, 16, 17, 127, 128, 129, 300])
+@pytest.mark.parametrize("H,Hkv,n", [(3, 1, 2), (29, 29, 6)])
+def test_prefill_query_rows_key_tiles(alibi, longest, pre, H, Hkv, n):
+    """Keys on the M side: 1 to 48 query rows, documents and preambles around the 128 keys of a tile, items of one key to several
+    tiles; few items (P as two numbers) and many (with at most 32 rows and 128 of preamble: for the first keys); bit-identical repeats."""
+    docs = [0, 1, 15, 95, 96, 97, 127, 128, 129, 260]
+    qry = [x for x in QRY_EDGES if x <= longest]
+    qry = (qry * 2)[:len(docs)]
+    lay = build_layout([pre] * n, [docs] * n, [qry[i:] + qry[:i] for i in range(n)])
+    _prefill(lay, H, Hkv, 128, rows=sp.SP_ROWS_QUERY_ONLY, alibi=alibi, repeats=1)
+
+
+@pytest.mark.parametrize("alibi", [False, True])
+@pytest.mark.parametrize("pre,longest", [(21, 32), (200, 32), (21, 48)])
+def test_prefill_query_rows_key_tiles_keep_values_to_their_path(alibi, pre, longest):
+    """NaN and Inf in every third path, which the padding behind preambles and paths reaches into: the others keep their bits."""
+    rng = np.random.default_rng(7)
+    docs, qry = ([[int(x) for x in rng.integers(lo, hi, n)] for n in (50, 45)] for lo, hi in ((0, 60), (1, longest + 1)))
+    qry[0][1] = longest
+    lay = build_layout([pre, pre], docs, qry)
+    T, H, D = lay.total_tokens, 15, 128
+    q, k, v = (_randn((T, H, D), i) for i in (1, 2, 3))
+    pos, slopes = torch.rand(T, generator=torch.Generator().manual_seed(4)).mul(300).float(), torch.linspace(0.01, 0.5, H)
+    dl = sp.DeviceLayout.from_host(lay)
+    ws = workspace(sp.sp_prefill_workspace_bytes(dl, H, D, sp.SP_BF16))
+
+    def run():
+        out, lse = torch.zeros((T, H, D), dtype=torch.bfloat16, device="cuda"), torch.zeros((H, T), device="cuda")
+        args = (dev(q), dev(k), dev(v), dl)
+        if alibi:
+            sp.sp_superpose_prefill_alibi(*args, dev(pos), dev(slopes), D ** -0.5, out, lse, ws, rows=sp.SP_ROWS_QUERY_ONLY)
+        else:
+            sp.sp_superpose_prefill(*args, D ** -0.5, out, lse, ws, rows=sp.SP_ROWS_QUERY_ONLY)
+        sp.sp_check_status(ws)
+        return f32(out), lse.cpu().numpy()
+
+    out0, lse0 = run()
+    others = np.ones(T, bool)
+    for i in range(0, lay.n_paths, 3):
+        r = slice(int(lay.path_start[i]), int(lay.path_start[i] + lay.doc_len[i] + lay.qry_len[i]))
+        q[r], k[r], v[r], others[r] = float("nan"), float("inf"), float("nan"), False
+    out1, lse1 = run()
+    np.testing.assert_array_equal(out0[others], out1[others])
+    np.testing.assert_array_equal(lse0[:, others], lse1[:, others])
