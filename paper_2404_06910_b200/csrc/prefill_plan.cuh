@@ -52,7 +52,6 @@ struct PlanArgs {
     int64_t total_tokens;             // T: every segment must lie inside [0, T)
     int64_t max_tiles;                // capacity of the tile list
     int sort_from;                    // pairs: lists of at least so many records are sorted
-    int across;                       // pairs: tiles over the rows of consecutive paths
     TcHeader *hdr;
     void *list;                       // TcTile or TcPair
 };
@@ -74,7 +73,8 @@ struct PlanArgs {
 // 801 / 784; back to back 2491 / 2464 / 2447 / 2461, 2670 / 2668 / 2646 / 2657, 913 / 904 / 896 / 888, query rows only 609 / 596 /
 // 590 / 597.
 constexpr int kSortWindow = 16;
-template <bool PAIRS>
+// ACROSS (pairs): tiles over the rows of consecutive paths.  A kernel of its own: what it has more costs a small launch 0.3 us.
+template <bool PAIRS, bool ACROSS = false>
 static __global__ void __launch_bounds__(1024) prefill_plan_kernel(const PlanArgs a)
 {
     __shared__ int warp_tot[32];
@@ -93,7 +93,7 @@ static __global__ void __launch_bounds__(1024) prefill_plan_kernel(const PlanArg
         }
         return lo;
     };
-    bool across = PAIRS && a.across;
+    bool across = ACROSS;
     if (across) {                     // what the host saw in its mirror, in the arrays themselves; otherwise segment by segment
         bool fit = true;
         for (int i = threadIdx.x; i < a.n_paths && fit; i += 1024) {
@@ -137,15 +137,23 @@ static __global__ void __launch_bounds__(1024) prefill_plan_kernel(const PlanArg
         // path writes the records of the pairs that start in it.
         const bool own = !(across && s >= a.n_prompts && rows > 0);
         int run0 = 0, run = rows, last = 0;                       // rows cut as one run, the first one's number; its last path
-        if (PAIRS && !own) {
+        if (ACROSS && !own) {
             const int b = prompt_of(s - a.n_prompts);
             last = a.ppo[b + 1] - 1;
             run0 = a.path_start[a.ppo[b]];
             run = a.path_start[last] + a.doc_len[last] + a.qry_len[last] - run0;
         }
-        const int height = PAIRS ? even_height(run, a.tile_rows) : a.tile_rows, nt = (rows + height - 1) / height;
-        const int at = own_row - run0, w0 = own ? 0 : (at + 2 * height - 1) / (2 * height);
-        const int n_rec = !PAIRS ? nt : (own ? (nt + 1) / 2 : (at + rows + 2 * height - 1) / (2 * height) - w0);
+        int nt = (rows + a.tile_rows - 1) / a.tile_rows, height = a.tile_rows;
+        if (PAIRS && (nt > 1 || !own)) {
+            height = even_height(run, a.tile_rows);
+            nt = (rows + height - 1) / height;
+        }
+        const int at = own_row - run0;
+        int w0 = 0, n_rec = PAIRS ? (nt + 1) / 2 : nt;
+        if (ACROSS && !own) {
+            w0 = (at + 2 * height - 1) / (2 * height);
+            n_rec = (at + rows + 2 * height - 1) / (2 * height) - w0;
+        }
         int incl = n_rec;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -158,7 +166,7 @@ static __global__ void __launch_bounds__(1024) prefill_plan_kernel(const PlanArg
         for (int w = 0; w < warp; ++w) before += warp_tot[w];
         const int off = before + incl - n_rec;
         for (int t = 0; t < n_rec && off + t < a.max_tiles; ++t) {
-            if (PAIRS && !own) {
+            if (ACROSS && !own) {
                 const int q0 = (w0 + t) * 2 * height, rows_a = min(height, run - q0), rows_b = min(height, run - q0 - rows_a);
                 TcPair pr;
                 const int p16 = (pre_n + 15) & ~15;
@@ -185,8 +193,8 @@ static __global__ void __launch_bounds__(1024) prefill_plan_kernel(const PlanArg
                 pr.q_u = pr.p16 + first + t0 * height;
                 pr.pre_row = pre_row; pr.pre_len = pre_n;
                 pr.rows_ab = rows_a | rows_b << 16;
-                pr.steps_a = a.across ? 0 : (pr.q_u + rows_a + kPairKeys - 1) / kPairKeys;
-                if (a.across) pr.p16 = -1;
+                pr.steps_a = ACROSS ? 0 : (pr.q_u + rows_a + kPairKeys - 1) / kPairKeys;
+                if (ACROSS) pr.p16 = -1;
                 pr.steps = (pr.q_u + rows_a + rows_b + kPairKeys - 1) / kPairKeys;
                 static_cast<TcPair *>(a.list)[off + t] = pr;
             } else {

@@ -218,7 +218,8 @@ template <int N> struct Ring {        // stage and parity of a ring of N barrier
 };
 
 // One row (key number `last`, own keys from number `from` up; dst: where this thread has stored it) in fp32 arithmetic over exactly the
-// keys it sees: its values that are not finite are replaced.  Rare, so small: 16 bytes at a time.
+// keys it sees: its values that are not finite are replaced.  Rare, so small: 16 bytes at a time.  For tiles across paths; in place of
+// exact_row64 it made head_dim 64 with ALiBi slower (16 prompts x 20 documents 388 -> 403 us).
 template <int D, bool ALIBI>
 __device__ __forceinline__ void exact_row(const TcParams &p, const TcPair &t, int head, int kv_head, int from, int last, unsigned char *dst)
 {
@@ -271,6 +272,70 @@ __device__ __forceinline__ void exact_row(const TcParams &p, const TcPair &t, in
             if ((y[i] & 0x7f800000u) == 0x7f800000u) y[i] = (y[i] & 0xffffu) | (x & 0xffff0000u);
         }
         *at = o;
+    }
+}
+
+// One row (key number `last`, 64 columns; o: bf16 pairs) in fp32 arithmetic over exactly the keys it sees: its values that are not
+// finite are replaced.
+template <bool ALIBI>
+__device__ __forceinline__ void exact_row64(const TcParams &p, const TcPair &t, int head, int kv_head, int last, uint32_t (&o)[32])
+{
+    const int64_t own = t.own_base + last;
+    const uint4 *q = reinterpret_cast<const uint4 *>(p.q + (own * p.n_heads + head) * 64);
+    const float pq = ALIBI ? p.pos[own] : 0.f, slope = ALIBI ? p.slopes[head] * kLog2eT : 0.f;
+    auto packed_row = [&](int u) { return (int64_t)u + (u < t.pre_len ? t.pre_row : t.own_base); };
+    auto score = [&](int64_t row) {
+        const uint4 *k = reinterpret_cast<const uint4 *>(p.k + (row * p.n_kv_heads + kv_head) * 64);
+        float s = 0.f;
+#pragma unroll 1
+        for (int c = 0; c < 8; ++c) {
+            const uint4 x = q[c], y = k[c];
+            s = fmaf(bf16_lo(x.x), bf16_lo(y.x), s); s = fmaf(bf16_hi(x.x), bf16_hi(y.x), s);
+            s = fmaf(bf16_lo(x.y), bf16_lo(y.y), s); s = fmaf(bf16_hi(x.y), bf16_hi(y.y), s);
+            s = fmaf(bf16_lo(x.z), bf16_lo(y.z), s); s = fmaf(bf16_hi(x.z), bf16_hi(y.z), s);
+            s = fmaf(bf16_lo(x.w), bf16_lo(y.w), s); s = fmaf(bf16_hi(x.w), bf16_hi(y.w), s);
+        }
+        s *= p.scale_log2e;
+        return ALIBI ? s - slope * fabsf(pq - p.pos[row]) : s;
+    };
+    float m = -INFINITY, l = 0.f;
+#pragma unroll 1
+    for (int u = 0; u <= last; ++u) {
+        if (u >= t.pre_len && u < t.p16) continue;
+        const float s = score(packed_row(u));
+        if (s > m) { l *= ex2(m - s); m = s; }
+        l += ex2(s - m);
+    }
+    const float inv = 1.f / l;
+#pragma unroll
+    for (int part = 0; part < 4; ++part) {               // 16 columns at a time
+        float acc[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) acc[i] = 0.f;
+#pragma unroll 1
+        for (int u = 0; u <= last; ++u) {
+            if (u >= t.pre_len && u < t.p16) continue;
+            const int64_t row = packed_row(u);
+            const float w = ex2(score(row) - m);
+            const uint4 *v = reinterpret_cast<const uint4 *>(p.v + (row * p.n_kv_heads + kv_head) * 64) + 2 * part;
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const uint4 y = v[c];
+                const uint32_t wd[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    acc[8 * c + 2 * e] = fmaf(w, bf16_lo(wd[e]), acc[8 * c + 2 * e]);
+                    acc[8 * c + 2 * e + 1] = fmaf(w, bf16_hi(wd[e]), acc[8 * c + 2 * e + 1]);
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {                    // the finite ones are right as they are
+            const uint32_t x = pack_bf16x2(acc[2 * i] * inv, acc[2 * i + 1] * inv);
+            uint32_t &y = o[8 * part + i];
+            if ((y & 0x7f80u) == 0x7f80u) y = (y & 0xffff0000u) | (x & 0xffffu);
+            if ((y & 0x7f800000u) == 0x7f800000u) y = (y & 0xffffu) | (x & 0xffff0000u);
+        }
     }
 }
 
@@ -619,6 +684,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
                         if (c == 1 && see <= 32) break;
+                        // keys this row may not see (causal diagonal, ragged end) or that do not exist -> -inf
+                        const uint32_t vis = low_bits(lim - c * 32) & (low_bits(g0 - c * 32) | ~low_bits(g1 - c * 32));
                         if (ALIBI) {              // score - slope * |distance|; key positions are broadcast reads
                             const uint64_t pq2 = pack_f32x2(-pq, -pq), ns2 = pack_f32x2(neg_slope, neg_slope);
 #pragma unroll
@@ -633,8 +700,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                                 }
                             }
                         }
-                        // keys this row may not see (causal diagonal, ragged end) or that do not exist -> -inf
-                        const uint32_t vis = low_bits(lim - c * 32) & (low_bits(g0 - c * 32) | ~low_bits(g1 - c * 32));
                         if (__any_sync(0xffffffffu, vis != 0xffffffffu)) {
 #pragma unroll
                             for (int i = 0; i < 32; ++i) r[c][i] = vis & (1u << i) ? r[c][i] : 0xff800000u;
@@ -762,7 +827,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&bars[C::BAR_O_FREE + ln]);
                     }
-                    if (C::EXACT || ACROSS) {
+                    if (C::EXACT && !ACROSS && hr < t.rows) {
+                        uint32_t nan = 0u;
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) asm("fma.rn.bf16x2 %0, %1, %2, %0;" : "+r"(nan) : "r"(o[i]), "r"(0u));
+                        if (nan & 0x7fff7fffu)
+                            exact_row64<ALIBI>(p, w.t, (w.h << (7 - log_rows)) + (row >> log_rows), w.h / p.units_per_kv, t.q_u + hr, o);
+                    }
+                    if (ACROSS) {
 #pragma unroll
                         for (int i = 0; i < 32; ++i) asm("fma.rn.bf16x2 %0, %1, %2, %0;" : "+r"(nan) : "r"(o[i]), "r"(0u));
                     }
@@ -781,7 +853,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                 // where a tile holds keys of paths that a row does not see, a row with a value that is not finite is computed again over
                 // its own keys.  The look at the row costs nothing that shows; looking through the V tiles instead cost the ALiBi variant
                 // 14 % (one more warp on the SM partition of two softmax warps).
-                if ((C::EXACT || ACROSS) && hr < t.rows && (nan & 0x7fff7fffu)) {
+                if (ACROSS && hr < t.rows && (nan & 0x7fff7fffu)) {
                     int start = w.t.own_base + w.t.p16;                    // of the row's own path
                     const int row_p = w.t.own_base + t.q_u + hr;
                     if (ACROSS && w.first_path >= 0)
@@ -950,9 +1022,9 @@ static int launch_tc(const void *q, const void *k, const void *v, const sp_layou
     // the sort takes a microsecond: worth it from a dozen items per block
     pa.sort_from = 12 * num_sms() / (n_heads >> log_g);
     // (not with the rotation folded in: Q is then where the output goes, and a row that has to be computed again would not find it)
-    pa.across = log_g == 0 && rows == SP_ROWS_ALL && !rope && across_pays(lay, n_heads);
+    const bool across = log_g == 0 && rows == SP_ROWS_ALL && !rope && across_pays(lay, n_heads);
     pa.hdr = hdr; pa.list = pairs;
-    if (int rc = launch(prefill_plan_kernel<true>, 1, 1024, 0, st, 1, pa)) return rc;
+    if (int rc = launch(across ? prefill_plan_kernel<true, true> : prefill_plan_kernel<true>, 1, 1024, 0, st, 1, pa)) return rc;
     if (pa.max_tiles == 0) return SP_OK;              // no segment can have a row
     if (rope) {
         RopeRows r = *rope;
@@ -975,7 +1047,7 @@ static int launch_tc(const void *q, const void *k, const void *v, const sp_layou
     const int64_t items = pa.max_tiles * p.n_units;
     const int grid = (int)std::min<int64_t>(items, num_sms());
     using Launch = int (*)(const TcParams &, int, cudaStream_t);
-    const auto run = [&](Launch segment, Launch heads, Launch across) { return (pa.across ? across : (log_g ? heads : segment))(p, grid, st); };
+    const auto run = [&](Launch segment, Launch heads, Launch paths) { return (across ? paths : (log_g ? heads : segment))(p, grid, st); };
     if (head_dim == 64)
         return pos ? run(launch_kernel<64, true, SEGMENT_ROWS, true>, launch_kernel<64, true, HEAD_ROWS, true>, launch_kernel<64, true, ACROSS_ROWS, true>)
                    : run(launch_kernel<64, false, SEGMENT_ROWS, true>, launch_kernel<64, false, HEAD_ROWS, true>, launch_kernel<64, false, ACROSS_ROWS, true>);
