@@ -8,10 +8,8 @@
 // keeps an online softmax per key group and writes one partial (max, sum, unnormalised output)
 // per head into the shared memory of the cluster's first block, which merges them in split
 // order, so results do not depend on scheduling.  sp_pruned_decode_static merges through global
-// memory instead.  bf16 with several query heads to a KV head: decode_mma.cuh.
-// Measured, 2 prompts x 32 heads, 8 kept of 400 paths of 160-544 rows, 95 MB: 24.6 us (26.6 with
-// partials fetched by the first block and without programmatic dependent launch), 14.5 at the
-// copy bandwidth; what is left is launch, index loads and one wave's ramp.
+// memory instead.  bf16 mostly runs on tensor-core instructions (decode_mma.cuh; rule and figures: mma_launch()); the kernel here serves fp32,
+// and bf16 with single heads where few keys per head start sooner in it or fill its waves.
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -300,7 +298,7 @@ template <typename T> struct DecodeSmem {
         end = reinterpret_cast<float *>(pos + n_seg);
     }
 };
-static size_t decode_table_bytes(int n_seg) { return round_up((n_seg + 1) * sizeof(int), 16) + 3 * n_seg * sizeof(void *); }
+__host__ __device__ constexpr size_t decode_table_bytes(int n_seg) { return round_up((n_seg + 1) * sizeof(int), 16) + 3 * n_seg * sizeof(void *); }
 
 // Segments of prompt b: 0 = preamble, 1..k = kept paths, k+1 = tail; lengths land in lo[s+1].
 template <typename T, bool ALIBI>
@@ -680,22 +678,69 @@ static int launch_cluster_kernel(K kern, const DecodeArgs &a, const DecodeRope &
     return launch(kern, dim3(a.n_splits, blocks_y, n_prompts), threads, smem, st, a.n_splits, a, rope, pairing);
 }
 
+// bf16, which kernel; units: a prompt and a KV head's block of up to 8 query heads each.  us, cold reads, D = 128.
+//  - The tensor-core kernel with rings in shared memory: almost always.  What served it before (grouped heads: loads held in registers;
+//    single heads: decode_cluster_kernel) / ring, 3 000 keys: 8 units 15.4 / 8.8, 32 18.8 / 13.5, 64 24.5 / 21.5, 192 65.4 / 54.2, 384 118 / 98;
+//    430 keys: 64 9.2 / 7.6, 192 15.2 / 12.0, 512 29.5 / 25.4; groups of 4, 3 000 keys: 32 18.6 / 16.4, 128 49.2 / 38.8, 256 87.9 / 66.4, 512
+//    136.5 / 125.7; 430 keys: 128 15.1 / 12.0, 512 27.6 / 26.0; groups of 2: 1 024 units 58.4 / 45.3.
+//  - Few units and keys: the kernels that hold loads in registers, whose blocks start sooner: 8 units of 430 keys 7.7 / 7.8, 16 5.6 / 5.9 (reads
+//    from L2), groups of 4 8.1 / 8.3; with 1 300 keys 9.0 / 7.0.
+//  - Grouped heads, few keys, and units that leave a ring two warps but registers four: 384 units of 430 keys 22.3 / 22.6.
+//  - Single heads, few keys, units that fill the waves of decode_cluster_kernel: 1 024 43.6 / 44.2, 2 048 75.3 / 77.1; but 1 536 66.3 / 61.7.
+struct MmaLaunch { bool ring; int n_splits, warps; size_t smem; };
+
+template <int D> static MmaLaunch mma_launch(DecodeArgs a, int n_prompts, int64_t max_keys)
+{
+    const int group = a.n_heads / a.n_kv_heads, blocks_y = a.n_kv_heads * ((group + kMmaHeads - 1) / kMmaHeads), sms = num_sms();
+    const int64_t units = (int64_t)n_prompts * blocks_y;
+    const size_t partial = std::min(group, kMmaHeads) * (D + 2) * sizeof(float);
+    MmaLaunch r = {};
+    const auto in_registers = [&]() {
+        // three blocks per SM for both head sizes: with four, 2 prompts x 16 KV heads of 64 become clusters of 16, which the SMs take in
+        // less evenly than clusters of 8 (12.1 us against 8.0)
+        r.ring = false;
+        r.n_splits = cluster_splits(n_prompts, blocks_y, max_keys, kMmaMaxWarps * kMmaKeys, 3);
+        r.warps = kMmaMaxWarps;
+        r.smem = decode_table_bytes(a.k + 2) + (D / 2) * sizeof(float2) + (r.warps + r.n_splits) * partial;
+        return r;
+    };
+    const bool few_keys = max_keys < 1024;
+    if (units <= 24 && few_keys) return in_registers();
+    r.ring = true;
+    const auto bytes = [&](int n, int w) {
+        a.n_splits = n;
+        return mma_ring_offset<D>(a, (int)partial) + w * std::max(partial, (size_t)MmaRing<D>::BYTES);
+    };
+    const auto blocks_per_sm = [&](int n, int w) { return (int)std::min<size_t>(228 * 1024 / (bytes(n, w) + 1024), mma_warps_per_sm(D, true) / w); };
+    // Splits: the largest cluster for which all blocks find a place at once, and a turn of keys for each of its warps (five where the merge
+    // is all that two blocks add: groups of 4, 128 units of 430 keys 12.0 us unsplit, 12.9 split).  Larger clusters do not fill the chip:
+    // 16 units in clusters of 8, 128 blocks where 148 fit (groups of 4), take 18.6 us, in clusters of 4 15.0; 16 in clusters of 16 13.3, of 8 10.2.
+    r.warps = kMmaMaxWarps;
+    for (r.n_splits = 16; r.n_splits > 1; r.n_splits /= 2) {
+        const int n = r.n_splits, per_sm = blocks_per_sm(n, r.warps), percent = n == 16 ? 45 : (n == 8 && per_sm < 2 ? 50 : (n == 2 ? 100 : 87));
+        if (n * units * 100 <= (int64_t)per_sm * sms * percent && n * r.warps * kMmaKeys * (n == 2 ? 5 : 1) <= max_keys) break;
+    }
+    // Unsplit: as many warps a block as still leave every block resident; where even blocks of one warp do not fit, two (1 536 units: one warp
+    // 68.5 us, two 61.7, four 71.9).
+    if (r.n_splits == 1) {
+        while (r.warps > 1 && (int64_t)blocks_per_sm(1, r.warps) * sms < units) --r.warps;
+        if ((int64_t)blocks_per_sm(1, r.warps) * sms < units) r.warps = 2;
+        if (few_keys && group > 1 && r.warps == 2 && units * kMmaMaxWarps <= mma_warps_per_sm(D, false) * sms) return in_registers();
+        const int64_t wave = 7 * sms, waves = (units + wave - 1) / wave;
+        if (few_keys && group == 1 && units * 100 >= waves * wave * 95) r.ring = false;
+    }
+    while (bytes(r.n_splits, r.warps) > 200 * 1024 && r.warps > 1) --r.warps;      // the table of thousands of kept paths takes the place of rings
+    r.smem = bytes(r.n_splits, r.warps);
+    return r;
+}
+
 template <int D, bool ALIBI, bool ROPE>
-static int launch_decode_mma(DecodeArgs a, const DecodeRope &rope, int pairing, int n_prompts, int64_t max_keys, cudaStream_t st)
+static int launch_decode_mma(DecodeArgs a, const MmaLaunch &m, const DecodeRope &rope, int pairing, int n_prompts, cudaStream_t st)
 {
     const int group = a.n_heads / a.n_kv_heads, blocks_y = a.n_kv_heads * ((group + kMmaHeads - 1) / kMmaHeads);
-    const int warps = mma_warps_per_sm(D) * num_sms();
-    const int64_t units = (int64_t)n_prompts * blocks_y;
-    // three blocks per SM for both head sizes: with four, 2 prompts x 16 KV heads of 64 become clusters of 16, which the SMs take in
-    // less evenly than clusters of 8 (12.1 us against 8.0)
-    a.n_splits = cluster_splits(n_prompts, blocks_y, max_keys, kMmaMaxWarps * kMmaKeys, mma_warps_per_sm(128) / kMmaMaxWarps);
-    // Unsplit launches take as many warps a block as still leave every block resident at once: 64 prompts x 8 KV heads fit with
-    // three (30 us a step); blocks of four need a second wave (33).
-    int w = kMmaMaxWarps;
-    if (a.n_splits == 1) w = (int)std::max<int64_t>(1, std::min<int64_t>(w, warps / units));
-    const size_t smem = decode_table_bytes(a.k + 2) + (size_t)(w + a.n_splits) * std::min(group, kMmaHeads) * (D + 2) * sizeof(float) +
-                        (D / 2) * sizeof(float2);
-    return launch_cluster_kernel(decode_mma_kernel<D, ALIBI, ROPE>, a, rope, pairing, blocks_y, n_prompts, 32 * w, smem, st);
+    a.n_splits = m.n_splits;
+    const auto kern = m.ring ? decode_mma_kernel<D, ALIBI, ROPE, true> : decode_mma_kernel<D, ALIBI, ROPE, false>;
+    return launch_cluster_kernel(kern, a, rope, pairing, blocks_y, n_prompts, 32 * m.warps, m.smem, st);
 }
 
 template <typename T, int D, int GRP, bool ALIBI, bool ROPE>
@@ -720,7 +765,8 @@ static int launch_decode_grp(const DecodeArgs &a, const DecodeRope &rope, int pa
 {
     const int group = a.n_heads / a.n_kv_heads;
     if constexpr (sizeof(T) == 2) {
-        if (group > 1) return launch_decode_mma<D, ALIBI, ROPE>(a, rope, pairing, n_prompts, max_keys, st);
+        const MmaLaunch m = mma_launch<D>(a, n_prompts, max_keys);
+        if (group > 1 || m.ring) return launch_decode_mma<D, ALIBI, ROPE>(a, m, rope, pairing, n_prompts, st);
     } else {
         // query heads per block: the largest of 4, 2, 1 that divides the group, so grouped heads share
         // one pass over their K and V rows

@@ -1,14 +1,19 @@
-// One-token decode attention for query heads that share a KV head (bf16): both products on warp-level tensor-core
-// instructions (mma.sync m16n8k16), fragments loaded straight from global memory.
+// One-token decode attention in bf16: both products on warp-level tensor-core instructions (mma.sync m16n8k16), for query heads that
+// share a KV head and for single ones.
 //
 // With g query heads per KV head a step still reads every K and V row once, but the SIMT kernel pays 2 g D multiply-adds a
 // key, which bounds it long before HBM does (g = 4: 0.24 of the copy bandwidth).  Here a warp takes 16 keys at a time:
 //   S [heads x keys] = Q K^T      A = Q, up to 8 heads in rows 0-7 of the fragment, B = K
 //   O^T [d x heads] += V^T P^T    A = V^T, B = P^T, which is the S fragment as it is
-// A contraction may run over its elements in any order and output rows may be any permutation, so every thread loads
-// contiguous 16-byte pieces of K and V rows and uses them as fragments: no shared memory, no ldmatrix.  Only V needs a
-// byte permute to pair two keys.  P is carried as the sum of two bf16 numbers (16 bits of mantissa), so the result is as
-// good as with fp32 products, values that are not finite included.
+// A contraction may run over its elements in any order and output rows may be any permutation, so every thread uses
+// contiguous 16-byte pieces of K and V rows as fragments: no ldmatrix.  Only V needs a byte permute to pair two keys.  P is carried as
+// the sum of two bf16 numbers (16 bits of mantissa), so the result is as good as with fp32 products (1.6555e-3 of the norm from 64-bit
+// results with either, the rounding of the output), values that are not finite included.
+// What bounds it is latency: a turn of 16 keys is a chain of 0.65 us for a warp (products, maximum, exponentials), and where loads go to
+// registers nothing is in flight meanwhile.  So K and V rows run through a ring in shared memory (cp.async), two turns of 8 KB
+// ahead of a warp's arithmetic: 8 warps per SM keep 128 KB in flight.  Two chains of products for S instead of one and fewer instructions per
+// copy changed nothing.  Cold reads, 2 prompts x 32 heads, 8 kept of long documents 24.5 -> 21.6 us (14.5 at the copy bandwidth); which
+// launches take which form, and the figures: mma_launch() in decode.cu.
 #pragma once
 
 namespace sp {
@@ -16,9 +21,30 @@ namespace sp {
 constexpr int kMmaHeads = 8;         // query heads per block at most
 constexpr int kMmaKeys = 16;         // keys per warp and turn
 constexpr int kMmaMaxWarps = 4;      // warps per block at most
-// Warps resident per SM, by the registers that a warp's loads and accumulators take: 168 with head_dim 128, less than 128 with 64
-// (64 prompts x 16 KV heads of 64: one warp to a block and 44.8 us with a budget of 12, two and 29.4 with 16).
-constexpr int mma_warps_per_sm(int D) { return D == 64 ? 16 : 12; }
+constexpr int kMmaStages = 3;        // RING: turns of a warp in shared memory
+// Warps resident per SM, by the registers that a warp's loads and accumulators take or (RING) the shared memory of its ring; held in
+// registers: 64 prompts x 16 KV heads of 64: one warp to a block and 44.8 us with a budget of 12, two and 29.4 with 16.
+constexpr int mma_warps_per_sm(int D, bool ring) { return D == 64 ? 16 : (ring ? 8 : 12); }
+template <int D> struct MmaRing {    // a warp's: [stage]([K][V] rows of the turn's keys | positions)
+    static constexpr int ROW = D * 2, V = kMmaKeys * ROW, POS = 2 * V, STAGE = POS + 128, BYTES = kMmaStages * STAGE;
+};
+
+// Start of the rings in shared memory: behind the segment table (whose size is no multiple of 16 with an odd number of segments), the
+// angles and the cluster's partials, of partial_bytes each.  A multiple of 128: 16 bytes off a 32-byte sector, every copy is split (48
+// units in 4 blocks of 4 warps each: 11.0 against 12.7 us).
+template <int D> __host__ __device__ __forceinline__ size_t mma_ring_offset(const DecodeArgs &a, int partial_bytes)
+{
+    return round_up(decode_table_bytes(a.k + 2) + (D / 2) * sizeof(float2) + (a.n_splits > 1 ? (size_t)a.n_splits * partial_bytes : 0), 128);
+}
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool valid)
+{
+    const int n = valid ? 16 : 0;        // 0: zero-filled, nothing is read
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void *src) { asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory"); }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 __device__ __forceinline__ void mma_16n8k16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
 {
@@ -29,8 +55,10 @@ __device__ __forceinline__ void mma_16n8k16(float (&d)[4], uint32_t a0, uint32_t
 static __device__ const uint4 g_zero_row[16] = {};
 
 // Grid (n_splits, KV heads x blocks of up to 8 query heads, prompts); the n_splits blocks of a (prompt, y) are a cluster.
-template <int D, bool ALIBI, bool ROPE>
-__global__ void __launch_bounds__(32 * kMmaMaxWarps, mma_warps_per_sm(D) / kMmaMaxWarps)
+// RING: K and V rows go through a ring in shared memory, two turns ahead of the arithmetic; otherwise a turn's loads go to registers
+// and nothing is in flight while a warp computes.
+template <int D, bool ALIBI, bool ROPE, bool RING>
+__global__ void __launch_bounds__(32 * kMmaMaxWarps, mma_warps_per_sm(D, RING) / kMmaMaxWarps)
 decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ DecodeRope rope, int rope_pairing)
 {
     using T = __nv_bfloat16;
@@ -39,7 +67,7 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
     constexpr int NM = D / 16;              // 16-row tiles of O^T
     constexpr int PS = D + 2;               // one partial: D outputs, max, sum
 
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    extern __shared__ __align__(128) unsigned char smem_raw[];
     const int n_seg = a.k + 2;
     const DecodeSmem<T> sm(smem_raw, n_seg);
     const int split = blockIdx.x, b = blockIdx.z;
@@ -51,6 +79,12 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
     float2 *cs = reinterpret_cast<float2 *>(sm.end);            // [D/2] (cos, sin), ROPE only
     float *red = reinterpret_cast<float *>(cs + D / 2);         // [W][nh][PS]
     float *part = red + W * nh * PS;                            // first block of the cluster: [n_splits][nh][PS]
+    unsigned char *rings = nullptr;                             // RING: behind `part`, and `red` takes their place in the end
+    if constexpr (RING) {
+        part = red;
+        rings = smem_raw + mma_ring_offset<D>(a, min(group, kMmaHeads) * PS * (int)sizeof(float));
+        red = reinterpret_cast<float *>(rings);
+    }
 
     decode_cluster_begin(a);
     pdl_wait();
@@ -172,29 +206,91 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
         prefetch_l2((lane < 2 ? sm.k : sm.v)[n_seg - 1] + new_off + (lane & 1) * (D / 2));
 
     int seg = 0;
-    for (int base = lo + warp * kMmaKeys; base < hi_loop; base += W * kMmaKeys) {
-        const int n = min(kMmaKeys, hi_loop - base);
-        // lane i (and i + 16) finds key i of the turn; keys that do not exist read the last one's K and get no weight, which is not
-        // enough where V holds an Inf: they read a V row of zeros
-        const int j = base + min(lane & 15, n - 1);
-        while (j >= sm.lo[seg + 1]) ++seg;                  // keys ascend: segments only advance
-        const int64_t off = (int64_t)(j - sm.lo[seg]) * row_elems;
-        const float kpos = ALIBI ? sm.pos[seg][j - sm.lo[seg]] : 0.f;
-        const unsigned long long kp = reinterpret_cast<unsigned long long>(sm.k[seg] + off), vp = reinterpret_cast<unsigned long long>((lane & 15) < n ? sm.v[seg] + off : reinterpret_cast<const T *>(g_zero_row));
-        uint4 kr[2][NC], vr[4][NV];
+    if constexpr (RING) {
+        // Rows are stored in 16-byte pieces permuted so that the fragments' reads are free of conflicts: K by the row's parity, V by the
+        // row pair.
+        const unsigned char *ring = rings + warp * MmaRing<D>::BYTES;
+        const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
+        constexpr int PIECES = D / 8, PER = 32 / PIECES;             // of a row; rows per copy instruction
+        const int piece = lane % PIECES, row0 = lane / PIECES;
+        auto fetch = [&](int base, int stage) {
+            if (base < hi_loop) {
+                const int n = min(kMmaKeys, hi_loop - base), j = base + min(lane & 15, n - 1);
+                while (j >= sm.lo[seg + 1]) ++seg;                  // lane i (and i + 16) finds key i of the turn; keys ascend: segments only advance
+                const int64_t off = (int64_t)(j - sm.lo[seg]) * row_elems;
+                const char *kp = reinterpret_cast<const char *>(sm.k[seg] + off), *vp = reinterpret_cast<const char *>(sm.v[seg] + off);
+                const uint32_t dst = ring_s + stage * MmaRing<D>::STAGE;
+                auto copy = [&](int r, const char *krow, const char *vrow, bool exists) {
+                    cp_async16(dst + r * MmaRing<D>::ROW + ((piece ^ ((r & 1) << 2)) << 4), krow + piece * 16, true);
+                    cp_async16(dst + MmaRing<D>::V + r * MmaRing<D>::ROW + ((piece ^ (r & 6)) << 4), vrow + piece * 16, exists);
+                };
+                if (n == kMmaKeys && __all_sync(0xffffffffu, seg == __shfl_sync(0xffffffffu, seg, 0))) {        // rows one after another
+                    const char *k0 = reinterpret_cast<const char *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(kp), 0)) + row0 * row_elems * 2;
+                    const char *v0 = reinterpret_cast<const char *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(vp), 0)) + row0 * row_elems * 2;
 #pragma unroll
-        for (int t = 0; t < 2; ++t) {
-            const uint4 *src = reinterpret_cast<const uint4 *>(__shfl_sync(0xffffffffu, kp, gid + 8 * t));
+                    for (int i = 0; i < kMmaKeys / PER; ++i, k0 += PER * row_elems * 2, v0 += PER * row_elems * 2) copy(i * PER + row0, k0, v0, true);
+                } else {
+                    // keys that do not exist read the last one's K and get no weight, which is not enough where V holds an Inf: zeros for V
+#pragma unroll 2
+                    for (int i = 0; i < kMmaKeys / PER; ++i) {
+                        const int r = i * PER + row0;
+                        copy(r, reinterpret_cast<const char *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(kp), r)),
+                             reinterpret_cast<const char *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(vp), r)), r < n);
+                    }
+                }
+                if (ALIBI && lane < 16) cp_async4(dst + MmaRing<D>::POS + lane * 4, sm.pos[seg] + (j - sm.lo[seg]));
+            }
+            cp_async_commit();
+        };
+        int stage = 0;
 #pragma unroll
-            for (int c = 0; c < NC; ++c) kr[t][c] = ld_stream16(src + tig + 4 * c);
+        for (int i = 0; i < kMmaStages - 1; ++i) fetch(lo + (warp + i * W) * kMmaKeys, i);
+        for (int base = lo + warp * kMmaKeys; base < hi_loop; base += W * kMmaKeys) {
+            cp_async_wait<kMmaStages - 2>();
+            __syncwarp();                                           // every lane's copies have landed, and the turn before this one has been read
+            fetch(base + (kMmaStages - 1) * W * kMmaKeys, stage == 0 ? kMmaStages - 1 : stage - 1);
+            const unsigned char *kt = ring + stage * MmaRing<D>::STAGE, *vt = kt + MmaRing<D>::V;
+            uint4 kr[2][NC], vr[4][NV];
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int c = 0; c < NC; ++c) kr[t][c] = *reinterpret_cast<const uint4 *>(kt + (gid + 8 * t) * MmaRing<D>::ROW + (((tig + 4 * c) ^ ((gid & 1) << 2)) << 4));
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int r = 2 * tig + (t & 1) + 8 * (t >> 1);
+#pragma unroll
+                for (int c = 0; c < NV; ++c) vr[t][c] = *reinterpret_cast<const uint4 *>(vt + r * MmaRing<D>::ROW + (((gid + 8 * c) ^ (r & 6)) << 4));
+            }
+            attend(kr, vr, min(kMmaKeys, hi_loop - base), ALIBI ? *reinterpret_cast<const float *>(kt + MmaRing<D>::POS + (lane & 15) * 4) : 0.f);
+            if (++stage == kMmaStages) stage = 0;
         }
+        cp_async_wait<0>();
+        __syncthreads();                                        // the rings are done with
+    } else {
+        for (int base = lo + warp * kMmaKeys; base < hi_loop; base += W * kMmaKeys) {
+            const int n = min(kMmaKeys, hi_loop - base);
+            // lane i (and i + 16) finds key i of the turn; keys that do not exist read the last one's K and get no weight, which is not
+            // enough where V holds an Inf: they read a V row of zeros
+            const int j = base + min(lane & 15, n - 1);
+            while (j >= sm.lo[seg + 1]) ++seg;              // keys ascend: segments only advance
+            const int64_t off = (int64_t)(j - sm.lo[seg]) * row_elems;
+            const float kpos = ALIBI ? sm.pos[seg][j - sm.lo[seg]] : 0.f;
+            const unsigned long long kp = reinterpret_cast<unsigned long long>(sm.k[seg] + off), vp = reinterpret_cast<unsigned long long>((lane & 15) < n ? sm.v[seg] + off : reinterpret_cast<const T *>(g_zero_row));
+            uint4 kr[2][NC], vr[4][NV];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const uint4 *src = reinterpret_cast<const uint4 *>(__shfl_sync(0xffffffffu, vp, 2 * tig + (t & 1) + 8 * (t >> 1)));
+            for (int t = 0; t < 2; ++t) {
+                const uint4 *src = reinterpret_cast<const uint4 *>(__shfl_sync(0xffffffffu, kp, gid + 8 * t));
 #pragma unroll
-            for (int c = 0; c < NV; ++c) vr[t][c] = ld_stream16(src + gid + 8 * c);
+                for (int c = 0; c < NC; ++c) kr[t][c] = ld_stream16(src + tig + 4 * c);
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const uint4 *src = reinterpret_cast<const uint4 *>(__shfl_sync(0xffffffffu, vp, 2 * tig + (t & 1) + 8 * (t >> 1)));
+#pragma unroll
+                for (int c = 0; c < NV; ++c) vr[t][c] = ld_stream16(src + gid + 8 * c);
+            }
+            attend(kr, vr, n, kpos);
         }
-        attend(kr, vr, n, kpos);
     }
 
     if (mine_new) {

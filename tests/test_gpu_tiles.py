@@ -406,3 +406,32 @@ def test_prefill_query_rows_key_tiles_keep_values_to_their_path(alibi, pre, long
     out1, lse1 = run()
     np.testing.assert_array_equal(out0[others], out1[others])
     np.testing.assert_array_equal(lse0[:, others], lse1[:, others])
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("k", [1, 2, 3, 6, 7])
+@pytest.mark.parametrize("H,Hkv,n_prompts,longest", [(8, 8, 1, 70), (32, 32, 3, 300), (8, 4, 40, 70), (16, 2, 60, 40), (40, 40, 30, 30), (12, 4, 9, 400), (64, 64, 20, 20)])
+def test_decode_keys_through_a_ring(D, k, H, Hkv, n_prompts, longest):
+    """Segment tables of odd and even size in front of the rings, single and grouped heads, from few units, each split over a cluster, to
+    more than there are warps; turns of 16 keys within a segment and across its end, prompts with fewer keys than warps."""
+    rng = np.random.default_rng(k)
+    lay = build_layout([int(x) for x in rng.integers(0, 40, n_prompts)], [[int(x) for x in rng.integers(0, longest, 8)] for _ in range(n_prompts)],
+                       [[int(x) for x in rng.integers(1, 9, 8)] for _ in range(n_prompts)])
+    T, cap = lay.total_tokens, 5
+    q, kc, vc = _randn((n_prompts, H, D), 1), _randn((T, Hkv, D), 2), _randn((T, Hkv, D), 3)
+    tk, tv = _randn((n_prompts, cap, Hkv, D), 4), _randn((n_prompts, cap, Hkv, D), 5)
+    kept = np.stack([lay.prompt_path_off[b] + rng.permutation(8)[:k] for b in range(n_prompts)]).astype(np.int32)
+    tl = rng.integers(0, cap + 1, n_prompts).astype(np.int32)
+    ref_o, ref_l = oracle.pruned_decode(f32(q), f32(kc), f32(vc), lay, kept, f32(tk), f32(tv), tl, 1 / math.sqrt(D))
+    args = (dev(q), dev(kc), dev(vc), sp.DeviceLayout.from_host(lay), dev(kept), k, dev(tk), dev(tv), dev(tl), cap, 1 / math.sqrt(D))
+    ws = workspace(sp.sp_decode_workspace_bytes(n_prompts, H, D))
+    outs = []
+    for _ in range(2):
+        out, lse = torch.full((n_prompts, H, D), float("nan"), dtype=torch.bfloat16, device="cuda"), torch.full((n_prompts, H), float("nan"), device="cuda")
+        sp.sp_pruned_decode(*args, out, lse, ws)
+        outs.append((f32(out), lse.cpu().numpy()))
+    np.testing.assert_array_equal(outs[0][0], outs[1][0])
+    assert rel_l2(outs[0][0], ref_o) <= TOL[torch.bfloat16]
+    fin = np.isfinite(ref_l)
+    np.testing.assert_allclose(outs[0][1][fin], ref_l[fin], atol=2e-2)
+    np.testing.assert_array_equal(outs[0][1][~fin], ref_l[~fin])
