@@ -58,20 +58,16 @@ template <> __device__ __forceinline__ void load_stream<float>(const float *p, f
 // Masked logits (-inf, or the type's lowest value) are ordinary input and add nothing: the running maximum may still be -inf,
 // or so large that its product with log2 e is not finite, when they are met.  Both are kept out of the sum by a clamp; a row
 // whose maximum itself is that large is summed again (a test of the maximum inside the loop: 508 us where this takes 500).
-template <typename T, int kScoreThreads>
-__global__ void __launch_bounds__(kScoreThreads)
-row_logp_kernel(const T *logits, int64_t ld, const int32_t *targets, int vocab, float *row_logp)
+// One row by kScoreThreads threads (tid); sync() is their barrier, sm / ss a number per warp.
+template <typename T, int kScoreThreads, typename Sync>
+__device__ __forceinline__ void score_row(const T *logits, int64_t ld, int64_t t, int y, int vocab, float *row_logp, int tid, float *sm, float *ss, Sync sync)
 {
-    pdl_wait();
-    pdl_trigger();
-    const int64_t t = blockIdx.x;
-    const int32_t y = targets[t];
     if (y < 0 || y >= vocab) {           // no target: contributes nothing, row is not read
-        if (threadIdx.x == 0) row_logp[t] = 0.f;
+        if (tid == 0) row_logp[t] = 0.f;
         return;
     }
     const T *row = logits + t * ld;
-    const float picked = threadIdx.x == 0 ? to_float(row[y]) : 0.f;      // ahead of the stream, not behind it
+    const float picked = tid == 0 ? to_float(row[y]) : 0.f;              // ahead of the stream, not behind it
     float m = -INFINITY, s = 0.f;
 
     constexpr int N = Vec<T>::N;
@@ -80,12 +76,12 @@ row_logp_kernel(const T *logits, int64_t ld, const int32_t *targets, int vocab, 
     const T *body = row + head;
     // the ends first: their latency hides behind the body's
     const int n_ends = vocab - nvec * N;
-    for (int c = threadIdx.x; c < n_ends; c += kScoreThreads) {
+    for (int c = tid; c < n_ends; c += kScoreThreads) {
         const float xv = to_float(row[c < head ? c : c + nvec * N]);
         if (xv > m) { s *= fast_exp2((m - xv) * kLog2e); m = xv; }
         if (xv != -INFINITY) s += fast_exp2((xv - m) * kLog2e);
     }
-    for (int i0 = threadIdx.x; i0 < nvec; i0 += kScoreThreads * kScoreUnroll) {
+    for (int i0 = tid; i0 < nvec; i0 += kScoreThreads * kScoreUnroll) {
         float f[kScoreUnroll][N];
 #pragma unroll
         for (int u = 0; u < kScoreUnroll; ++u) {
@@ -121,10 +117,9 @@ row_logp_kernel(const T *logits, int64_t ld, const int32_t *targets, int vocab, 
         const float s2 = __shfl_xor_sync(0xffffffffu, s, o);
         merge_ms(m, s, m2, s2);
     }
-    __shared__ float sm[kScoreThreads / 32], ss[kScoreThreads / 32];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = tid >> 5, lane = tid & 31;
     if (lane == 0) { sm[warp] = m; ss[warp] = s; }
-    __syncthreads();
+    sync();
     if (warp > 0) return;
     m = sm[0]; s = ss[0];
     for (int w = 1; w < kScoreThreads / 32; ++w) merge_ms(m, s, sm[w], ss[w]);
@@ -139,17 +134,23 @@ row_logp_kernel(const T *logits, int64_t ld, const int32_t *targets, int vocab, 
     if (lane == 0) row_logp[t] = picked - (m + logf(s));
 }
 
-// scores[i] = weight[i] * sum_t row_logp[t] + prior[i]; one warp per path, fixed order.
-__global__ void __launch_bounds__(256)
-path_sum_kernel(const float *row_logp, const int32_t *row_off, int n_paths, const float *prior, const float *weight, float *scores)
+template <typename T, int kScoreThreads>
+__global__ void __launch_bounds__(kScoreThreads)
+row_logp_kernel(const T *logits, int64_t ld, const int32_t *targets, int vocab, float *row_logp)
 {
+    __shared__ float sm[kScoreThreads / 32], ss[kScoreThreads / 32];
     pdl_wait();
     pdl_trigger();
-    const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (i >= n_paths) return;
+    const int64_t t = blockIdx.x;
+    score_row<T, kScoreThreads>(logits, ld, t, targets[t], vocab, row_logp, threadIdx.x, sm, ss, []() { __syncthreads(); });
+}
+
+// scores[i] = weight[i] * sum_t row_logp[t] + prior[i], t in [t0, t1); one warp, fixed order.
+__device__ __forceinline__ void path_sum(const float *row_logp, int i, int t0, int t1, const float *prior, const float *weight, float *scores)
+{
     const int lane = threadIdx.x & 31;
     double acc = 0.0;
-    for (int t = row_off[i] + lane; t < row_off[i + 1]; t += 32) acc += (double)row_logp[t];
+    for (int t = t0 + lane; t < t1; t += 32) acc += (double)__ldcg(row_logp + t);       // other blocks have written them
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) {
@@ -157,6 +158,40 @@ path_sum_kernel(const float *row_logp, const int32_t *row_off, int n_paths, cons
         const double pr = prior ? (double)prior[i] : 0.0;
         scores[i] = (float)(w * acc + pr);
     }
+}
+
+__global__ void __launch_bounds__(256)
+path_sum_kernel(const float *row_logp, const int32_t *row_off, int n_paths, const float *prior, const float *weight, float *scores)
+{
+    pdl_wait();
+    pdl_trigger();
+    const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (i < n_paths) path_sum(row_logp, i, row_off[i], row_off[i + 1], prior, weight, scores);
+}
+
+// So few logits that launches are all that counts: the rows of a path are worked on by the blocks of one cluster, kRowsAtOnce a block at a
+// time, and the first block adds them up: one launch instead of two.  Rows in front of the first path and behind the last one go with
+// those.
+constexpr int kRowsAtOnce = 4;
+template <typename T>
+__global__ void __launch_bounds__(256 * kRowsAtOnce)
+path_scores_kernel(const T *logits, int64_t ld, const int32_t *targets, const int32_t *row_off, int n_rows, int vocab, const float *prior,
+                   const float *weight, float *row_logp, float *scores)
+{
+    __shared__ float sm[kRowsAtOnce][8], ss[kRowsAtOnce][8];
+    pdl_wait();
+    pdl_trigger();
+    const int path = blockIdx.y, rank = blockIdx.x, blocks = gridDim.x, group = threadIdx.x >> 8;
+    const int t0 = row_off[path], t1 = row_off[path + 1];
+    const int first = path == 0 ? 0 : max(t0, 0), last = path == (int)gridDim.y - 1 ? n_rows : min(t1, n_rows);
+    auto sync = [&]() { asm volatile("barrier.cta.sync %0, 256;" ::"r"(group + 1) : "memory"); };
+    for (int t = first + group * blocks + rank; t < last; t += blocks * kRowsAtOnce) {
+        score_row<T, 256>(logits, ld, t, targets[t], vocab, row_logp, threadIdx.x & 255, sm[group], ss[group], sync);
+        sync();                                             // the numbers of this row's warps have been read
+    }
+    if (blocks > 1) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    else __syncthreads();
+    if (rank == 0 && threadIdx.x < 32) path_sum(row_logp, path, t0, t1, prior, weight, scores);
 }
 
 }  // namespace sp
@@ -190,18 +225,25 @@ extern "C" int sp_path_scores(const void *logits, int64_t ld_logits, const int32
         rows_out = reinterpret_cast<float *>(static_cast<char *>(ws) + 256);
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (n_rows > 0) {
+    const auto go = [&](auto *p) {
+        using T = std::remove_const_t<std::remove_pointer_t<decltype(p)>>;
+        // One launch for up to 4 MB of logits.  us, two launches / one: a step of 4 paths x 8 rows of 512 (host-bound) 29.0 / 26.8, scores and
+        // top-k of 480 rows of 8 000 (8 MB) 11.4 / 11.2, of 32 000 12.3 / 17.2: blocks of four rows are too few to ask for all of it at once.
+        if (n_rows > 0 && n_rows <= 256 && n_paths <= 65535 && n_rows * vocab * (int64_t)sizeof(T) <= 4 << 20) {
+            const int64_t rows = (n_rows + n_paths - 1) / n_paths;
+            int blocks = 1;
+            while (blocks < 8 && blocks * kRowsAtOnce < rows) blocks *= 2;
+            return launch(path_scores_kernel<T>, dim3(blocks, n_paths), 256 * kRowsAtOnce, 0, st, blocks, p, ld_logits, targets, row_off, (int)n_rows, vocab,
+                          prior, weight, rows_out, scores);
+        }
         // Many rows: small blocks, of which more are in flight at different stages of a row; few rows: the block that is done with its
         // row sooner.  us with 128 / 256 threads: 30 720 rows 480 / 487, 30 720 short rows (8 000) 86 / 105, 1 920 rows 40 / 38, 480
         // rows 19.4 / 15.9.
         const bool many = n_rows >= 24 * (int64_t)num_sms();
-        auto go = [&](auto kern, auto *p) { return launch(kern, (unsigned)n_rows, many ? 128 : 256, 0, st, 1, p, ld_logits, targets, vocab, rows_out); };
-        auto pick = [&](auto *p) {
-            using T = std::remove_const_t<std::remove_pointer_t<decltype(p)>>;
-            return many ? go(row_logp_kernel<T, 128>, p) : go(row_logp_kernel<T, 256>, p);
-        };
-        const int rc = dtype == SP_BF16 ? pick(static_cast<const __nv_bfloat16 *>(logits)) : pick(static_cast<const float *>(logits));
-        if (rc) return rc;
-    }
-    return launch(path_sum_kernel, (n_paths + 7) / 8, 256, 0, st, 1, rows_out, row_off, n_paths, prior, weight, scores);
+        if (n_rows > 0)
+            if (int rc = launch(many ? row_logp_kernel<T, 128> : row_logp_kernel<T, 256>, (unsigned)n_rows, many ? 128 : 256, 0, st, 1, p, ld_logits, targets,
+                                vocab, rows_out)) return rc;
+        return launch(path_sum_kernel, (n_paths + 7) / 8, 256, 0, st, 1, rows_out, row_off, n_paths, prior, weight, scores);
+    };
+    return dtype == SP_BF16 ? go(static_cast<const __nv_bfloat16 *>(logits)) : go(static_cast<const float *>(logits));
 }

@@ -435,3 +435,26 @@ def test_decode_keys_through_a_ring(D, k, H, Hkv, n_prompts, longest):
     fin = np.isfinite(ref_l)
     np.testing.assert_allclose(outs[0][1][fin], ref_l[fin], atol=2e-2)
     np.testing.assert_array_equal(outs[0][1][~fin], ref_l[~fin])
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("lens,vocab", [([1], 5), ([4, 5], 700), ([8, 9, 16, 17, 33], 1001), ([100, 0, 1], 64), ([33] * 7, 2051), ([250, 6], 4096), ([257], 64)])
+def test_path_scores_in_one_launch(dtype, lens, vocab):
+    """The rows of a path over one to eight blocks of a cluster, four a block at a time; paths without rows, rows in front of the first and
+    behind the last path; a row more than one launch takes.  Bit-identical repeats; tolerance 1e-3 per row as in the parity suite."""
+    before, behind = 3, 2
+    off = np.concatenate([[before], before + np.cumsum(lens)]).astype(np.int32)
+    rows = int(off[-1]) + behind
+    logits = _randn((rows, vocab), 7, dtype) * 3
+    tgt = torch.randint(-1, vocab, (rows,), generator=torch.Generator().manual_seed(8), dtype=torch.int32)
+    prior, weight = _randn((len(lens),), 9, torch.float32), torch.full((len(lens),), 0.125)
+    ref_s, ref_r = oracle.path_scores(f32(logits), tgt.numpy(), off, prior.numpy(), weight.numpy())
+    got = []
+    for _ in range(2):
+        scores, row_logp = torch.full((len(lens),), float("nan"), device="cuda"), torch.full((rows,), float("nan"), device="cuda")
+        sp.sp_path_scores(dev(logits), dev(tgt), dev(off), scores, dev(prior), dev(weight), row_logp)
+        got.append((scores.cpu().numpy(), row_logp.cpu().numpy()))
+    np.testing.assert_array_equal(got[0][0], got[1][0])
+    want = torch.log_softmax(logits.double(), 1).gather(1, tgt.clamp(min=0).long()[:, None])[:, 0].masked_fill(tgt < 0, 0).numpy()
+    np.testing.assert_allclose(got[0][1], want, atol=1e-3)
+    np.testing.assert_allclose(got[0][0], ref_s, atol=1e-3 * max(max(lens), 1))
