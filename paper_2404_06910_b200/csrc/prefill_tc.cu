@@ -1021,8 +1021,10 @@ static int launch_tc(const void *q, const void *k, const void *v, const sp_layou
     pa.max_tiles = plan_max_tiles(lay->n_prompts, lay->n_paths, lay->max_pre_len, lay->max_path_len, 2 * pa.tile_rows);
     // the sort takes a microsecond: worth it from a dozen items per block
     pa.sort_from = 12 * num_sms() / (n_heads >> log_g);
-    // (not with the rotation folded in: Q is then where the output goes, and a row that has to be computed again would not find it)
-    const bool across = log_g == 0 && rows == SP_ROWS_ALL && !rope && across_pays(lay, n_heads);
+    // (not where the output takes Q's place, as it does with the rotation folded in: a row that has to be computed again would not find it)
+    const uintptr_t q_at = reinterpret_cast<uintptr_t>(q), out_at = reinterpret_cast<uintptr_t>(out), q_bytes = (uintptr_t)lay->total_tokens * q_cols * 2;
+    const bool over_q = rope || (out_at < q_at + q_bytes && q_at < out_at + q_bytes);
+    const bool across = log_g == 0 && rows == SP_ROWS_ALL && !over_q && across_pays(lay, n_heads);
     pa.hdr = hdr; pa.list = pairs;
     if (int rc = launch(across ? prefill_plan_kernel<true, true> : prefill_plan_kernel<true>, 1, 1024, 0, st, 1, pa)) return rc;
     if (pa.max_tiles == 0) return SP_OK;              // no segment can have a row

@@ -357,6 +357,32 @@ def test_prefill_tiles_across_paths_keep_values_to_their_path(D, alibi):
     assert np.abs(out0[others] - out1[others]).max() <= 2 ** -7 * np.abs(out0).max()
 
 
+@pytest.mark.parametrize("alibi", [False, True])
+def test_prefill_short_paths_with_the_output_in_place_of_the_queries(alibi):
+    """Output over the queries, with values that are not finite: nothing reads a row of queries again once its result is stored, so the
+    bits are those of tiles segment by segment (which a layout without its host mirror always gets) into a buffer of their own."""
+    lay = _short_paths(40, 4, 90, 24)
+    H, D, T = 20, 128, lay.total_tokens
+    q, k, v = (_randn((T, H, D), i) for i in (1, 2, 3))
+    v[int(lay.path_start[120])] = float("inf")
+    pos, slopes = torch.rand(T, generator=torch.Generator().manual_seed(4)).mul(300).float(), torch.linspace(0.01, 0.5, H)
+
+    def run(in_place):
+        dl = sp.DeviceLayout.from_host(lay, mirror=in_place)
+        ws = workspace(sp.sp_prefill_workspace_bytes(dl, H, D, sp.SP_BF16))
+        qd, lse = dev(q), torch.zeros((H, T), device="cuda")
+        out = qd if in_place else torch.zeros_like(qd)
+        if alibi:
+            sp.sp_superpose_prefill_alibi(qd, dev(k), dev(v), dl, dev(pos), dev(slopes), D ** -0.5, out, lse, ws)
+        else:
+            sp.sp_superpose_prefill(qd, dev(k), dev(v), dl, D ** -0.5, out, lse, ws)
+        sp.sp_check_status(ws)
+        return f32(out), lse.cpu().numpy()
+
+    for a, b in zip(run(True), run(False)):
+        np.testing.assert_array_equal(a, b)
+
+
 QRY_EDGES = [1, 8, 15, 16, 17, 31, 32, 33, 47, 48]
 
 
