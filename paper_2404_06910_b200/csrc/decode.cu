@@ -8,8 +8,9 @@
 // keeps an online softmax per key group and writes one partial (max, sum, unnormalised output)
 // per head into the shared memory of the cluster's first block, which merges them in split
 // order, so results do not depend on scheduling.  sp_pruned_decode_static merges through global
-// memory instead.  bf16 mostly runs on tensor-core instructions (decode_mma.cuh; rule and figures: mma_launch()); the kernel here serves fp32,
-// and bf16 with single heads where few keys per head start sooner in it or fill its waves.
+// memory instead.  bf16 mostly runs in decode_mma.cuh (K and V through rings in shared memory, grouped heads on tensor-core
+// instructions; rule and figures: mma_launch()); the kernel here serves fp32, and bf16 with single heads where few keys per head start sooner
+// in it or fill its waves.
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -679,7 +680,7 @@ static int launch_cluster_kernel(K kern, const DecodeArgs &a, const DecodeRope &
 }
 
 // bf16, which kernel; units: a prompt and a KV head's block of up to 8 query heads each.  us, cold reads, D = 128.
-//  - The tensor-core kernel with rings in shared memory: almost always.  What served it before (grouped heads: loads held in registers;
+//  - The kernel with rings in shared memory: almost always.  What served it before (grouped heads: loads held in registers;
 //    single heads: decode_cluster_kernel) / ring, 3 000 keys: 8 units 15.4 / 8.8, 32 18.8 / 13.5, 64 24.5 / 21.5, 192 65.4 / 54.2, 384 118 / 98;
 //    430 keys: 64 9.2 / 7.6, 192 15.2 / 12.0, 512 29.5 / 25.4; groups of 4, 3 000 keys: 32 18.6 / 16.4, 128 49.2 / 38.8, 256 87.9 / 66.4, 512
 //    136.5 / 125.7; 430 keys: 128 15.1 / 12.0, 512 27.6 / 26.0; groups of 2: 1 024 units 58.4 / 45.3.
@@ -739,7 +740,8 @@ static int launch_decode_mma(DecodeArgs a, const MmaLaunch &m, const DecodeRope 
 {
     const int group = a.n_heads / a.n_kv_heads, blocks_y = a.n_kv_heads * ((group + kMmaHeads - 1) / kMmaHeads);
     a.n_splits = m.n_splits;
-    const auto kern = m.ring ? decode_mma_kernel<D, ALIBI, ROPE, true> : decode_mma_kernel<D, ALIBI, ROPE, false>;
+    const auto kern = group == 1 ? decode_mma_kernel<D, ALIBI, ROPE, true, true>
+                                 : (m.ring ? decode_mma_kernel<D, ALIBI, ROPE, true, false> : decode_mma_kernel<D, ALIBI, ROPE, false, false>);
     return launch_cluster_kernel(kern, a, rope, pairing, blocks_y, n_prompts, 32 * m.warps, m.smem, st);
 }
 

@@ -1,5 +1,5 @@
-// One-token decode attention in bf16: both products on warp-level tensor-core instructions (mma.sync m16n8k16), for query heads that
-// share a KV head and for single ones.
+// One-token decode attention in bf16: for query heads that share a KV head both products on warp-level tensor-core instructions
+// (mma.sync m16n8k16), for single heads in fp32 arithmetic.
 //
 // With g query heads per KV head a step still reads every K and V row once, but the SIMT kernel pays 2 g D multiply-adds a
 // key, which bounds it long before HBM does (g = 4: 0.24 of the copy bandwidth).  Here a warp takes 16 keys at a time:
@@ -9,6 +9,9 @@
 // contiguous 16-byte pieces of K and V rows as fragments: no ldmatrix.  Only V needs a byte permute to pair two keys.  P is carried as
 // the sum of two bf16 numbers (16 bits of mantissa), so the result is as good as with fp32 products (1.6555e-3 of the norm from 64-bit
 // results with either, the rounding of the output), values that are not finite included.
+// Single heads, where the SIMT kernel's multiply-adds cost nothing that shows, keep its arithmetic: with the products above their
+// log-sum-exp was up to 4.6e-6 from 64 bits where it is 1.9e-6 now and was before, the output 3e-6 of its distance further off, at the same
+// times (2 prompts x 32 heads, 8 kept of long documents 16.4 us above, 16.7 so; 16 x 32 heads 23.1 / 23.1; D = 64 18.2 / 18.2).
 // What bounds it is latency: a turn of 16 keys is a chain of 0.65 us for a warp (products, maximum, exponentials), and where loads go to
 // registers nothing is in flight meanwhile.  So K and V rows run through a ring in shared memory (cp.async), two turns of 8 KB
 // ahead of a warp's arithmetic: 8 warps per SM keep 128 KB in flight.  Two chains of products for S instead of one and fewer instructions per
@@ -57,7 +60,8 @@ static __device__ const uint4 g_zero_row[16] = {};
 // Grid (n_splits, KV heads x blocks of up to 8 query heads, prompts); the n_splits blocks of a (prompt, y) are a cluster.
 // RING: K and V rows go through a ring in shared memory, two turns ahead of the arithmetic; otherwise a turn's loads go to registers
 // and nothing is in flight while a warp computes.
-template <int D, bool ALIBI, bool ROPE, bool RING>
+// SINGLE (with RING): one head to a KV head, in fp32 arithmetic: D / 8 lanes to a key, a running softmax per group of such lanes.
+template <int D, bool ALIBI, bool ROPE, bool RING, bool SINGLE>
 __global__ void __launch_bounds__(32 * kMmaMaxWarps, mma_warps_per_sm(D, RING) / kMmaMaxWarps)
 decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ DecodeRope rope, int rope_pairing)
 {
@@ -86,12 +90,18 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
         red = reinterpret_cast<float *>(rings);
     }
 
+    constexpr int LPK = D / 8, KG = 32 / LPK;                   // SINGLE: lanes to a key, groups of them
+    const int sub = lane % LPK, kg = lane / LPK;
+
     decode_cluster_begin(a);
     pdl_wait();
     uint4 qf[NC];                            // query head h0 + gid, unscaled bf16; on its way while the table is built
+    uint4 q1 = make_uint4(0u, 0u, 0u, 0u);   // SINGLE: its piece `sub`
 #pragma unroll
     for (int c = 0; c < NC; ++c) qf[c] = make_uint4(0u, 0u, 0u, 0u);
-    if (gid < nh) {
+    if (SINGLE) {
+        q1 = reinterpret_cast<const uint4 *>(static_cast<const T *>(a.q) + ((int64_t)b * a.n_heads + h0) * D)[sub];
+    } else if (gid < nh) {
         const uint4 *src = reinterpret_cast<const uint4 *>(static_cast<const T *>(a.q) + ((int64_t)b * a.n_heads + h0 + gid) * D);
 #pragma unroll
         for (int c = 0; c < NC; ++c) qf[c] = src[tig + 4 * c];
@@ -141,13 +151,80 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
         }
     };
 
-    if (ROPE) rotate(qf);
+    // SINGLE: the same for the eight elements of piece `sub`, rounded as they are stored
+    auto rotate1 = [&](uint4 &x) {
+        uint32_t *wd = reinterpret_cast<uint32_t *>(&x);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            float n0, n1;
+            if (rope_pairing == SP_ROPE_HALF_SPLIT) {
+                const bool upper = sub >= LPK / 2;
+                const uint32_t other = __shfl_xor_sync(0xffffffffu, wd[e], LPK / 2), lo_w = upper ? other : wd[e], hi_w = upper ? wd[e] : other;
+                const float2 w0 = cs[8 * (sub % (LPK / 2)) + 2 * e], w1 = cs[8 * (sub % (LPK / 2)) + 2 * e + 1];
+                float n2, n3;
+                rope_rotate(bf16_lo(lo_w), bf16_lo(hi_w), w0.x, w0.y, n0, n2);
+                rope_rotate(bf16_hi(lo_w), bf16_hi(hi_w), w1.x, w1.y, n1, n3);
+                if (upper) { n0 = n2; n1 = n3; }
+            } else {
+                const float2 w = cs[4 * sub + e];
+                rope_rotate(bf16_lo(wd[e]), bf16_hi(wd[e]), w.x, w.y, n0, n1);
+            }
+            wd[e] = pack_bf16x2(n0, n1);
+        }
+    };
+
+    if (ROPE && !SINGLE) rotate(qf);
+    if (ROPE && SINGLE) rotate1(q1);
+    float qs[8], acc[8];                     // SINGLE: the query's elements in log2 units, the group's output
+    Raw16<T>::unpack(q1, qs);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) { qs[e] *= a.scale_log2e; acc[e] = 0.f; }
 
     float m = -INFINITY, l = 0.f, o[NM][4];  // head gid: maximum, this thread's share of the sum; O^T rows, heads 2 tig, + 1
 #pragma unroll
     for (int i = 0; i < NM; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
     const float q_pos = ALIBI ? a.q_pos[b] : 0.f;
-    const float slope_l2 = (ALIBI && gid < nh) ? a.slopes[h0 + gid] * kLog2eD : 0.f;
+    const float slope_l2 = (ALIBI && (SINGLE || gid < nh)) ? a.slopes[h0 + (SINGLE ? 0 : gid)] * kLog2eD : 0.f;
+
+    // SINGLE: N keys to a group of lanes, their pieces `sub` in kr and vr; key u exists where u < n.
+    auto attend1 = [&](const auto &kr, const auto &vr, const auto &kpos, int n) {
+        constexpr int N = sizeof(kr) / sizeof(kr[0]);
+        float x[N], top = -INFINITY;
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            float kf[8];
+            Raw16<T>::unpack(kr[u], kf);
+            x[u] = 0.f;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) x[u] = fmaf(qs[e], kf[e], x[u]);
+        }
+#pragma unroll
+        for (int s = LPK / 2; s > 0; s >>= 1)
+#pragma unroll
+            for (int u = 0; u < N; ++u) x[u] += __shfl_xor_sync(0xffffffffu, x[u], s);
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            if (ALIBI) x[u] -= slope_l2 * fabsf(q_pos - kpos[u]);
+            if (u >= n) x[u] = -INFINITY;
+            top = fmaxf(top, x[u]);
+        }
+        if (top > m) {
+            const float r = ex2f(m - top);
+            l *= r;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] *= r;
+            m = top;
+        }
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            const float p = u < n ? ex2f(x[u] - m) : 0.f;
+            float vf[8];
+            Raw16<T>::unpack(vr[u], vf);
+            l += p;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] = fmaf(p, vf[e], acc[e]);
+        }
+    };
 
     // 16 keys: kr = K rows gid, gid + 8; vr = V rows 2 tig, 2 tig + 1, 2 tig + 8, 2 tig + 9.  n: keys that exist.
     auto attend = [&](const uint4 (&kr)[2][NC], const uint4 (&vr)[4][NV], int n, float kpos) {
@@ -250,19 +327,33 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
             __syncwarp();                                           // every lane's copies have landed, and the turn before this one has been read
             fetch(base + (kMmaStages - 1) * W * kMmaKeys, stage == 0 ? kMmaStages - 1 : stage - 1);
             const unsigned char *kt = ring + stage * MmaRing<D>::STAGE, *vt = kt + MmaRing<D>::V;
-            uint4 kr[2][NC], vr[4][NV];
-#pragma unroll
-            for (int t = 0; t < 2; ++t)
-#pragma unroll
-                for (int c = 0; c < NC; ++c) kr[t][c] = *reinterpret_cast<const uint4 *>(kt + (gid + 8 * t) * MmaRing<D>::ROW + (((tig + 4 * c) ^ ((gid & 1) << 2)) << 4));
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const int r = 2 * tig + (t & 1) + 8 * (t >> 1);
-#pragma unroll
-                for (int c = 0; c < NV; ++c) vr[t][c] = *reinterpret_cast<const uint4 *>(vt + r * MmaRing<D>::ROW + (((gid + 8 * c) ^ (r & 6)) << 4));
-            }
-            attend(kr, vr, min(kMmaKeys, hi_loop - base), ALIBI ? *reinterpret_cast<const float *>(kt + MmaRing<D>::POS + (lane & 15) * 4) : 0.f);
             if (++stage == kMmaStages) stage = 0;
+            if constexpr (SINGLE) {                                 // group kg: rows kg, kg + KG, ..
+                constexpr int N = kMmaKeys / KG;
+                uint4 kr[N], vr[N];
+                float kpos[N];
+#pragma unroll
+                for (int u = 0; u < N; ++u) {
+                    const int r = kg + u * KG;
+                    kr[u] = *reinterpret_cast<const uint4 *>(kt + r * MmaRing<D>::ROW + ((sub ^ ((r & 1) << 2)) << 4));
+                    vr[u] = *reinterpret_cast<const uint4 *>(vt + r * MmaRing<D>::ROW + ((sub ^ (r & 6)) << 4));
+                    kpos[u] = ALIBI ? *reinterpret_cast<const float *>(kt + MmaRing<D>::POS + r * 4) : 0.f;
+                }
+                attend1(kr, vr, kpos, (min(kMmaKeys, hi_loop - base) - kg + KG - 1) / KG);
+            } else {
+                uint4 kr[2][NC], vr[4][NV];
+#pragma unroll
+                for (int t = 0; t < 2; ++t)
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) kr[t][c] = *reinterpret_cast<const uint4 *>(kt + (gid + 8 * t) * MmaRing<D>::ROW + (((tig + 4 * c) ^ ((gid & 1) << 2)) << 4));
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    const int r = 2 * tig + (t & 1) + 8 * (t >> 1);
+#pragma unroll
+                    for (int c = 0; c < NV; ++c) vr[t][c] = *reinterpret_cast<const uint4 *>(vt + r * MmaRing<D>::ROW + (((gid + 8 * c) ^ (r & 6)) << 4));
+                }
+                attend(kr, vr, min(kMmaKeys, hi_loop - base), ALIBI ? *reinterpret_cast<const float *>(kt + MmaRing<D>::POS + (lane & 15) * 4) : 0.f);
+            }
         }
         cp_async_wait<0>();
         __syncthreads();                                        // the rings are done with
@@ -293,7 +384,15 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
         }
     }
 
-    if (mine_new) {
+    if (SINGLE && mine_new) {                                // as below
+        uint4 *krow = reinterpret_cast<uint4 *>(const_cast<T *>(sm.k[n_seg - 1]) + new_off);
+        uint4 kr[1] = {krow[sub]}, vr[1] = {reinterpret_cast<const uint4 *>(sm.v[n_seg - 1] + new_off)[sub]};
+        const float kpos[1] = {0.f};
+        rotate1(kr[0]);
+        __syncwarp();
+        if (kg == 0) krow[sub] = kr[0];
+        attend1(kr, vr, kpos, kg == 0 ? 1 : 0);
+    } else if (mine_new) {
         // The newest key: rotated, rounded and written back for the later steps, then one more turn with one key.
         uint4 *krow = reinterpret_cast<uint4 *>(const_cast<T *>(sm.k[n_seg - 1]) + new_off);
         const uint4 *vrow = reinterpret_cast<const uint4 *>(sm.v[n_seg - 1] + new_off);
@@ -316,16 +415,39 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
     }
 
     // ---- combine the warps of this block (fixed order) --------------------------------
-    l += __shfl_xor_sync(0xffffffffu, l, 1);
-    l += __shfl_xor_sync(0xffffffffu, l, 2);
+    if constexpr (SINGLE) {                                  // the groups of this warp first
+        float top = m;
 #pragma unroll
-    for (int r = 0; r < 2; ++r)
-        if (2 * tig + r < nh) {
-            float *mine = red + (warp * nh + 2 * tig + r) * PS + 8 * gid;
+        for (int s = LPK; s < 32; s <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, s));
+        const float r = m == -INFINITY ? 0.f : ex2f(m - top);
+        m = top;
+        l *= r;
 #pragma unroll
-            for (int i = 0; i < NM; ++i) { mine[i] = o[i][r]; mine[D == 128 ? i + 64 : i + 4] = o[i][2 + r]; }
+        for (int e = 0; e < 8; ++e) acc[e] *= r;
+#pragma unroll
+        for (int s = LPK; s < 32; s <<= 1) {
+            l += __shfl_xor_sync(0xffffffffu, l, s);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], s);
         }
-    if (tig == 0 && gid < nh) { red[(warp * nh + gid) * PS + D] = m; red[(warp * nh + gid) * PS + D + 1] = l; }
+        float *mine = red + warp * PS;
+        if (kg == 0) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) mine[sub * 8 + e] = acc[e];
+        }
+        if (lane == 0) { mine[D] = m; mine[D + 1] = l; }
+    } else {
+        l += __shfl_xor_sync(0xffffffffu, l, 1);
+        l += __shfl_xor_sync(0xffffffffu, l, 2);
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+            if (2 * tig + r < nh) {
+                float *mine = red + (warp * nh + 2 * tig + r) * PS + 8 * gid;
+#pragma unroll
+                for (int i = 0; i < NM; ++i) { mine[i] = o[i][r]; mine[D == 128 ? i + 64 : i + 4] = o[i][2 + r]; }
+            }
+        if (tig == 0 && gid < nh) { red[(warp * nh + gid) * PS + D] = m; red[(warp * nh + gid) * PS + D + 1] = l; }
+    }
     __syncthreads();
 
     float *mine = decode_cluster_target(a, part, nh * PS);

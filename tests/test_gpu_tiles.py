@@ -463,6 +463,37 @@ def test_decode_keys_through_a_ring(D, k, H, Hkv, n_prompts, longest):
     np.testing.assert_array_equal(outs[0][1][~fin], ref_l[~fin])
 
 
+@pytest.mark.parametrize("H,D", [(32, 128), (40, 64)])
+@pytest.mark.parametrize("alibi", [False, True])
+def test_decode_single_heads_in_fp32_arithmetic(H, D, alibi):
+    """Scores, probabilities and sums of single heads in bf16 are fp32 numbers.  An error of 2^-22 puts an output on the other side of a
+    rounding boundary, bf16 numbers being 2^-8 apart, in one of 2^13 cases, 0.012 %; four times that are allowed.  Probabilities cut off behind 16
+    bits came to 0.27 and 0.31 %."""
+    rng = np.random.default_rng(0)
+    lay = build_layout([64, 64], [[int(x) for x in rng.integers(128, 513, 8)] for _ in range(2)], [[24] * 8] * 2)
+    T, cap, k = lay.total_tokens, 256, 8
+    q, kc, vc, tk, tv = _randn((2, H, D), 1), _randn((T, H, D), 2), _randn((T, H, D), 3), _randn((2, cap, H, D), 4), _randn((2, cap, H, D), 5)
+    kept, tl = np.arange(16, dtype=np.int32).reshape(2, 8), np.array([200, 31], np.int32)
+    q_pos, pos, tail_pos = torch.tensor([700.0, 650.0]), torch.rand(T, generator=torch.Generator().manual_seed(6)) * 600, torch.full((2, cap), 640.0)
+    slopes = torch.exp2(-8.0 * (torch.arange(H) + 1) / H).float()
+    out, lse = torch.zeros((2, H, D), dtype=torch.bfloat16, device="cuda"), torch.zeros((2, H), device="cuda")
+    args = (dev(q), dev(kc), dev(vc), sp.DeviceLayout.from_host(lay), dev(kept), k, dev(tk), dev(tv), dev(tl), cap)
+    ws = workspace(sp.sp_decode_workspace_bytes(2, H, D))
+    if alibi:
+        sp.sp_pruned_decode_alibi(*args, dev(q_pos), dev(pos), dev(tail_pos), dev(slopes), D ** -0.5, out, lse, ws)
+    else:
+        sp.sp_pruned_decode(*args, D ** -0.5, out, lse, ws)
+    wrong = 0
+    for b in range(2):
+        (lo, hi), n = lay.prompt_row_range(b), int(tl[b])
+        keys, values = torch.cat([kc[lo:hi], tk[b, :n]]).double(), torch.cat([vc[lo:hi], tv[b, :n]]).double()
+        s = torch.einsum("hd,khd->hk", q[b].double(), keys) * D ** -0.5
+        if alibi:
+            s -= slopes.double()[:, None] * (q_pos[b].double() - torch.cat([pos[lo:hi], tail_pos[b, :n]]).double()).abs()
+        wrong += int((out[b].cpu() != torch.einsum("hk,khd->hd", torch.softmax(s, 1), values).float().bfloat16()).sum())
+    assert wrong <= 5e-4 * 2 * H * D
+
+
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("lens,vocab", [([1], 5), ([4, 5], 700), ([8, 9, 16, 17, 33], 1001), ([100, 0, 1], 64), ([33] * 7, 2051), ([250, 6], 4096), ([257], 64)])
 def test_path_scores_in_one_launch(dtype, lens, vocab):
