@@ -140,8 +140,8 @@ int sp_rope_apply_pair(void *xq, int64_t ld_q, int n_heads_q, void *xk, int64_t 
  * of every path (the cached, online case of Algorithm 3); other rows of out are untouched.
  * head_dim in {64, 128}.  SP_BF16 runs on the tensor cores: the softmax probabilities are
  * rounded to bf16 before the second product with head_dim 128, carried as the sum of two bf16
- * numbers with head_dim 64 and with SP_ROWS_QUERY_ONLY (there, with many paths of at most 640 keys
- * behind at most 128 preamble rows: for the first keys only).  SP_F32 runs an fp32 SIMT kernel.
+ * numbers with head_dim 64 and with SP_ROWS_QUERY_ONLY (there, without ALiBi and with many paths of at
+ * most 640 keys behind at most 128 preamble rows: for the first keys only).  SP_F32 runs an fp32 SIMT kernel.
  * ws: at least sp_prefill_workspace_bytes() bytes, 256-byte aligned.
  */
 size_t sp_prefill_workspace_bytes(int n_prompts, int n_paths, int max_pre_len, int max_path_len,

@@ -41,10 +41,12 @@ namespace sp {
 //    48 rows 734 / 553, behind 600 2270 / 1290; ALiBi 32 rows 762 / 480, 48 rows 792 / 718; 1 prompt x 20 documents 22.0 / 17.4.
 // The number of query rows is known from the host mirror only; without one the kernel for all rows, but for many items behind a preamble
 // from which on it loses more than the other one does with more than 48 rows.
-// P as two bf16 numbers, but with many items (path, head) of a few key tiles: there it is one number except for an item's first 32
-// keys, which is as exact as what served them before (2.09e-3 of the norm from 64-bit results at 8 x 100 documents behind 48 rows, 2.13e-3
-// before; two numbers 1.66e-3) and 0 to 3 % faster (documents of 32-64 rows 100.5 / 104.0 us, ALiBi 476 / 480).  With more key tiles
-// the running maximum it needs costs more than the second number (behind 384 rows 836 / 721).
+// P as two bf16 numbers, but without a bias and with many items (path, head) of a few key tiles: there it is one number except for an
+// item's first 32 keys, which is more exact than what served them before (of the norm from 64-bit results, 40 prompts of 10 or 20
+// documents: 2.01e-3 to 2.14e-3, 2.09e-3 to 2.16e-3 before; two numbers 1.66e-3) and 0 to 3 % faster (documents of 32-64 rows 100.5 / 104.0 us).
+// With more key tiles the running maximum it needs costs more than the second number (behind 384 rows 836 / 721).  Under ALiBi the
+// weight is on the nearest keys, which 32 fixed ones do not catch: 1.82e-3 to 1.89e-3 where it was 1.88e-3 before; two numbers 1.66e-3, at up
+// to 3 % of the time (behind 48 rows 474 / 476, documents of 40 rows 259 / 267).
 static int qonly_rows(const sp_layout *lay, bool alibi, int n_heads, int n_kv_heads)      // 0: the kernel for all rows
 {
     if (n_heads / n_kv_heads % 2 == 0) return 0;
@@ -53,9 +55,9 @@ static int qonly_rows(const sp_layout *lay, bool alibi, int n_heads, int n_kv_he
     for (int i = 0; i < lay->n_paths; ++i) longest = std::max(longest, lay->host_mirror->qry_len[i]);
     return longest <= 48 ? longest : 0;
 }
-static bool qonly_split(const sp_layout *lay, int n_heads)
+static bool qonly_split(const sp_layout *lay, bool alibi, int n_heads)
 {
-    return (int64_t)lay->n_paths * n_heads <= 9 * (int64_t)num_sms() || lay->max_pre_len > 128 || (int64_t)lay->max_pre_len + lay->max_path_len > 640;
+    return alibi || (int64_t)lay->n_paths * n_heads <= 9 * (int64_t)num_sms() || lay->max_pre_len > 128 || (int64_t)lay->max_pre_len + lay->max_path_len > 640;
 }
 
 static int prefill_entry(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
@@ -83,7 +85,7 @@ static int prefill_entry(const void *q, const void *k, const void *v, const sp_l
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (dtype == SP_BF16 && head_dim == 128 && rows == SP_ROWS_QUERY_ONLY)
         if (const int longest = qonly_rows(lay, pos != nullptr, n_heads, n_kv_heads))
-            return launch_prefill_qonly(q, k, v, lay, pos, slopes, n_heads, n_kv_heads, scale, longest, qonly_split(lay, n_heads), out, lse, ws, st);
+            return launch_prefill_qonly(q, k, v, lay, pos, slopes, n_heads, n_kv_heads, scale, longest, qonly_split(lay, pos != nullptr, n_heads), out, lse, ws, st);
     // bf16 goes to the tensor cores for both head sizes (head_dim 64, 8 prompts x 20 documents, 32 heads: 0.17 ms; the fp32
     // SIMT kernel, which served it before, took 9.4 ms)
     if (dtype == SP_BF16)

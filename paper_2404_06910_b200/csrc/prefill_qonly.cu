@@ -11,8 +11,8 @@
 // clk of an SM's share of HBM: K and V stages are all that has to be kept in flight.
 // Work item: the query rows of one path (at most NQ) and a head, heads fastest, one persistent block per SM.  Items alternate
 // between two softmax warpgroups ("lanes") with S^T, P^T and O^T of their own; loads and products run in item order.
-// P is (SPLIT) the sum of two bf16 numbers, side by side as columns of one product, or one number relative to the running maximum and
-// two for an item's first 32 keys (the rule, and what both cost: prefill.cu).
+// P is (SPLIT) the sum of two bf16 numbers, side by side as columns of one product, or, without a bias, one number relative to the running
+// maximum and two for an item's first 32 keys (the rule, and what both cost: prefill.cu).
 // Measured (32 heads, 8 x 100 documents of 64-256 rows behind 48): 470 us = 0.95 of the copy bandwidth, 610 with warp-level products
 // (mma.sync, two warps to a scheduler, the chain product - softmax - product exposed); 48 rows 553 us = 0.93.
 // Behind long preambles (384 rows: 724 us, 456 at the copy bandwidth) it is bound by what L2 gives the SMs, 10 TB/s: every
@@ -585,12 +585,14 @@ template <int NQ, bool SPLIT> static int launch_qonly(QoParams &p, const void *q
 {
     using C = QoConfig<NQ, SPLIT>;
     if (int rc = encode_rows_map(&p.q, q, p.total_tokens, (int64_t)p.n_heads * 128, NQ, 1)) return rc;
-    auto kern = p.pos ? prefill_qonly_kernel<NQ, SPLIT, true> : prefill_qonly_kernel<NQ, SPLIT, false>;
+    auto kern = prefill_qonly_kernel<NQ, SPLIT, false>;
+    if constexpr (SPLIT)
+        if (p.pos) kern = prefill_qonly_kernel<NQ, SPLIT, true>;
     SP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
     return launch(kern, grid, kQThreads, C::SMEM, st, 1, p);
 }
 
-// longest: query rows of a path at most; split: P as the sum of two bf16 numbers (always with more than 32 rows)
+// longest: query rows of a path at most; split: P as the sum of two bf16 numbers (always with more than 32 rows and with ALiBi)
 int launch_prefill_qonly(const void *q, const void *k, const void *v, const sp_layout *lay, const float *pos,
                          const float *slopes, int n_heads, int n_kv_heads, float scale, int longest, bool split, void *out,
                          float *lse, void *ws, cudaStream_t st)
