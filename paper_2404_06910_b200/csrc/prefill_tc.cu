@@ -217,61 +217,105 @@ template <int N> struct Ring {        // stage and parity of a ring of N barrier
     __device__ __forceinline__ void next() { skip(1); }
 };
 
-// One row (key number `last`, own keys from number `from` up; dst: where this thread has stored it) in fp32 arithmetic over exactly the
-// keys it sees: its values that are not finite are replaced.  Rare, so small: 16 bytes at a time.  For tiles across paths; in place of
-// exact_row64 it made head_dim 64 with ALiBi slower (16 prompts x 20 documents 388 -> 403 us).
-template <int D, bool ALIBI>
-__device__ __forceinline__ void exact_row(const TcParams &p, const TcPair &t, int head, int kv_head, int from, int last, unsigned char *dst)
+// ---- rows with values that are not finite ------------------------------------------------
+// Keys that a row does not see have a P of exactly zero, but 0 x Inf and 0 x NaN reach O.  Where such keys share tiles with those it does
+// see, the row's values that are not finite are computed again, in fp32 over exactly the keys it sees, by the row's warp: a lane takes
+// every 32nd key's score, then D / 32 columns of the sums.  Not where nothing hidden can be the cause: a value of the preamble or of the row's
+// own keys belongs there.  A row of 740 keys takes its warp 36 us; a look at the rows alone doubles a launch's time.
+// A lane's columns of a row: D / 64 words of two bf16 numbers each.
+template <int D> struct Words {
+    uint32_t w[D / 64];
+    __device__ __forceinline__ void load(const void *row)
+    {
+        if constexpr (D == 128) { const uint2 x = static_cast<const uint2 *>(row)[threadIdx.x & 31]; w[0] = x.x; w[1] = x.y; }
+        else w[0] = static_cast<const uint32_t *>(row)[threadIdx.x & 31];
+    }
+    __device__ __forceinline__ void store(void *row) const
+    {
+        if constexpr (D == 128) static_cast<uint2 *>(row)[threadIdx.x & 31] = make_uint2(w[0], w[1]);
+        else static_cast<uint32_t *>(row)[threadIdx.x & 31] = w[0];
+    }
+};
+// Ones in the halves of a word that are not finite, or NaN.
+__device__ __forceinline__ uint32_t not_finite(uint32_t x)
 {
+    return ((x & 0x7f80u) == 0x7f80u ? 0xffffu : 0u) | ((x & 0x7f800000u) == 0x7f800000u ? 0xffff0000u : 0u);
+}
+__device__ __forceinline__ uint32_t is_nan(uint32_t x) { return ((x & 0x7fffu) > 0x7f80u ? 0xffffu : 0u) | ((x & 0x7fff0000u) > 0x7f800000u ? 0xffff0000u : 0u); }
+template <int D> __device__ __forceinline__ const __nv_bfloat16 *value_row(const TcParams &p, int64_t row, int kv_head) { return p.v + (row * p.n_kv_heads + kv_head) * D; }
+
+// The first and the last of the segment's keys [u0, u1) whose values are not all finite.
+template <int D>
+__device__ __forceinline__ void bad_values(const TcParams &p, const TcPair &t, int kv_head, int u0, int u1, int &first, int &last)
+{
+    constexpr int PIECES = D / 8;                        // of 16 bytes in a row
+    const int lane = threadIdx.x & 31;
+    first = INT_MAX; last = -1;
+#pragma unroll 8
+    for (int u = u0 + lane / PIECES; u < u1; u += 32 / PIECES) {
+        const uint4 v = reinterpret_cast<const uint4 *>(value_row<D>(p, t.own_base + u, kv_head))[lane % PIECES];
+        if (not_finite(v.x) | not_finite(v.y) | not_finite(v.z) | not_finite(v.w)) { first = min(first, u); last = u; }
+    }
+    first = __reduce_min_sync(0xffffffffu, first);
+    last = __reduce_max_sync(0xffffffffu, last);
+}
+
+// The row with key number `last`, whose own keys start at number `from`; y: its columns of this lane.
+template <int D, bool ALIBI>
+__device__ __forceinline__ void exact_row(const TcParams &p, const TcPair &t, int head, int kv_head, int from, int last, Words<D> &y)
+{
+    const int lane = threadIdx.x & 31, n = t.pre_len + last - from + 1;
     const int64_t own = t.own_base + last;
+    Words<D> v;
+    v.load(value_row<D>(p, own, kv_head));
+    bool cause = false;                                  // a NaN of the row's own value is its own
+#pragma unroll
+    for (int i = 0; i < D / 64; ++i) cause |= (not_finite(y.w[i]) & ~is_nan(v.w[i])) != 0u;
+    if (!__any_sync(0xffffffffu, cause)) return;
     const uint4 *q = reinterpret_cast<const uint4 *>(p.q + (own * p.n_heads + head) * D);
     const float pq = ALIBI ? p.pos[own] : 0.f, slope = ALIBI ? p.slopes[head] * kLog2eT : 0.f;
-    auto packed_row = [&](int u) { return (int64_t)u + (u < t.pre_len ? t.pre_row : t.own_base); };
-    auto score = [&](int64_t row) {
+    auto packed_row = [&](int i) { return (int64_t)i + (i < t.pre_len ? t.pre_row : t.own_base + from - t.pre_len); };
+    float m = -INFINITY, l = 0.f, acc[D / 32];
+#pragma unroll
+    for (int e = 0; e < D / 32; ++e) acc[e] = 0.f;
+#pragma unroll 1
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        const int64_t row = packed_row(min(i0 + lane, n - 1));
         const uint4 *k = reinterpret_cast<const uint4 *>(p.k + (row * p.n_kv_heads + kv_head) * D);
         float s = 0.f;
-#pragma unroll 1
+#pragma unroll 4
         for (int c = 0; c < D / 8; ++c) {
-            const uint4 x = q[c], y = k[c];
-            s = fmaf(bf16_lo(x.x), bf16_lo(y.x), s); s = fmaf(bf16_hi(x.x), bf16_hi(y.x), s);
-            s = fmaf(bf16_lo(x.y), bf16_lo(y.y), s); s = fmaf(bf16_hi(x.y), bf16_hi(y.y), s);
-            s = fmaf(bf16_lo(x.z), bf16_lo(y.z), s); s = fmaf(bf16_hi(x.z), bf16_hi(y.z), s);
-            s = fmaf(bf16_lo(x.w), bf16_lo(y.w), s); s = fmaf(bf16_hi(x.w), bf16_hi(y.w), s);
+            const uint4 x = q[c], z = k[c];
+            s = fmaf(bf16_lo(x.x), bf16_lo(z.x), s); s = fmaf(bf16_hi(x.x), bf16_hi(z.x), s);
+            s = fmaf(bf16_lo(x.y), bf16_lo(z.y), s); s = fmaf(bf16_hi(x.y), bf16_hi(z.y), s);
+            s = fmaf(bf16_lo(x.z), bf16_lo(z.z), s); s = fmaf(bf16_hi(x.z), bf16_hi(z.z), s);
+            s = fmaf(bf16_lo(x.w), bf16_lo(z.w), s); s = fmaf(bf16_hi(x.w), bf16_hi(z.w), s);
         }
         s *= p.scale_log2e;
-        return ALIBI ? s - slope * fabsf(pq - p.pos[row]) : s;
-    };
-    float m = -INFINITY, l = 0.f;
-#pragma unroll 1
-    for (int u = 0; u <= last; ++u) {
-        if (u >= t.pre_len && u < from) continue;
-        const float s = score(packed_row(u));
-        if (s > m) { l *= ex2(m - s); m = s; }
-        l += ex2(s - m);
+        if (ALIBI) s -= slope * fabsf(pq - p.pos[row]);
+        if (i0 + lane >= n) s = -INFINITY;
+        const float m_new = fmaxf(m, warp_max(s)), ref = m_new == -INFINITY ? 0.f : m_new, a = ex2(m - ref), w = ex2(s - ref);
+        m = m_new;
+        l = fmaf(l, a, warp_sum(w));
+#pragma unroll
+        for (int e = 0; e < D / 32; ++e) acc[e] *= a;
+        const int here = min(32, n - i0);
+#pragma unroll 8
+        for (int j = 0; j < here; ++j) {
+            const float wj = __shfl_sync(0xffffffffu, w, j);
+            v.load(value_row<D>(p, packed_row(i0 + j), kv_head));
+#pragma unroll
+            for (int i = 0; i < D / 64; ++i) {
+                acc[2 * i] = fmaf(wj, bf16_lo(v.w[i]), acc[2 * i]);
+                acc[2 * i + 1] = fmaf(wj, bf16_hi(v.w[i]), acc[2 * i + 1]);
+            }
+        }
     }
     const float inv = 1.f / l;
-#pragma unroll 1
-    for (int c = 0; c < D / 8; ++c) {
-        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll 1
-        for (int u = 0; u <= last; ++u) {
-            if (u >= t.pre_len && u < from) continue;
-            const int64_t row = packed_row(u);
-            const float w = ex2(score(row) - m);
-            float v[8];
-            Vec<__nv_bfloat16>::load(p.v + (row * p.n_kv_heads + kv_head) * D + c * 8, v);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) acc[e] = fmaf(w, v[e], acc[e]);
-        }
-        uint4 *at = reinterpret_cast<uint4 *>(dst) + c, o = *at;
-        uint32_t *y = reinterpret_cast<uint32_t *>(&o);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {                    // the finite ones are right as they are
-            const uint32_t x = pack_bf16x2(acc[2 * i] * inv, acc[2 * i + 1] * inv);
-            if ((y[i] & 0x7f80u) == 0x7f80u) y[i] = (y[i] & 0xffff0000u) | (x & 0xffffu);
-            if ((y[i] & 0x7f800000u) == 0x7f800000u) y[i] = (y[i] & 0xffffu) | (x & 0xffff0000u);
-        }
-        *at = o;
+    for (int i = 0; i < D / 64; ++i) {                   // the finite ones are right as they are
+        const uint32_t again = not_finite(y.w[i]);
+        y.w[i] = (y.w[i] & ~again) | (pack_bf16x2(acc[2 * i] * inv, acc[2 * i + 1] * inv) & again);
     }
 }
 
@@ -786,6 +830,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
         const int quad = warp - WARP_EPI, row = quad * 32 + lane;
         const int hr = row & ((1 << log_rows) - 1), hr0 = quad * 32 & ((1 << log_rows) - 1);
         uint32_t ph = 0, g[2] = {0, 0};                  // tiles so far, mod 2, a bit per lane; key tiles so far
+        bool not_all_finite = false;                     // ACROSS: some value that this thread has stored is not finite
 #pragma unroll 1
         for (Walk w(p); ok && w.next();) {
 #pragma unroll 1
@@ -849,16 +894,45 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                         }
                     }
                 }
-                // Hidden keys have a P of exactly zero, but 0 x Inf and 0 x NaN reach O: with head_dim 64 (as precise as fp32 arithmetic) and
-                // where a tile holds keys of paths that a row does not see, a row with a value that is not finite is computed again over
-                // its own keys.  The look at the row costs nothing that shows; looking through the V tiles instead cost the ALiBi variant
-                // 14 % (one more warp on the SM partition of two softmax warps).
-                if (ACROSS && hr < t.rows && (nan & 0x7fff7fffu)) {
-                    int start = w.t.own_base + w.t.p16;                    // of the row's own path
-                    const int row_p = w.t.own_base + t.q_u + hr;
-                    if (ACROSS && w.first_path >= 0)
-                        for (int i = w.first_path + 1; i < p.n_paths && p.path_start[i] > start && p.path_start[i] <= row_p; ++i) start = p.path_start[i];
-                    exact_row<D, ALIBI>(p, w.t, (w.h << (7 - log_rows)) + (row >> log_rows), w.h / p.units_per_kv, start - w.t.own_base, t.q_u + hr, dst);
+                not_all_finite |= hr < t.rows && (nan & 0x7fff7fffu);
+            }
+        }
+        if (ACROSS && ok && __any_sync(0xffffffffu, not_all_finite)) {
+            // Rows that other paths' values may have reached, once more: behind the last item, when no other warp waits for this one, and from
+            // the stored output, in which the rows that one warp has written are its own.
+#pragma unroll 1
+            for (Walk w(p); w.next();) {
+                // rows of one segment meet only their own later rows, head_dim 128: as in a launch without tiles across paths
+                if (D == 128 && w.first_path < 0) continue;
+#pragma unroll 1
+                for (int b = 0; b < w.n_q(); ++b) {
+                    const LaneTile t(w, w.lane_a() ^ b);
+                    const int kv_head = w.h / p.units_per_kv, row0 = w.t.own_base + t.q_u + quad * 32, n = min(32, t.rows - quad * 32);
+                    auto out_row = [&](int r) { return p.out + ((int64_t)(row0 + r) * p.n_heads + w.h) * D; };
+                    uint32_t rows = 0u;                  // a bit per row with values that are not finite
+#pragma unroll 4
+                    for (int r = 0; r < n; ++r) {
+                        Words<D> y;
+                        y.load(out_row(r));
+#pragma unroll
+                        for (int i = 0; i < D / 64; ++i) rows |= not_finite(y.w[i]) ? 1u << r : 0u;
+                    }
+                    rows = __reduce_or_sync(0xffffffffu, rows);
+                    int bad_first = INT_MAX, bad_last = -1;
+                    if (rows) bad_values<D>(p, w.t, kv_head, w.t.p16, min((t.end + 15) & ~15, w.end()), bad_first, bad_last);
+#pragma unroll 1
+                    for (; rows; rows &= rows - 1) {
+                        const int r = __ffs(rows) - 1, last = t.q_u + quad * 32 + r;
+                        int start = w.t.own_base + w.t.p16;               // of the row's own path
+                        if (w.first_path >= 0)
+                            for (int i = w.first_path + 1; i < p.n_paths && p.path_start[i] > start && p.path_start[i] <= row0 + r; ++i) start = p.path_start[i];
+                        const int from = start - w.t.own_base;
+                        if (bad_first >= from && bad_last <= last) continue;
+                        Words<D> y;
+                        y.load(out_row(r));
+                        exact_row<D, ALIBI>(p, w.t, w.h, kv_head, from, last, y);
+                        y.store(out_row(r));
+                    }
                 }
             }
         }

@@ -22,6 +22,18 @@ def _randn(shape, seed, dtype=torch.bfloat16):
     return torch.randn(*shape, generator=torch.Generator().manual_seed(seed)).to(dtype)
 
 
+def _median_ms(call, n=5):
+    times = []
+    for _ in range(n):
+        begin, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        begin.record()
+        call()
+        end.record()
+        end.synchronize()
+        times.append(begin.elapsed_time(end))
+    return sorted(times)[n // 2]
+
+
 def _prefill(lay, H, Hkv, D, dtype=torch.bfloat16, rows=sp.SP_ROWS_ALL, alibi=False, shift=0, mirror=True, repeats=0):
     """Runs and checks one prefill, and repeats, which have to give the same bits; shift: elements by which the output's address misses 32-byte alignment."""
     T = lay.total_tokens
@@ -373,6 +385,78 @@ def test_prefill_tiles_across_paths_keep_values_to_their_path(D, alibi):
     out1, lse1 = run(k2, v2)
     np.testing.assert_array_equal(lse0[:, others], lse1[:, others])
     assert np.abs(out0[others] - out1[others]).max() <= 2 ** -7 * np.abs(out0).max()
+
+
+def _short_path_call(lay, H, D, alibi, q, k, v):
+    """A call over tiles across paths, and its outputs."""
+    T = lay.total_tokens
+    pos, slopes = dev(torch.rand(T, generator=torch.Generator().manual_seed(4)).mul(300).float()), dev(torch.linspace(0.01, 0.5, H))
+    dl = sp.DeviceLayout.from_host(lay)
+    ws = workspace(sp.sp_prefill_workspace_bytes(dl, H, D, sp.SP_BF16))
+    args, out, lse = (dev(q), dev(k), dev(v), dl), torch.zeros((T, H, D), dtype=torch.bfloat16, device="cuda"), torch.zeros((H, T), device="cuda")
+
+    def call():
+        if alibi:
+            sp.sp_superpose_prefill_alibi(*args, pos, slopes, D ** -0.5, out, lse, ws)
+        else:
+            sp.sp_superpose_prefill(*args, D ** -0.5, out, lse, ws)
+
+    call()
+    sp.sp_check_status(ws)
+    return call, f32(out), lse.cpu().numpy()
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("alibi", [False, True])
+@pytest.mark.parametrize("where", ["a preamble", "everywhere"])
+def test_prefill_tiles_across_paths_values_that_rows_see(D, alibi, where):
+    """A NaN that every row of a prompt sees, or that fills V: it is each row's own and costs a look at the keys, not the row's
+    computation anew (by one thread, at some 300 times the launch).  Every bit that does not depend on it stays."""
+    H, n = 20, 60
+    rng = np.random.default_rng(6)
+    lay = build_layout([700] * 4, [[int(x) for x in rng.integers(8, 60, n)] for _ in range(4)], [[8] * n] * 4)
+    q, k, v = (_randn((lay.total_tokens, H, D), i) for i in (1, 2, 3))
+    clean, out0, lse0 = _short_path_call(lay, H, D, alibi, q, k, v)
+    v2 = v.clone()
+    paths = slice(int(lay.path_start[n]), int(lay.path_start[2 * n - 1] + lay.doc_len[2 * n - 1] + lay.qry_len[2 * n - 1]))
+    if where == "everywhere":
+        v2[:] = float("nan")
+    else:
+        v2[int(lay.pre_start[1]) + 3, :, 7] = float("nan")
+    bad, out1, lse1 = _short_path_call(lay, H, D, alibi, q, k, v2)
+    np.testing.assert_array_equal(lse0, lse1)
+    if where == "everywhere":
+        assert np.isnan(out1).all()
+    else:
+        assert np.isnan(out1[paths][:, :, 7]).all()
+        out0[paths][:, :, 7] = out1[paths][:, :, 7] = 0
+        same = np.ones(lay.total_tokens, bool)
+        same[int(lay.pre_start[1]):int(lay.pre_start[1] + lay.pre_len[1])] = False
+        np.testing.assert_array_equal(out0[same], out1[same])
+    assert _median_ms(bad) <= 10 * _median_ms(clean)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("first", [False, True])
+def test_prefill_tiles_across_paths_scores_of_minus_infinity(D, first):
+    """Rows computed again because of an Inf in another path's V while a key of theirs, the first one or another, scores -Inf: that key has no
+    weight.  Tolerance as for other rows that are computed again: 2^-7 of the largest value."""
+    lay = _short_paths(40, 4, 90, 24)
+    H, T = 20, lay.total_tokens
+    q, k, v = (_randn((T, H, D), i) for i in (1, 2, 3))
+    q[:, :, 5] = q[:, :, 5].abs() + 0.125
+    k[torch.from_numpy(lay.pre_start).long() + (0 if first else 17), :, 5] = float("-inf")
+    _, out0, lse0 = _short_path_call(lay, H, D, False, q, k, v)
+    others, v2 = np.ones(T, bool), v.clone()
+    for b in range(4):                                       # a preamble's rows in front of that key see nothing else
+        others[int(lay.pre_start[b]):int(lay.pre_start[b]) + 18] = False
+    for i in (5, 120, 200, 355):
+        r = slice(int(lay.path_start[i]), int(lay.path_start[i] + lay.doc_len[i] + lay.qry_len[i]))
+        v2[r], others[r] = float("inf"), False
+    _, out1, lse1 = _short_path_call(lay, H, D, False, q, k, v2)
+    assert np.isfinite(out0[others]).all()
+    np.testing.assert_array_equal(lse0[:, others], lse1[:, others])
+    assert np.abs(out0[others] - out1[others]).max() <= 2 ** -7 * np.abs(out0[others]).max()
 
 
 @pytest.mark.parametrize("alibi", [False, True])
