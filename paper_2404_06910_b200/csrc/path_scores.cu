@@ -169,10 +169,10 @@ path_sum_kernel(const float *row_logp, const int32_t *row_off, int n_paths, cons
     if (i < n_paths) path_sum(row_logp, i, row_off[i], row_off[i + 1], prior, weight, scores);
 }
 
-// So few logits that launches are all that counts: the rows of a path are worked on by the blocks of one cluster, kRowsAtOnce a block at a
-// time, and the first block adds them up: one launch instead of two.  Rows in front of the first path and behind the last one go with
+// So few logits that launches are all that counts: the rows of a path are worked on by the blocks of one cluster, kRowsAtOnce a block, all at
+// once, and the first block adds them up: one launch instead of two.  Rows in front of the first path and behind the last one go with
 // those.
-constexpr int kRowsAtOnce = 4;
+constexpr int kRowsAtOnce = 4, kScoreCluster = 8;
 template <typename T>
 __global__ void __launch_bounds__(256 * kRowsAtOnce)
 path_scores_kernel(const T *logits, int64_t ld, const int32_t *targets, const int32_t *row_off, int n_rows, int vocab, const float *prior,
@@ -227,12 +227,16 @@ extern "C" int sp_path_scores(const void *logits, int64_t ld_logits, const int32
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const auto go = [&](auto *p) {
         using T = std::remove_const_t<std::remove_pointer_t<decltype(p)>>;
-        // One launch for up to 4 MB of logits.  us, two launches / one: a step of 4 paths x 8 rows of 512 (host-bound) 29.0 / 26.8, scores and
-        // top-k of 480 rows of 8 000 (8 MB) 11.4 / 11.2, of 32 000 12.3 / 17.2: blocks of four rows are too few to ask for all of it at once.
-        if (n_rows > 0 && n_rows <= 256 && n_paths <= 65535 && n_rows * vocab * (int64_t)sizeof(T) <= 4 << 20) {
-            const int64_t rows = (n_rows + n_paths - 1) / n_paths;
-            int blocks = 1;
-            while (blocks < 8 && blocks * kRowsAtOnce < rows) blocks *= 2;
+        // One launch where the host's share of two is what a caller waits for and the GPU's time no longer: up to 32 rows, eight to a path in the
+        // mean, 128 KB of logits, no more paths than rows.  A block to each of eight rows while those fit on the SMs; its other three are for paths
+        // that have more.  Scores and top-k, us called one by one (queued ahead), two launches / one: 4 x 8 rows of 512 in fp32
+        // 18.4 / 15.9 (5.9 / 5.5), 8 x 4 of 2 048 in bf16 18.6 / 16.1 (5.9 / 5.7), 32 x 1 of 2 048 18.6 / 16.3 (5.9 / 5.9), 1 x 8 of 8 192
+        // 18.6 / 16.1 (5.7 / 5.9).  Not with more: blocks that take rows one after another, or blocks by the thousand (cold, scores alone: 1 x 256
+        // of 8 000 11.3 / 32.8, 65 535 paths without rows 17 / 418), or rows so long that four in a block are slow (4 x 8 of 50 432 9.1 / 14.7).
+        if (n_rows > 0 && n_rows <= kScoreCluster * kRowsAtOnce && n_rows <= kScoreCluster * (int64_t)n_paths && n_paths <= n_rows &&
+            n_rows * vocab * (int64_t)sizeof(T) <= 128 << 10) {
+            int blocks = kScoreCluster;
+            while (blocks > 1 && (blocks / 2 >= n_rows || blocks * n_paths > num_sms())) blocks /= 2;
             return launch(path_scores_kernel<T>, dim3(blocks, n_paths), 256 * kRowsAtOnce, 0, st, blocks, p, ld_logits, targets, row_off, (int)n_rows, vocab,
                           prior, weight, rows_out, scores);
         }

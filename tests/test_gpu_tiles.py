@@ -597,10 +597,11 @@ def test_decode_single_heads_in_fp32_arithmetic(H, D, alibi):
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
-@pytest.mark.parametrize("lens,vocab", [([1], 5), ([4, 5], 700), ([8, 9, 16, 17, 33], 1001), ([100, 0, 1], 64), ([33] * 7, 2051), ([250, 6], 4096), ([257], 64)])
+@pytest.mark.parametrize("lens,vocab", [([1], 5), ([4, 5], 700), ([8, 9, 16, 17, 33], 1001), ([100, 0, 1], 64), ([33] * 7, 2051), ([250, 6], 4096), ([257], 64),
+                                        ([27], 300), ([25, 1, 1, 0], 64), ([0, 26, 0, 1], 1000), ([1] * 27, 129), ([2, 0, 1], 2051), ([25, 1, 1, 1], 64)])
 def test_path_scores_in_one_launch(dtype, lens, vocab):
     """The rows of a path over one to eight blocks of a cluster, four a block at a time; paths without rows, rows in front of the first and
-    behind the last path; a row more than one launch takes.  Bit-identical repeats; tolerance 1e-3 per row as in the parity suite."""
+    behind the last path; one path with nearly all rows, as many blocks as fit; a row more than one launch takes.  Bit-identical repeats; tolerance 1e-3 per row as in the parity suite."""
     before, behind = 3, 2
     off = np.concatenate([[before], before + np.cumsum(lens)]).astype(np.int32)
     rows = int(off[-1]) + behind
@@ -617,3 +618,23 @@ def test_path_scores_in_one_launch(dtype, lens, vocab):
     want = torch.log_softmax(logits.double(), 1).gather(1, tgt.clamp(min=0).long()[:, None])[:, 0].masked_fill(tgt < 0, 0).numpy()
     np.testing.assert_allclose(got[0][1], want, atol=1e-3)
     np.testing.assert_allclose(got[0][0], ref_s, atol=1e-3 * max(max(lens), 1))
+
+
+@pytest.mark.parametrize("rows,paths,vocab,more_rows,more_paths", [(8, 65535, 512, 0, 1), (8, 4096, 512, 512, 0), (256, 1, 8000, 4, 0), (128, 1, 8000, 132, 0),
+                                                                   (32, 4, 60000, 228, 0)])
+def test_path_scores_of_few_rows_take_no_longer_than_of_more(rows, paths, vocab, more_rows, more_paths):
+    """Paths without rows by the thousand, one path with all rows, long rows: not above what a call with more rows or paths takes, which
+    always goes through two launches.  A quarter for the clock's steps of 1 us and what a cold start varies."""
+    def call(rows, paths):
+        logits, tgt = torch.randn(rows, vocab, device="cuda").bfloat16(), torch.zeros(rows, dtype=torch.int32, device="cuda")
+        off = torch.full((paths + 1,), rows, dtype=torch.int32, device="cuda")
+        off[:2] = torch.tensor([0, rows if paths == 1 else rows // 2])
+        scores, row_logp = torch.empty(paths, device="cuda"), torch.empty(rows, device="cuda")
+
+        def many():
+            for _ in range(20):
+                sp.sp_path_scores(logits, tgt, off, scores, None, None, row_logp)
+        many()
+        return _median_ms(many, 9)
+
+    assert call(rows, paths) <= 1.25 * call(rows + more_rows, paths + more_paths)
