@@ -688,6 +688,10 @@ static int launch_cluster_kernel(K kern, const DecodeArgs &a, const DecodeRope &
 //    from L2), groups of 4 8.1 / 8.3; with 1 300 keys 9.0 / 7.0.
 //  - Grouped heads, few keys, and units that leave a ring two warps but registers four: 384 units of 430 keys 22.3 / 22.6.
 //  - Single heads, few keys, units that fill the waves of decode_cluster_kernel: 1 024 43.6 / 44.2, 2 048 75.3 / 77.1; but 1 536 66.3 / 61.7.
+//  - Grouped heads, a table of hundreds of kept paths, which takes the place of rings: registers, if rings leave half as many warps or fewer and
+//    those blocks are resident at once.  Registers / ring, kept paths of 1-8 rows, groups of 8, one unit: 1 000 66.8 / 61.4, 2 500 160 / 194,
+//    4 096 272 / 803; groups of 2, four units: 2 500 169 / 146, 4 096 276 / 339; 64 units in groups of 4: 1 000 192 / 197, 4 096 (not resident)
+//    1348 / 971.  Single heads keep their rings (4 096, 32 units 2455 / 604).
 struct MmaLaunch { bool ring; int n_splits, warps; size_t smem; };
 
 template <int D> static MmaLaunch mma_launch(DecodeArgs a, int n_prompts, int64_t max_keys)
@@ -697,11 +701,11 @@ template <int D> static MmaLaunch mma_launch(DecodeArgs a, int n_prompts, int64_
     const size_t partial = std::min(group, kMmaHeads) * (D + 2) * sizeof(float);
     MmaLaunch r = {};
     const auto in_registers = [&]() {
+        MmaLaunch r = {};
+        r.warps = kMmaMaxWarps;
         // three blocks per SM for both head sizes: with four, 2 prompts x 16 KV heads of 64 become clusters of 16, which the SMs take in
         // less evenly than clusters of 8 (12.1 us against 8.0)
-        r.ring = false;
         r.n_splits = cluster_splits(n_prompts, blocks_y, max_keys, kMmaMaxWarps * kMmaKeys, 3);
-        r.warps = kMmaMaxWarps;
         r.smem = decode_table_bytes(a.k + 2) + (D / 2) * sizeof(float2) + (r.warps + r.n_splits) * partial;
         return r;
     };
@@ -732,6 +736,11 @@ template <int D> static MmaLaunch mma_launch(DecodeArgs a, int n_prompts, int64_
     }
     while (bytes(r.n_splits, r.warps) > 200 * 1024 && r.warps > 1) --r.warps;      // the table of thousands of kept paths takes the place of rings
     r.smem = bytes(r.n_splits, r.warps);
+    if (group > 1 && decode_table_bytes(a.k + 2) >= MmaRing<D>::BYTES) {
+        const MmaLaunch o = in_registers();
+        const int64_t places = (int64_t)std::min<size_t>(228 * 1024 / (o.smem + 1024), 3) * sms;
+        if (2 * r.n_splits * r.warps <= o.n_splits * o.warps && o.n_splits * units <= places) return o;
+    }
     return r;
 }
 

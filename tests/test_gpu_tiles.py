@@ -596,6 +596,29 @@ def test_decode_single_heads_in_fp32_arithmetic(H, D, alibi):
     assert wrong <= 5e-4 * 2 * H * D
 
 
+@pytest.mark.parametrize("H,Hkv", [(8, 1), (8, 4)])
+def test_decode_thousands_of_kept_paths(H, Hkv):
+    """The table of 4 096 kept paths, 112 KB, leaves shared memory for little else: twice the keys of 2 048 paths, and not above three times
+    their time (six where rings were kept at the cost of splits)."""
+    D, cap, n = 128, 4, 4096
+    rng = np.random.default_rng(3)
+    lay = build_layout([9], [[int(x) for x in rng.integers(1, 9, n)]], [[1] * n])
+    T = lay.total_tokens
+    q, kc, vc, tk, tv = _randn((1, H, D), 1), _randn((T, Hkv, D), 2), _randn((T, Hkv, D), 3), _randn((1, cap, Hkv, D), 4), _randn((1, cap, Hkv, D), 5)
+    tl, dl, ws = np.array([3], np.int32), sp.DeviceLayout.from_host(lay), workspace(sp.sp_decode_workspace_bytes(1, H, D))
+    cache, took = (dev(q), dev(kc), dev(vc), dl), []
+    for k in (n, n // 2):
+        kept = rng.permutation(n)[:k].astype(np.int32)[None]
+        args = (*cache, dev(kept), k, dev(tk), dev(tv), dev(tl), cap, D ** -0.5)
+        out, lse = torch.full((1, H, D), float("nan"), dtype=torch.bfloat16, device="cuda"), torch.full((1, H), float("nan"), device="cuda")
+        sp.sp_pruned_decode(*args, out, lse, ws)
+        ref_o, ref_l = oracle.pruned_decode(f32(q), f32(kc), f32(vc), lay, kept, f32(tk), f32(tv), tl, D ** -0.5)
+        assert rel_l2(f32(out), ref_o) <= TOL[torch.bfloat16]
+        np.testing.assert_allclose(lse.cpu().numpy(), ref_l, atol=2e-2)
+        took.append(_median_ms(lambda: [sp.sp_pruned_decode(*args, out, lse, ws) for _ in range(20)], 9))
+    assert took[0] <= 3 * took[1]
+
+
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("lens,vocab", [([1], 5), ([4, 5], 700), ([8, 9, 16, 17, 33], 1001), ([100, 0, 1], 64), ([33] * 7, 2051), ([250, 6], 4096), ([257], 64),
                                         ([27], 300), ([25, 1, 1, 0], 64), ([0, 26, 0, 1], 1000), ([1] * 27, 129), ([2, 0, 1], 2051), ([25, 1, 1, 1], 64)])
