@@ -20,6 +20,9 @@ namespace sp {
 constexpr int kDecThreads = 128;
 constexpr int kDecUnroll = 4;        // keys in flight per key group (kept small: occupancy hides latency better)
 constexpr int kDecMaxSplits = 64;
+// Shared memory of a block at most.  What a kernel is allowed belongs to the function, for all threads of the process, so it is set to this for
+// every launch: set to what one launch needs, it could be lowered between another thread's setting and its launch.
+constexpr int kDecMaxSmem = 200 * 1024;
 constexpr float kLog2eD = 1.4426950408889634f;
 constexpr float kLn2D = 0.6931471805599453f;
 
@@ -264,9 +267,9 @@ static int launch_decode(const DecodeArgs &a, int n_prompts, cudaStream_t st)
     constexpr int G = kDecThreads / (D / Vec<T>::N);
     const int n_seg = a.k + 2;
     const size_t smem = round_up((n_seg + 1) * sizeof(int), 16) + 2 * n_seg * sizeof(void *) + (size_t)G * (D + 2) * sizeof(float);
-    SP_REQUIRE(smem <= 200 * 1024, SP_ERR_UNSUPPORTED, "sp_pruned_decode: k = %d needs too much shared memory", a.k);
+    SP_REQUIRE(smem <= kDecMaxSmem, SP_ERR_UNSUPPORTED, "sp_pruned_decode: k = %d needs too much shared memory", a.k);
     if (smem > 48 * 1024)
-        SP_CUDA(cudaFuncSetAttribute(decode_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        SP_CUDA(cudaFuncSetAttribute(decode_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecMaxSmem));
     dim3 grid(a.n_splits, a.n_heads, n_prompts);
     return launch(decode_kernel<T, D>, grid, kDecThreads, smem, st, 1, a);
 }
@@ -671,9 +674,9 @@ template <typename K>
 static int launch_cluster_kernel(K kern, const DecodeArgs &a, const DecodeRope &rope, int pairing, int blocks_y, int n_prompts, int threads,
                                  size_t smem, cudaStream_t st)
 {
-    SP_REQUIRE(smem <= 200 * 1024, SP_ERR_UNSUPPORTED, "sp_pruned_decode: k = %d needs too much shared memory", a.k);
+    SP_REQUIRE(smem <= kDecMaxSmem, SP_ERR_UNSUPPORTED, "sp_pruned_decode: k = %d needs too much shared memory", a.k);
     if (smem > 48 * 1024)
-        SP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        SP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecMaxSmem));
     if (a.n_splits > 8)
         SP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     return launch(kern, dim3(a.n_splits, blocks_y, n_prompts), threads, smem, st, a.n_splits, a, rope, pairing);
@@ -734,7 +737,7 @@ template <int D> static MmaLaunch mma_launch(DecodeArgs a, int n_prompts, int64_
         const int64_t wave = 7 * sms, waves = (units + wave - 1) / wave;
         if (few_keys && group == 1 && units * 100 >= waves * wave * 95) r.ring = false;
     }
-    while (bytes(r.n_splits, r.warps) > 200 * 1024 && r.warps > 1) --r.warps;      // the table of thousands of kept paths takes the place of rings
+    while (bytes(r.n_splits, r.warps) > kDecMaxSmem && r.warps > 1) --r.warps;      // the table of thousands of kept paths takes the place of rings
     r.smem = bytes(r.n_splits, r.warps);
     if (group > 1 && decode_table_bytes(a.k + 2) >= MmaRing<D>::BYTES) {
         const MmaLaunch o = in_registers();
