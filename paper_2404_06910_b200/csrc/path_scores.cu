@@ -189,6 +189,7 @@ path_scores_kernel(const T *logits, int64_t ld, const int32_t *targets, const in
         score_row<T, 256>(logits, ld, t, targets[t], vocab, row_logp, threadIdx.x & 255, sm[group], ss[group], sync);
         sync();                                             // the numbers of this row's warps have been read
     }
+    __syncwarp();                                           // rows that end in their first warp's first thread leave warps diverged
     if (blocks > 1) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     else __syncthreads();
     if (rank == 0 && threadIdx.x < 32) path_sum(row_logp, path, t0, t1, prior, weight, scores);
