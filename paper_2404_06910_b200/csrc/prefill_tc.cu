@@ -89,7 +89,8 @@ template <int D, bool ALIBI, bool SPLIT> struct TcConfig {
     // what the others give back, which has to add up; only they grow.
     static constexpr int R_LAUNCH = 96, R_SOFT = 128, R_EPI = 96, R_LOAD = 56, R_MMA = 64;
     static_assert(2 * R_SOFT + R_EPI + R_LOAD + R_MMA <= kTcThreads / 128 * R_LAUNCH, "registers of a block");
-    static_assert(R_SOFT >= R_LAUNCH && R_EPI <= R_LAUNCH && R_LOAD <= R_LAUNCH && R_MMA <= R_LAUNCH, "direction of setmaxnreg");
+    static_assert(R_EPI == R_LAUNCH, "a function called from the epilogue may use what the kernel was launched with");
+    static_assert(R_SOFT >= R_LAUNCH && R_LOAD <= R_LAUNCH && R_MMA <= R_LAUNCH, "direction of setmaxnreg");
 };
 static_assert(TcConfig<128, false, false>::SMEM <= 232448 && TcConfig<128, true, false>::SMEM <= 232448, "one block's shared memory");
 
@@ -319,69 +320,84 @@ __device__ __forceinline__ void exact_row(const TcParams &p, const TcPair &t, in
     }
 }
 
-// One row (key number `last`, 64 columns; o: bf16 pairs) in fp32 arithmetic over exactly the keys it sees: its values that are not
-// finite are replaced.
-template <bool ALIBI>
-__device__ __forceinline__ void exact_row64(const TcParams &p, const TcPair &t, int head, int kv_head, int last, uint32_t (&o)[32])
+// The same for tiles of one segment, head_dim 64, before a row is stored (the output may take Q's place): the rows of the warp that
+// are not finite; o: the bf16 pairs of this thread's.  Rows in front of one whose values are not finite share tiles with it.  Called, not
+// inlined, because it is rare and the loop it is called from is sensitive to registers (inlined, ALiBi, 16 prompts x 20 documents: 344 -> 357
+// us); the epilogue's warps keep the registers that the kernel was launched with, so any called function has enough.
+template <bool ALIBI, TileRows ROWS>
+__device__ __noinline__ void exact_rows64(const TcParams &p, uint32_t pair, int unit, int b, int quad, uint32_t *o)
 {
-    const int64_t own = t.own_base + last;
-    const uint4 *q = reinterpret_cast<const uint4 *>(p.q + (own * p.n_heads + head) * 64);
-    const float pq = ALIBI ? p.pos[own] : 0.f, slope = ALIBI ? p.slopes[head] * kLog2eT : 0.f;
-    auto packed_row = [&](int u) { return (int64_t)u + (u < t.pre_len ? t.pre_row : t.own_base); };
-    auto score = [&](int64_t row) {
-        const uint4 *k = reinterpret_cast<const uint4 *>(p.k + (row * p.n_kv_heads + kv_head) * 64);
-        float s = 0.f;
+    const TcPair t = p.pairs[pair];
+    const int lane = threadIdx.x & 31, log_rows = ROWS == HEAD_ROWS ? p.log_rows : 7, row = quad * 32 + lane, hr = row & ((1 << log_rows) - 1);
+    const int rows_a = t.rows_ab & 0xffff, rows_b = t.rows_ab >> 16, q_u = t.q_u + (b ? rows_a : 0), n_rows = b ? rows_b : rows_a;
+    const int kv_head = unit / p.units_per_kv, head = (unit << (7 - log_rows)) + (row >> log_rows);
+    uint32_t bad = 0u;
+    for (int i = 0; i < 32; ++i) bad |= not_finite(o[i]);
+    uint32_t rows = __ballot_sync(0xffffffffu, bad && hr < n_rows);
+    int bad_first, bad_last;
+    bad_values<64>(p, t, kv_head, q_u, min((q_u + n_rows + 15) & ~15, t.q_u + rows_a + rows_b), bad_first, bad_last);
 #pragma unroll 1
-        for (int c = 0; c < 8; ++c) {
-            const uint4 x = q[c], y = k[c];
-            s = fmaf(bf16_lo(x.x), bf16_lo(y.x), s); s = fmaf(bf16_hi(x.x), bf16_hi(y.x), s);
-            s = fmaf(bf16_lo(x.y), bf16_lo(y.y), s); s = fmaf(bf16_hi(x.y), bf16_hi(y.y), s);
-            s = fmaf(bf16_lo(x.z), bf16_lo(y.z), s); s = fmaf(bf16_hi(x.z), bf16_hi(y.z), s);
-            s = fmaf(bf16_lo(x.w), bf16_lo(y.w), s); s = fmaf(bf16_hi(x.w), bf16_hi(y.w), s);
+    for (; rows; rows &= rows - 1) {
+        const int r = __ffs(rows) - 1, last = q_u + __shfl_sync(0xffffffffu, hr, r);
+        if (bad_last <= last) continue;
+        Words<64> y;                                     // row r from its thread to a lane each, and back
+#pragma unroll 1
+        for (int i = 0; i < 32; ++i) {
+            const uint32_t x = __shfl_sync(0xffffffffu, o[i], r);
+            if (lane == i) y.w[0] = x;
         }
-        s *= p.scale_log2e;
-        return ALIBI ? s - slope * fabsf(pq - p.pos[row]) : s;
-    };
-    float m = -INFINITY, l = 0.f;
+        exact_row<64, ALIBI>(p, t, __shfl_sync(0xffffffffu, head, r), kv_head, t.p16, last, y);
 #pragma unroll 1
-    for (int u = 0; u <= last; ++u) {
-        if (u >= t.pre_len && u < t.p16) continue;
-        const float s = score(packed_row(u));
-        if (s > m) { l *= ex2(m - s); m = s; }
-        l += ex2(s - m);
-    }
-    const float inv = 1.f / l;
-#pragma unroll
-    for (int part = 0; part < 4; ++part) {               // 16 columns at a time
-        float acc[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-#pragma unroll 1
-        for (int u = 0; u <= last; ++u) {
-            if (u >= t.pre_len && u < t.p16) continue;
-            const int64_t row = packed_row(u);
-            const float w = ex2(score(row) - m);
-            const uint4 *v = reinterpret_cast<const uint4 *>(p.v + (row * p.n_kv_heads + kv_head) * 64) + 2 * part;
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const uint4 y = v[c];
-                const uint32_t wd[4] = {y.x, y.y, y.z, y.w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    acc[8 * c + 2 * e] = fmaf(w, bf16_lo(wd[e]), acc[8 * c + 2 * e]);
-                    acc[8 * c + 2 * e + 1] = fmaf(w, bf16_hi(wd[e]), acc[8 * c + 2 * e + 1]);
-                }
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {                    // the finite ones are right as they are
-            const uint32_t x = pack_bf16x2(acc[2 * i] * inv, acc[2 * i + 1] * inv);
-            uint32_t &y = o[8 * part + i];
-            if ((y & 0x7f80u) == 0x7f80u) y = (y & 0xffff0000u) | (x & 0xffffu);
-            if ((y & 0x7f800000u) == 0x7f800000u) y = (y & 0xffffu) | (x & 0xffff0000u);
+        for (int i = 0; i < 32; ++i) {
+            const uint32_t x = __shfl_sync(0xffffffffu, y.w[0], i);
+            if (lane == r) o[i] = x;
         }
     }
 }
+
+// Tiles across paths: the rows that other paths' values may have reached, once more, by the warp that has stored them: behind the last item,
+// when no other warp waits for this one, and from the stored output.
+template <int D, bool ALIBI> __device__ __forceinline__ void exact_rows_across(const TcParams &p, int quad)
+{
+#pragma unroll 1
+    for (Walk<true> w(p); w.next();) {
+        // rows of one segment meet only their own later rows, head_dim 128: as in a launch without tiles across paths
+        if (D == 128 && w.first_path < 0) continue;
+#pragma unroll 1
+        for (int b = 0; b < w.n_q(); ++b) {
+            const LaneTile t(w, w.lane_a() ^ b);
+            const int kv_head = w.h / p.units_per_kv, row0 = w.t.own_base + t.q_u + quad * 32, n = min(32, t.rows - quad * 32);
+            auto out_row = [&](int r) { return p.out + ((int64_t)(row0 + r) * p.n_heads + w.h) * D; };
+            uint32_t rows = 0u;                  // a bit per row with values that are not finite
+#pragma unroll 4
+            for (int r = 0; r < n; ++r) {
+                Words<D> y;
+                y.load(out_row(r));
+#pragma unroll
+                for (int i = 0; i < D / 64; ++i) rows |= not_finite(y.w[i]) ? 1u << r : 0u;
+            }
+            rows = __reduce_or_sync(0xffffffffu, rows);
+            int bad_first = INT_MAX, bad_last = -1;
+            if (rows) bad_values<D>(p, w.t, kv_head, w.t.p16, min((t.end + 15) & ~15, w.end()), bad_first, bad_last);
+#pragma unroll 1
+            for (; rows; rows &= rows - 1) {
+                const int r = __ffs(rows) - 1, last = t.q_u + quad * 32 + r;
+                int start = w.t.own_base + w.t.p16;               // of the row's own path
+                if (w.first_path >= 0)
+                    for (int i = w.first_path + 1; i < p.n_paths && p.path_start[i] > start && p.path_start[i] <= row0 + r; ++i) start = p.path_start[i];
+                const int from = start - w.t.own_base;
+                if (bad_first >= from && bad_last <= last) continue;
+                Words<D> y;
+                y.load(out_row(r));
+                exact_row<D, ALIBI>(p, w.t, w.h, kv_head, from, last, y);
+                y.store(out_row(r));
+            }
+        }
+    }
+}
+
+// Inlined it made head_dim 64 slower (16 prompts x 17 paths behind 390 rows 459 -> 473 us), called head_dim 128 (497 -> 507).
+template <bool ALIBI> __device__ __noinline__ void exact_rows_across64(const TcParams &p, int quad) { exact_rows_across<64, ALIBI>(p, quad); }
 
 template <int N> __device__ __forceinline__ void reg_alloc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
 template <int N> __device__ __forceinline__ void reg_dealloc() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
@@ -872,16 +888,22 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&bars[C::BAR_O_FREE + ln]);
                     }
-                    if (C::EXACT && !ACROSS && hr < t.rows) {
-                        uint32_t nan = 0u;
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) asm("fma.rn.bf16x2 %0, %1, %2, %0;" : "+r"(nan) : "r"(o[i]), "r"(0u));
-                        if (nan & 0x7fff7fffu)
-                            exact_row64<ALIBI>(p, w.t, (w.h << (7 - log_rows)) + (row >> log_rows), w.h / p.units_per_kv, t.q_u + hr, o);
-                    }
                     if (ACROSS) {
 #pragma unroll
                         for (int i = 0; i < 32; ++i) asm("fma.rn.bf16x2 %0, %1, %2, %0;" : "+r"(nan) : "r"(o[i]), "r"(0u));
+                    }
+                    if constexpr (C::EXACT && !ACROSS) {
+                        uint32_t nan = 0u;
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) asm("fma.rn.bf16x2 %0, %1, %2, %0;" : "+r"(nan) : "r"(o[i]), "r"(0u));
+                        if (__any_sync(0xffffffffu, hr < t.rows && (nan & 0x7fff7fffu))) {
+                            uint32_t copy[32];
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) copy[i] = o[i];
+                            exact_rows64<ALIBI, ROWS>(p, w.pair, w.h, b, quad, copy);
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) o[i] = copy[i];
+                        }
                     }
                     if (hr < t.rows) {
                         if (p.wide_stores) {
@@ -898,43 +920,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_
             }
         }
         if (ACROSS && ok && __any_sync(0xffffffffu, not_all_finite)) {
-            // Rows that other paths' values may have reached, once more: behind the last item, when no other warp waits for this one, and from
-            // the stored output, in which the rows that one warp has written are its own.
-#pragma unroll 1
-            for (Walk w(p); w.next();) {
-                // rows of one segment meet only their own later rows, head_dim 128: as in a launch without tiles across paths
-                if (D == 128 && w.first_path < 0) continue;
-#pragma unroll 1
-                for (int b = 0; b < w.n_q(); ++b) {
-                    const LaneTile t(w, w.lane_a() ^ b);
-                    const int kv_head = w.h / p.units_per_kv, row0 = w.t.own_base + t.q_u + quad * 32, n = min(32, t.rows - quad * 32);
-                    auto out_row = [&](int r) { return p.out + ((int64_t)(row0 + r) * p.n_heads + w.h) * D; };
-                    uint32_t rows = 0u;                  // a bit per row with values that are not finite
-#pragma unroll 4
-                    for (int r = 0; r < n; ++r) {
-                        Words<D> y;
-                        y.load(out_row(r));
-#pragma unroll
-                        for (int i = 0; i < D / 64; ++i) rows |= not_finite(y.w[i]) ? 1u << r : 0u;
-                    }
-                    rows = __reduce_or_sync(0xffffffffu, rows);
-                    int bad_first = INT_MAX, bad_last = -1;
-                    if (rows) bad_values<D>(p, w.t, kv_head, w.t.p16, min((t.end + 15) & ~15, w.end()), bad_first, bad_last);
-#pragma unroll 1
-                    for (; rows; rows &= rows - 1) {
-                        const int r = __ffs(rows) - 1, last = t.q_u + quad * 32 + r;
-                        int start = w.t.own_base + w.t.p16;               // of the row's own path
-                        if (w.first_path >= 0)
-                            for (int i = w.first_path + 1; i < p.n_paths && p.path_start[i] > start && p.path_start[i] <= row0 + r; ++i) start = p.path_start[i];
-                        const int from = start - w.t.own_base;
-                        if (bad_first >= from && bad_last <= last) continue;
-                        Words<D> y;
-                        y.load(out_row(r));
-                        exact_row<D, ALIBI>(p, w.t, w.h, kv_head, from, last, y);
-                        y.store(out_row(r));
-                    }
-                }
-            }
+            if constexpr (D == 128) exact_rows_across<D, ALIBI>(p, quad);
+            else exact_rows_across64<ALIBI>(p, quad);
         }
     }
 

@@ -387,11 +387,11 @@ def test_prefill_tiles_across_paths_keep_values_to_their_path(D, alibi):
     assert np.abs(out0[others] - out1[others]).max() <= 2 ** -7 * np.abs(out0).max()
 
 
-def _short_path_call(lay, H, D, alibi, q, k, v):
-    """A call over tiles across paths, and its outputs."""
+def _short_path_call(lay, H, D, alibi, q, k, v, mirror=True):
+    """A call, over tiles across paths where the layout has its host mirror, and its outputs."""
     T = lay.total_tokens
     pos, slopes = dev(torch.rand(T, generator=torch.Generator().manual_seed(4)).mul(300).float()), dev(torch.linspace(0.01, 0.5, H))
-    dl = sp.DeviceLayout.from_host(lay)
+    dl = sp.DeviceLayout.from_host(lay, mirror=mirror)
     ws = workspace(sp.sp_prefill_workspace_bytes(dl, H, D, sp.SP_BF16))
     args, out, lse = (dev(q), dev(k), dev(v), dl), torch.zeros((T, H, D), dtype=torch.bfloat16, device="cuda"), torch.zeros((H, T), device="cuda")
 
@@ -483,6 +483,33 @@ def test_prefill_short_paths_with_the_output_in_place_of_the_queries(alibi):
 
     for a, b in zip(run(True), run(False)):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("alibi", [False, True])
+@pytest.mark.parametrize("H,Hkv", [(10, 10), (8, 2)])
+def test_prefill_head64_values_that_rows_see(alibi, H, Hkv):
+    """Tiles of one segment, head_dim 64: a NaN in a preamble, which every row of a prompt sees, is no reason to compute rows again; an Inf
+    is, for the rows in front of it, and keys that score -Inf, the first one among them, then have no weight."""
+    rng = np.random.default_rng(6)
+    lay = build_layout([300] * 4, [[int(x) for x in rng.integers(8, 200, 12)] for _ in range(4)], [[8] * 12] * 4)
+    T, D = lay.total_tokens, 64
+    q, k, v = _randn((T, H, D), 1), _randn((T, Hkv, D), 2), _randn((T, Hkv, D), 3)
+    q[:, :, 5] = q[:, :, 5].abs() + 0.125
+    k[torch.from_numpy(lay.pre_start).long(), :, 5] = float("-inf")
+    clean, out0, lse0 = _short_path_call(lay, H, D, alibi, q, k, v, mirror=False)
+    v2 = v.clone()
+    v2[int(lay.pre_start[1]) + 3, :, 7] = float("nan")
+    bad, out1, lse1 = _short_path_call(lay, H, D, alibi, q, k, v2, mirror=False)
+    assert _median_ms(bad) <= 10 * _median_ms(clean)
+    np.testing.assert_array_equal(lse0, lse1)
+    rows = slice(int(lay.path_start[12]), int(lay.path_start[23] + lay.doc_len[23] + lay.qry_len[23]))
+    assert np.isnan(out1[rows][:, :, 7]).all()
+    v2 = v.clone()
+    r = int(lay.path_start[12]) + 13
+    v2[r, :, 7] = float("inf")
+    _, out2, _ = _short_path_call(lay, H, D, alibi, q, k, v2, mirror=False)
+    first = slice(int(lay.path_start[12]), r)
+    assert np.abs(out2[first] - out0[first]).max() <= 2 ** -7 * np.abs(out0[first]).max()
 
 
 QRY_EDGES = [1, 8, 15, 16, 17, 31, 32, 33, 47, 48]
