@@ -384,9 +384,10 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
         }
     }
 
-    if (SINGLE && mine_new) {                                // as below
+    if (SINGLE && mine_new) {                                // as below; the key is the first group's, the others' value is zero: 0 x Inf is not
         uint4 *krow = reinterpret_cast<uint4 *>(const_cast<T *>(sm.k[n_seg - 1]) + new_off);
-        uint4 kr[1] = {krow[sub]}, vr[1] = {reinterpret_cast<const uint4 *>(sm.v[n_seg - 1] + new_off)[sub]};
+        uint4 kr[1] = {krow[sub]}, vr[1] = {make_uint4(0u, 0u, 0u, 0u)};
+        if (kg == 0) vr[0] = reinterpret_cast<const uint4 *>(sm.v[n_seg - 1] + new_off)[sub];
         const float kpos[1] = {0.f};
         rotate1(kr[0]);
         __syncwarp();
