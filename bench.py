@@ -46,12 +46,12 @@ PREFILL_LAUNCHES = 2           # kernels sp_superpose_prefill launches per call 
 # Each entry names the hash of the kernel sources it was taken from: after a kernel change the
 # figure is withheld (null in the JSON line) until the capture is repeated.
 NCU_TRAFFIC = {
-    ("prefill", "cfg2_batched_serving"): {"bytes_per_unit": 2439558144.0 / 74087, "unit": "token",
-                                          "capture": "the cfg2 shape with 20 prompts (74 087 tokens), one launch",
-                                          "source_hash": "13831cadeac3"},
-    ("decode", "cfg3_llama2_7b"): {"bytes_per_unit": 108792320.0 / 6548, "unit": "gathered key",
+    ("prefill", "cfg2_batched_serving"): {"bytes_per_unit": 2439235925.0 / 74087, "unit": "token",
+                                          "capture": "the cfg2 shape with 20 prompts (74 087 tokens), three launches averaged",
+                                          "source_hash": "317c51d742d0"},
+    ("decode", "cfg3_llama2_7b"): {"bytes_per_unit": 108933760.0 / 6548, "unit": "gathered key",
                                    "capture": "cfg3 (8 prompts, 6 548 keys per launch), two launches averaged",
-                                   "source_hash": "34d267c625a9"},
+                                   "source_hash": "971024e5f7c8"},
 }
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
@@ -302,7 +302,7 @@ class HotPath:
 
 
 STAGES = ("rope", "prefill", "path_scores", "topk", "decode")
-PREFILL_SOURCES = ("prefill_tc.cu", "prefill_plan.cuh", "tc_ptx.cuh")
+PREFILL_SOURCES = ("prefill_tc.cu", "prefill_plan.cuh", "tc_ptx.cuh", "tensor_map.cuh")
 DECODE_SOURCES = ("decode.cu", "decode_mma.cuh")
 
 

@@ -202,7 +202,9 @@ int sp_prune_topk(const float *scores, const int32_t *prompt_path_off, int n_pro
  * partial results through distributed shared memory in split order (results do not depend on
  * scheduling); the workspace is therefore not written, and its status word is not touched
  * (this call has no bounded waits).  Query heads that share a KV head (n_kv_heads < n_heads) are
- * served together, up to 8 to a block (SP_F32: 4, 2 or 1), so K and V rows are read once per block.
+ * served together, up to 8 to a block (SP_F32: 4, 2 or 1), so K and V rows are read once per block;
+ * with SP_BF16 their products run on the tensor cores, the softmax probabilities as the sum of two
+ * bf16 numbers.  Single heads (n_kv_heads == n_heads) and SP_F32 are computed in fp32 arithmetic.
  */
 size_t sp_decode_workspace_bytes(int n_prompts, int n_heads, int head_dim);
 int sp_pruned_decode(const void *q, const void *k_cache, const void *v_cache,

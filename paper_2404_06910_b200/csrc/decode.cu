@@ -721,13 +721,16 @@ template <int D> static MmaLaunch mma_launch(DecodeArgs a, int n_prompts, int64_
     };
     const auto blocks_per_sm = [&](int n, int w) { return (int)std::min<size_t>(228 * 1024 / (bytes(n, w) + 1024), mma_warps_per_sm(D, true) / w); };
     // Splits: the largest cluster for which all blocks find a place at once, and a turn of keys for each of its warps (five where the merge
-    // is all that two blocks add: groups of 4, 128 units of 430 keys 12.0 us unsplit, 12.9 split).  Larger clusters do not fill the chip:
-    // 16 units in clusters of 8, 128 blocks where 148 fit (groups of 4), take 18.6 us, in clusters of 4 15.0; 16 in clusters of 16 13.3, of 8 10.2.
+    // is all that two blocks add: groups of 4, 128 units of 430 keys 12.0 us unsplit, 12.9 split).  percent: how much of the chip's places (SMs x
+    // blocks per SM) clusters of n fill.  A cluster's blocks share a GPC, whose SMs are no multiple of 8 or 16, so the larger it is the more of
+    // them stay empty: 16 units in clusters of 8, 128 blocks where 148 fit (groups of 4), take 18.6 us, in clusters of 4 15.0; 16 in clusters of
+    // 16 13.3, of 8 10.2.
     r.warps = kMmaMaxWarps;
     for (r.n_splits = 16; r.n_splits > 1; r.n_splits /= 2) {
         const int n = r.n_splits, per_sm = blocks_per_sm(n, r.warps), percent = n == 16 ? 45 : (n == 8 && per_sm < 2 ? 50 : (n == 2 ? 100 : 87));
         if (n * units * 100 <= (int64_t)per_sm * sms * percent && n * r.warps * kMmaKeys * (n == 2 ? 5 : 1) <= max_keys) break;
     }
+    // 24 units and 1 024 keys above, 95 % of the waves below: the nearest round numbers between the measured shapes at the head of this rule.
     // Unsplit: as many warps a block as still leave every block resident; where even blocks of one warp do not fit, two (1 536 units: one warp
     // 68.5 us, two 61.7, four 71.9).
     if (r.n_splits == 1) {

@@ -43,7 +43,8 @@ namespace sp {
 // from which on it loses more than the other one does with more than 48 rows.
 // P as two bf16 numbers, but without a bias and with many items (path, head) of a few key tiles: there it is one number except for an
 // item's first 32 keys, which is more exact than what served them before (of the norm from 64-bit results, 40 prompts of 10 or 20
-// documents: 2.01e-3 to 2.14e-3, 2.09e-3 to 2.16e-3 before; two numbers 1.66e-3) and 0 to 3 % faster (documents of 32-64 rows 100.5 / 104.0 us).
+// documents: 2.01e-3 to 2.14e-3, 2.09e-3 to 2.16e-3 before; two numbers 1.66e-3) and 0 to 3 % faster (documents of 32-64 rows 100.5 / 104.0 us); a
+// probability is then off by 2^-9 of itself at most.
 // With more key tiles the running maximum it needs costs more than the second number (behind 384 rows 836 / 721).  Under ALiBi the
 // weight is on the nearest keys, which 32 fixed ones do not catch: 1.82e-3 to 1.89e-3 where it was 1.88e-3 before; two numbers 1.66e-3, at up
 // to 3 % of the time (behind 48 rows 474 / 476, documents of 40 rows 259 / 267).

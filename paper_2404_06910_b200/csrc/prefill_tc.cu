@@ -404,8 +404,8 @@ template <int N> __device__ __forceinline__ void reg_dealloc() { asm volatile("s
 
 // ALIBI: scores get -slope_h * |pos_q - pos_k| before the softmax (Section 3.2.2: real-valued positions are no obstacle
 // for ALiBi).
-// GROUPED: tiles of several heads.  A kernel of its own: the index arithmetic costs a launch of single heads 1.5 % (32 query rows of
-// 800 paths, 621 against 630 us).
+// ROWS: what makes up a tile.  Tiles of several heads are a kernel of their own because their index arithmetic cost a launch of single heads
+// 1.5 % (630 against 621 us, measured on 32 query rows of 800 paths, which go to prefill_qonly.cu now).
 template <int D, bool ALIBI, TileRows ROWS, bool SPLIT>
 __global__ void __launch_bounds__(kTcThreads, 1) prefill_tc_kernel(const __grid_constant__ TcParams p)
 {

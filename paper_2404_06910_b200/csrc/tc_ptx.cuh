@@ -51,7 +51,8 @@ __device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity)
 }
 // Bounded wait: false when the limit ran out (the caller records a timeout and unwinds).  A probe suspends the thread for
 // up to the hint, so the limit is a few seconds at most and some 0.1 s at least, thousands of times the longest wait of a
-// launch that makes progress.  Counted, not timed: the loop is inlined at two dozen places of a kernel that is sensitive to
+// launch that makes progress (but for head_dim 64 with values that are not finite: exact_rows64() in prefill_tc.cu holds a tile up for at most
+// 32 rows x 4 us per hundred keys).  Counted, not timed: the loop is inlined at two dozen places of a kernel that is sensitive to
 // the size of its code (reading a clock in each took 4.6 KB of 35).
 constexpr uint32_t kWaitProbes = 3000000u;
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity)
