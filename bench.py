@@ -49,9 +49,9 @@ NCU_TRAFFIC = {
     ("prefill", "cfg2_batched_serving"): {"bytes_per_unit": 2439235925.0 / 74087, "unit": "token",
                                           "capture": "the cfg2 shape with 20 prompts (74 087 tokens), three launches averaged",
                                           "source_hash": "317c51d742d0"},
-    ("decode", "cfg3_llama2_7b"): {"bytes_per_unit": 108933760.0 / 6548, "unit": "gathered key",
+    ("decode", "cfg3_llama2_7b"): {"bytes_per_unit": 108784512.0 / 6548, "unit": "gathered key",
                                    "capture": "cfg3 (8 prompts, 6 548 keys per launch), two launches averaged",
-                                   "source_hash": "971024e5f7c8"},
+                                   "source_hash": "95cd14eef97f"},
 }
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
@@ -303,7 +303,7 @@ class HotPath:
 
 STAGES = ("rope", "prefill", "path_scores", "topk", "decode")
 PREFILL_SOURCES = ("prefill_tc.cu", "prefill_plan.cuh", "tc_ptx.cuh", "tensor_map.cuh")
-DECODE_SOURCES = ("decode.cu", "decode_mma.cuh")
+DECODE_SOURCES = ("decode.cu", "decode_mma.cuh", "tc_ptx.cuh")
 
 
 def source_hash(names) -> str:

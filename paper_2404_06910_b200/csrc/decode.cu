@@ -14,6 +14,7 @@
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace sp {
 

@@ -10,8 +10,8 @@
 // the sum of two bf16 numbers (16 bits of mantissa), so the result is as good as with fp32 products (1.6555e-3 of the norm from 64-bit
 // results with either, the rounding of the output), values that are not finite included.
 // Single heads, where the SIMT kernel's multiply-adds cost nothing that shows, keep its arithmetic: with the products above their
-// log-sum-exp was up to 4.6e-6 from 64 bits where it is 1.9e-6 now and was before, the output 3e-6 of its distance further off, at the same
-// times (2 prompts x 32 heads, 8 kept of long documents 16.4 us above, 16.7 so; 16 x 32 heads 23.1 / 23.1; D = 64 18.2 / 18.2).
+// log-sum-exp was up to 4.6e-6 from 64 bits where it is 1.9e-6 now and was before, and the output 3e-6 of its distance further off, at no better
+// times (2 prompts x 32 heads, 8 kept of long documents 16.2 us with products, 16.0 so; 16 x 32 heads 23.2 / 22.7; D = 64 18.1 / 17.7).
 // What bounds it is latency: a turn of 16 keys is a chain of 0.65 us for a warp (products, maximum, exponentials), and where loads go to
 // registers nothing is in flight meanwhile.  So K and V rows run through a ring in shared memory (cp.async), two turns of 8 KB
 // ahead of a warp's arithmetic: 8 warps per SM keep 128 KB in flight.  Two chains of products for S instead of one and fewer instructions per
@@ -175,10 +175,13 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
 
     if (ROPE && !SINGLE) rotate(qf);
     if (ROPE && SINGLE) rotate1(q1);
-    float qs[8], acc[8];                     // SINGLE: the query's elements in log2 units, the group's output
-    Raw16<T>::unpack(q1, qs);
+    uint64_t qs[4], acc[4];                  // SINGLE: the query's elements in log2 units, the group's output, two numbers each
+    {
+        float f[8];
+        Raw16<T>::unpack(q1, f);
 #pragma unroll
-    for (int e = 0; e < 8; ++e) { qs[e] *= a.scale_log2e; acc[e] = 0.f; }
+        for (int e = 0; e < 4; ++e) { qs[e] = ptx::pack_f32x2(f[2 * e] * a.scale_log2e, f[2 * e + 1] * a.scale_log2e); acc[e] = 0ull; }
+    }
 
     float m = -INFINITY, l = 0.f, o[NM][4];  // head gid: maximum, this thread's share of the sum; O^T rows, heads 2 tig, + 1
 #pragma unroll
@@ -186,43 +189,58 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
     const float q_pos = ALIBI ? a.q_pos[b] : 0.f;
     const float slope_l2 = (ALIBI && (SINGLE || gid < nh)) ? a.slopes[h0 + (SINGLE ? 0 : gid)] * kLog2eD : 0.f;
 
-    // SINGLE: N keys to a group of lanes, their pieces `sub` in kr and vr; key u exists where u < n.
-    auto attend1 = [&](const auto &kr, const auto &vr, const auto &kpos, int n) {
-        constexpr int N = sizeof(kr) / sizeof(kr[0]);
-        float x[N], top = -INFINITY;
+    // SINGLE: LPK / 2 keys to a group of LPK lanes, their pieces `sub` in kr and vr; key u exists where u < n and is lanes 2 u's and 2 u + 1's (kpos)
+    // once its products have been added up (half as many shuffles as if every lane had every sum, and one exponential a lane: with those, 25
+    // prompts x 32 heads, 5 warps to an SM, took 114.5 us where this takes 112.2).
+    constexpr int KEYS1 = LPK / 2;
+    auto attend1 = [&](const uint4 (&kr)[KEYS1], const uint4 (&vr)[KEYS1], float kpos, int n) {
+        auto pairs = [](const uint4 &w, uint64_t (&f)[4]) {
+            const uint32_t x[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-        for (int u = 0; u < N; ++u) {
-            float kf[8];
-            Raw16<T>::unpack(kr[u], kf);
-            x[u] = 0.f;
+            for (int e = 0; e < 4; ++e) f[e] = ptx::pack_f32x2(bf16_lo(x[e]), bf16_hi(x[e]));
+        };
+        float x[KEYS1];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) x[u] = fmaf(qs[e], kf[e], x[u]);
+        for (int u = 0; u < KEYS1; ++u) {
+            uint64_t f[4], d = 0ull;
+            pairs(kr[u], f);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) d = ptx::fma_f32x2(qs[e], f[e], d);
+            float d0, d1;
+            ptx::unpack_f32x2(d, d0, d1);
+            x[u] = d0 + d1;
         }
 #pragma unroll
-        for (int s = LPK / 2; s > 0; s >>= 1)
+        for (int c = KEYS1 / 2, s = LPK / 2; s > 1; c /= 2, s /= 2) {          // halves of the keys change hands
+            const bool up = sub & s;
 #pragma unroll
-            for (int u = 0; u < N; ++u) x[u] += __shfl_xor_sync(0xffffffffu, x[u], s);
-#pragma unroll
-        for (int u = 0; u < N; ++u) {
-            if (ALIBI) x[u] -= slope_l2 * fabsf(q_pos - kpos[u]);
-            if (u >= n) x[u] = -INFINITY;
-            top = fmaxf(top, x[u]);
+            for (int u = 0; u < c; ++u) {
+                const float keep = up ? x[u + c] : x[u], give = up ? x[u] : x[u + c];
+                x[u] = keep + __shfl_xor_sync(0xffffffffu, give, s);
+            }
         }
+        x[0] += __shfl_xor_sync(0xffffffffu, x[0], 1);
+        if (ALIBI) x[0] -= slope_l2 * fabsf(q_pos - kpos);
+        if (sub / 2 >= n) x[0] = -INFINITY;
+        float top = x[0];
+#pragma unroll
+        for (int s = LPK / 2; s > 1; s /= 2) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, s));
         if (top > m) {
             const float r = ex2f(m - top);
             l *= r;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) acc[e] *= r;
+            for (int e = 0; e < 4; ++e) acc[e] = ptx::mul_f32x2(acc[e], ptx::pack_f32x2(r, r));
             m = top;
         }
+        const float p = sub / 2 < n ? ex2f(x[0] - m) : 0.f;
+        l += p;                                                                 // of this lane's keys
 #pragma unroll
-        for (int u = 0; u < N; ++u) {
-            const float p = u < n ? ex2f(x[u] - m) : 0.f;
-            float vf[8];
-            Raw16<T>::unpack(vr[u], vf);
-            l += p;
+        for (int u = 0; u < KEYS1; ++u) {
+            const float w = __shfl_sync(0xffffffffu, p, 2 * u, LPK);
+            uint64_t f[4];
+            pairs(vr[u], f);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) acc[e] = fmaf(p, vf[e], acc[e]);
+            for (int e = 0; e < 4; ++e) acc[e] = ptx::fma_f32x2(ptx::pack_f32x2(w, w), f[e], acc[e]);
         }
     };
 
@@ -329,16 +347,14 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
             const unsigned char *kt = ring + stage * MmaRing<D>::STAGE, *vt = kt + MmaRing<D>::V;
             if (++stage == kMmaStages) stage = 0;
             if constexpr (SINGLE) {                                 // group kg: rows kg, kg + KG, ..
-                constexpr int N = kMmaKeys / KG;
-                uint4 kr[N], vr[N];
-                float kpos[N];
+                uint4 kr[KEYS1], vr[KEYS1];
 #pragma unroll
-                for (int u = 0; u < N; ++u) {
+                for (int u = 0; u < KEYS1; ++u) {
                     const int r = kg + u * KG;
                     kr[u] = *reinterpret_cast<const uint4 *>(kt + r * MmaRing<D>::ROW + ((sub ^ ((r & 1) << 2)) << 4));
                     vr[u] = *reinterpret_cast<const uint4 *>(vt + r * MmaRing<D>::ROW + ((sub ^ (r & 6)) << 4));
-                    kpos[u] = ALIBI ? *reinterpret_cast<const float *>(kt + MmaRing<D>::POS + r * 4) : 0.f;
                 }
+                const float kpos = ALIBI ? *reinterpret_cast<const float *>(kt + MmaRing<D>::POS + (kg + sub / 2 * KG) * 4) : 0.f;
                 attend1(kr, vr, kpos, (min(kMmaKeys, hi_loop - base) - kg + KG - 1) / KG);
             } else {
                 uint4 kr[2][NC], vr[4][NV];
@@ -384,15 +400,19 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
         }
     }
 
-    if (SINGLE && mine_new) {                                // as below; the key is the first group's, the others' value is zero: 0 x Inf is not
+    if (SINGLE && mine_new) {                                // as below; the key is the first group's first, all else zero: 0 x Inf is not
         uint4 *krow = reinterpret_cast<uint4 *>(const_cast<T *>(sm.k[n_seg - 1]) + new_off);
-        uint4 kr[1] = {krow[sub]}, vr[1] = {make_uint4(0u, 0u, 0u, 0u)};
-        if (kg == 0) vr[0] = reinterpret_cast<const uint4 *>(sm.v[n_seg - 1] + new_off)[sub];
-        const float kpos[1] = {0.f};
+        uint4 kr[KEYS1], vr[KEYS1];
+#pragma unroll
+        for (int u = 0; u < KEYS1; ++u) kr[u] = vr[u] = make_uint4(0u, 0u, 0u, 0u);
+        kr[0] = krow[sub];
         rotate1(kr[0]);
         __syncwarp();
-        if (kg == 0) krow[sub] = kr[0];
-        attend1(kr, vr, kpos, kg == 0 ? 1 : 0);
+        if (kg == 0) {
+            krow[sub] = kr[0];
+            vr[0] = reinterpret_cast<const uint4 *>(sm.v[n_seg - 1] + new_off)[sub];
+        }
+        attend1(kr, vr, 0.f, kg == 0 ? 1 : 0);
     } else if (mine_new) {
         // The newest key: rotated, rounded and written back for the later steps, then one more turn with one key.
         uint4 *krow = reinterpret_cast<uint4 *>(const_cast<T *>(sm.k[n_seg - 1]) + new_off);
@@ -424,18 +444,19 @@ decode_mma_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
         m = top;
         l *= r;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) acc[e] *= r;
+        for (int s = 2; s < 32; s <<= 1) l += __shfl_xor_sync(0xffffffffu, l, s);
 #pragma unroll
-        for (int s = LPK; s < 32; s <<= 1) {
-            l += __shfl_xor_sync(0xffffffffu, l, s);
+        for (int e = 0; e < 4; ++e) {
+            float f[2];
+            ptx::unpack_f32x2(ptx::mul_f32x2(acc[e], ptx::pack_f32x2(r, r)), f[0], f[1]);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], s);
+            for (int i = 0; i < 2; ++i) {
+#pragma unroll
+                for (int s = LPK; s < 32; s <<= 1) f[i] += __shfl_xor_sync(0xffffffffu, f[i], s);
+                if (kg == 0) red[warp * PS + sub * 8 + 2 * e + i] = f[i];
+            }
         }
         float *mine = red + warp * PS;
-        if (kg == 0) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) mine[sub * 8 + e] = acc[e];
-        }
         if (lane == 0) { mine[D] = m; mine[D + 1] = l; }
     } else {
         l += __shfl_xor_sync(0xffffffffu, l, 1);
